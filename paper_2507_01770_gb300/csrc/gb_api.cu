@@ -333,6 +333,17 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     if ((e = upload(&d_groups, H.groups.data(), H.groups.size(), A))) return bad(e, "upload program");
     if ((e = upload(&d_dirty, H.dirty.data(), H.dirty.size(), A))) return bad(e, "upload program");
     if ((e = upload(&d_leaves, H.var_leaves.data(), H.var_leaves.size(), A))) return bad(e, "upload program");
+    for (int L = 0; L < GB_BOX_LISTS; L++) {
+        GbBoxTile* d_bt;
+        if ((e = upload(&d_bt, H.box_tiles[L].data(), H.box_tiles[L].size(), A))) return bad(e, "upload program");
+        P.box_tiles[L] = d_bt;
+        P.n_box_tiles[L] = (int)H.box_tiles[L].size();
+    }
+    P.n_tins = (int)H.tins.size();
+    for (const GbSum& S : H.sums) {
+        P.max_terms = std::max(P.max_terms, S.count);
+        P.box_leaves = std::max(P.box_leaves, S.nvar_leaves);
+    }
     if ((e = upload(&d_l, l, (size_t)n, A))) return bad(e, "upload bounds");
     if ((e = upload(&d_u, u, (size_t)n, A))) return bad(e, "upload bounds");
     std::vector<const double*> t64(n_tables > 0 ? n_tables : 1, nullptr);  // kept until the final sync
@@ -1125,7 +1136,7 @@ gb_status gb_eval_boxes(gb_problem* p, const double* d_lo, const double* d_hi, i
     GB_CU(cudaSetDevice(p->device));
     cudaStream_t s = (cudaStream_t)stream;
     float* scratch = nullptr;
-    if (fp32) {
+    if (fp32 && !gb_box_coop(p->P, nbox)) {   // the FP32 copy of the boxes (the cooperative kernel converts as it loads)
         size_t cnt = (size_t)nbox * p->n * 2;
         GB_CU(cudaMallocAsync((void**)&scratch, cnt * sizeof(float), s));
     }

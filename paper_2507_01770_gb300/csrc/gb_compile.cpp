@@ -268,6 +268,25 @@ std::string gb_compile(const gb_node* nd, int32_t nn, int32_t root, const int64_
             P->dirty[(size_t)b * ns + k] = int2{g0, g1};
         }
 
+    // tiles of the from-scratch box evaluation: whole groups, greedily
+    for (int L = 0; L < GB_BOX_LISTS; L++) {
+        const int T = GB_BOX_T[L];
+        std::vector<GbBoxTile>& out = P->box_tiles[L];
+        bool fits = true;
+        for (int k = 0; k < ns && fits; k++) {
+            const GbSum& S = P->sums[k];
+            for (int g = 0; g < S.ngroups && fits; g++) {
+                const GbGroup& G = P->groups[S.group0 + g];
+                fits = G.count <= T;
+                if (g == 0 || out.back().nt + G.count > T) out.push_back(GbBoxTile{k, G.t0, 0, g, 0, 0});
+                out.back().nt += G.count;
+                out.back().ng++;
+                out.back().cmax = std::max(out.back().cmax, G.count);
+            }
+        }
+        if (!fits) out.clear();
+    }
+
     // group ownership for the block-record pool
     {
         const int NG = (int)P->groups.size();

@@ -130,6 +130,18 @@ struct GbJkD {
     uint16_t mask;
 };
 
+// A tile of a from-scratch box evaluation (k_box): consecutive whole groups of
+// one sum, at most GB_BOX_T[list] terms, whose term values are reduced
+// together in shared memory.
+struct GbBoxTile {
+    int32_t sum;
+    int32_t t0, nt;           // term ordinals [t0, t0 + nt) of the sum
+    int32_t g0, ng;           // its groups [g0, g0 + ng) (local indices)
+    int32_t cmax;             // terms of the largest of them
+};
+#define GB_BOX_LISTS 2
+constexpr int GB_BOX_T[GB_BOX_LISTS] = {128, 512};
+
 // Outer VAR leaf: register and coordinate (for the gradient).
 struct GbVarLeaf { int32_t reg, coord; };
 
@@ -170,6 +182,11 @@ struct GbProg {
     int32_t samples;                 // GUB samples per box (0: midpoint; S: diagonal points j / (S + 1))
     int32_t mono_all;                // first-order test on every coordinate
     int32_t any_prod;                // some reduction is an IPROD
+    // from-scratch box evaluation: tiles of every sum's terms, one list per tile size
+    const GbBoxTile* box_tiles[GB_BOX_LISTS];
+    int32_t n_box_tiles[GB_BOX_LISTS];   // 0: a group exceeds the list's tile size
+    int32_t n_tins, max_terms, box_leaves;   // template instructions, terms of the longest sum, IVAR leaves of
+                                     //    the widest template
 };
 
 // Host-side compiled program (arrays in host memory before upload).
@@ -186,6 +203,7 @@ struct GbHostProg {
     std::vector<int2> dirty;
     std::vector<GbVarLeaf> var_leaves;
     int64_t ops_eval = 0, ops_mid = 0;   // static directed-op counts (see gb_compile.cpp)
+    std::vector<GbBoxTile> box_tiles[GB_BOX_LISTS];
     // block records: group ownership (a group lives in the record of its lowest touched block)
     int32_t GPB = 1, span = 0;
     std::vector<int2> gown;

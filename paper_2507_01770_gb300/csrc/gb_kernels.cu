@@ -1938,9 +1938,9 @@ cudaError_t gb_launch_output(const GbEntries& E, long long count, const GbPool& 
     return cudaGetLastError();
 }
 
-cudaError_t gb_launch_eval_boxes(const GbProg& P, const double* lo, const double* hi, float* scratch32,
-                                 long long nbox, int blk, int fp32, double* F, double* Fmid, double* G, int* mono,
-                                 cudaStream_t s) {
+cudaError_t gb_launch_eval_boxes_thread(const GbProg& P, const double* lo, const double* hi, float* scratch32,
+                                        long long nbox, int blk, int fp32, double* F, double* Fmid, double* G,
+                                        int* mono, cudaStream_t s) {
     float* lo32 = nullptr;
     float* hi32 = nullptr;
     if (fp32) {

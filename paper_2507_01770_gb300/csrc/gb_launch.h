@@ -215,6 +215,12 @@ cudaError_t gb_launch_output(const GbEntries& E, long long count, const GbPool& 
 cudaError_t gb_launch_eval_boxes(const GbProg& P, const double* lo, const double* hi, float* scratch32,
                                  long long nbox, int blk, int fp32, double* F, double* Fmid, double* G,
                                  int* mono, cudaStream_t s);
+// The same, one thread per box (any program; scratch32 as above).
+cudaError_t gb_launch_eval_boxes_thread(const GbProg& P, const double* lo, const double* hi, float* scratch32,
+                                        long long nbox, int blk, int fp32, double* F, double* Fmid, double* G,
+                                        int* mono, cudaStream_t s);
+// 1: gb_launch_eval_boxes evaluates nbox boxes with the cooperative kernel, which needs no scratch32.
+int gb_box_coop(const GbProg& P, long long nbox);
 cudaError_t gb_launch_peak(int which, int iters, int blocks, void* sink, cudaStream_t s);
 long long gb_launches_so_far();
 // Streaming multiprocessors of the current device (queried once per device).
