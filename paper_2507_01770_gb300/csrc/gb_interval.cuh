@@ -83,6 +83,8 @@ __device__ __forceinline__ bool same_value(double x, double y) {
     unsigned long long a = (unsigned long long)__double_as_longlong(x), b = (unsigned long long)__double_as_longlong(y);
     return (a == b && (a & 0x7fffffffffffffffULL) <= 0x7ff0000000000000ULL) || ((a | b) << 1) == 0;
 }
+__device__ __forceinline__ bool zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool zero_bits(float x) { return (__float_as_int(x) << 1) == 0; }
 __device__ __forceinline__ bool is_one(double x) { return __double_as_longlong(x) == 0x3ff0000000000000LL; }
 __device__ __forceinline__ bool gt_zero(float x) {
     int b = __float_as_int(x);
@@ -166,31 +168,27 @@ template <typename T> __device__ __forceinline__ T pmul_ru(T a, T b) {
 // Eq. 5, sign-case form.  P: lo >= +0 (sign bit clear), N: hi has its sign
 // bit set, M: otherwise.  -0 endpoints are classified by sign bit; every
 // case still selects the products that attain the extremes because a zero
-// endpoint contributes a zero product.
+// endpoint contributes a zero product.  The operands are selected on the
+// integer pipe and the two products formed once for all lanes (a warp's FP64
+// instruction holds the pipe ~16 clocks whatever its active lanes, so one
+// product per case would cost one slot per case present in the warp); only
+// M x M, which needs all four products, adds a branch.
 template <typename I> __device__ __forceinline__ I imul(I x, I y) {
     typedef decltype(x.lo) T;
-    T a = x.lo, b = x.hi, c = y.lo, d = y.hi;
+    const T a = x.lo, b = x.hi, c = y.lo, d = y.hi;
     I r;
     if (__builtin_expect(any_inf(a, b, c, d), 0)) {
         r.lo = fmin(fmin(pmul_rd(a, c), pmul_rd(a, d)), fmin(pmul_rd(b, c), pmul_rd(b, d)));
         r.hi = fmax(fmax(pmul_ru(a, c), pmul_ru(a, d)), fmax(pmul_ru(b, c), pmul_ru(b, d)));
         return r;
     }
-    int cx = !sgn(a) ? 0 : (sgn(b) ? 1 : 2);
-    int cy = !sgn(c) ? 0 : (sgn(d) ? 1 : 2);
-    switch (cx * 3 + cy) {
-    case 0: r.lo = mul_rd(a, c); r.hi = mul_ru(b, d); break;  // P P
-    case 1: r.lo = mul_rd(b, c); r.hi = mul_ru(a, d); break;  // P N
-    case 2: r.lo = mul_rd(b, c); r.hi = mul_ru(b, d); break;  // P M
-    case 3: r.lo = mul_rd(a, d); r.hi = mul_ru(b, c); break;  // N P
-    case 4: r.lo = mul_rd(b, d); r.hi = mul_ru(a, c); break;  // N N
-    case 5: r.lo = mul_rd(a, d); r.hi = mul_ru(a, c); break;  // N M
-    case 6: r.lo = mul_rd(a, d); r.hi = mul_ru(b, d); break;  // M P
-    case 7: r.lo = mul_rd(b, c); r.hi = mul_ru(a, c); break;  // M N
-    default:                                                   // M M
-        r.lo = fmin(mul_rd(a, d), mul_rd(b, c));
-        r.hi = fmax(mul_ru(a, c), mul_ru(b, d));
-        break;
+    const bool px = !sgn(a), nx = sgn(a) && sgn(b), mx = sgn(a) && !sgn(b);
+    const bool ny = sgn(c) && sgn(d), my = sgn(c) && !sgn(d);
+    r.lo = mul_rd((ny || (px && my)) ? b : a, (nx || (mx && !ny)) ? d : c);
+    r.hi = mul_ru((ny || (nx && my)) ? a : b, (nx || (mx && ny)) ? c : d);
+    if (mx && my) {   // [a d, b d] so far
+        r.lo = fmin(r.lo, mul_rd(b, c));
+        r.hi = fmax(mul_ru(a, c), r.hi);
     }
     return r;
 }
@@ -222,8 +220,8 @@ template <typename I> __device__ __forceinline__ I isqr(I x) {
 template <typename I> __device__ __forceinline__ I iscale(I x, decltype(x.lo) c) {
     typedef decltype(x.lo) T;
     I r;
-    if (c == (T)0) { r.lo = r.hi = (T)0; return r; }
-    if (c > (T)0) { r.lo = mul_rd(x.lo, c); r.hi = mul_ru(x.hi, c); }
+    if (zero_bits(c)) { r.lo = r.hi = (T)0; return r; }
+    if (!sgn(c)) { r.lo = mul_rd(x.lo, c); r.hi = mul_ru(x.hi, c); }
     else { r.lo = mul_rd(x.hi, c); r.hi = mul_ru(x.lo, c); }
     return r;
 }
@@ -232,7 +230,7 @@ template <typename I> __device__ __forceinline__ I iscale(I x, decltype(x.lo) c)
 template <typename I> __device__ __forceinline__ I ircp(I y) {
     typedef decltype(y.lo) T;
     I r;
-    if (y.lo > (T)0 || y.hi < (T)0) { r.lo = rcp_rd(y.hi); r.hi = rcp_ru(y.lo); }
+    if (gt_zero(y.lo) || lt_zero(y.hi)) { r.lo = rcp_rd(y.hi); r.hi = rcp_ru(y.lo); }
     else { r.lo = -inf_v<T>(); r.hi = inf_v<T>(); }
     return r;
 }
