@@ -104,6 +104,8 @@ struct gb_problem {
     GbSplit sp{};
     GbTabs tabs{};
     bool use_tabs = false;
+    GbPaper paper{};
+    bool use_paper = false;        // paper mode from per-parent tables
     GbState* st = nullptr;         // device
     GbState* st_host = nullptr;    // pinned host
     unsigned* out_list = nullptr;
@@ -195,8 +197,10 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     if (opt.pool_mode < 0 || opt.pool_mode > 2) return fail(GB_E_INVALID, "pool_mode must be 0, 1 or 2");
     if (opt.eval_mode < 0 || opt.eval_mode > 4) return fail(GB_E_INVALID, "eval_mode must be 0 .. 4");
     if (opt.samples < 0 || opt.samples > 64) return fail(GB_E_INVALID, "samples must be 0 .. 64");
-    if (opt.samples > 0 || opt.mono_all) {   // paper mode: full evaluations in the interpreter
+    bool paper_tabs = false;
+    if (opt.samples > 0 || opt.mono_all) {   // paper mode: its own tables (eval_mode 0, where they fit) or the interpreter
         if (opt.eval_mode >= 2) return fail(GB_E_INVALID, "samples > 0 and mono_all need eval_mode 0 or 1");
+        paper_tabs = opt.eval_mode == 0 && !opt.fp32_prefilter;
         opt.eval_mode = 1;
     }
     if (opt.max_records < 0) return fail(GB_E_INVALID, "max_records must be >= 0");
@@ -253,6 +257,25 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             gb_build_tables(&p->hp, opt.split_m, opt.split_d, sbits);
             if (!p->hp.tab_ok || (double)K * p->hp.max_srows * per_row <= budget) break;
         }
+    }
+    // paper mode: tables when a parent has at least 16 children, they fit
+    // max(64 MiB, pool budget / 8) for all parents of a generation and the
+    // objective's outer expression allows them
+    if (paper_tabs) {
+        const int flog2 = opt.split_d * mshift;
+        const long long K = std::max(1LL, (long long)opt.max_children >> flog2);
+        const int nk = 1 + (opt.samples > 0 ? opt.samples : 1);
+        const double budget = std::max(64.0 * (1 << 20), (double)opt.pool_bytes / 8.0);
+        paper_tabs = flog2 >= 4 && K <= 65535;
+        for (int sbits = GB_TAB_SBITS; paper_tabs; sbits--) {
+            gb_build_tables(&p->hp, opt.split_m, opt.split_d, sbits, true);
+            const GbHostProg& T = p->hp;
+            const double per = 16.0 * (nk * ((double)T.max_arows + T.max_srows + T.max_hrows + T.tree_nodes) +
+                                       (double)T.max_arows * T.max_leaves + T.max_drows);
+            if (T.tab_ok && K * per <= budget) break;
+            if (!T.tab_ok || sbits == 0) paper_tabs = false;
+        }
+        if (!paper_tabs) p->hp.tab_ok = 0;
     }
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev <= opt.device || opt.device < 0) {
@@ -576,6 +599,63 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             p->use_tabs = true;
         }
     }
+    if (paper_tabs) {
+        const GbHostProg& Hh = p->hp;
+        GbPaper& T = p->paper;
+        int32_t* d_spc;
+        GbSplitPos* d_sps;
+        GbDTerm* d_dt;
+        int2* d_jk;
+        GbContrib* d_cb;
+        GbJkD* d_jkd;
+        GbSeg* d_segs;
+        GbPaperSum* d_ps;
+        GbHoistPos* d_hp;
+        int32_t* d_hn;
+        GbOIns* d_op;
+        if ((e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||
+            (e = upload(&d_sps, Hh.sps.data(), Hh.sps.size(), A)) ||
+            (e = upload(&d_dt, Hh.dterms.data(), Hh.dterms.size(), A)) ||
+            (e = upload(&d_jk, Hh.jk.data(), Hh.jk.size(), A)) ||
+            (e = upload(&d_cb, Hh.contribs.data(), Hh.contribs.size(), A)) ||
+            (e = upload(&d_jkd, Hh.jkd.data(), Hh.jkd.size(), A)) ||
+            (e = upload(&d_segs, Hh.segs.data(), Hh.segs.size(), A)) ||
+            (e = upload(&d_ps, Hh.psums.data(), Hh.psums.size(), A)) ||
+            (e = upload(&d_hp, Hh.hoist_pos.data(), Hh.hoist_pos.size(), A)) ||
+            (e = upload(&d_hn, Hh.hoist_node.data(), Hh.hoist_node.size(), A)) ||
+            (e = upload(&d_op, Hh.oprog.data(), Hh.oprog.size(), A)))
+            return bad(e, "upload table layouts");
+        P.m = Hh.m;
+        P.mshift = Hh.mshift;
+        P.max_rows = Hh.max_rows;
+        P.sp_of_cyc = d_spc;
+        P.sps = d_sps;
+        P.dterms = d_dt;
+        P.jk = d_jk;
+        P.contribs = d_cb;
+        P.jkd = d_jkd;
+        P.segs = d_segs;
+        T.nk = 1 + (opt.samples > 0 ? opt.samples : 1);
+        T.n_hoist = (int)Hh.hoist_node.size();
+        T.n_oprog = (int)Hh.oprog.size();
+        T.arows = std::max(1, Hh.max_arows);
+        T.srows = std::max(1, Hh.max_srows);
+        T.drows = std::max(1, Hh.max_drows);
+        T.hrows = std::max(1, Hh.max_hrows);
+        T.tree_nodes = std::max(1, Hh.tree_nodes);
+        T.max_leaves = std::max(1, Hh.max_leaves);
+        T.psums = d_ps;
+        T.hoist_pos = d_hp;
+        T.hoist_node = d_hn;
+        T.oprog = d_op;
+        T.indep = Hh.indep;
+        const size_t kk = K * (size_t)T.nk;
+        if ((e = alloc(&T.tv, kk * T.arows, A)) || (e = alloc(&T.ts, kk * T.srows, A)) ||
+            (e = alloc(&T.nd, kk * T.tree_nodes, A)) || (e = alloc(&T.hv, kk * T.hrows, A)) ||
+            (e = alloc(&T.tl, K * (size_t)T.arows * T.max_leaves, A)) || (e = alloc(&T.td, K * (size_t)T.drows, A)))
+            return bad(e, "allocate paper-mode tables");
+        p->use_paper = true;
+    }
     p->G.K = p->K;
     p->G.flog2 = d * mshift;
     p->G.fp32 = fp32;
@@ -711,7 +791,7 @@ static cudaError_t capture_graphs(gb_problem* p) {
             long long n1 = 0;
             e = gb_launch_generation(p->P, p->pool, p->E[b], p->E[1 - b], p->par, p->ch, p->sp, p->sc,
                                      p->use_tabs ? &p->tabs : nullptr, p->G, p->cap, p->Cmax, p->st, s, nullptr,
-                                     &n1, 0, &p->fork);
+                                     &n1, 0, &p->fork, p->use_paper ? &p->paper : nullptr);
             nl += n1;
         }
         cudaError_t e2 = cudaStreamEndCapture(s, &g);
@@ -784,7 +864,7 @@ __attribute__((visibility("hidden"))) int solve_advance(gb_problem* p, bool bloc
         long long nl = 0;
         e = gb_launch_generation(p->P, p->pool, p->E[cur], p->E[1 - cur], p->par, p->ch, p->sp, p->sc,
                                  p->use_tabs ? &p->tabs : nullptr, p->G, p->cap, p->Cmax, p->st, s, &p->ev[2], &nl, 0,
-                                 &p->fork);
+                                 &p->fork, p->use_paper ? &p->paper : nullptr);
         if (e != cudaSuccess) return stop(cuda_fail(e, "generation launch"));
         R.timed64 = true;
         R.timed32 = p->opt.fp32_prefilter != 0;

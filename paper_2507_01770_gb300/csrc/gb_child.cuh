@@ -186,6 +186,41 @@ __device__ __forceinline__ void warp_group(const GbProg& P, const GbSplitPos& SP
         for (int t = 0; t < NV; t++) out[t] = tr[t].result();
 }
 
+// Path of sum k's pairwise group tree above its dirty groups [dr.x, dr.y)
+// (values cur[0 .. dr.y - dr.x)), with the parent's tree nodes (node(i),
+// level-major) for the clean siblings; returns the sum (PROD: the product).
+template <bool PROD = false, typename I, typename N>
+__device__ __forceinline__ I tab_path(const GbSum& S, int2 dr, I* cur, N node, int& ops) {
+    I tmp[GB_TAB_MAX_DIRTY];
+    if (S.ngroups == 0 || S.nnodes <= 0) {
+        I z;
+        z.lo = PROD ? 1 : 0;
+        z.hi = PROD ? 1 : 0;
+        return z;
+    }
+    int lo = dr.x, hi = dr.y, off = 0;
+    if (lo >= hi) return node(S.nnodes - 1);   // no dirty group: the parent's root
+    for (int mL = S.ngroups; mL > 1; mL = (mL + 1) / 2) {
+        const int nlo = lo >> 1, nhi = ((hi - 1) >> 1) + 1;
+        for (int q = nlo; q < nhi; q++) {
+            const int a = 2 * q;
+            I left = (a >= lo && a < hi) ? cur[a - lo] : node(off + a);
+            I v = left;
+            if (a + 1 < mL) {
+                I right = (a + 1 >= lo && a + 1 < hi) ? cur[a + 1 - lo] : node(off + a + 1);
+                v = Tree<I, PROD>::comb(left, right);
+                ops += PROD ? 8 : 2;
+            }
+            tmp[q - nlo] = v;
+        }
+        for (int q = 0; q < nhi - nlo; q++) cur[q] = tmp[q];
+        lo = nlo;
+        hi = nhi;
+        off += mL;
+    }
+    return cur[0];
+}
+
 // A block's arrival at a grid-wide counter of n blocks; every thread calls
 // it and gets true in the last block to arrive.  The block's writes before
 // the call (any thread's: the barrier orders them before thread 0's release

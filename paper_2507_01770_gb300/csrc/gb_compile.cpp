@@ -340,7 +340,64 @@ std::string gb_compile(const gb_node* nd, int32_t nn, int32_t root, const int64_
 }
 
 // Per-split-position layouts of the per-parent term tables (see GbSplitPos).
-void gb_build_tables(GbHostProg* P, int m, int d, int sbits) {
+// Outer values that no reduction enters (coordinates and constants only) and
+// the program over them and the reductions that a child runs.  false: too
+// many of them, or one depends on more digits than a table holds.
+static bool build_hoists(GbHostProg* P, std::vector<std::vector<int>>* vars) {
+    const int no = (int)P->outer.size();
+    std::vector<char> dep(no, 0);
+    std::vector<std::vector<int>> coords(no);
+    P->indep = 0;
+    P->oprog.clear();
+    P->hoist_node.clear();
+    vars->clear();
+    auto binary = [](int op) { return op == D_ADD || op == D_SUB || op == D_MUL || op == D_DIV; };
+    auto leaf = [](int op) { return op == D_CONST || op == D_PI || op == D_EULER || op == D_VAR || op == D_ISUMV; };
+    for (int t = 0; t < no; t++) {
+        const GbIns& I = P->outer[t];
+        if (I.op == D_ISUMV) dep[t] = 1;
+        if (I.op == D_VAR) coords[t].push_back(I.aux);
+        if (!leaf(I.op)) {
+            dep[t] = dep[I.a] || (binary(I.op) && dep[I.b]);
+            coords[t] = coords[I.a];
+            if (binary(I.op)) coords[t].insert(coords[t].end(), coords[I.b].begin(), coords[I.b].end());
+        }
+        if (!dep[t]) P->indep |= 1u << t;
+    }
+    auto slot = [&](int reg, bool rcp) {
+        const int key = reg | (rcp ? 1 << 16 : 0);
+        for (size_t h = 0; h < P->hoist_node.size(); h++)
+            if (P->hoist_node[h] == key) return (int)h;
+        P->hoist_node.push_back(key);
+        vars->push_back(coords[reg]);
+        return (int)P->hoist_node.size() - 1;
+    };
+    if (no == 0 || !dep[P->outer_root]) return false;   // no reduction reaches the root: nothing to tabulate
+    for (int t = 0; t < no; t++) {
+        const GbIns& I = P->outer[t];
+        if (!dep[t]) continue;
+        GbOIns o{};
+        o.op = I.op;
+        o.dst = (uint8_t)t;
+        o.a = I.a;
+        o.b = I.b;
+        o.c = I.c;
+        if (I.op == D_ISUMV) {
+            o.a = (uint8_t)I.aux;
+        } else {
+            if (!dep[I.a]) o.a = (uint8_t)slot(I.a, false), o.ha = 1;
+            if (binary(I.op) && !dep[I.b]) {
+                if (I.op == D_DIV) o.op = D_MUL;
+                o.b = (uint8_t)slot(I.b, I.op == D_DIV);
+                o.hb = 1;
+            }
+        }
+        P->oprog.push_back(o);
+    }
+    return P->hoist_node.size() <= GB_MAX_HOIST;
+}
+
+void gb_build_tables(GbHostProg* P, int m, int d, int sbits, bool paper) {
     P->tab_ok = 0;
     P->m = m;
     P->mshift = m == 2 ? 1 : 2;
@@ -355,7 +412,15 @@ void gb_build_tables(GbHostProg* P, int m, int d, int sbits) {
     P->max_srows = 0;
     P->max_nseg = 0;
     P->max_rows = P->max_dterm = 0;
-    if (P->any_prod) return;   // the tables hold sums only: products run on the interpreter
+    if (P->any_prod && !paper) return;   // these tables hold sums only: products run on the interpreter
+    std::vector<std::vector<int>> hvars;
+    P->psums.clear();
+    P->hoist_pos.clear();
+    P->max_arows = P->max_hrows = 0;
+    if (paper && !build_hoists(P, &hvars)) return;
+    int reach = 0;   // widest template's coordinate range
+    for (const GbSum& S : P->sums)
+        if (S.has_var) reach = std::max(reach, S.off_max - S.off_min);
     const int n = P->n, B = P->B, ns = (int)P->sums.size();
     int node = 0, max_leaves = 0;
     for (GbSum& S : P->sums) {
@@ -466,16 +531,76 @@ void gb_build_tables(GbHostProg* P, int m, int d, int sbits) {
             if (rows > GB_TAB_MAX_ROWS) return;
             P->max_rows = std::max(P->max_rows, rows);
             P->max_dterm = std::max(P->max_dterm, sp.ndterm);
-            // gradient contributions of every block coordinate, per sum, in
-            // ascending term and ascending leaf order
-            for (int j = bs; j < be; j++) {
+            sp.ja = bs;
+            sp.jb = be;
+            // the dterms of each sum in ascending term order, for the partials
+            std::vector<std::vector<int>> order(ns);
+            for (int q = 0; q < sp.ndterm; q++) order[P->dterms[sp.dterm0 + q].sum].push_back(q);
+            if (paper) {
+                sp.ja = std::max(0, bs - reach);
+                sp.jb = std::min(n, be + reach);
+                for (int k = 0; k < ns; k++) {
+                    const GbSum& S = P->sums[k];
+                    const int2 dr = P->dirty[(size_t)b * ns + k];
+                    GbPaperSum ps{0, 0, order[k].empty() ? 0 : order[k][0], -1};
+                    if (dr.y > dr.x) {
+                        ps.t_lo = P->groups[S.group0 + dr.x].t0;
+                        const GbGroup& Z = P->groups[S.group0 + dr.y - 1];
+                        ps.t_hi = Z.t0 + Z.count;
+                    }
+                    auto add = [&](int t) {
+                        GbDTerm D{};
+                        D.sum = (int16_t)k;
+                        D.group = -1;
+                        D.term = t;
+                        D.row = rows++;
+                        P->dterms.push_back(D);
+                        sp.nx++;
+                        return (int)P->dterms.size() - 1 - sp.dterm0;
+                    };
+                    if (S.prod) {   // every other term's value
+                        if (rows + S.count > GB_TAB_MAX_ROWS) return;
+                        ps.x0 = sp.ndterm + sp.nx;
+                        for (int t = 0; t < S.count; t++)
+                            if (t < ps.t_lo || t >= ps.t_hi) add(t);
+                    } else if (S.has_var) {   // the clean terms that touch [ja, jb)
+                        std::vector<int> before, after;
+                        for (int t = 0; t < S.count; t++) {
+                            const int i = S.first + t * S.step;
+                            if (i + S.off_max < sp.ja || (t >= ps.t_lo && t < ps.t_hi)) continue;
+                            if (i + S.off_min >= sp.jb) break;
+                            (t < ps.t_lo ? before : after).push_back(add(t));
+                        }
+                        order[k].insert(order[k].begin(), before.begin(), before.end());
+                        order[k].insert(order[k].end(), after.begin(), after.end());
+                    }
+                    P->psums.push_back(ps);
+                }
+                if (rows > GB_TAB_MAX_ROWS) return;
+                P->max_arows = std::max(P->max_arows, rows);
+                for (const std::vector<int>& hv : hvars) {
+                    int lo = 1 << 30, hi = 0;
+                    for (int j : hv)
+                        if (j >= c && j < c + dd) {
+                            lo = std::min(lo, (j - c) * P->mshift);
+                            hi = std::max(hi, (j - c + 1) * P->mshift);
+                        }
+                    if (lo > hi) lo = hi = 0;
+                    if (hi - lo > GB_TAB_SBITS) return;
+                    P->hoist_pos.push_back(GbHoistPos{sp.hrows, (int16_t)lo, (uint16_t)((1u << (hi - lo)) - 1u)});
+                    sp.hrows += 1 << (hi - lo);
+                }
+                P->max_hrows = std::max(P->max_hrows, sp.hrows);
+            }
+            // gradient contributions of every block coordinate (paper mode: of
+            // [ja, jb)), per sum, in ascending term and ascending leaf order
+            for (int j = sp.ja; j < sp.jb; j++) {
                 for (int k = 0; k < ns; k++) {
                     const GbSum& S = P->sums[k];
                     const int start = (int)P->contribs.size();
-                    if (S.has_var) {
-                        for (int q = 0; q < sp.ndterm; q++) {
+                    if (S.has_var && !S.prod) {
+                        for (int q : order[k]) {
                             const GbDTerm& D = P->dterms[sp.dterm0 + q];
-                            if (D.sum != k) continue;
                             const int i = S.first + D.term * S.step;
                             int leaf = 0;
                             for (int t = S.ins0; t < S.ins0 + S.nins; t++) {

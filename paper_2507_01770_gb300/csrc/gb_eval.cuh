@@ -16,6 +16,8 @@
 //    [1, 1]; leaf adjoints are accumulated per coordinate in ascending term
 //    and leaf order, then multiplied by the sum's outer adjoint.
 #pragma once
+#include <type_traits>
+
 #include "gb_internal.h"
 #include "gb_interval.cuh"
 
@@ -482,42 +484,48 @@ __device__ __noinline__ typename Prec<T>::I prod_term_seed(const GbProg& P, int 
     return tree_item_adjoint(a, G.count, tt - G.t0, tval, ops);
 }
 
+// Value of one outer instruction from the registers before it.
+template <typename T, typename V>
+__device__ __forceinline__ typename Prec<T>::I outer_ins(const GbIns& in, const V& X, const typename Prec<T>::I* sums,
+                                                          const typename Prec<T>::I* O) {
+    typename Prec<T>::I v;
+    switch (in.op) {
+    case D_CONST: v = Prec<T>::cst(in); break;
+    case D_PI: v = pi_iv((T)0); break;
+    case D_EULER: v = e_iv((T)0); break;
+    case D_VAR: v = X.get(in.aux); break;
+    case D_ISUMV: v = sums[in.aux]; break;
+    case D_ADD: v = iadd(O[in.a], O[in.b]); break;
+    case D_SUB: v = isub(O[in.a], O[in.b]); break;
+    case D_MUL: v = imul(O[in.a], O[in.b]); break;
+    case D_NEG: v = ineg(O[in.a]); break;
+    case D_SQR: v = isqr(O[in.a]); break;
+    case D_DIV:
+    case D_SQRT:
+    case D_EXP:
+    case D_SIN:
+    case D_STEP:
+    case D_COS: v = slow_fwd(in.op, O[in.a], O[in.b]); break;
+    case D_SCALE:
+        if (in.clo32 == in.chi32 || sizeof(T) == 8)
+            v = iscale(O[in.a], sizeof(T) == 8 ? (T)in.c : (T)in.clo32);
+        else
+            v = imul(O[in.a], mk<T>((T)in.clo32, (T)in.chi32));
+        break;
+    default: v.lo = 0; v.hi = 0; break;
+    }
+    return v;
+}
+
 // Outer forward pass; O receives all outer registers, returns F.
 template <typename T, typename V>
 __device__ __forceinline__ typename Prec<T>::I outer_fwd(const GbProg& P, const V& X,
                                                           const typename Prec<T>::I* sums,
                                                           typename Prec<T>::I* O, int& ops) {
-    typedef typename Prec<T>::I I;
     for (int t = 0; t < P.n_outer; t++) {
-        GbIns in = P.outer[t];
+        const GbIns in = P.outer[t];
         ops += in.pad & 0xff;
-        I v;
-        switch (in.op) {
-        case D_CONST: v = Prec<T>::cst(in); break;
-        case D_PI: v = pi_iv((T)0); break;
-        case D_EULER: v = e_iv((T)0); break;
-        case D_VAR: v = X.get(in.aux); break;
-        case D_ISUMV: v = sums[in.aux]; break;
-        case D_ADD: v = iadd(O[in.a], O[in.b]); break;
-        case D_SUB: v = isub(O[in.a], O[in.b]); break;
-        case D_MUL: v = imul(O[in.a], O[in.b]); break;
-        case D_NEG: v = ineg(O[in.a]); break;
-        case D_SQR: v = isqr(O[in.a]); break;
-        case D_DIV:
-        case D_SQRT:
-        case D_EXP:
-        case D_SIN:
-        case D_STEP:
-        case D_COS: v = slow_fwd(in.op, O[in.a], O[in.b]); break;
-        case D_SCALE:
-            if (in.clo32 == in.chi32 || sizeof(T) == 8)
-                v = iscale(O[in.a], sizeof(T) == 8 ? (T)in.c : (T)in.clo32);
-            else
-                v = imul(O[in.a], mk<T>((T)in.clo32, (T)in.chi32));
-            break;
-        default: v.lo = 0; v.hi = 0; break;
-        }
-        O[t] = v;
+        O[t] = outer_ins<T>(in, X, sums, O);
     }
     return O[P.outer_root];
 }
@@ -528,12 +536,14 @@ __device__ __forceinline__ typename Prec<T>::I outer_fwd(const GbProg& P, const 
 // receives the partials of the block.  Needs the outer registers O of the
 // forward pass.  A product's term templates are seeded with the term's
 // adjoint in the product (prod_term_seed; group values from gcache except
-// the groups dirty for block dblk, all recomputed when gcache is null).
-template <bool PR, typename T, typename V, typename C>
+// the groups dirty for block dblk, all recomputed when gcache is null), or by
+// seeder(k, term ordinal) when it is not a null pointer.
+template <bool PR, typename T, typename V, typename C, typename Seed = const int*>
 __device__ __forceinline__ bool block_mono(const GbProg& P, int blk, const V& X, const View<double>& X64,
                                            const typename Prec<T>::I* O, typename Prec<T>::I* OA,
                                            typename Prec<T>::I* R, typename Prec<T>::I* RA,
-                                           double* Gout, const CacheRef<C>* gcache, int dblk, int& ops) {
+                                           double* Gout, const CacheRef<C>* gcache, int dblk, int& ops,
+                                           const Seed& seeder = nullptr) {
     typedef typename Prec<T>::I I;
     // outer adjoints
     for (int t = 0; t < P.n_outer; t++) OA[t] = mk<T>((T)0, (T)0);
@@ -567,7 +577,12 @@ __device__ __forceinline__ bool block_mono(const GbProg& P, int blk, const V& X,
                 int i = S.first + cur[k] * S.step;
                 I seed = mk<T>((T)1, (T)1);
                 if constexpr (PR) {
-                    if (S.prod) seed = prod_term_seed<T>(P, k, cur[k], X, gcache, dblk, R, ops);
+                    if (S.prod) {
+                        if constexpr (std::is_pointer<Seed>::value)
+                            seed = prod_term_seed<T>(P, k, cur[k], X, gcache, dblk, R, ops);
+                        else
+                            seed = seeder(k, cur[k]);
+                    }
                 }
                 term_fwd<T>(P, S, i, X, R, ops);
                 for (int t = 0; t < S.nins; t++) RA[t] = mk<T>((T)0, (T)0);

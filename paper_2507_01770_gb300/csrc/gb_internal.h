@@ -84,7 +84,29 @@ struct GbSplitPos {
     int32_t drows;            // rows of the per-parent partial tables
     int32_t seg0, nseg;       // segments [seg0, seg0 + nseg) of the dirty groups' term trees
     int32_t srows;            // rows of the per-parent segment tables
-    int32_t pad;
+    // paper mode: terms [dterm0 + ndterm, + nx) that no split coordinate touches but whose adjoints (sums) or
+    // values (products) the first-order test needs, one table row each from row tab_entries on; the partials
+    // tabulated are those of coordinates [ja, jb), the block and a term's reach beyond it
+    int32_t nx, ja, jb;
+    int32_t hrows;            // rows of the hoisted outer values
+};
+// Paper mode, per (split position, reduction): its dirty terms [t_lo, t_hi)
+// are dterms d0 ..., the other terms of a product, in order, dterms x0 ...
+// (all relative to dterm0; x0 < 0: not tabulated).
+struct GbPaperSum { int32_t t_lo, t_hi, d0, x0; };
+// Paper mode, per (split position, hoisted outer value): its row for a child
+// index r is base + ((r >> shift) & mask).
+#define GB_MAX_HOIST 16
+struct GbHoistPos { int32_t base; int16_t shift; uint16_t mask; };
+// The outer expression as a child evaluates it: the nodes that depend on a
+// reduction, in order; operands are outer registers or (ha, hb) hoisted
+// values -- nodes that depend on no reduction, tabulated per parent; a
+// division by such a node multiplies by its hoisted reciprocal (Eq. 6).
+struct GbOIns {
+    uint8_t op, dst, a, b;
+    uint8_t ha, hb;
+    uint16_t pad;
+    double c;
 };
 // A segment of a dirty group's term tree: the aligned block of 2^level terms
 // starting at dirty term dterm (relative to the split position's dterm0),
@@ -204,6 +226,13 @@ struct GbHostProg {
     std::vector<GbVarLeaf> var_leaves;
     int64_t ops_eval = 0, ops_mid = 0;   // static directed-op counts (see gb_compile.cpp)
     std::vector<GbBoxTile> box_tiles[GB_BOX_LISTS];
+    // paper mode tables
+    std::vector<GbPaperSum> psums;       // [split positions][n_sum]
+    std::vector<GbHoistPos> hoist_pos;   // [split positions][hoists]
+    std::vector<int32_t> hoist_node;     // outer register, | 1 << 16: its reciprocal
+    std::vector<GbOIns> oprog;
+    int32_t max_arows = 0, max_hrows = 0;
+    uint32_t indep = 0;                  // outer registers that depend on no reduction
     // block records: group ownership (a group lives in the record of its lowest touched block)
     int32_t GPB = 1, span = 0;
     std::vector<int2> gown;
@@ -223,7 +252,8 @@ struct GbHostProg {
 // Builds the per-split-position table layouts for pieces m and split width d;
 // leaves tab_ok = 0 when a layout exceeds the table limits.
 // sbits: largest digit-bit count of a tabulated term-tree segment (<= GB_TAB_SBITS).
-void gb_build_tables(GbHostProg* P, int m, int d, int sbits = GB_TAB_SBITS);
+// paper: layouts of the paper-mode tables (products included; see GbSplitPos).
+void gb_build_tables(GbHostProg* P, int m, int d, int sbits = GB_TAB_SBITS, bool paper = false);
 // Compiles and validates a DAG; returns an empty string or an error message.
 std::string gb_compile(const gb_node* nodes, int32_t nn, int32_t root, const int64_t* tlen,
                        int32_t ntab, int32_t n, int32_t B, GbHostProg* out);

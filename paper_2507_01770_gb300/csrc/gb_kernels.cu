@@ -23,6 +23,7 @@
 #include "gb_child.cuh"
 #include "gb_eval.cuh"
 #include "gb_launch.h"
+#include "gb_paper.cuh"
 
 using namespace gb;
 
@@ -1062,12 +1063,14 @@ __device__ __forceinline__ void tab_dirty_groups(const GbProg& P, const GbPool& 
 // ---------------------------------------------------------------------------
 // Survivors into free slots: coordinates, FP32 shadow, group caches (dirty
 // groups recomputed, the rest copied from the parent), pool entry.
-template <bool PR, bool TAB>
+// TAB: 0 the interpreter, 1 the term tables, 2 the paper-mode tables.
+template <bool PR, int TAB>
 __device__ __forceinline__ void materialize_one(const GbProg& P, const GbPool& pool, const GbParents& par,
                                                 const GbChildren& ch, const GbSplit& sp, const GbEntries& En,
                                                 double tol_x, const GbState* st, long long s, int lane,
-                                                const GbTabs& Tb, double2* shF, double2* shM, float2* sh32) {
-    constexpr bool tab = TAB;
+                                                const GbTabs& Tb, const GbPaper& PT, double2* shF, double2* shM,
+                                                float2* sh32) {
+    constexpr bool tab = TAB == 1;
     const long long nfree = st->nfree, bump = st->bump, kept_old = st->kept_old;
     const long long ci = ch.surv[s];
     ChildCtx c = child_ctx(par, ci, sp);
@@ -1095,6 +1098,13 @@ __device__ __forceinline__ void materialize_one(const GbProg& P, const GbPool& p
     iv64 R[TAB ? 1 : GB_MAX_TREGS];
     iv32 R32[TAB ? 1 : GB_MAX_TREGS];
     int slot_k = 0, ops = 0;
+    if constexpr (TAB == 2)   // the dirty groups' values, one (group, kind) per lane
+        paper_dirty_groups(P, pool, PT, c, lane, [&](int gg, int kind, iv64 v) {
+            const size_t at = (size_t)ns * pool.NG + gg;
+            if (kind == 0) pool.gsum[at] = make_double2(v.lo, v.hi);
+            else if (P.samples == 0) pool.gmid[at] = make_double2(v.lo, v.hi);
+            else pool.gsamp[((size_t)ns * pool.S + (kind - 1)) * pool.NG + gg] = make_double2(v.lo, v.hi);
+        });
     for (int k = 0; k < P.n_sum; k++) {
         GbSum S = P.sums[k];
         int2 dr = P.dirty[blk * P.n_sum + k];
@@ -1108,11 +1118,11 @@ __device__ __forceinline__ void materialize_one(const GbProg& P, const GbPool& p
                 pool.gsamp[((size_t)ns * pool.S + j) * pool.NG + S.group0 + g] =
                     pool.gsamp[((size_t)c.slot * pool.S + j) * pool.NG + S.group0 + g];
         }
-        for (int g = dr.x; g < dr.y; g++, slot_k++) {
+        for (int g = dr.x; TAB != 2 && g < dr.y; g++, slot_k++) {
             if ((slot_k & 31) != lane) continue;
             size_t dst = (size_t)ns * pool.NG + S.group0 + g;
             iv64 a, b;
-            if constexpr (TAB) {
+            if constexpr (tab) {
                 const int at = k * GB_TAB_MAX_DIRTY + (g - dr.x);
                 a = iv64{shF[at].x, shF[at].y};
                 b = iv64{shM[at].x, shM[at].y};
@@ -1127,12 +1137,20 @@ __device__ __forceinline__ void materialize_one(const GbProg& P, const GbPool& p
             }
             pool.gsum[dst] = make_double2(a.lo, a.hi);
             pool.gmid[dst] = make_double2(b.lo, b.hi);
-            if constexpr (!TAB)   // diagonal samples: paper mode runs on the interpreter only
+            if constexpr (!TAB)   // diagonal samples (the term tables have none)
                 for (int j = 1; pool.gsamp && j <= pool.S; j++) {
                     const iv64 v = group_sum<PR, double>(P, S, g, SampleView{X, j, pool.S + 1}, R, ops);
                     pool.gsamp[((size_t)ns * pool.S + (j - 1)) * pool.NG + S.group0 + g] = make_double2(v.lo, v.hi);
                 }
         }
+    }
+    if (TAB == 2 && pool.gdp) {   // coordinate partials: from the tables where the split reaches, else the parent's
+        const GbSplitPos SP = P.sps[P.sp_of_cyc[c.info.x]];
+        const double2* src = pool.gdp + (size_t)c.slot * P.n_sum * n;
+        double2* dst = pool.gdp + (size_t)ns * P.n_sum * n;
+        for (int k = 0; k < P.n_sum; k++)
+            for (int j = lane; j < n; j += 32)
+                dst[(size_t)k * n + j] = j < SP.ja || j >= SP.jb ? src[(size_t)k * n + j] : paper_D_row(P, PT, SP, c.p, j, k, c.r);
     }
     if (!TAB && pool.gdp) {   // coordinate partials: the parent's, recomputed where the split reaches
         const int2 ab = d_affected(P, blk);
@@ -1237,12 +1255,13 @@ __global__ void k_gc_scatter(GbPool pool, const GbState* st, const int* tile_off
 // with those entries replaced.  A new record holds the child's coordinates of
 // its block and the cached sums of the groups it owns (groups of the dirty
 // ranges recomputed, the others copied from the parent's record).
-template <bool PR, bool TAB>
+template <bool PR, int TAB>
 __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& pool, const GbParents& par,
                                                 const GbChildren& ch, const GbSplit& sp, const GbEntries& En,
                                                 double tol_x, const GbState* st, long long s, int lane,
-                                                const GbTabs& Tb, double2* shF, double2* shM, float2* sh32) {
-    constexpr bool tab = TAB;
+                                                const GbTabs& Tb, const GbPaper& PT, double2* shF, double2* shM,
+                                                float2* sh32) {
+    constexpr bool tab = TAB == 1;
     const long long nfree = st->nfree, bump = st->bump, kept_old = st->kept_old;
     const long long rnf = st->rec_nfree, rbump = st->rec_bump;
     const long long ci = ch.surv[s];
@@ -1326,6 +1345,14 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
     iv64 R[TAB ? 1 : GB_MAX_TREGS];
     iv32 R32[TAB ? 1 : GB_MAX_TREGS];
     int ops = 0;
+    if constexpr (TAB == 2)   // the dirty groups' values, one (group, kind) per lane, into their owners' records
+        paper_dirty_groups(P, pool, PT, c, lane, [&](int gg, int kind, iv64 v) {
+            const int2 o = P.gown[gg];
+            const size_t at = (size_t)crow[o.x] * GPB + o.y;
+            if (kind == 0) pool.rgsum[at] = make_double2(v.lo, v.hi);
+            else if (P.samples == 0) pool.rgmid[at] = make_double2(v.lo, v.hi);
+            else pool.rgsamp[(size_t)(kind - 1) * pool.R * GPB + at] = make_double2(v.lo, v.hi);
+        });
     for (int it = lane; it < nrec * GPB; it += 32) {
         const int t = it / GPB, o = it - t * GPB, b = blk - t;
         if (b < 0) continue;
@@ -1345,13 +1372,14 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
             for (int j = 0; pool.rgsamp && j < pool.S; j++) pool.rgsamp[j * sstep + dst] = pool.rgsamp[j * sstep + src];
             continue;
         }
-        if constexpr (!TAB)   // diagonal samples: paper mode runs on the interpreter only
+        if constexpr (TAB == 2) continue;   // written above
+        if constexpr (!TAB)   // diagonal samples (the term tables have none)
             for (int j = 1; pool.rgsamp && j <= pool.S; j++) {
                 const iv64 v = group_sum<PR, double>(P, S, gl, SampleView{X, j, pool.S + 1}, R, ops);
                 pool.rgsamp[(j - 1) * sstep + dst] = make_double2(v.lo, v.hi);
             }
         iv64 a, m;
-        if constexpr (TAB) {
+        if constexpr (tab) {
             const int at = k * GB_TAB_MAX_DIRTY + (gl - dr.x);
             a = iv64{shF[at].x, shF[at].y};
             m = iv64{shM[at].x, shM[at].y};
@@ -1366,6 +1394,19 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
         }
         pool.rgsum[dst] = make_double2(a.lo, a.hi);
         pool.rgmid[dst] = make_double2(m.lo, m.hi);
+    }
+    if (TAB == 2 && pool.rgdp) {   // coordinate partials of each new record's block, from the tables or the parent's
+        const GbSplitPos SP = P.sps[P.sp_of_cyc[c.info.x]];
+        for (int t = 0; t < nrec && blk - t >= 0; t++) {
+            const int b = blk - t, j0 = b * B, w = min(n, j0 + B) - j0;
+            const double2* src = pool.rgdp + (size_t)prow[b] * P.n_sum * B;
+            double2* dst = pool.rgdp + (size_t)crow[b] * P.n_sum * B;
+            for (int i = lane; i < P.n_sum * w; i += 32) {
+                const int k = i / w, j = j0 + i - k * w;
+                dst[(size_t)k * B + (j - j0)] = j < SP.ja || j >= SP.jb ? src[(size_t)k * B + (j - j0)]
+                                                                      : paper_D_row(P, PT, SP, c.p, j, k, c.r);
+            }
+        }
     }
     if (!TAB && pool.rgdp) {   // coordinate partials of each new record's block (templates within one coordinate)
         iv64 RA[GB_MAX_TREGS];
@@ -1394,10 +1435,10 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
 // the next selection.  For K = 1 the smallest selectable key of the new pool
 // is all the selection needs: its entry is the next parent when it is below
 // the new incumbent's cut-off threshold, and if it is not, no entry is.
-template <bool PR, bool RECS, bool TAB>
+template <bool PR, bool RECS, int TAB>
 __global__ void __launch_bounds__(128) k_materialize(GbProg P, GbPool pool, GbParents par, GbChildren ch,
                                                      GbSplit sp, GbEntries En, double tol_x, GbState* st,
-                                                     GbTabs Tb, GbGenConst G, int npart, unsigned long long* pkey,
+                                                     GbTabs Tb, GbPaper PT, GbGenConst G, int npart, unsigned long long* pkey,
                                                      long long* ppos) {
     gb_grid_trigger();
     gb_grid_wait();
@@ -1415,9 +1456,11 @@ __global__ void __launch_bounds__(128) k_materialize(GbProg P, GbPool pool, GbPa
     long long bq = -1;
     for (long long s = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; s < kept; s += nwarps) {
         if constexpr (RECS)
-            materialize_rec<PR, TAB>(P, pool, par, ch, sp, En, tol_x, st, s, lane, Tb, shF[w], shM[w], sh32[w]);
+            materialize_rec<PR, TAB>(P, pool, par, ch, sp, En, tol_x, st, s, lane, Tb, PT, shF[w], shM[w],
+                                     sh32[w]);
         else
-            materialize_one<PR, TAB>(P, pool, par, ch, sp, En, tol_x, st, s, lane, Tb, shF[w], shM[w], sh32[w]);
+            materialize_one<PR, TAB>(P, pool, par, ch, sp, En, tol_x, st, s, lane, Tb, PT, shF[w], shM[w],
+                                     sh32[w]);
         __syncwarp();
         if (pkey && lane == 0) {   // the entry lane 0 has just written
             const long long e = kept_old + s;
@@ -1746,7 +1789,7 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
                                  const GbParents& par, const GbChildren& ch, const GbSplit& sp, const GbScan& sc,
                                  const GbTabs* tabs, const GbGenConst& G, long long cap, long long Cmax,
                                  GbState* st, cudaStream_t s, cudaEvent_t* ev, long long* nlaunch, int part,
-                                 const GbFork* fork) {
+                                 const GbFork* fork, const GbPaper* paper) {
     long long n0 = gb_launch_count;
     cudaError_t e;
     const unsigned gpool = (unsigned)std::min<long long>(grid_for(cap, 256), gb_sm_count() * 8);
@@ -1825,6 +1868,7 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
         k_prep<<<grid_for(G.K * (long long)sp.dmax, 128), 128, 0, s>>>(P, pool, par, sp, st);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (ev && part == 0) cudaEventRecord(ev[0], s);
+        if (paper && (e = gb_launch_paper_tables(P, pool, par, *paper, G.K, sp, st, s)) != cudaSuccess) return e;
     } else if (!sel_tabs) {
         if ((e = tables()) != cudaSuccess) return e;
     }
@@ -1867,6 +1911,8 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
             gb_launch_count++;
             if ((e = gb_launch_eval64_tab(P, pool, par, *tabs, ch, Cmax, sp, G.fp32 != 0, st, s)) != cudaSuccess)
                 return e;
+        } else if (paper) {
+            if ((e = gb_launch_paper_eval(P, pool, par, *paper, ch, Cmax, sp, st, s)) != cudaSuccess) return e;
         } else {
             gb_launch_count++;
             if (P.any_prod) k_eval64<true><<<gch, 128, 0, s>>>(P, pool, par, ch, sp, G.fp32, st);
@@ -1891,6 +1937,7 @@ after_eval:
     }
     GbTabs Tb{};
     if (tabs) Tb = *tabs;
+    const GbPaper PT = paper ? *paper : GbPaper{};
     gb_launch_count++;
     const unsigned gmat = gmat_max;
     // K = 1: the generation ends in k_materialize's last block (no k_stats pass)
@@ -1899,17 +1946,19 @@ after_eval:
     const int np = 1;   // the partition's combined pair
 #define GB_MAT(PR, RECS, TAB)                                                                                      \
     e = gb_launch_ex(k_materialize<PR, RECS, TAB>, gmat, 128, 0, s, true, P, pool, par, ch, sp, E_new, G.tol_x,   \
-                     st, Tb, G, np, pk, pq)
-    // products never use term tables
-    if (P.any_prod) {
-        if (pool.recs) GB_MAT(true, true, false);
-        else GB_MAT(true, false, false);
+                     st, Tb, PT, G, np, pk, pq)
+    if (paper) {   // (products included: a group's value comes from the tables)
+        if (pool.recs) GB_MAT(false, true, 2);
+        else GB_MAT(false, false, 2);
+    } else if (P.any_prod) {   // products never use the term tables
+        if (pool.recs) GB_MAT(true, true, 0);
+        else GB_MAT(true, false, 0);
     } else if (tabs) {
-        if (pool.recs) GB_MAT(false, true, true);
-        else GB_MAT(false, false, true);
+        if (pool.recs) GB_MAT(false, true, 1);
+        else GB_MAT(false, false, 1);
     } else {
-        if (pool.recs) GB_MAT(false, true, false);
-        else GB_MAT(false, false, false);
+        if (pool.recs) GB_MAT(false, true, 0);
+        else GB_MAT(false, false, 0);
     }
 #undef GB_MAT
     if (e != cudaSuccess) return e;

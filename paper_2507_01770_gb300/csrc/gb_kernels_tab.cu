@@ -422,41 +422,6 @@ __global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents
 }
 
 // ---------------------------------------------------------------------------
-// Path of sum k's pairwise group tree above its dirty groups [dr.x, dr.y)
-// (values cur[0 .. dr.y - dr.x)), with the parent's tree nodes (node(i),
-// level-major) for the clean siblings; returns the sum.
-template <typename I, typename N>
-__device__ __forceinline__ I tab_path(const GbSum& S, int2 dr, I* cur, N node, int& ops) {
-    I tmp[GB_TAB_MAX_DIRTY];
-    if (S.ngroups == 0 || S.nnodes <= 0) {
-        I z;
-        z.lo = 0;
-        z.hi = 0;
-        return z;
-    }
-    int lo = dr.x, hi = dr.y, off = 0;
-    if (lo >= hi) return node(S.nnodes - 1);   // no dirty group: the parent's root
-    for (int mL = S.ngroups; mL > 1; mL = (mL + 1) / 2) {
-        const int nlo = lo >> 1, nhi = ((hi - 1) >> 1) + 1;
-        for (int q = nlo; q < nhi; q++) {
-            const int a = 2 * q;
-            I left = (a >= lo && a < hi) ? cur[a - lo] : node(off + a);
-            I v = left;
-            if (a + 1 < mL) {
-                I right = (a + 1 >= lo && a + 1 < hi) ? cur[a + 1 - lo] : node(off + a + 1);
-                v = iadd(left, right);
-                ops += 2;
-            }
-            tmp[q - nlo] = v;
-        }
-        for (int q = 0; q < nhi - nlo; q++) cur[q] = tmp[q];
-        lo = nlo;
-        hi = nhi;
-        off += mL;
-    }
-    return cur[0];
-}
-
 // tab_path for a warp whose lanes all walk the same path (one child per
 // warp): the clean sibling nodes the walk reads depend only on the tree's
 // shape and the dirty range, so they are listed first (lane t takes the t-th

@@ -115,6 +115,25 @@ struct GbTabs {
     // most GB_REG_DIRTY groups of fewer than 2^GB_REG_LEVELS terms each)
     int reg;
 };
+// Paper mode (diagonal samples, first-order test on every coordinate) from
+// per-parent tables.  Kind 0 is the box, kinds 1 .. nk - 1 its sample points
+// (samples S: the S diagonal points; 0: the midpoint).  Arrays are indexed
+// by (parent * nk + kind) * rows, tl and td by parent * rows.
+struct GbPaper {
+    int nk, n_hoist, n_oprog;
+    int arows, srows, drows, hrows, tree_nodes, max_leaves;   // rows per (parent, kind)
+    double2* tv;      // term values of the dirty terms' rows, then of the clean ones a product needs (kind 0)
+    double2* tl;      // leaf adjoints of the sums' terms (kind 0), max_leaves per row
+    double2* ts;      // term-tree segments
+    double2* nd;      // group trees of the parent's cached values
+    double2* td;      // partial sums D by digit combination
+    double2* hv;      // hoisted outer values
+    const GbPaperSum* psums;
+    const GbHoistPos* hoist_pos;
+    const int32_t* hoist_node;
+    const GbOIns* oprog;
+    uint32_t indep;
+};
 constexpr int GB_CG = GB_MAX_ISUM * GB_TAB_MAX_DIRTY;
 constexpr int GB_MV_BITS = 6;
 constexpr int GB_REG_DIRTY = 4;
@@ -189,7 +208,13 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
                                  const GbParents& par, const GbChildren& ch, const GbSplit& sp, const GbScan& sc,
                                  const GbTabs* tabs, const GbGenConst& G, long long cap, long long Cmax,
                                  GbState* st, cudaStream_t s, cudaEvent_t* ev, long long* nlaunch, int part = 0,
-                                 const GbFork* fork = nullptr);
+                                 const GbFork* fork = nullptr, const GbPaper* paper = nullptr);
+// Paper mode: the tables of every parent (after k_prep), then the children from them.
+cudaError_t gb_launch_paper_tables(const GbProg& P, const GbPool& pool, const GbParents& par, const GbPaper& T,
+                                   long long K, const GbSplit& sp, GbState* st, cudaStream_t s);
+cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbParents& par, const GbPaper& T,
+                                 const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
+                                 cudaStream_t s);
 
 // One problem of a fused child evaluation: the arguments of its
 // k_eval3264_tabw launch (term tables, one child per warp, FP32 then FP64).
