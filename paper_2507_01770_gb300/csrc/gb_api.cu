@@ -362,6 +362,13 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         P.box_tiles[L] = d_bt;
         P.n_box_tiles[L] = (int)H.box_tiles[L].size();
     }
+    for (int b = 0; b < H.nb; b++)
+        for (size_t k = 0; k < H.sums.size(); k++) {
+            const int2 dr = H.dirty[(size_t)b * H.sums.size() + k];
+            int t = 0;
+            for (int g = dr.x; g < dr.y; g++) t += H.groups[H.sums[k].group0 + g].count;
+            P.max_dirty_terms = std::max(P.max_dirty_terms, t);
+        }
     P.n_tins = (int)H.tins.size();
     for (const GbSum& S : H.sums) {
         P.max_terms = std::max(P.max_terms, S.count);
@@ -513,6 +520,9 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     if (opt.eval_mode != 1) {
         const bool want = opt.eval_mode >= 2 || p->fan >= 16;
         if (p->hp.tab_ok && want) {
+            const bool warp = opt.eval_mode == 4 || (opt.eval_mode != 3 && gb_warp_per_child(p->Cmax));
+            const bool dec = !warp && P.n_var_leaves == 0 && (P.outer_unit || (P.outer_sum && P.n_sum == 1)) &&
+                             gb_build_endpoints(&p->hp, false);
             const GbHostProg& Hh = p->hp;
             int32_t* d_spc;
             GbSplitPos* d_sps;
@@ -566,7 +576,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             if (fp32 && ((e = alloc(&T.tv32, rows, A)) || (e = alloc(&T.tl32, rows * T.max_leaves, A)) ||
                          (e = alloc(&T.nf32, nodes, A))))
                 return bad(e, "allocate term tables");
-            T.warp = opt.eval_mode == 4 ? 1 : opt.eval_mode == 3 ? 0 : (gb_warp_per_child(p->Cmax) ? 1 : 0);
+            T.warp = warp ? 1 : 0;
             T.reg = 0;
             if (P.outer_sum && P.n_sum == 1 && P.n_var_leaves == 0) {   // the register-resident walk of the one sum
                 const GbSum& S0 = Hh.sums[0];
@@ -578,6 +588,12 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
                         fits = Hh.groups[S0.group0 + g].count < (1 << GB_REG_LEVELS);
                 }
                 T.reg = fits ? 1 : 0;
+            }
+            T.dec = dec ? 1 : 0;
+            if (dec) {
+                GbUop* d_u;
+                if ((e = upload(&d_u, Hh.uops.data(), Hh.uops.size(), A))) return bad(e, "upload table layouts");
+                P.uops = d_u;
             }
             T.max_sum_nodes = 1;
             for (const GbSum& S : Hh.sums) T.max_sum_nodes = std::max(T.max_sum_nodes, (int)S.nnodes);
@@ -600,6 +616,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         }
     }
     if (paper_tabs) {
+        const bool dec = gb_build_endpoints(&p->hp, true);
         const GbHostProg& Hh = p->hp;
         GbPaper& T = p->paper;
         int32_t* d_spc;
@@ -613,7 +630,9 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         GbHoistPos* d_hp;
         int32_t* d_hn;
         GbOIns* d_op;
-        if ((e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||
+        GbUop* d_u;
+        if ((e = upload(&d_u, Hh.uops.data(), Hh.uops.size(), A)) ||
+            (e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||
             (e = upload(&d_sps, Hh.sps.data(), Hh.sps.size(), A)) ||
             (e = upload(&d_dt, Hh.dterms.data(), Hh.dterms.size(), A)) ||
             (e = upload(&d_jk, Hh.jk.data(), Hh.jk.size(), A)) ||
@@ -649,12 +668,15 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         T.hoist_node = d_hn;
         T.oprog = d_op;
         T.indep = Hh.indep;
+        T.dec = dec ? 1 : 0;
+        P.uops = d_u;
         const size_t kk = K * (size_t)T.nk;
         if ((e = alloc(&T.tv, kk * T.arows, A)) || (e = alloc(&T.ts, kk * T.srows, A)) ||
             (e = alloc(&T.nd, kk * T.tree_nodes, A)) || (e = alloc(&T.hv, kk * T.hrows, A)) ||
             (e = alloc(&T.tl, K * (size_t)T.arows * T.max_leaves, A)) || (e = alloc(&T.td, K * (size_t)T.drows, A)))
-            return bad(e, "allocate paper-mode tables");
-        p->use_paper = true;
+            cudaGetLastError();   // no room for the tables: the interpreter
+        else
+            p->use_paper = true;
     }
     p->G.K = p->K;
     p->G.flog2 = d * mshift;

@@ -310,4 +310,19 @@ __device__ __forceinline__ void set_survivors(const GbGenConst& G, GbState* st, 
     st->overflow = (S > room || (G.nrec && S * G.nrec > st->rec_nfree + (G.R - st->rec_bump))) ? 1 : 0;
 }
 
+// The kernel's last block to finish lists the generation's survivors (at most
+// 64 children per thread of it) against the final incumbent.
+__device__ __forceinline__ void list_survivors_last(const GbChildren& ch, long long nch, const GbGenConst& G,
+                                                    GbState* st) {
+    __shared__ int s_sw[32];
+    __shared__ bool s_last;
+    if (!arrive_last(&st->cc_done, gridDim.x, &s_last)) return;
+    const double gub_new = gb_key_value(__ldcg((const unsigned long long*)&st->gub_new_key));
+    const long long S = survivor_list_block(ch, nch, gub_new, true, s_sw);
+    if (threadIdx.x == 0) {
+        st->cc_done = 0;
+        set_survivors(G, st, S);
+    }
+}
+
 }  // namespace gb

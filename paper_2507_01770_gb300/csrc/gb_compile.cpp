@@ -397,6 +397,180 @@ static bool build_hoists(GbHostProg* P, std::vector<std::vector<int>>* vars) {
     return P->hoist_node.size() <= GB_MAX_HOIST;
 }
 
+namespace {
+
+// Endpoint program of one split position (see GbUop).
+struct DecBuilder {
+    GbHostProg* P;
+    const GbSplitPos* sp;
+    bool paper;
+    const GbHoistPos* hoists;   // this split position's (paper)
+    std::vector<GbUop> u;
+    int depth = 0, max_depth = 0;
+    std::vector<char> seen;
+
+    GbUop make(int op, int base = 0, int shift = 0, unsigned mask = 0) {
+        GbUop x{};
+        x.op = (uint8_t)op;
+        x.base = base;
+        x.shift = (int16_t)shift;
+        x.mask = (uint16_t)mask;
+        return x;
+    }
+    void push(const GbUop& x) {
+        u.push_back(x);
+        max_depth = std::max(max_depth, ++depth);
+    }
+    void add() {
+        u.push_back(make(U_ADD));
+        depth--;
+    }
+    // group g of sum k: its segments through the binary counter (the levels
+    // present lie on the stack, the lowest on top)
+    void group(int k, int g) {
+        unsigned cnt = 0;
+        for (int q = sp->seg0; q < sp->seg0 + sp->nseg; q++) {
+            const GbSeg& G = P->segs[q];
+            if (G.sum != k || G.group != g) continue;
+            push(make(G.level ? U_SEG : U_ROW, G.base, G.shift, G.mask));
+            for (unsigned c = cnt >> G.level; c & 1u; c >>= 1) add();
+            cnt += 1u << G.level;
+        }
+        if (!cnt) push(make(U_ZERO));
+        for (int n = __builtin_popcount(cnt); n > 1; n--) add();
+    }
+    // node q of level L of sum k's group tree (level sizes and offsets given), dirty nodes [lo[L], hi[L])
+    void node(int k, int L, int q, const std::vector<int>& size, const std::vector<int>& off,
+              const std::vector<int>& lo, const std::vector<int>& hi) {
+        if (L == 0) return group(k, q);
+        const int a = 2 * q, b = a + 1;
+        const bool da = a >= lo[L - 1] && a < hi[L - 1], db = b >= lo[L - 1] && b < hi[L - 1], hb = b < size[L - 1];
+        if (da) node(k, L - 1, a, size, off, lo, hi);
+        if (hb && db) node(k, L - 1, b, size, off, lo, hi);
+        if (!hb) return;
+        if (da && db) return add();
+        u.push_back(make(U_ADDN, P->sums[k].node0 + off[L - 1] + (da ? b : a)));
+    }
+    void sum(int k) {
+        const GbSum& S = P->sums[k];
+        const int2 dr = P->dirty[(size_t)sp->block * P->sums.size() + k];
+        if (S.ngroups == 0 || S.nnodes <= 0) return push(make(U_ZERO));
+        if (dr.x >= dr.y) return push(make(U_NODE, S.node0 + S.nnodes - 1));
+        std::vector<int> size{S.ngroups}, off{0}, lo{dr.x}, hi{dr.y};
+        while (size.back() > 1) {
+            off.push_back(off.back() + size.back());
+            const int l = lo.back(), h = hi.back();
+            lo.push_back(l >> 1);
+            hi.push_back(((h - 1) >> 1) + 1);
+            size.push_back((size.back() + 1) / 2);
+        }
+        node(k, (int)size.size() - 1, 0, size, off, lo, hi);
+    }
+    bool konst(int t, double* lo, double* hi) const {
+        const GbIns& I = P->outer[t];
+        if (I.op == D_CONST) *lo = *hi = I.c;
+        else if (I.op == D_PI) *lo = 3.141592653589793, *hi = std::nextafter(*lo, 4.0);
+        else if (I.op == D_EULER) *lo = 2.718281828459045, *hi = std::nextafter(*lo, 3.0);
+        else return false;
+        return true;
+    }
+    // operand t without a reduction: op + a constant or (paper) a hoisted value
+    bool operand(int t, int opc, int oph, bool rcp) {
+        GbUop x = make(opc);
+        if (!rcp && konst(t, &x.lo, &x.hi)) {
+            u.push_back(x);
+            return true;
+        }
+        if (!paper) return false;
+        const int key = t | (rcp ? 1 << 16 : 0);
+        for (size_t h = 0; h < P->hoist_node.size(); h++)
+            if (P->hoist_node[h] == key) {
+                u.push_back(make(oph, hoists[h].base, hoists[h].shift, hoists[h].mask));
+                return true;
+            }
+        return false;
+    }
+    bool outer(int t) {
+        const GbIns& I = P->outer[t];
+        if (seen[t]) return false;   // a shared subexpression would run twice
+        seen[t] = 1;
+        auto dep = [&](int q) { return !((P->indep >> q) & 1u); };
+        double lo, hi;
+        switch (I.op) {
+        case D_ISUMV: sum(I.aux); return true;
+        case D_ADD:
+            if (dep(I.a) && dep(I.b)) {
+                if (!outer(I.a) || !outer(I.b)) return false;
+                add();
+                return true;
+            }
+            return outer(dep(I.a) ? I.a : I.b) && operand(dep(I.a) ? I.b : I.a, U_ADDC, U_ADDH, false);
+        case D_SUB: return dep(I.a) && !dep(I.b) && outer(I.a) && operand(I.b, U_SUBC, U_SUBH, false);
+        case D_SCALE: {
+            if (!(I.c > 0.0)) return false;
+            if (!outer(I.a)) return false;
+            GbUop x = make(U_SCALE);
+            x.lo = x.hi = I.c;
+            u.push_back(x);
+            return true;
+        }
+        case D_MUL: {
+            if (dep(I.a) && dep(I.b)) return false;
+            const int c = dep(I.a) ? I.b : I.a;
+            return konst(c, &lo, &hi) && lo > 0.0 && outer(dep(I.a) ? I.a : I.b) && operand(c, U_MULC, U_MULH, false);
+        }
+        case D_DIV:   // by a positive constant: times its (outward rounded) reciprocal
+            return !dep(I.b) && konst(I.b, &lo, &hi) && lo > 0.0 && std::isfinite(1.0 / lo) && outer(I.a) &&
+                   operand(I.b, U_MULC, U_MULH, true);
+        default: return false;
+        }
+    }
+};
+
+// The endpoint programs of every split position; false if the objective or
+// the stack depth does not allow them.
+bool build_endpoint_programs(GbHostProg* P, bool paper) {
+    P->uops.clear();
+    const int no = (int)P->outer.size();
+    if (P->any_prod || no == 0) return false;
+    if (!paper) {   // which outer registers depend on a sum (paper mode: build_hoists)
+        P->indep = 0;
+        for (int t = 0; t < no; t++) {
+            const GbIns& I = P->outer[t];
+            const bool leaf = I.op == D_CONST || I.op == D_PI || I.op == D_EULER || I.op == D_VAR || I.op == D_ISUMV;
+            const bool bin = I.op == D_ADD || I.op == D_SUB || I.op == D_MUL || I.op == D_DIV;
+            bool ind = I.op != D_ISUMV;
+            if (!leaf) ind = ((P->indep >> I.a) & 1u) && (!bin || ((P->indep >> I.b) & 1u));
+            if (ind) P->indep |= 1u << t;
+        }
+    }
+    if ((P->indep >> P->outer_root) & 1u) return false;
+    for (size_t i = 0; i < P->sps.size(); i++) {
+        GbSplitPos& sp = P->sps[i];
+        DecBuilder B;
+        B.P = P;
+        B.sp = &sp;
+        B.paper = paper;
+        B.hoists = paper ? P->hoist_pos.data() + i * P->hoist_node.size() : nullptr;
+        B.seen.assign(no, 0);
+        if (!B.outer(P->outer_root) || B.max_depth > GB_DEC_DEPTH) return false;
+        sp.u0 = (int)P->uops.size();
+        sp.nu = (int)B.u.size();
+        sp.nsuf = 0;
+        while (sp.nsuf < sp.nu) {
+            const GbUop& x = B.u[sp.nu - 1 - sp.nsuf];
+            if (x.op <= U_ADD || ((x.op == U_ADDH || x.op == U_SUBH || x.op == U_MULH) && x.mask != 0)) break;
+            sp.nsuf++;
+        }
+        P->uops.insert(P->uops.end(), B.u.begin(), B.u.end());
+    }
+    return true;
+}
+
+}  // namespace
+
+bool gb_build_endpoints(GbHostProg* P, bool paper) { return P->tab_ok && build_endpoint_programs(P, paper); }
+
 void gb_build_tables(GbHostProg* P, int m, int d, int sbits, bool paper) {
     P->tab_ok = 0;
     P->m = m;

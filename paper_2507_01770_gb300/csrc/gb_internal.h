@@ -89,7 +89,26 @@ struct GbSplitPos {
     // tabulated are those of coordinates [ja, jb), the block and a term's reach beyond it
     int32_t nx, ja, jb;
     int32_t hrows;            // rows of the hoisted outer values
+    int32_t u0, nu, nsuf;     // endpoint program uops [u0, u0 + nu); the last nsuf read no digit and push nothing
 };
+// Endpoint program of a split position: F's lower end (or a sample's upper
+// end) of a child as a postfix program over one double per stack entry, for
+// objectives whose outer expression adds the sums (and, scaled by positive
+// constants, what no sum enters): then each end of the result depends on the
+// same end of every operand alone.  Pushes read a term row, a segment row or
+// a tree node of the parent; ADD combines the two top entries.
+enum GbUopCode : uint8_t {
+    U_ROW = 0, U_SEG, U_NODE, U_ZERO, U_ADD, U_ADDN, U_ADDH, U_SUBH, U_MULH, U_ADDC, U_SUBC, U_MULC, U_SCALE
+};
+struct GbUop {
+    uint8_t op, pad;
+    int16_t shift;
+    uint16_t mask, pad2;
+    int32_t base;      // row or node; for a table, of its entry 0
+    int32_t pad3;
+    double lo, hi;     // constant operand
+};  // 32 bytes
+#define GB_DEC_DEPTH 4
 // Paper mode, per (split position, reduction): its dirty terms [t_lo, t_hi)
 // are dterms d0 ..., the other terms of a product, in order, dterms x0 ...
 // (all relative to dterm0; x0 < 0: not tabulated).
@@ -196,6 +215,7 @@ struct GbProg {
     const GbContrib* contribs;
     const GbJkD* jkd;                // parallel to jk: partial-table rows
     int32_t max_drows;
+    const GbUop* uops;               // endpoint programs of every split position
     const GbSeg* segs;               // term-tree segments of every split position
     int32_t max_srows, max_nseg;
     int32_t outer_sum;               // 1: the outer expression is one sum (F = that sum, adjoint [1, 1])
@@ -209,6 +229,7 @@ struct GbProg {
     int32_t n_box_tiles[GB_BOX_LISTS];   // 0: a group exceeds the list's tile size
     int32_t n_tins, max_terms, box_leaves;   // template instructions, terms of the longest sum, IVAR leaves of
                                      //    the widest template
+    int32_t max_dirty_terms;         // terms of a sum's groups that a block touches, at most
 };
 
 // Host-side compiled program (arrays in host memory before upload).
@@ -231,6 +252,7 @@ struct GbHostProg {
     std::vector<GbHoistPos> hoist_pos;   // [split positions][hoists]
     std::vector<int32_t> hoist_node;     // outer register, | 1 << 16: its reciprocal
     std::vector<GbOIns> oprog;
+    std::vector<GbUop> uops;
     int32_t max_arows = 0, max_hrows = 0;
     uint32_t indep = 0;                  // outer registers that depend on no reduction
     // block records: group ownership (a group lives in the record of its lowest touched block)
@@ -254,6 +276,8 @@ struct GbHostProg {
 // sbits: largest digit-bit count of a tabulated term-tree segment (<= GB_TAB_SBITS).
 // paper: layouts of the paper-mode tables (products included; see GbSplitPos).
 void gb_build_tables(GbHostProg* P, int m, int d, int sbits = GB_TAB_SBITS, bool paper = false);
+// Endpoint programs (GbUop) of every split position of the layouts just built; false: not for this objective.
+bool gb_build_endpoints(GbHostProg* P, bool paper);
 // Compiles and validates a DAG; returns an empty string or an error message.
 std::string gb_compile(const gb_node* nodes, int32_t nn, int32_t root, const int64_t* tlen,
                        int32_t ntab, int32_t n, int32_t B, GbHostProg* out);
@@ -308,6 +332,7 @@ struct GbState {
     int gc;                            // block records: collect before this generation's inserts
     unsigned stats_done;               // blocks of k_stats finished (the last one starts the generation)
     unsigned cc_done;                  // blocks of the child kernel finished (the last one lists the survivors)
+    int cc_listed;                     // the child kernel has listed the survivors (written by k_child_box alone)
     unsigned part_done;                // blocks of the partition finished (the last one combines their keys)
     unsigned long long min_key;        // smallest active key (K = 1 selection)
     long long evals32, evals64, mids;  // running counters

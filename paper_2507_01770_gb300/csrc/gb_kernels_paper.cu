@@ -25,6 +25,7 @@
 
 #include <algorithm>
 
+#include "gb_dec.cuh"
 #include "gb_paper.cuh"
 
 using namespace gb;
@@ -456,6 +457,19 @@ __global__ void __launch_bounds__(128) k_pp_eval(GbProg P, GbPool pool, GbParent
     }
 }
 
+// The same from the endpoint programs.
+__global__ void __launch_bounds__(128) k_pp_dec(GbProg P, GbPool pool, GbParents par, GbPaper T, GbDec D, GbChildren ch,
+                                                GbSplit sp, int one, GbState* st) {
+    if (st->halt) return;
+    __shared__ unsigned s_queue[4][64];
+    int ops = 0;
+    dec_children<6>(P, par, ch, sp, D, false, one != 0, st, s_queue[threadIdx.x >> 5], [&](unsigned ci) {
+        const ChildCtx c = child_ctx(par, ci, sp);
+        return paper_mono<false>(P, pool, par, T, c, sp, P.sp_of_cyc[c.info.x], ops);
+    });
+    warp_add_ops(ops, &st->ops64);
+}
+
 unsigned grid_for(long long items, int per_block) {
     const long long g = (items + per_block - 1) / per_block;
     return (unsigned)(g < 1 ? 1 : g);
@@ -481,6 +495,16 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
                                  cudaStream_t s) {
     gb_launch_count++;
+    if (T.dec) {
+        const GbDec D{T.tv, T.ts, T.nd, T.hv, (long long)T.nk * T.arows, (long long)T.nk * T.srows,
+                      (long long)T.nk * T.tree_nodes, (long long)T.nk * T.hrows, T.arows, T.srows, T.tree_nodes, T.hrows,
+                      T.nk};
+        const bool one = (Cmax >> sp.flog2) <= 1;
+        // one parent: as many threads as stay resident, each taking several children
+        const unsigned gd = std::min<unsigned>(grid_for(Cmax, 128), (unsigned)gb_sm_count() * (one ? 8 : 32));
+        k_pp_dec<<<gd, 128, 0, s>>>(P, pool, par, T, D, ch, sp, one ? 1 : 0, st);
+        return cudaGetLastError();
+    }
     const unsigned g = std::min<unsigned>(grid_for(Cmax, 128), (unsigned)gb_sm_count() * 32);
     if (P.any_prod) k_pp_eval<true><<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, st);
     else k_pp_eval<false><<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, st);

@@ -12,7 +12,9 @@
 // same order as the interpreter kernels, so the results are bit-identical.
 #include <cuda_runtime.h>
 
-#include "gb_child.cuh"
+#include <algorithm>
+
+#include "gb_dec.cuh"
 
 using namespace gb;
 
@@ -367,13 +369,24 @@ __global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents
         if (tl32) T.td32[o] = make_float2(D32.lo, D32.hi);
     }
     // (2) segment tables
-    const int nw_items = SP.nseg << GB_TAB_SBITS;
+    const int nw_items = SP.srows;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const size_t rb = (size_t)p * T.max_rows;
     for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw_items; w += nwarps) {
-        const int si = w >> GB_TAB_SBITS, c = w & ((1 << GB_TAB_SBITS) - 1);
+        // the tabulated segment owning row w (a lane per segment)
+        int si = -1;
+        for (int s0 = 0; s0 < SP.nseg && si < 0; s0 += 32) {
+            bool mine = false;
+            if (s0 + lane < SP.nseg) {
+                const GbSeg G = P.segs[SP.seg0 + s0 + lane];
+                mine = G.level != 0 && G.base <= w && w <= G.base + (int)G.mask;
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, mine);
+            if (b) si = s0 + __ffs(b) - 1;
+        }
+        if (si < 0) continue;   // the same for the whole warp
         const GbSeg G = P.segs[SP.seg0 + si];
-        if (G.level == 0 || c > (int)G.mask) continue;   // the same for the whole warp
+        const int c = w - G.base;
         const unsigned r = (unsigned)c << G.shift;
         const int L = G.level, sub = L > 5 ? L - 5 : 0, width = 1 << (L - sub);
         iv64 f{0.0, 0.0}, m{0.0, 0.0};
@@ -1258,6 +1271,31 @@ __global__ void __launch_bounds__(128, REG ? GB_TAB_MINB_REG : GB_TAB_MINB) k_ev
     }
 }
 
+// One child per thread from the endpoint programs (every sum enters F with
+// adjoint [1, 1], so the first-order test needs no outer values).
+__global__ void __launch_bounds__(128) k_eval64_dec(GbProg P, GbPool pool, GbParents par, GbTabs Tb, GbDec D,
+                                                    GbChildren ch, GbSplit sp, int from_list, int one, GbState* st) {
+    gb_grid_trigger();
+    gb_grid_wait();
+    if (st->halt) return;
+    __shared__ unsigned s_queue[4][64];
+    int ops = 0;
+    dec_children<2>(P, par, ch, sp, D, from_list != 0, one != 0, st, s_queue[threadIdx.x >> 5], [&](unsigned ci) {
+        const ChildCtx c = child_ctx(par, ci, sp);
+        const GbSplitPos SP = P.sps[P.sp_of_cyc[c.info.x]];
+        const View<double> X = view64(pool, par, c, sp);
+        const int c0 = c.info.z * P.B, c1 = min(P.n, c0 + P.B);
+        const double2* tl = leaf_tab<double>(Tb, c.p);
+        const double2* td = part_tab<double>(Tb, c.p);
+        for (int j = c0; j < c1; j++) {
+            const iv64 g = tab_partial<double>(P, Tb, tl, td, SP, j, c0, c.r, (const iv64*)nullptr, 0xffffffffu, ops);
+            if (mono_hit(P, X, j, gt_zero(g.lo), lt_zero(g.hi))) return true;
+        }
+        return false;
+    });
+    warp_add_ops(ops, &st->ops64);
+}
+
 __global__ void __launch_bounds__(128, GB_TAB_MINB) k_eval32_tab(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
                                                     GbChildren ch, GbSplit sp, GbState* st) {
     if (st->halt) return;
@@ -1577,8 +1615,10 @@ __device__ __forceinline__ bool eval64_tab_child_w(const GbProg& P, const GbPool
     return true;
 }
 
+// cc: as k_eval3264_tabw.
 __global__ void __launch_bounds__(128, 1) k_eval64_tabw(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
-                                                     GbChildren ch, GbSplit sp, int from_list, GbState* st) {
+                                                     GbChildren ch, GbSplit sp, int from_list, GbState* st,
+                                                     GbGenConst G, int cc) {
     if (st->halt) return;
     const long long lim = from_list ? st->n32 : st->nch;
     const double gub_prev = gb_key_value(st->gub_key);
@@ -1603,6 +1643,7 @@ __global__ void __launch_bounds__(128, 1) k_eval64_tabw(GbProg P, GbPool pool, G
         atomicAdd((unsigned long long*)&st->mids, nv);
         if (!from_list) atomicAdd((unsigned long long*)&st->children, nv);
     }
+    if (cc) list_survivors_last(ch, st->nch, G, st);
 }
 
 // FP32 pass of one child by a warp: writes flag32 (and resets the FP64 flag
@@ -1725,16 +1766,7 @@ __global__ void __launch_bounds__(128, 1) k_eval3264_tabw(GbProg P, GbPool pool,
         atomicAdd((unsigned long long*)&st->kept32, n32);
         atomicAdd((unsigned long long*)&st->n32, n32);
     }
-    if (!cc) return;
-    __shared__ int s_sw[32];
-    __shared__ bool s_last;
-    if (!arrive_last(&st->cc_done, gridDim.x, &s_last)) return;
-    const double gub_new = gb_key_value(__ldcg((const unsigned long long*)&st->gub_new_key));
-    const long long S = survivor_list_block(ch, lim, gub_new, true, s_sw);
-    if (threadIdx.x == 0) {
-        st->cc_done = 0;
-        set_survivors(G, st, S);
-    }
+    if (cc) list_survivors_last(ch, lim, G, st);
 }
 
 // The same FP32-then-FP64 warp-per-child evaluation over the children of
@@ -1835,14 +1867,24 @@ cudaError_t gb_launch_ptab(const GbProg& P, const GbPool& pool, const GbParents&
 
 cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, bool from_list,
-                                 GbState* st, cudaStream_t s) {
+                                 GbState* st, cudaStream_t s, const GbGenConst* cc) {
     if (T.warp) {
         unsigned g = grid_for(Cmax * 32, 128);
         if (g > gb_sm_count() * 32) g = gb_sm_count() * 32;
-        k_eval64_tabw<<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, from_list ? 1 : 0, st);
+        k_eval64_tabw<<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, from_list ? 1 : 0, st, cc ? *cc : GbGenConst{},
+                                        cc ? 1 : 0);
         return cudaGetLastError();
     }
     unsigned g = grid_for(Cmax, 128);
+    if (T.dec) {
+        const GbDec D{T.tv64, T.ts64, T.nf64, nullptr, T.max_rows, T.max_srows, T.tree_nodes, 0,
+                      T.tm64 - T.tv64, T.tsm64 - T.ts64, T.nm64 - T.nf64, 0, 2};
+        const bool one = (Cmax >> sp.flog2) <= 1;
+        // one parent: as many threads as stay resident, each taking several children
+        g = std::min<unsigned>(g, (unsigned)gb_sm_count() * (one ? 12 : 32));
+        return gb_launch_ex(k_eval64_dec, g, 128, 0, s, true, P, pool, par, T, D, ch, sp, from_list ? 1 : 0, one ? 1 : 0,
+                            st);
+    }
     if (g > gb_sm_count() * GB_TAB_GRID) g = gb_sm_count() * GB_TAB_GRID;
     return gb_launch_ex(P.outer_sum ? (T.reg ? k_eval64_tab<true, true> : k_eval64_tab<true, false>)
                                     : k_eval64_tab<false, false>,
@@ -1853,7 +1895,7 @@ cudaError_t gb_launch_ptab_d(const GbProg& P, const GbPool& pool, const GbParent
                              long long K, int B, GbState* st, cudaStream_t s, bool fixed) {
     // threads for the partial-table entries, warps for the segment entries
     const long long items = std::max<long long>((long long)B * P.n_sum << GB_TAB_DBITS,
-                                                (long long)P.max_nseg << (GB_TAB_SBITS + 5));
+                                                (long long)P.max_srows << 5);
     unsigned g = grid_for(items, 128);
     if (g > (unsigned)gb_sm_count() * 16) g = gb_sm_count() * 16;
     return gb_launch_ex(k_ptab_d, dim3(g, (unsigned)K), 128, 0, s, true, P, pool, par, T, st, fixed ? 1 : 0);

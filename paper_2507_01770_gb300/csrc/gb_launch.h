@@ -114,6 +114,7 @@ struct GbTabs {
     // 1 when every block's dirty groups fit the register-resident walk (at
     // most GB_REG_DIRTY groups of fewer than 2^GB_REG_LEVELS terms each)
     int reg;
+    int dec;          // one child per thread: endpoint programs (P.uops) evaluate the children
 };
 // Paper mode (diagonal samples, first-order test on every coordinate) from
 // per-parent tables.  Kind 0 is the box, kinds 1 .. nk - 1 its sample points
@@ -133,6 +134,15 @@ struct GbPaper {
     const int32_t* hoist_node;
     const GbOIns* oprog;
     uint32_t indep;
+    int dec;          // 1: endpoint programs (P.uops) evaluate the children
+};
+// Tables of the endpoint programs (gb_dec.cuh): kind 0's arrays with the
+// strides of a parent (p) and of the next kind (k).
+struct GbDec {
+    const double2 *tv, *ts, *nd, *hv;
+    long long tvp, tsp, ndp, hvp;
+    long long tvk, tsk, ndk, hvk;
+    int nk;
 };
 constexpr int GB_CG = GB_MAX_ISUM * GB_TAB_MAX_DIRTY;
 constexpr int GB_MV_BITS = 6;
@@ -244,6 +254,13 @@ cudaError_t gb_launch_eval_boxes(const GbProg& P, const double* lo, const double
 cudaError_t gb_launch_eval_boxes_thread(const GbProg& P, const double* lo, const double* hi, float* scratch32,
                                         long long nbox, int blk, int fp32, double* F, double* Fmid, double* G,
                                         int* mono, cudaStream_t s);
+// FP64 children by the interpreter, several threads per child (gb_kernels_box.cu);
+// the last block lists the survivors when there are at most 8192 children.
+// gb_child_box: threads per child, 0 when the program does not fit.
+int gb_child_box(const GbProg& P);
+constexpr long long GB_CHILD_BOX_MAX = 16384;   // children of a generation it takes (more: it returns at once)
+cudaError_t gb_launch_child_box(const GbProg& P, const GbPool& pool, const GbParents& par, const GbChildren& ch,
+                                long long Cmax, const GbSplit& sp, GbState* st, const GbGenConst& G, cudaStream_t s);
 // 1: gb_launch_eval_boxes evaluates nbox boxes with the cooperative kernel, which needs no scratch32.
 int gb_box_coop(const GbProg& P, long long nbox);
 cudaError_t gb_launch_peak(int which, int iters, int blocks, void* sink, cudaStream_t s);
@@ -304,7 +321,7 @@ cudaError_t gb_launch_ptab(const GbProg& P, const GbPool& pool, const GbParents&
                            const GbEntries* Esel = nullptr);
 cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, bool from_list,
-                                 GbState* st, cudaStream_t s);
+                                 GbState* st, cudaStream_t s, const GbGenConst* cc = nullptr);
 // FP32 prefilter + FP64 evaluation fused, one child per warp (tables).
 // Partial tables of every parent (after gb_launch_ptab).
 // fixed: the generation has K parents for certain (do not read the count the partition writes).
