@@ -102,6 +102,13 @@ struct MidView {
     }
 };
 
+// The box (point 0) or its midpoint sample (point 1), per lane.
+struct PointView {
+    View<double> v;
+    int point;
+    __device__ __forceinline__ iv64 get(int j) const { return point ? MidView{v}.get(j) : v.get(j); }
+};
+
 // Diagonal sample point j of S: coordinate i is boundary j of the (S + 1)-piece
 // partition of [lo_i, hi_i], RN(lo + RN(RN(RN(hi - lo) / (S + 1)) * j)) (the
 // split-boundary rounding), j in 1 .. S.

@@ -312,19 +312,24 @@ __global__ void __launch_bounds__(256) k_stats(GbEntries E, GbGenConst G, GbStat
     __shared__ unsigned long long s_c[8], s_k[8];
     __shared__ long long s_q[8];
     __shared__ bool s_last;
+    // blocks without entries (or parents) of their own leave at once: a small
+    // pool's statistics wait for a few blocks, not for the largest pool's grid
+    const long long own = !finish ? st->pool : max(st->parents, st->kept_old + (st->overflow ? st->parents : st->kept));
+    const unsigned nblk = (unsigned)min((long long)gridDim.x, max(1LL, (own + blockDim.x - 1) / blockDim.x));
+    if (blockIdx.x >= nblk) return;
     // at the end of a generation (finish): the parents' slots go back to the
     // free list (on overflow the parents go back into the pool), and the new
     // pool and incumbent are read from the generation's counters; the last
     // block rolls the counters forward
     if (finish) free_parents(par, pool, E, st, blockIdx.x * (long long)blockDim.x + threadIdx.x,
-                             (long long)gridDim.x * blockDim.x);
+                             (long long)nblk * blockDim.x);
     const long long count = !finish ? st->pool
                                     : st->kept_old + (st->overflow ? st->parents : st->kept);
     const double thr = thr_of(gb_key_value(finish ? st->gub_new_key : st->gub_key), G.tol_f);
     long long c = 0, kq = -1;
     unsigned long long kmin = ~0ull;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < count;
-         q += (long long)gridDim.x * blockDim.x) {
+         q += (long long)nblk * blockDim.x) {
         const double f = E.flo[q];
         if (f < thr && !((unsigned)E.cyc[q] & GB_FINAL_BIT)) {
             c++;
@@ -348,11 +353,11 @@ __global__ void __launch_bounds__(256) k_stats(GbEntries E, GbGenConst G, GbStat
         bkey[blockIdx.x] = tk;
         bpos[blockIdx.x] = tq;
     }
-    if (!arrive_last(&st->stats_done, gridDim.x, &s_last)) return;
+    if (!arrive_last(&st->stats_done, nblk, &s_last)) return;
     // last block: combine every block's pair, then start the next generation
     kmin = ~0ull;
     kq = -1;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) better_key(kmin, kq, __ldcg(bkey + b), __ldcg(bpos + b));
+    for (int b = threadIdx.x; b < (int)nblk; b += blockDim.x) better_key(kmin, kq, __ldcg(bkey + b), __ldcg(bpos + b));
     for (int o = 16; o; o >>= 1) {
         const unsigned long long k2 = __shfl_down_sync(0xffffffffu, kmin, o);
         const long long q2 = __shfl_down_sync(0xffffffffu, kq, o);
@@ -369,11 +374,81 @@ __global__ void __launch_bounds__(256) k_stats(GbEntries E, GbGenConst G, GbStat
     open_generation(G, st, active, mk, mq);
 }
 
-// Radix select (16-bit digits, 4 passes) of the K-th smallest active key.
-__global__ void k_radix_hist(GbEntries E, GbGenConst G, int pass, const GbState* st, unsigned* hist) {
+// The K-th smallest active key.  Pools of at most SEL_SMALL entries (most of
+// them: the select used to spend 67 of 150 us a generation in eight launches
+// on pools of a few thousand): one block loads every key once into registers
+// and narrows it down 8 bits at a time over a shared histogram (pass 0; the
+// other passes return).  Larger pools: 16-bit digits, 4 passes over a global
+// histogram, whose last block picks the digit.
+constexpr int SEL_T = 1024, SEL_PER = 16;
+constexpr long long SEL_SMALL = (long long)SEL_T * SEL_PER;
+
+__device__ __forceinline__ void select_small(const GbEntries& E, double thr, long long count, GbState* st) {
+    __shared__ unsigned bins[256];
+    __shared__ unsigned long long s_prefix;
+    __shared__ long long s_rank, s_below, s_ties;
+    const int lane = threadIdx.x & 31;
+    unsigned long long key[SEL_PER];
+    bool act[SEL_PER];
+#pragma unroll
+    for (int u = 0; u < SEL_PER; u++) {
+        const long long q = u * (long long)SEL_T + threadIdx.x;
+        double f = 0.0;
+        int cy = 0;
+        if (q < count) f = E.flo[q], cy = E.cyc[q];
+        act[u] = q < count && f < thr && !((unsigned)cy & GB_FINAL_BIT);
+        key[u] = gb_order_key(f);
+    }
+    if (threadIdx.x == 0) s_prefix = 0, s_rank = st->radix_rank, s_below = 0, s_ties = 0;
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        for (int i = threadIdx.x; i < 256; i += SEL_T) bins[i] = 0;
+        __syncthreads();
+        const unsigned long long prefix = s_prefix;
+#pragma unroll
+        for (int u = 0; u < SEL_PER; u++)
+            if (act[u] && (shift == 56 || (key[u] >> (shift + 8)) == prefix)) atomicAdd(&bins[(key[u] >> shift) & 255u], 1u);
+        __syncthreads();
+        if (threadIdx.x < 32) {   // the bin holding the rank: 8 bins a lane, a scan over the lanes
+            long long c[8], sum = 0;
+            for (int i = 0; i < 8; i++) c[i] = bins[lane * 8 + i], sum += c[i];
+            long long inc = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            const long long rank = s_rank;
+            long long before = inc - sum;
+            __syncwarp();
+            for (int i = 0; i < 8; i++) {
+                if (before < rank && rank <= before + c[i]) {
+                    s_prefix = (prefix << 8) | (unsigned long long)(lane * 8 + i);
+                    s_rank = rank - before;
+                    s_below += before;
+                    s_ties = c[i];
+                }
+                before += c[i];
+            }
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        st->radix_prefix = st->sel_T = s_prefix;
+        st->radix_rank = st->sel_need = s_rank;
+        st->sel_below += s_below;
+        st->sel_ties = s_ties;
+        if (s_ties == 0) st->error |= 1;
+    }
+}
+
+__global__ void __launch_bounds__(SEL_T) k_radix(GbEntries E, GbGenConst G, int pass, GbState* st, unsigned* hist) {
     if (st->halt || st->sel_mode != 2) return;
     const long long count = st->pool;
     const double thr = thr_of(gub_of(st), G.tol_f);
+    if (count <= SEL_SMALL) {
+        if (pass == 0 && blockIdx.x == 0) select_small(E, thr, count, st);
+        return;
+    }
+    __shared__ bool s_last;
     const unsigned long long prefix = st->radix_prefix;
     const int shift = 48 - 16 * pass;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < count;
@@ -384,23 +459,22 @@ __global__ void k_radix_hist(GbEntries E, GbGenConst G, int pass, const GbState*
         if (pass > 0 && (key >> (shift + 16)) != prefix) continue;
         atomicAdd(&hist[(key >> shift) & 0xffffu], 1u);
     }
-}
-
-// One block of 1024 threads (32 warps, each owning 2048 consecutive bins):
-// coalesced warp totals, a scan over the 32 totals, then the owning warp
-// walks its chunk 32 bins at a time.  Clears the histogram for the next pass.
-__global__ void __launch_bounds__(1024) k_radix_pick(int pass, GbState* st, unsigned* hist) {
-    if (st->halt || st->sel_mode != 2) return;
+    if (!arrive_last(&st->stats_done, gridDim.x, &s_last)) return;
+    // the last block: 32 warps, each owning 2048 consecutive bins: warp
+    // totals, a scan over them, then the owning warp walks its chunk 32 bins
+    // at a time; the histogram is cleared for the next pass
     __shared__ long long wtot[32];
     __shared__ long long wpre[33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned* h = hist + w * 2048;
     long long s = 0;
-    for (int k = 0; k < 64; k++) s += h[k * 32 + lane];
+#pragma unroll 16
+    for (int k = 0; k < 64; k++) s += __ldcg(h + k * 32 + lane);
     for (int o = 16; o; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) wtot[w] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
+        st->stats_done = 0;
         long long acc = 0;
         for (int i = 0; i < 32; i++) {
             wpre[i] = acc;
@@ -413,7 +487,7 @@ __global__ void __launch_bounds__(1024) k_radix_pick(int pass, GbState* st, unsi
     if (wpre[w] < rank && rank <= wpre[w] + wtot[w]) {
         long long acc = wpre[w];
         for (int k = 0; k < 64; k++) {
-            long long c = h[k * 32 + lane];
+            long long c = __ldcg(h + k * 32 + lane);
             long long inc = c;
             for (int o = 1; o < 32; o <<= 1) {
                 long long v = __shfl_up_sync(0xffffffffu, inc, o);
@@ -423,7 +497,7 @@ __global__ void __launch_bounds__(1024) k_radix_pick(int pass, GbState* st, unsi
             bool hit = before < rank && rank <= before + c;
             unsigned b = __ballot_sync(0xffffffffu, hit);
             if (hit) {
-                st->radix_prefix = (st->radix_prefix << 16) | (unsigned long long)(w * 2048 + k * 32 + lane);
+                st->radix_prefix = (prefix << 16) | (unsigned long long)(w * 2048 + k * 32 + lane);
                 st->radix_rank = rank - before;
                 st->sel_below += before;
                 if (pass == 3) st->sel_ties = c;   // entries whose whole key equals the threshold
@@ -464,6 +538,7 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(int narr, const int* tile_c
     gb_grid_wait();
     if (what != 3 && st->halt) return;
     if (what == 4 && !st->gc) return;
+    if (what == 2 && st->cc_listed) return;
     __shared__ long long part[1024];
     __shared__ long long tot[3];
     const long long items = what == 3 ? out_count : what == 4 ? st->rec_bump : st->nch;
@@ -768,10 +843,10 @@ __global__ void k_prep(GbProg P, GbPool pool, GbParents par, GbSplit sp, GbState
         st->children = 0;
         st->overflow = 0;
     }
-    const long long npar = st->parents;
-    const long long p = idx / sp.dmax;
-    const int k = (int)(idx - p * sp.dmax);
-    if (p >= npar) return;
+    const long long items = st->parents * sp.dmax;
+    for (long long it = idx; it < items; it += (long long)gridDim.x * blockDim.x) {
+    const long long p = it / sp.dmax;
+    const int k = (int)(it - p * sp.dmax);
     const int n = P.n, B = P.B;
     int c = par.cyc[p] & 0x7fffffff;
     int b = c / B;
@@ -795,6 +870,7 @@ __global__ void k_prep(GbProg P, GbPool pool, GbParents par, GbSplit sp, GbState
             par.bnd_rd[o] = __double2float_rd(v);
             par.bnd_ru[o] = __double2float_ru(v);
         }
+    }
     }
 }
 
@@ -888,8 +964,8 @@ __device__ __forceinline__ bool eval64_child(const GbProg& P, const GbPool& pool
 
 template <bool PR>
 __global__ void __launch_bounds__(128) k_eval64(GbProg P, GbPool pool, GbParents par, GbChildren ch, GbSplit sp,
-                                                int from_list, GbState* st) {
-    if (st->halt) return;
+                                                int from_list, GbState* st, long long above) {
+    if (st->halt || st->nch <= above) return;   // above: smaller generations went to k_child_box
     const long long lim = from_list ? st->n32 : st->nch;
     const double gub_prev = gub_of(st);
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -969,7 +1045,7 @@ __device__ __forceinline__ bool child_pred(const GbChildren& ch, long long i, lo
 __global__ void k_cc_count(GbChildren ch, int mode, const GbState* st, int* tile_cnt) {
     gb_grid_trigger();
     gb_grid_wait();
-    if (st->halt) return;
+    if (st->halt || (mode == 1 && st->cc_listed)) return;
     __shared__ int sw[PT / 32 + 1];
     const long long n = st->nch;
     const double gub_new = gb_key_value(st->gub_new_key);
@@ -988,7 +1064,7 @@ __global__ void k_cc_count(GbChildren ch, int mode, const GbState* st, int* tile
 __global__ void k_cc_scatter(GbChildren ch, int mode, const GbState* st, const int* tile_off, unsigned* out) {
     gb_grid_trigger();
     gb_grid_wait();
-    if (st->halt) return;
+    if (st->halt || (mode == 1 && st->cc_listed)) return;
     __shared__ int sw[PT / 32 + 1];
     const long long n = st->nch;
     const double gub_new = gb_key_value(st->gub_new_key);
@@ -1119,6 +1195,22 @@ __device__ __forceinline__ void materialize_one(const GbProg& P, const GbPool& p
                     pool.gsamp[((size_t)c.slot * pool.S + j) * pool.NG + S.group0 + g];
         }
         for (int g = dr.x; TAB != 2 && g < dr.y; g++, slot_k++) {
+            if constexpr (!TAB && !PR) {   // a small group by the whole warp: F's terms in lanes 0-15, the midpoint's in 16-31
+                const GbGroup G = P.groups[S.group0 + g];
+                if (G.count <= 16 && !pool.gsamp && !pool.fp32) {
+                    const int t = lane & 15;
+                    iv64 v{0.0, 0.0};
+                    if (t < G.count)
+                        v = term_fwd<double>(P, S, S.first + (G.t0 + t) * S.step, PointView{X, lane >> 4}, R, ops);
+                    for (int s2 = 1; s2 < 16; s2 <<= 1) {   // the in-place pairwise tree of each half
+                        const iv64 o = shfl_iv(v, (lane & 16) | ((t + s2) & 15));
+                        if ((t & (2 * s2 - 1)) == 0 && t + s2 < G.count) v = iadd(v, o);
+                    }
+                    if (t == 0)
+                        (lane ? pool.gmid : pool.gsum)[(size_t)ns * pool.NG + S.group0 + g] = make_double2(v.lo, v.hi);
+                    continue;
+                }
+            }
             if ((slot_k & 31) != lane) continue;
             size_t dst = (size_t)ns * pool.NG + S.group0 + g;
             iv64 a, b;
@@ -1176,7 +1268,7 @@ __device__ __forceinline__ void materialize_one(const GbProg& P, const GbPool& p
 __global__ void __launch_bounds__(1024) k_cc_small(GbChildren ch, GbGenConst G, GbState* st) {
     gb_grid_trigger();
     gb_grid_wait();
-    if (st->halt) return;
+    if (st->halt || st->cc_listed) return;
     __shared__ int sw[32];
     const long long S = survivor_list_block(ch, st->nch, gb_key_value(st->gub_new_key), false, sw);
     if (threadIdx.x == 0) set_survivors(G, st, S);
@@ -1792,7 +1884,6 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
                                  const GbFork* fork, const GbPaper* paper) {
     long long n0 = gb_launch_count;
     cudaError_t e;
-    const unsigned gpool = (unsigned)std::min<long long>(grid_for(cap, 256), gb_sm_count() * 8);
     const unsigned gtile_pool = (unsigned)std::min<long long>(grid_for(cap, GB_TILE), gb_sm_count() * 8);
     const unsigned gtile_ch = (unsigned)std::min<long long>(grid_for(Cmax, GB_TILE), gb_sm_count() * 8);
     const unsigned gch = (unsigned)std::min<long long>(grid_for(Cmax, 128), gb_sm_count() * 32);
@@ -1806,10 +1897,12 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
     {
     // (the selection was chosen at the end of the last generation)
     if (G.K > 1) {
-        for (int pass = 0; pass < 4; pass++) {
-            gb_launch_count += 2;
-            k_radix_hist<<<gpool, 256, 0, s>>>(E, G, pass, st, sc.hist);
-            k_radix_pick<<<1, 1024, 0, s>>>(pass, st, sc.hist);
+        // (small pools: block 0 of the first launch does it all)
+        const unsigned gsel = (unsigned)std::min<long long>(grid_for(cap, SEL_T), gb_sm_count() * 2);
+        const int passes = cap <= SEL_SMALL ? 1 : 4;
+        for (int pass = 0; pass < passes; pass++) {
+            gb_launch_count++;
+            k_radix<<<gsel, SEL_T, 0, s>>>(E, G, pass, st, sc.hist);
         }
     }
     // K = 1 with term tables: the parent is the pool entry the last k_stats
@@ -1865,7 +1958,7 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
     }
     if (!tabs) {   // with term tables k_ptab splits the parents itself
         gb_launch_count++;
-        k_prep<<<grid_for(G.K * (long long)sp.dmax, 128), 128, 0, s>>>(P, pool, par, sp, st);
+        k_prep<<<std::min<unsigned>(grid_for(G.K * (long long)sp.dmax, 128), gb_sm_count() * 16), 128, 0, s>>>(P, pool, par, sp, st);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (ev && part == 0) cudaEventRecord(ev[0], s);
         if (paper && (e = gb_launch_paper_tables(P, pool, par, *paper, G.K, sp, st, s)) != cudaSuccess) return e;
@@ -1909,14 +2002,23 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
         }
         if (tabs) {
             gb_launch_count++;
-            if ((e = gb_launch_eval64_tab(P, pool, par, *tabs, ch, Cmax, sp, G.fp32 != 0, st, s)) != cudaSuccess)
+            cc_done = tabs->warp && !G.fp32 && Cmax <= 64LL * 128;
+            if ((e = gb_launch_eval64_tab(P, pool, par, *tabs, ch, Cmax, sp, G.fp32 != 0, st, s, cc_done ? &G : nullptr)) !=
+                cudaSuccess)
                 return e;
         } else if (paper) {
             if ((e = gb_launch_paper_eval(P, pool, par, *paper, ch, Cmax, sp, st, s)) != cudaSuccess) return e;
+        } else if (!G.fp32 && P.samples == 0 && !P.mono_all && gb_child_box(P)) {
+            gb_launch_count++;
+            if ((e = gb_launch_child_box(P, pool, par, ch, Cmax, sp, st, G, s)) != cudaSuccess) return e;
+            if (Cmax > GB_CHILD_BOX_MAX) {
+                gb_launch_count++;
+                k_eval64<false><<<gch, 128, 0, s>>>(P, pool, par, ch, sp, 0, st, GB_CHILD_BOX_MAX);
+            }
         } else {
             gb_launch_count++;
-            if (P.any_prod) k_eval64<true><<<gch, 128, 0, s>>>(P, pool, par, ch, sp, G.fp32, st);
-            else k_eval64<false><<<gch, 128, 0, s>>>(P, pool, par, ch, sp, G.fp32, st);
+            if (P.any_prod) k_eval64<true><<<gch, 128, 0, s>>>(P, pool, par, ch, sp, G.fp32, st, 0);
+            else k_eval64<false><<<gch, 128, 0, s>>>(P, pool, par, ch, sp, G.fp32, st, 0);
         }
         if (ev) cudaEventRecord(ev[1], s);
     }
@@ -1924,6 +2026,8 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
 after_eval:
     if (cc_done) {
         // (listed by the child kernel's last block)
+    } else if (Cmax <= 64LL * 128 && !tabs && !paper && !G.fp32 && P.samples == 0 && !P.mono_all && gb_child_box(P)) {
+        // (always listed by the child kernel's last block)
     } else if (Cmax <= (1LL << 16)) {
         gb_launch_count++;
         if ((e = gb_launch_ex(k_cc_small, 1, 1024, 0, s, true, ch, G, st)) != cudaSuccess) return e;

@@ -19,7 +19,7 @@
 
 #include <algorithm>
 
-#include "gb_eval.cuh"
+#include "gb_child.cuh"
 #include "gb_launch.h"
 
 using namespace gb;
@@ -330,6 +330,224 @@ BoxPick box_pick(const GbProg& P, long long nbox) {
     return none;
 }
 
+// ---------------------------------------------------------------------------
+// FP64 children of small programs (no term tables: fewer than 16 children a
+// parent), W threads per child: the terms of the dirty groups, F and midpoint
+// side by side, the clean groups from the parent's cache, then the trees, the
+// outer expression and the block's partials as in k_box.  A generation of
+// such a solve holds a few dozen children, so it waits for one child's chain:
+// one thread per child walked midpoint, F and partials one term after the
+// other (n = 2: 70 us a generation).  W <= 16, so warps never wait for one
+// another, and every loop around a __syncwarp has the same trip count in all
+// lanes whatever their children's blocks.  Generations above
+// GB_CHILD_BOX_MAX children fill the chip one thread per child (which tests
+// only the children that pass the cut-off): k_eval64.
+template <typename C>
+__global__ void __launch_bounds__(128) k_child_box(GbProg P, GbPool pool, GbParents par, GbChildren ch, GbSplit sp,
+                                                   GbState* st, GbGenConst G) {
+    constexpr int W = C::W, TT = C::TT, CH = C::CH, BPB = C::BPB;
+    if (st->halt) return;
+    if (st->nch > GB_CHILD_BOX_MAX) {   // k_eval64 takes them
+        if (blockIdx.x == 0 && threadIdx.x == 0) st->cc_listed = 0;
+        return;
+    }
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x % W, bx = threadIdx.x / W;
+    GbIns* s_ins = (GbIns*)smem;
+    int* s_leaf = (int*)(s_ins + P.n_tins);
+    {
+        const int4* src = (const int4*)P.tins;
+        int4* dst = (int4*)s_ins;
+        for (int i = threadIdx.x; i < P.n_tins * (int)(sizeof(GbIns) / 16); i += blockDim.x) dst[i] = src[i];
+        __syncthreads();
+        if ((int)threadIdx.x < P.n_sum) {
+            const GbSum S = P.sums[threadIdx.x];
+            int l = 0;
+            for (int t = 0; t < S.nins; t++)
+                if (s_ins[S.ins0 + t].op == D_IVAR) s_leaf[threadIdx.x * GB_MAX_TREGS + l++] = s_ins[S.ins0 + t].aux;
+        }
+    }
+    unsigned char* q = (unsigned char*)(s_leaf + GB_MAX_ISUM * GB_MAX_TREGS) + bx * ((box_smem<C, iv64>(P) + 15) / 16 * 16);
+    auto take = [&](size_t bytes) {
+        unsigned char* r = q;
+        q += bytes;
+        return r;
+    };
+    iv64* v64 = (iv64*)take(2 * (size_t)TT * 16);   // [F | midpoint]
+    iv64* gmid = (iv64*)take((size_t)P.n_groups * 16);
+    iv64* oa = (iv64*)take((size_t)GB_MAX_OREGS * 16);
+    iv64* gF = (iv64*)take((size_t)P.n_groups * 16);
+    iv64* acc = (iv64*)take((size_t)P.n_sum * CH * 16);
+    iv64* adj = (iv64*)take((size_t)(CH + GB_MAX_WIN) * P.box_leaves * 16);
+    ushort2* place = (ushort2*)take((size_t)TT * 4);
+    int* s_mono = (int*)take(16);
+    unsigned char* touched = take((size_t)P.n_sum * CH);
+    __syncthreads();
+
+    const long long nch = st->nch;
+    const double gub_prev = gb_key_value(st->gub_key);
+    unsigned long long key = ~0ull, nv = 0;
+    int ops = 0;
+    iv64 R[GB_MAX_TREGS];
+    const int wfirst = (threadIdx.x & ~31) / W;   // the warp's first slot
+    for (long long base = (long long)blockIdx.x * BPB; base + wfirst < nch; base += (long long)gridDim.x * BPB) {
+        const long long ci0 = base + bx;
+        const bool in = ci0 < nch;
+        const long long ci = in ? ci0 : nch - 1;   // (a spare slot repeats the last child, unwritten)
+        const ChildCtx c = child_ctx(par, ci, sp);
+        const int blk = c.info.z;
+        const View<double> X = view64(pool, par, c, sp);
+        const CacheRef<double2> cf = cache64(pool, P, c.slot, 0), cm = cache64(pool, P, c.slot, 1);
+        for (int k = 0; k < P.n_sum; k++) {
+            const GbSum S = P.sums[k];
+            const int2 dr = P.dirty[blk * P.n_sum + k];
+            const GbGroup* GR = P.groups + S.group0;
+            for (int g = lane; g < S.ngroups; g += W)
+                if (g < dr.x || g >= dr.y) {
+                    const double2 a = cf[S.group0 + g], b = cm[S.group0 + g];
+                    gF[S.group0 + g] = iv64{a.x, a.y};
+                    gmid[S.group0 + g] = iv64{b.x, b.y};
+                }
+            const int t0 = dr.x < dr.y ? GR[dr.x].t0 : 0;
+            const int nt = dr.x < dr.y ? GR[dr.y - 1].t0 + GR[dr.y - 1].count - t0 : 0;
+            for (int t = lane; t < nt; t += W) {
+                int g = dr.x;
+                while (g + 1 < dr.y && GR[g + 1].t0 <= t0 + t) g++;
+                place[t] = make_ushort2((unsigned short)(t0 + t - GR[g].t0), (unsigned short)GR[g].count);
+            }
+            for (int it = lane; it < 2 * nt; it += W) {
+                const int role = it >= nt ? 1 : 0, t = it - role * nt;
+                v64[role * TT + t] = term_fwd<double>(P, S, S.first + (t0 + t) * S.step, PointView{X, role}, R, ops,
+                                                      s_ins + S.ins0);
+            }
+            __syncwarp();
+            for (int s = 1; s < TT; s <<= 1) {
+                for (int t = lane; t < nt; t += W) {
+                    const ushort2 pl = place[t];
+                    if ((pl.x & (2 * s - 1)) == 0 && pl.x + s < pl.y) {
+                        v64[t] = iadd(v64[t], v64[t + s]);
+                        v64[TT + t] = iadd(v64[TT + t], v64[TT + t + s]);
+                    }
+                }
+                __syncwarp();
+            }
+            for (int g = dr.x + lane; g < dr.y; g += W) {
+                gF[S.group0 + g] = v64[GR[g].t0 - t0];
+                gmid[S.group0 + g] = v64[TT + GR[g].t0 - t0];
+            }
+            __syncwarp();
+        }
+        for (int k = 0; k < P.n_sum; k++) {
+            const GbSum S = P.sums[k];
+            iv64* f = gF + S.group0;
+            iv64* m = gmid + S.group0;
+            for (int s = 1; s < S.ngroups; s <<= 1) {
+                for (int g = lane * 2 * s; g + s < S.ngroups; g += W * 2 * s) {
+                    f[g] = iadd(f[g], f[g + s]);
+                    m[g] = iadd(m[g], m[g + s]);
+                }
+                __syncwarp();
+            }
+        }
+        iv64 F{0.0, 0.0};
+        if (lane < 2) {   // lane 0: F and its adjoints, lane 1: the midpoint sample
+            iv64 sums[GB_MAX_ISUM], O[GB_MAX_OREGS];
+            for (int k = 0; k < P.n_sum; k++) {
+                const GbSum S = P.sums[k];
+                sums[k] = S.ngroups ? (lane ? gmid : gF)[S.group0] : iv64{0.0, 0.0};
+            }
+            F = outer_fwd<double>(P, PointView{X, lane}, sums, O, ops);
+            if (lane == 0) {
+                iv64 OA[GB_MAX_OREGS];
+                for (int t = 0; t < P.n_outer; t++) OA[t] = iv64{0.0, 0.0};
+                OA[P.outer_root] = iv64{1.0, 1.0};
+                reverse_sweep<double>(P.outer, P.n_outer, O, OA, ops);
+                for (int t = 0; t < P.n_outer; t++) oa[t] = OA[t];
+                *s_mono = 0;
+            } else if (in && c.valid && F.hi == F.hi) {
+                const unsigned long long k2 = gb_order_key(F.hi);
+                key = k2 < key ? k2 : key;
+            }
+        }
+        __syncwarp();
+        const int c0 = blk * P.B, c1 = min(P.n, c0 + P.B);   // (at most CH coordinates)
+        for (int k = 0; k < P.n_sum; k++) {
+            const GbSum S = P.sums[k];
+            if (!S.has_var) {
+                for (int jj = lane; jj < c1 - c0; jj += W) touched[k * CH + jj] = 0;
+                continue;
+            }
+            const GbIns* ins = s_ins + S.ins0;
+            const int a = c0 - S.off_max - S.first, z = c1 - 1 - S.off_min - S.first;
+            const int ta = a <= 0 ? 0 : (a + S.step - 1) / S.step;
+            const int tz = z < 0 ? 0 : min(S.count, z / S.step + 1);
+            for (int t = ta + lane; t < tz; t += W) {
+                iv64 RA[GB_MAX_TREGS];
+                term_fwd<double>(P, S, S.first + t * S.step, X, R, ops, ins);
+                for (int i = 0; i < S.nins; i++) RA[i] = iv64{0.0, 0.0};
+                RA[S.nins - 1] = iv64{1.0, 1.0};
+                reverse_sweep<double>(ins, S.nins, R, RA, ops);
+                int l = 0;
+                for (int i = 0; i < S.nins; i++)
+                    if (ins[i].op == D_IVAR) adj[(t - ta) * P.box_leaves + l++] = RA[i];
+            }
+            __syncwarp();
+            for (int jj = lane; jj < c1 - c0; jj += W) {
+                const int j = c0 + jj;
+                const int ja = j - S.off_max - S.first, jz = j - S.off_min - S.first;
+                const int a2 = ja <= 0 ? 0 : (ja + S.step - 1) / S.step;
+                const int z2 = jz < 0 ? 0 : min(S.count, jz / S.step + 1);
+                iv64 w{0.0, 0.0};
+                bool any = false;
+                for (int t = a2; t < z2; t++)
+                    for (int l = 0; l < S.nvar_leaves; l++)
+                        if (S.first + t * S.step + s_leaf[k * GB_MAX_TREGS + l] == j) {
+                            w = iadd(w, adj[(t - ta) * P.box_leaves + l]);
+                            any = true;
+                        }
+                acc[k * CH + jj] = w;
+                touched[k * CH + jj] = any ? 1 : 0;
+            }
+            __syncwarp();
+        }
+        bool hit = false;
+        for (int jj = lane; jj < c1 - c0; jj += W) {
+            const int j = c0 + jj;
+            iv64 g{0.0, 0.0};
+            for (int v = 0; v < P.n_var_leaves; v++) {
+                const GbVarLeaf V = P.var_leaves[v];
+                if (V.coord == j) g = iadd(g, oa[V.reg]);
+            }
+            for (int k = 0; k < P.n_sum; k++)
+                if (touched[k * CH + jj]) g = iadd(g, imul(oa[P.sums[k].outer_reg], acc[k * CH + jj]));
+            if (!gt_zero(g.lo) && !lt_zero(g.hi)) continue;
+            const iv64 x = X.get(j);
+            hit |= (gt_zero(g.lo) && !same_value(x.lo, __ldg(P.l + j))) ||
+                   (lt_zero(g.hi) && !same_value(x.hi, __ldg(P.u + j)));
+        }
+        if (hit) atomicOr(s_mono, 1);
+        __syncwarp();
+        if (lane == 0 && in) {
+            const bool keep = c.valid && !(F.lo > gub_prev) && *s_mono == 0;
+            ch.flo[ci] = c.valid ? canon_lo(F.lo) : __longlong_as_double(0x7ff0000000000000LL);
+            ch.flag[ci] = keep ? 1 : 0;
+            if (c.valid) nv++;
+        }
+        __syncwarp();
+    }
+    warp_min_gub(key, key != ~0ull, st);
+    warp_add_ops(ops, &st->ops64);
+    for (int o = 16; o; o >>= 1) nv += __shfl_down_sync(0xffffffffu, nv, o);
+    if ((threadIdx.x & 31) == 0 && nv) {
+        atomicAdd((unsigned long long*)&st->evals64, nv);
+        atomicAdd((unsigned long long*)&st->mids, nv);
+        atomicAdd((unsigned long long*)&st->children, nv);
+    }
+    const bool list = nch <= 64LL * 128;
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->cc_listed = list ? 1 : 0;
+    if (list) list_survivors_last(ch, nch, G, st);
+}
+
 template <typename C, typename T>
 cudaError_t launch_box(const GbProg& P, int list, const double* lo, const double* hi, long long nbox, int blk,
                        double* F, double* Fmid, double* G, int* mono, cudaStream_t s) {
@@ -361,6 +579,41 @@ cudaError_t launch_pick(const GbProg& P, BoxPick k, const double* lo, const doub
 extern thread_local long long gb_launch_count;   // kernels launched by this thread (gb_kernels.cu)
 
 int gb_box_coop(const GbProg& P, long long nbox) { return box_pick(P, nbox).cfg >= 0 ? 1 : 0; }
+
+// The dirty terms of a sum, the block's coordinates and the groups must fit a
+// child's share of shared memory (W = 16: a warp per two children).
+int gb_child_box(const GbProg& P) {
+    if (P.any_prod || P.n_groups > 64) return 0;
+    const int need = std::max(P.max_dirty_terms, P.B);
+    if (need <= 4 && box_smem_block<Cfg4, iv64>(P) <= 100 * 1024) return 4;
+    if (need <= 8 && box_smem_block<Cfg8, iv64>(P) <= 100 * 1024) return 8;
+    if (need <= 16 && box_smem_block<Cfg16, iv64>(P) <= 100 * 1024) return 16;
+    return 0;
+}
+
+namespace {
+template <typename C>
+cudaError_t launch_child_box(const GbProg& P, const GbPool& pool, const GbParents& par, const GbChildren& ch,
+                             long long Cmax, const GbSplit& sp, GbState* st, const GbGenConst& G, cudaStream_t s) {
+    const size_t smem = box_smem_block<C, iv64>(P);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_child_box<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const unsigned g = (unsigned)std::min<long long>((Cmax + C::BPB - 1) / C::BPB, gb_sm_count() * 8);
+    k_child_box<C><<<g, 128, smem, s>>>(P, pool, par, ch, sp, st, G);
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t gb_launch_child_box(const GbProg& P, const GbPool& pool, const GbParents& par, const GbChildren& ch,
+                                long long Cmax, const GbSplit& sp, GbState* st, const GbGenConst& G, cudaStream_t s) {
+    switch (gb_child_box(P)) {
+    case 4: return launch_child_box<Cfg4>(P, pool, par, ch, Cmax, sp, st, G, s);
+    case 8: return launch_child_box<Cfg8>(P, pool, par, ch, Cmax, sp, st, G, s);
+    default: return launch_child_box<Cfg16>(P, pool, par, ch, Cmax, sp, st, G, s);
+    }
+}
 
 cudaError_t gb_launch_eval_boxes(const GbProg& P, const double* lo, const double* hi, float* scratch32,
                                  long long nbox, int blk, int fp32, double* F, double* Fmid, double* G, int* mono,
