@@ -351,7 +351,6 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     GbVarLeaf* d_leaves;
     double *d_l, *d_u;
     if ((e = upload(&d_outer, H.outer.data(), H.outer.size(), A))) return bad(e, "upload program");
-    if ((e = upload(&d_tins, H.tins.data(), H.tins.size(), A))) return bad(e, "upload program");
     if ((e = upload(&d_sums, H.sums.data(), H.sums.size(), A))) return bad(e, "upload program");
     if ((e = upload(&d_groups, H.groups.data(), H.groups.size(), A))) return bad(e, "upload program");
     if ((e = upload(&d_dirty, H.dirty.data(), H.dirty.size(), A))) return bad(e, "upload program");
@@ -376,7 +375,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     }
     if ((e = upload(&d_l, l, (size_t)n, A))) return bad(e, "upload bounds");
     if ((e = upload(&d_u, u, (size_t)n, A))) return bad(e, "upload bounds");
-    std::vector<const double*> t64(n_tables > 0 ? n_tables : 1, nullptr);  // kept until the final sync
+    std::vector<const double*> t64(n_tables > 0 ? n_tables : 1, nullptr);
     std::vector<const float2*> t32(n_tables > 0 ? n_tables : 1, nullptr);
     for (int t = 0; t < n_tables; t++) {
         double* d64;
@@ -389,18 +388,16 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         t64[t] = d64;
         t32[t] = d32;
     }
-    const double** d_t64;
-    const float2** d_t32;
-    if ((e = upload(&d_t64, t64.data(), t64.size(), A))) return bad(e, "upload tables");
-    if ((e = upload(&d_t32, t32.data(), t32.size(), A))) return bad(e, "upload tables");
+    std::vector<GbIns> tins = H.tins;   // kept until the final sync
+    for (GbIns& I : tins)
+        if (I.op == D_COEF) I.coef64 = t64[I.aux], I.coef32 = t32[I.aux];
+    if ((e = upload(&d_tins, tins.data(), tins.size(), A))) return bad(e, "upload program");
     P.outer = d_outer;
     P.tins = d_tins;
     P.sums = d_sums;
     P.groups = d_groups;
     P.dirty = d_dirty;
     P.var_leaves = d_leaves;
-    P.tab64 = d_t64;
-    P.tab32 = d_t32;
     P.l = d_l;
     P.u = d_u;
     int2* d_gown;
@@ -597,7 +594,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             }
             T.max_sum_nodes = 1;
             for (const GbSum& S : Hh.sums) T.max_sum_nodes = std::max(T.max_sum_nodes, (int)S.nnodes);
-            // no opt-in needed: the table kernel's static shared memory (about 7 KB) and the
+            // no opt-in needed: the table kernel's static shared memory (about 12 KB) and the
             // trees stay within the 48 KB a launch gets by default
             T.tree_smem = (size_t)T.max_sum_nodes * sizeof(double2) <= 32 * 1024 ? 1 : 0;
             if (T.warp) {   // per-child sums and dirty group values (k_child_sums)

@@ -120,6 +120,46 @@ bool mark_template(Ctx& c, int v, std::string& err) {
     return true;
 }
 
+// The GB_RV_* bits of a program (registers are the instruction indices; every
+// node but the last has a consumer after it).
+void mark_reverse(GbIns* ins, int n) {
+    std::vector<char> val(n, 0), seen(n, 0);
+    auto live = [&](int t) { return (ins[t].pad & GB_RV_LIVE) != 0; };
+    auto is_bin = [](int op) { return op == D_ADD || op == D_SUB || op == D_MUL || op == D_DIV; };
+    auto is_leaf = [](int op) { return op <= D_ISUMV; };
+    for (int t = 0; t < n; t++) {
+        GbIns& I = ins[t];
+        const bool leaf = is_leaf(I.op);
+        const bool la = !leaf && live(I.a), lb = !leaf && is_bin(I.op) && live(I.b);
+        if (I.op == D_VAR || I.op == D_IVAR || I.op == D_ISUMV || la || lb) I.pad |= GB_RV_LIVE;
+        if (la) I.pad |= GB_RV_A;
+        if (lb) I.pad |= GB_RV_B;
+    }
+    for (int t = n - 1; t >= 0; t--) {   // the sweep's order: a push into a, then into b
+        GbIns& I = ins[t];
+        if (!live(t)) continue;
+        if ((I.pad & GB_RV_A) && !seen[I.a]) seen[I.a] = 1, I.pad |= GB_RV_A0;
+        if ((I.pad & GB_RV_B) && !seen[I.b]) seen[I.b] = 1, I.pad |= GB_RV_B0;
+        switch (I.op) {   // values the push reads
+        case D_MUL:
+            if (I.pad & GB_RV_A) val[I.b] = 1;
+            if (I.pad & GB_RV_B) val[I.a] = 1;
+            break;
+        case D_DIV: val[I.b] = val[t] = 1; break;
+        case D_SQR: case D_SIN: case D_COS: case D_STEP: val[I.a] = 1; break;
+        case D_EXP: case D_SQRT: val[t] = 1; break;
+        default: break;
+        }
+    }
+    for (int t = n - 1; t >= 0; t--) {   // and what those are computed from
+        if (!val[t]) continue;
+        ins[t].pad |= GB_RV_VAL;
+        if (is_leaf(ins[t].op)) continue;
+        val[ins[t].a] = 1;
+        if (is_bin(ins[t].op)) val[ins[t].b] = 1;
+    }
+}
+
 }  // namespace
 
 std::string gb_compile(const gb_node* nd, int32_t nn, int32_t root, const int64_t* tlen,
@@ -217,6 +257,7 @@ std::string gb_compile(const gb_node* nd, int32_t nn, int32_t root, const int64_
             P->tins.push_back(J);
         }
         S.nins = (int)P->tins.size() - S.ins0;
+        mark_reverse(P->tins.data() + S.ins0, S.nins);
         if (S.nins > GB_MAX_TREGS) return "sum template exceeds the register limit";
         if (treg[q.a] != S.nins - 1) return "internal: template root is not last";
         S.first = q.b;
@@ -250,6 +291,7 @@ std::string gb_compile(const gb_node* nd, int32_t nn, int32_t root, const int64_
         S.ngroups = (int)P->groups.size() - S.group0;
         P->sums.push_back(S);
     }
+    mark_reverse(P->outer.data(), (int)P->outer.size());
     // dirty group ranges per block (local indices within each sum)
     int ns = (int)P->sums.size();
     P->dirty.assign((size_t)P->nb * ns, int2{0, 0});

@@ -26,16 +26,16 @@ namespace gb {
 template <typename T> struct Prec;
 template <> struct Prec<double> {
     typedef iv64 I;
-    static __device__ __forceinline__ I coef(const GbProg& P, int t, int idx) {
-        double c = __ldg(P.tab64[t] + idx);
+    static __device__ __forceinline__ I coef(const GbIns& in, int i) {
+        const double c = __ldg(in.coef64 + i + in.aux2);
         return I{c, c};
     }
     static __device__ __forceinline__ I cst(const GbIns& in) { return I{in.c, in.c}; }
 };
 template <> struct Prec<float> {
     typedef iv32 I;
-    static __device__ __forceinline__ I coef(const GbProg& P, int t, int idx) {
-        float2 c = __ldg(P.tab32[t] + idx);
+    static __device__ __forceinline__ I coef(const GbIns& in, int i) {
+        const float2 c = __ldg(in.coef32 + i + in.aux2);
         return I{c.x, c.y};
     }
     static __device__ __forceinline__ I cst(const GbIns& in) { return I{in.clo32, in.chi32}; }
@@ -233,7 +233,9 @@ template <typename I> __device__ __noinline__ void slow_rev_pair(int op, I g, I 
 // `sins` / `pre` (both or neither): the template's instructions and the
 // values of its coordinate and coefficient loads, staged by stage_term.
 // PAIR: run by lanes 0 and 1 of a warp together (slow_fwd_pair).
-template <typename T, typename V, bool PAIR = false>
+// VALS: only the nodes whose values the reverse sweep needs (the root may not
+// be one of them).
+template <typename T, typename V, bool PAIR = false, bool VALS = false>
 __device__ __forceinline__ typename Prec<T>::I term_fwd(const GbProg& P, const GbSum& S, int i,
                                                          const V& X, typename Prec<T>::I* R, int& ops,
                                                          const GbIns* sins = nullptr,
@@ -242,6 +244,7 @@ __device__ __forceinline__ typename Prec<T>::I term_fwd(const GbProg& P, const G
     const GbIns* ins = sins ? sins : P.tins + S.ins0;
     for (int t = 0; t < S.nins; t++) {
         GbIns in = ins[t];
+        if (VALS && !(in.pad & GB_RV_VAL)) continue;
         ops += in.pad & 0xff;
         I v;
         switch (in.op) {
@@ -249,7 +252,7 @@ __device__ __forceinline__ typename Prec<T>::I term_fwd(const GbProg& P, const G
         case D_PI: v = pi_iv((T)0); break;
         case D_EULER: v = e_iv((T)0); break;
         case D_IVAR: v = pre ? pre[t] : X.get(i + in.aux); break;
-        case D_COEF: v = pre ? pre[t] : Prec<T>::coef(P, in.aux, i + in.aux2); break;
+        case D_COEF: v = pre ? pre[t] : Prec<T>::coef(in, i); break;
         case D_ADD: v = iadd(R[in.a], R[in.b]); break;
         case D_SUB: v = isub(R[in.a], R[in.b]); break;
         case D_MUL: v = imul(R[in.a], R[in.b]); break;
@@ -274,77 +277,76 @@ __device__ __forceinline__ typename Prec<T>::I term_fwd(const GbProg& P, const G
     return R[S.nins - 1];
 }
 
-// Warp-cooperative staging for term_fwd: lane t (t < nins) loads instruction
-// t of the template into `sins` and, for a coordinate or coefficient load,
-// its value into `pre` -- the loads of all instructions in flight at once,
-// instead of one after the other in the interpreter loop.  Every lane of the
-// warp calls it (the views are the same in every lane).
+// Warp-cooperative staging for term_fwd: lane t (t < nins) loads the value of
+// instruction t of the template into `pre` when it is a coordinate or a
+// coefficient (vals: one that the reverse sweep needs) -- the loads of all
+// instructions in flight at once, instead of one after the other in the
+// interpreter loop.  Every lane of the warp calls it (the views are the same
+// in every lane).
 template <typename T, typename V>
-__device__ __forceinline__ void stage_term(const GbProg& P, const GbSum& S, int i, const V& X, GbIns* sins,
+__device__ __forceinline__ void stage_term(const GbIns* ins, int nins, int i, const V& X, bool vals,
                                            typename Prec<T>::I* pre, int lane) {
-    if (lane < S.nins) {
-        const GbIns in = P.tins[S.ins0 + lane];
-        sins[lane] = in;
+    if (lane < nins && (!vals || (ins[lane].pad & GB_RV_VAL))) {
+        const GbIns in = ins[lane];
         if (in.op == D_IVAR) pre[lane] = X.get(i + in.aux);
-        else if (in.op == D_COEF) pre[lane] = Prec<T>::coef(P, in.aux, i + in.aux2);
+        else if (in.op == D_COEF) pre[lane] = Prec<T>::coef(in, i);
     }
     __syncwarp();
 }
 
-// Reverse sweep over a bytecode list (forward values V, adjoints A already
+// A push of d into an adjoint: its first one is [0, 0] + d without the two
+// additions (RU(+0 + -0) is +0, the other sums are d's own ends).
+template <typename I> __device__ __forceinline__ void adj_push(I& A, I d, bool first) {
+    if (first) {
+        A.lo = d.lo;
+        A.hi = zero_bits(d.hi) ? (decltype(d.hi))0 : d.hi;
+    } else {
+        A = iadd(A, d);
+    }
+}
+
+// Reverse sweep over a bytecode list (forward values V, the root's adjoint
 // seeded).  Node t pushes into its first, then its second operand; a node's
 // adjoint thus receives its consumers' contributions in descending order.
+// Adjoints that no coordinate or reduction receives (of constants and
+// coefficients) are not formed.
 template <typename T, bool PAIR = false>
 __device__ __forceinline__ void reverse_sweep(const GbIns* ins, int nins, const typename Prec<T>::I* V,
                                               typename Prec<T>::I* A, int& ops) {
     typedef typename Prec<T>::I I;
     for (int t = nins - 1; t >= 0; t--) {
-        GbIns in = ins[t];
+        const GbIns in = ins[t];
         ops += (in.pad >> 8) & 0xff;
-        I g = A[t];
+        if (!(in.pad & (GB_RV_A | GB_RV_B))) continue;   // a leaf, or constants only
+        const I g = A[t];
+        I da = g, db = g;
         switch (in.op) {
-        case D_ADD:
-            A[in.a] = iadd(A[in.a], g);
-            A[in.b] = iadd(A[in.b], g);
-            break;
         case D_SUB:
-            A[in.a] = iadd(A[in.a], g);
-            A[in.b] = iadd(A[in.b], ineg(g));
+            db = ineg(g);
             break;
-        case D_MUL: {
-            I va = V[in.a], vb = V[in.b];
-            A[in.a] = iadd(A[in.a], imul(g, vb));
-            A[in.b] = iadd(A[in.b], imul(g, va));
+        case D_MUL:
+            if (in.pad & GB_RV_A) da = imul(g, V[in.b]);
+            if (in.pad & GB_RV_B) db = imul(g, V[in.a]);
             break;
-        }
-        case D_DIV: {
-            I da, db;
-            slow_rev(in.op, g, V[in.a], V[in.b], V[t], &da, &db);
-            A[in.a] = iadd(A[in.a], da);
-            A[in.b] = iadd(A[in.b], db);
-            break;
-        }
-        case D_NEG: A[in.a] = iadd(A[in.a], ineg(g)); break;
-        case D_SQR: A[in.a] = iadd(A[in.a], imul(g, iscale(V[in.a], (T)2))); break;
-        case D_EXP: A[in.a] = iadd(A[in.a], imul(g, V[t])); break;
+        case D_DIV: slow_rev(in.op, g, V[in.a], V[in.b], V[t], &da, &db); break;
+        case D_NEG: da = ineg(g); break;
+        case D_SQR: da = imul(g, iscale(V[in.a], (T)2)); break;
+        case D_EXP: da = imul(g, V[t]); break;
         case D_SQRT:
         case D_SIN:
         case D_STEP:
-        case D_COS: {
-            I da, db;
+        case D_COS:
             if (PAIR) slow_rev_pair(in.op, g, V[in.a], V[in.a], V[t], &da, &db);
             else slow_rev(in.op, g, V[in.a], V[in.a], V[t], &da, &db);
-            A[in.a] = iadd(A[in.a], da);
             break;
-        }
         case D_SCALE:
-            if (in.clo32 == in.chi32 || sizeof(T) == 8)
-                A[in.a] = iadd(A[in.a], iscale(g, sizeof(T) == 8 ? (T)in.c : (T)in.clo32));
-            else
-                A[in.a] = iadd(A[in.a], imul(g, mk<T>((T)in.clo32, (T)in.chi32)));
+            if (in.clo32 == in.chi32 || sizeof(T) == 8) da = iscale(g, sizeof(T) == 8 ? (T)in.c : (T)in.clo32);
+            else da = imul(g, mk<T>((T)in.clo32, (T)in.chi32));
             break;
-        default: break;
+        default: break;   // D_ADD
         }
+        if (in.pad & GB_RV_A) adj_push(A[in.a], da, (in.pad & GB_RV_A0) != 0);
+        if (in.pad & GB_RV_B) adj_push(A[in.b], db, (in.pad & GB_RV_B0) != 0);
     }
 }
 

@@ -43,11 +43,27 @@ struct GbIns {
     uint8_t a, b;     // operand registers
     int32_t aux;      // VAR coordinate | IVAR offset | COEF table | ISUMV slot
     int32_t aux2;     // COEF offset
-    float clo32;      // c rounded down to float
-    float chi32;      // c rounded up to float
-    int32_t pad;      // directed-op cost: forward (bits 0-7), reverse (bits 8-15)
-    double c;         // CONST value | SCALE factor
+    int32_t pad;      // directed-op cost: forward (bits 0-7), reverse (bits 8-15); GB_RV_* (bits 16-21)
+    union {           // COEF (on the device): its table, directly (one dependent load less than a table of tables)
+        struct {
+            float clo32, chi32;   // c rounded down / up to float
+        };
+        const float2* coef32;     // outward float pairs (lo, hi)
+    };
+    union {
+        double c;     // CONST value | SCALE factor
+        const double* coef64;
+    };
 };  // 32 bytes
+// What the reverse sweep can leave out (set by the compiler).  A node carries
+// an adjoint when a coordinate or a reduction lies below it; the others'
+// adjoints are read by nobody.
+#define GB_RV_LIVE (1 << 16)     // the node carries an adjoint
+#define GB_RV_A (1 << 17)        // its first operand carries one
+#define GB_RV_B (1 << 18)        // its second
+#define GB_RV_A0 (1 << 19)       // the push into the first operand is that operand's first
+#define GB_RV_B0 (1 << 20)
+#define GB_RV_VAL (1 << 21)      // the reverse sweep reads the node's value (or computes one from it)
 
 // One ISUM (or IPROD) node: its template bytecode and the grouping of its terms.
 // Terms are grouped into maximal runs with the same range of touched
@@ -198,8 +214,6 @@ struct GbProg {
     const GbGroup* groups;           // [n_groups]
     const int2* dirty;               // [nb * n_sum]: dirty local group range per block
     const GbVarLeaf* var_leaves;     // [n_var_leaves]
-    const double* const* tab64;      // [n_tables] table pointers
-    const float2* const* tab32;      // [n_tables] outward float pairs (lo, hi)
     const double* l;                 // [n]
     const double* u;                 // [n]
     // block records (pool mode 2): group -> (owner block, index in its record)

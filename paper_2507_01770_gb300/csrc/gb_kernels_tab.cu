@@ -57,25 +57,31 @@ __device__ __forceinline__ iv64 mid_node(const GbTabs& T, size_t i) { double2 v 
 // ---------------------------------------------------------------------------
 // k_ptab: per parent (blockIdx.y).  Blocks x < row_blocks: table row parts,
 // PTAB_ITEMS per block (one warp) -- rows are (dirty term, digit
-// combination) and each row has up to three independent parts: 0 the FP64
-// value and leaf adjoints (one forward pass, then the reverse sweep), 1 the
-// midpoint value, 2 the FP32 value and leaf adjoints.  A part is one serial
-// chain of FP64 work (a template's interval operations, transcendentals
-// included).  On GB300 a dependent FP64 operation takes ~30 ns and a warp's
-// FP64 instruction holds the SM's FP64 pipe for ~16 clocks whatever its
-// active lanes, so each part gets a warp of its own (parts in one warp would
-// diverge and run one after the other), spread over the SMs.  The warp's
-// lanes first stage the template's instructions and its coordinate and
-// coefficient values in shared memory (all loads in flight at once), then
-// lanes 0 and 1 interpret it together: both run every operation, and exp,
-// sin and cos evaluate their two endpoints one per lane (itrig_pair).
+// combination) and each row has up to five independent parts: 0 the FP64
+// value, 1 the midpoint value, 2 the FP64 leaf adjoints (the nodes the
+// reverse sweep reads, then the sweep), 3 the FP32 value, 4 the FP32 leaf
+// adjoints.  A part is one serial chain of FP64 work (a template's interval
+// operations, transcendentals included), so each gets a warp of its own
+// (parts in one warp would diverge and run one after the other), spread over
+// the SMs: on GB300 a dependent FP64 operation takes ~70 clocks and a warp's
+// FP64 instruction holds the SM's FP64 pipe for ~16 whatever its active
+// lanes.  Measured on the n = 10^4 family, one parent: value and adjoints in
+// one part 8.7k + 13.7k clocks, the longest chain of the kernel.  What the
+// templates are made of (instructions, sums, the split position's dirty
+// terms) is staged in shared memory while the parent is looked up -- a load
+// that misses L1 costs ~700 clocks, and these would otherwise follow one
+// another -- and a warp's lanes load the coordinate and coefficient values
+// together; then lanes 0 and 1 interpret the template together: both run
+// every operation, and exp, sin and cos evaluate their two endpoints one per
+// lane (itrig_pair).
 // Blocks x >= row_blocks: one group tree of the parent's cached sums each
 // (sum k, kind: F, midpoint, FP32), level by level.
 constexpr int PTAB_T = 128;
-constexpr int PTAB_ITEMS = 4;        // row parts per block: one per warp, in its lane 0
-constexpr int PTAB_SMEM_DT = 256;   // dirty terms staged in shared memory for the row lookup
+constexpr int PTAB_ITEMS = 4;        // row parts per block: one per warp, in its lanes 0 and 1
+constexpr int PTAB_SMEM_DT = 256;   // dirty terms staged in shared memory
+constexpr int PTAB_SMEM_INS = GB_MAX_ISUM * GB_MAX_TREGS;   // template instructions: all of them
 
-__host__ __device__ __forceinline__ int ptab_parts(const GbPool& pool) { return pool.fp32 ? 3 : 2; }
+__host__ __device__ __forceinline__ int ptab_parts(const GbPool& pool) { return pool.fp32 ? 5 : 3; }
 
 // One level-major pairwise group tree: the level-0 nodes (the parent's
 // cached group sums) are in a[0, ngroups); every level is formed from the one
@@ -159,6 +165,12 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
     __shared__ double s_bnd[GB_MAX_SPLIT_D * 5];
     __shared__ float s_brd[GB_MAX_SPLIT_D * 5], s_bru[GB_MAX_SPLIT_D * 5];
     const long long p = blockIdx.y;
+    __shared__ GbIns s_ins[PTAB_SMEM_INS];
+    __shared__ GbSum s_sum[GB_MAX_ISUM];
+    if ((int)blockIdx.x < row_blocks) {
+        for (int t = threadIdx.x; t < P.n_tins; t += blockDim.x) s_ins[t] = P.tins[t];
+        if (threadIdx.x < P.n_sum) s_sum[threadIdx.x] = P.sums[threadIdx.x];
+    }
     // from_sel: the one parent is pool entry sel_pos (the partition, which
     // writes the parent count, may be running)
     if (!from_sel && p >= st->parents) return;
@@ -182,14 +194,14 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
     // its dirty terms are staged while the split's box loads are in flight)
     const int spi = P.sp_of_cyc[cyc & 0x7fffffff];
     const bool rows = (int)blockIdx.x < row_blocks;
-    __shared__ int s_row[PTAB_SMEM_DT];
+    __shared__ GbDTerm s_dt[PTAB_SMEM_DT];
     GbSplitPos SP{};
     bool staged = false;
     if (rows && spi >= 0) {
         SP = P.sps[spi];
         staged = SP.ndterm <= PTAB_SMEM_DT;
         if (staged)
-            for (int t = threadIdx.x; t < SP.ndterm; t += blockDim.x) s_row[t] = P.dterms[SP.dterm0 + t].row;
+            for (int t = threadIdx.x; t < SP.ndterm; t += blockDim.x) s_dt[t] = P.dterms[SP.dterm0 + t];
     }
     int4 info = make_int4(0, 0, 0, 0);
     if (rows) info = parent_split(P, pool, par, sp, p, slot, cyc, s_bnd, s_brd, s_bru, blockIdx.x == 0);
@@ -214,8 +226,7 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
     const int parts = ptab_parts(pool);
     int ops = 0, ops32 = 0, spare = 0;   // (lane 1's interpreter counts go to `spare`)
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // per warp: the template's instructions and load values (stage_term)
-    __shared__ GbIns s_ins[PTAB_ITEMS][GB_MAX_TREGS];
+    // per warp: the template's load values (stage_term)
     __shared__ double2 s_pre[PTAB_ITEMS][GB_MAX_TREGS];
     for (int item = blockIdx.x * PTAB_ITEMS + wib; item < SP.tab_entries * parts; item += row_blocks * PTAB_ITEMS) {
         const int row = item / parts, part = item - row * parts;
@@ -223,16 +234,17 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
         int lo = 0, hi = SP.ndterm - 1;
         while (lo < hi) {
             int mid = (lo + hi + 1) >> 1;
-            const int r0 = staged ? s_row[mid] : P.dterms[SP.dterm0 + mid].row;
+            const int r0 = staged ? s_dt[mid].row : P.dterms[SP.dterm0 + mid].row;
             if (r0 <= row) lo = mid; else hi = mid - 1;
         }
-        const GbDTerm D = P.dterms[SP.dterm0 + lo];
+        const GbDTerm D = staged ? s_dt[lo] : P.dterms[SP.dterm0 + lo];
         const unsigned r = (unsigned)(row - D.row) << D.dshift;   // a child index with these digits
-        const GbSum S = P.sums[D.sum];
+        const GbSum S = s_sum[D.sum];
         const int i = S.first + D.term * S.step;
         const size_t orow = (size_t)p * T.max_rows + row;
-        const GbIns* ins = s_ins[wib];
-        if (part < 2) {
+        const GbIns* ins = s_ins + S.ins0;
+        const bool vals = part == 2 || part == 4;
+        if (part < 3) {
             iv64* pre = reinterpret_cast<iv64*>(s_pre[wib]);
             View<double> X = box_view64(pool, slot);
             X.blo = s_bnd;
@@ -242,30 +254,25 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
             X.mshift = sp.mshift;
             X.mstride = sp.m + 1;
             X.r = r;
-            if (part == 1) {
-                stage_term<double>(P, S, i, MidView{X}, s_ins[wib], pre, lane);
-                if (lane < 2) {
-                    iv64 R[GB_MAX_TREGS];
-                    const iv64 v = term_fwd<double, MidView, true>(P, S, i, MidView{X}, R, lane ? spare : ops, ins, pre);
-                    if (lane == 0) T.tm64[orow] = make_double2(v.lo, v.hi);
-                }
-            } else {
-                stage_term<double>(P, S, i, X, s_ins[wib], pre, lane);
-                if (lane < 2) {
-                    int& o = lane ? spare : ops;
-                    iv64 R[GB_MAX_TREGS], RA[GB_MAX_TREGS];
-                    const iv64 v = term_fwd<double, View<double>, true>(P, S, i, X, R, o, ins, pre);
+            const PointView PX{X, part & 1};
+            stage_term<double>(ins, S.nins, i, PX, vals, pre, lane);
+            if (lane < 2) {
+                int& o = lane ? spare : ops;
+                iv64 R[GB_MAX_TREGS];
+                if (!vals) {
+                    const iv64 v = term_fwd<double, PointView, true>(P, S, i, PX, R, o, ins, pre);
+                    if (lane == 0) (part ? T.tm64 : T.tv64)[orow] = make_double2(v.lo, v.hi);
+                } else {
+                    iv64 RA[GB_MAX_TREGS];
+                    term_fwd<double, PointView, true, true>(P, S, i, PX, R, o, ins, pre);
                     for (int t = 0; t < S.nins; t++) RA[t] = iv64{0.0, 0.0};
                     RA[S.nins - 1] = iv64{1.0, 1.0};
                     reverse_sweep<double, true>(ins, S.nins, R, RA, o);
-                    if (lane == 0) {
-                        T.tv64[orow] = make_double2(v.lo, v.hi);
-                        int leaf = 0;
-                        for (int t = 0; t < S.nins; t++) {
-                            if (ins[t].op != D_IVAR) continue;
-                            T.tl64[orow * T.max_leaves + leaf] = make_double2(RA[t].lo, RA[t].hi);
-                            leaf++;
-                        }
+                    int leaf = 0;
+                    for (int t = 0; t < S.nins && lane == 0; t++) {
+                        if (ins[t].op != D_IVAR) continue;
+                        T.tl64[orow * T.max_leaves + leaf] = make_double2(RA[t].lo, RA[t].hi);
+                        leaf++;
                     }
                 }
             }
@@ -279,18 +286,21 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
             X32.mshift = sp.mshift;
             X32.mstride = sp.m + 1;
             X32.r = r;
-            stage_term<float>(P, S, i, X32, s_ins[wib], pre, lane);
+            stage_term<float>(ins, S.nins, i, X32, vals, pre, lane);
             if (lane < 2) {
                 int& o = lane ? spare : ops32;
-                iv32 R32[GB_MAX_TREGS], RA32[GB_MAX_TREGS];
-                const iv32 f = term_fwd<float, View<float>, true>(P, S, i, X32, R32, o, ins, pre);
-                for (int t = 0; t < S.nins; t++) RA32[t] = iv32{0.f, 0.f};
-                RA32[S.nins - 1] = iv32{1.f, 1.f};
-                reverse_sweep<float, true>(ins, S.nins, R32, RA32, o);
-                if (lane == 0) {
-                    T.tv32[orow] = make_float2(f.lo, f.hi);
+                iv32 R32[GB_MAX_TREGS];
+                if (!vals) {
+                    const iv32 f = term_fwd<float, View<float>, true>(P, S, i, X32, R32, o, ins, pre);
+                    if (lane == 0) T.tv32[orow] = make_float2(f.lo, f.hi);
+                } else {
+                    iv32 RA32[GB_MAX_TREGS];
+                    term_fwd<float, View<float>, true, true>(P, S, i, X32, R32, o, ins, pre);
+                    for (int t = 0; t < S.nins; t++) RA32[t] = iv32{0.f, 0.f};
+                    RA32[S.nins - 1] = iv32{1.f, 1.f};
+                    reverse_sweep<float, true>(ins, S.nins, R32, RA32, o);
                     int leaf = 0;
-                    for (int t = 0; t < S.nins; t++) {
+                    for (int t = 0; t < S.nins && lane == 0; t++) {
                         if (ins[t].op != D_IVAR) continue;
                         T.tl32[orow * T.max_leaves + leaf] = make_float2(RA32[t].lo, RA32[t].hi);
                         leaf++;
