@@ -601,7 +601,7 @@ def roofline(m, w, opts, sm_mhz, sms, gb, local):
     if w.get("paper"):
         kname = "k_eval32 + k_eval64 (bytecode interpreter)" if w["fp32"] else "k_eval64 (bytecode interpreter)"
     elif w["fp32"] and warp:
-        kname = "k_ptab + k_ptab_d + k_eval3264_tabw (tables, then FP32 and FP64 in one warp-per-child kernel)"
+        kname = "k_ptab + k_ptab_d + k_eval_tabw (tables, then FP32 and FP64 in one warp-per-child kernel)"
     else:
         kname = ("k_ptab + k_ptab_d + " + ("k_eval32_tab + compaction + " if w["fp32"] else "") + "k_eval64_tab"
                  + ("w" if warp else ""))

@@ -209,7 +209,7 @@ template <typename I> __device__ __noinline__ void slow_rev(int op, I g, I va, I
     }
 }
 
-// The same, for lanes 0 and 1 of a warp interpreting the same template
+// The same, for an even lane and the next interpreting the same template
 // together (PAIR interpreters): exp, sin and cos evaluate their two
 // endpoints in the two lanes (iexp_pair, itrig_pair); the other operations
 // run in both lanes alike.
@@ -494,7 +494,7 @@ __device__ __noinline__ typename Prec<T>::I prod_term_seed(const GbProg& P, int 
 }
 
 // Value of one outer instruction from the registers before it.
-template <typename T, typename V>
+template <typename T, bool PAIR = false, typename V>
 __device__ __forceinline__ typename Prec<T>::I outer_ins(const GbIns& in, const V& X, const typename Prec<T>::I* sums,
                                                           const typename Prec<T>::I* O) {
     typename Prec<T>::I v;
@@ -514,7 +514,7 @@ __device__ __forceinline__ typename Prec<T>::I outer_ins(const GbIns& in, const 
     case D_EXP:
     case D_SIN:
     case D_STEP:
-    case D_COS: v = slow_fwd(in.op, O[in.a], O[in.b]); break;
+    case D_COS: v = PAIR ? slow_fwd_pair(in.op, O[in.a], O[in.b]) : slow_fwd(in.op, O[in.a], O[in.b]); break;
     case D_SCALE:
         if (in.clo32 == in.chi32 || sizeof(T) == 8)
             v = iscale(O[in.a], sizeof(T) == 8 ? (T)in.c : (T)in.clo32);
@@ -527,14 +527,14 @@ __device__ __forceinline__ typename Prec<T>::I outer_ins(const GbIns& in, const 
 }
 
 // Outer forward pass; O receives all outer registers, returns F.
-template <typename T, typename V>
+template <typename T, bool PAIR = false, typename V>
 __device__ __forceinline__ typename Prec<T>::I outer_fwd(const GbProg& P, const V& X,
                                                           const typename Prec<T>::I* sums,
                                                           typename Prec<T>::I* O, int& ops) {
     for (int t = 0; t < P.n_outer; t++) {
         const GbIns in = P.outer[t];
         ops += in.pad & 0xff;
-        O[t] = outer_ins<T>(in, X, sums, O);
+        O[t] = outer_ins<T, PAIR>(in, X, sums, O);
     }
     return O[P.outer_root];
 }

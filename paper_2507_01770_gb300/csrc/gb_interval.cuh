@@ -332,14 +332,17 @@ template <typename I> __device__ __forceinline__ I itrig(I x, bool is_cos) {
     return r;
 }
 
-// Two-lane forms of iexp and itrig for lanes 0 and 1 of a warp that hold the
-// same argument (both run the same interpreter; the table kernel does): lane
+// Two-lane forms of iexp and itrig for an even lane and the next that hold the
+// same argument (both run the same interpreter): lane
 // h evaluates the library function at endpoint h, and for itrig the
 // directed division of endpoint h by pi, and the two lanes exchange them --
 // the values of iexp / itrig, with the two endpoint evaluations side by side
 // instead of one after the other.  RU(a / b) is taken as -RD(-a / b), the
 // same number under IEEE directed rounding.
-template <typename T> __device__ __forceinline__ T pair_get(T v, int src) { return __shfl_sync(0x3u, v, src); }
+template <typename T> __device__ __forceinline__ T pair_get(T v, int src) {
+    const int l0 = threadIdx.x & 30;
+    return __shfl_sync(3u << l0, v, l0 + src);
+}
 
 template <typename I> __device__ __forceinline__ I iexp_pair(I x) {
     typedef decltype(x.lo) T;

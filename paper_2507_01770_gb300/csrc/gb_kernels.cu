@@ -1979,7 +1979,7 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
         if (ev) cudaEventRecord(ev[2], s), cudaEventRecord(ev[3], s);
         gb_launch_count++;
         cc_done = Cmax <= 64LL * 128;   // (at most 64 children per thread of the last block)
-        if ((e = gb_launch_eval3264_tabw(P, pool, par, *tabs, ch, Cmax, sp, st, s, cc_done ? &G : nullptr)) !=
+        if ((e = gb_launch_eval_tabw(P, pool, par, *tabs, ch, Cmax, sp, true, st, s, cc_done ? &G : nullptr)) !=
             cudaSuccess)
             return e;
         if (ev) cudaEventRecord(ev[1], s);

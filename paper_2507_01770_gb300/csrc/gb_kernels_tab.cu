@@ -445,77 +445,6 @@ __global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents
 }
 
 // ---------------------------------------------------------------------------
-// tab_path for a warp whose lanes all walk the same path (one child per
-// warp): the clean sibling nodes the walk reads depend only on the tree's
-// shape and the dirty range, so they are listed first (lane t takes the t-th
-// one the walk will read) and loaded by all lanes at once, one round of
-// memory latency instead of one per level; the walk then takes each from its
-// lane.  Same operations in the same order as tab_path, so the same sum,
-// returned in lane 0 (cur is read in lane 0 only).
-template <typename I, typename N>
-__device__ __forceinline__ I tab_path_w(const GbSum& S, int2 dr, I* cur, N node, int lane, int& ops) {
-    if (S.ngroups == 0 || S.nnodes <= 0) {
-        I z;
-        z.lo = 0;
-        z.hi = 0;
-        return z;
-    }
-    if (dr.x >= dr.y) return node(S.nnodes - 1);   // no dirty group: the parent's root
-    int mine = -1, cnt = 0;
-    {
-        int lo = dr.x, hi = dr.y, off = 0;
-        for (int mL = S.ngroups; mL > 1; mL = (mL + 1) / 2) {
-            const int nlo = lo >> 1, nhi = ((hi - 1) >> 1) + 1;
-            for (int q = nlo; q < nhi; q++) {
-                const int a = 2 * q;
-                if (!(a >= lo && a < hi)) mine = cnt++ == lane ? off + a : mine;
-                if (a + 1 < mL && !(a + 1 >= lo && a + 1 < hi)) mine = cnt++ == lane ? off + a + 1 : mine;
-            }
-            lo = nlo;
-            hi = nhi;
-            off += mL;
-        }
-    }
-    I pre;
-    pre.lo = 0;
-    pre.hi = 0;
-    if (mine >= 0) pre = node(mine);
-    I tmp[GB_TAB_MAX_DIRTY];
-    int lo = dr.x, hi = dr.y, off = 0, used = 0;
-    // every lane follows the walk (the shuffles), lane 0 alone computes it:
-    // cur and tmp are touched by one thread per warp
-    auto take = [&](int idx) {
-        const I v = shfl_iv(pre, used & 31);
-        return used++ < 32 ? v : node(idx);
-    };
-    for (int mL = S.ngroups; mL > 1; mL = (mL + 1) / 2) {
-        const int nlo = lo >> 1, nhi = ((hi - 1) >> 1) + 1;
-        for (int q = nlo; q < nhi; q++) {
-            const int a = 2 * q;
-            const bool la = a >= lo && a < hi, lb = a + 1 >= lo && a + 1 < hi;
-            I left = la ? pre : take(off + a);
-            I right = left;
-            if (a + 1 < mL) right = lb ? pre : take(off + a + 1);
-            if (lane == 0) {
-                if (la) left = cur[a - lo];
-                I v = left;
-                if (a + 1 < mL) {
-                    if (lb) right = cur[a + 1 - lo];
-                    v = iadd(left, right);
-                }
-                tmp[q - nlo] = v;
-            }
-            if (a + 1 < mL) ops += 2;
-        }
-        if (lane == 0)
-            for (int q = 0; q < nhi - nlo; q++) cur[q] = tmp[q];
-        lo = nlo;
-        hi = nhi;
-        off += mL;
-    }
-    return cur[0];   // defined in lane 0
-}
-
 // tab_path for 32 lanes that walk the same path (same tree and dirty range)
 // over their own dirty values: the sibling nodes are loaded once across the
 // lanes (lane t the t-th one the walk reads) and handed out by shuffles;
@@ -1349,12 +1278,19 @@ __global__ void __launch_bounds__(128, GB_TAB_MINB) k_eval32_tab(GbProg P, GbPoo
 }
 
 // ---------------------------------------------------------------------------
-// One child per warp (generations with few children): the lanes share the
-// dirty terms of each group (warp_group) and the coordinates of the
-// first-order test; the group-tree paths and the outer expression are
-// computed by every lane alike.  Same operations in the same order as the
-// per-thread kernels, so the results are identical.  Operation counts: the
-// work every lane repeats is counted once (lane 0), the shared work per lane.
+// One child per warp (generations with few children).  The sums come from
+// k_child_sums.  Four lanes evaluate the outer expression: lanes 0 and 1 over
+// the box, lanes 2 and 3 at the midpoint, the two of a pair sharing the
+// endpoints of exp, sin and cos; then lanes 0 and 1 sweep it in reverse and the
+// lanes share the coordinates of the first-order test.  Same operations in the
+// same order as the per-thread kernels, so the results are identical.
+//
+// Bound: latency, one child's chain of dependent loads and FP64 operations.
+// The outer instructions and the sums' descriptions, which the chain reads one
+// by one, are staged in shared memory at the start (a load that misses L1
+// costs ~700 clocks).  Measured before, with everything in lane 0 and the
+// program in global memory: n = 1000 exp/sqrt/cos family 37k clocks for the
+// FP32 test and 122k for a child that passes it, n = 10^4 family 13k and 25k.
 
 // The partial-table entries of a split position's block, (coordinate,
 // sum)-major, staged in shared memory by the warp that evaluates a child:
@@ -1362,30 +1298,48 @@ __global__ void __launch_bounds__(128, GB_TAB_MINB) k_eval32_tab(GbProg P, GbPoo
 constexpr int GB_WMETA = 384;
 struct WMeta { int x, y, base, sm; };
 
-// Per-warp shared scratch of the one-child-per-warp kernels: the outer
-// expression's values and adjoints (written by lane 0, read by every lane
-// in the first-order test) and the staged partial-table entries.
+// Per-warp shared scratch: each evaluating lane's sums and outer values, the
+// adjoints of lanes 0 and 1 (lane 0's are read by every lane in the first-order
+// test) and the staged partial-table entries.  A lane's registers are GB_WO
+// entries from the next's: an odd number of 16-byte entries, so four lanes
+// reading the same register meet no bank conflict.
+constexpr int GB_WO = GB_MAX_OREGS + 1;
 struct WScratch {
-    iv64* O64;
-    iv64* OA64;
-    iv32* O32;
-    iv32* OA32;
+    iv64 *S64, *O64, *OA64;   // the warp's; lane's copy at lane * GB_MAX_ISUM or lane * GB_WO
+    iv32 *S32, *O32, *OA32;
     WMeta* meta;
 };
-template <typename T> __device__ __forceinline__ typename TabPrec<T>::I* ws_O(const WScratch& w);
-template <> __device__ __forceinline__ iv64* ws_O<double>(const WScratch& w) { return w.O64; }
-template <> __device__ __forceinline__ iv32* ws_O<float>(const WScratch& w) { return w.O32; }
-template <typename T> __device__ __forceinline__ typename TabPrec<T>::I* ws_OA(const WScratch& w);
-template <> __device__ __forceinline__ iv64* ws_OA<double>(const WScratch& w) { return w.OA64; }
-template <> __device__ __forceinline__ iv32* ws_OA<float>(const WScratch& w) { return w.OA32; }
+template <typename T> __device__ __forceinline__ typename TabPrec<T>::I* ws_O(const WScratch& w, int lane);
+template <> __device__ __forceinline__ iv64* ws_O<double>(const WScratch& w, int lane) { return w.O64 + lane * GB_WO; }
+template <> __device__ __forceinline__ iv32* ws_O<float>(const WScratch& w, int lane) { return w.O32 + lane * GB_WO; }
+template <typename T> __device__ __forceinline__ typename TabPrec<T>::I* ws_OA(const WScratch& w, int lane);
+template <> __device__ __forceinline__ iv64* ws_OA<double>(const WScratch& w, int lane) { return w.OA64 + lane * GB_WO; }
+template <> __device__ __forceinline__ iv32* ws_OA<float>(const WScratch& w, int lane) { return w.OA32 + lane * GB_WO; }
 
 // The kernels' shared declarations: 4 warps per block.
-#define GB_WSCRATCH_DECL                                                   \
-    __shared__ WMeta s_meta[4][GB_WMETA];                                  \
-    __shared__ iv64 s_o64[4][GB_MAX_OREGS], s_oa64[4][GB_MAX_OREGS];       \
-    __shared__ iv32 s_o32[4][GB_MAX_OREGS], s_oa32[4][GB_MAX_OREGS];       \
-    const int wib_ = threadIdx.x >> 5;                                     \
-    const WScratch ws{s_o64[wib_], s_oa64[wib_], s_o32[wib_], s_oa32[wib_], s_meta[wib_]};
+#define GB_WSCRATCH_DECL                                                                                   \
+    __shared__ WMeta s_meta[4][GB_WMETA];                                                                  \
+    __shared__ __align__(16) iv64 s_s64[4][4 * GB_MAX_ISUM], s_o64[4][4 * GB_WO], s_oa64[4][2 * GB_WO];     \
+    __shared__ iv32 s_s32[4][2 * GB_MAX_ISUM], s_o32[4][2 * GB_WO], s_oa32[4][2 * GB_WO];                  \
+    const int wib_ = threadIdx.x >> 5;                                                                     \
+    const WScratch ws{s_s64[wib_], s_o64[wib_], s_oa64[wib_], s_s32[wib_], s_o32[wib_], s_oa32[wib_], s_meta[wib_]};
+
+// The outer instructions and the sums' descriptions into shared memory (16
+// bytes a thread); the caller's program then points at them.  A barrier of the
+// block follows before they are read.
+struct WProg {
+    GbIns outer[GB_MAX_OREGS];
+    GbSum sums[GB_MAX_ISUM];
+};
+__device__ __forceinline__ void stage_prog(GbProg& P, WProg& s) {
+    static_assert(sizeof(GbIns) == 32 && sizeof(GbSum) % 4 == 0, "copied in words");
+    const int* a = reinterpret_cast<const int*>(P.outer);
+    const int* b = reinterpret_cast<const int*>(P.sums);
+    for (int i = threadIdx.x; i < P.n_outer * (int)(sizeof(GbIns) / 4); i += blockDim.x) ((int*)s.outer)[i] = a[i];
+    for (int i = threadIdx.x; i < P.n_sum * (int)(sizeof(GbSum) / 4); i += blockDim.x) ((int*)s.sums)[i] = b[i];
+    P.outer = s.outer;
+    P.sums = s.sums;
+}
 
 __device__ __forceinline__ bool stage_meta(const GbProg& P, const GbSplitPos& SP, int cnt, WMeta* m, int lane) {
     if (cnt > GB_WMETA) return false;
@@ -1472,22 +1426,22 @@ __device__ __forceinline__ typename TabPrec<T>::I tab_partial_m(const GbProg& P,
 
 // First-order test, coordinates of the block spread over the lanes (the
 // block's partial-table entries staged in shared memory when they fit).
-// The outer adjoints are computed by lane 0 from the outer values in the
-// warp's scratch and shared through it.
+// The outer adjoints are computed by lanes 0 and 1 from their outer values in
+// the warp's scratch; lane 0's are shared through it.
 template <typename T>
 __device__ __forceinline__ bool tab_mono_w(const GbProg& P, const GbTabs& Tb, long long p, const GbSplitPos& SP,
                                            int blk, unsigned r, const View<double>& X64, const WScratch& ws,
                                            int& red, int& par, int lane) {
     typedef typename TabPrec<T>::I I;
-    I* O = ws_O<T>(ws);
-    I* OA = ws_OA<T>(ws);
+    const I* OA = ws_OA<T>(ws, 0);
     unsigned unit = P.outer_unit ? 0xffffffffu : 1u;   // a single outer sum: its adjoint is [1, 1]
     if (!P.outer_sum && !P.outer_unit) {
-        if (lane == 0) {
-            for (int t = 0; t < P.n_outer; t++) OA[t] = mk<T>((T)0, (T)0);
-            OA[P.outer_root] = mk<T>((T)1, (T)1);
-            reverse_sweep<T>(P.outer, P.n_outer, O, OA, red);
-            unit = unit_sums(P, OA);
+        if (lane < 2) {
+            I* A = ws_OA<T>(ws, lane);
+            for (int t = 0; t < P.n_outer; t++) A[t] = mk<T>((T)0, (T)0);
+            A[P.outer_root] = mk<T>((T)1, (T)1);
+            reverse_sweep<T, true>(P.outer, P.n_outer, ws_O<T>(ws, lane), A, red);
+            unit = unit_sums(P, A);
         }
         __syncwarp();
         unit = __shfl_sync(0xffffffffu, unit, 0);
@@ -1541,241 +1495,155 @@ __device__ __forceinline__ bool tab_mono_w(const GbProg& P, const GbTabs& Tb, lo
     return __any_sync(0xffffffffu, hit);
 }
 
-// F from lane 0's sums (the outer expression evaluated by lane 0 into the
-// warp's scratch), broadcast to every lane.
-template <typename T, typename V>
+// Sums of child ci that lane `lane` evaluates into its scratch: FP32 (lanes 0
+// and 1), FP64 over the box (lanes 0 and 1) and at the midpoint (2 and 3).  All
+// loads of a lane are in flight together.
+template <bool F32, bool F64>
+__device__ __forceinline__ void child_sums_w(const GbProg& P, const GbTabs& Tb, long long ci, const WScratch& ws,
+                                             int lane) {
+    if (lane >= 4) return;
+    const size_t at = (size_t)ci * P.n_sum;
+    const double2* s64 = lane < 2 ? Tb.cs64 : Tb.csm64;
+    double2 d[GB_MAX_ISUM];
+    float2 f[GB_MAX_ISUM];
+#pragma unroll
+    for (int k = 0; k < GB_MAX_ISUM; k++) {
+        if (k >= P.n_sum) continue;
+        if (F64) d[k] = s64[at + k];
+        if (F32 && lane < 2) f[k] = Tb.cs32[at + k];
+    }
+#pragma unroll
+    for (int k = 0; k < GB_MAX_ISUM; k++) {
+        if (k >= P.n_sum) continue;
+        if (F64) ws.S64[lane * GB_MAX_ISUM + k] = iv64{d[k].x, d[k].y};
+        if (F32 && lane < 2) ws.S32[lane * GB_MAX_ISUM + k] = iv32{f[k].x, f[k].y};
+    }
+}
+
+// F of a child by lanes 0 .. NL - 1 (pairs sharing endpoints); each lane's
+// value is returned in it.
+template <typename T, int NL, typename V>
 __device__ __forceinline__ typename TabPrec<T>::I outer_w(const GbProg& P, const V& X,
-                                                          const typename TabPrec<T>::I* sums, const WScratch& ws,
-                                                          int lane, int& red) {
-    typedef typename TabPrec<T>::I I;
-    I F{};
-    if (lane == 0) F = outer_value<T>(P, X, sums, ws_O<T>(ws), red);
+                                                          const typename TabPrec<T>::I* sums,
+                                                          typename TabPrec<T>::I* O, int lane, int& red) {
+    typename TabPrec<T>::I F{};
+    if (lane < NL) F = P.outer_sum ? sums[lane * GB_MAX_ISUM]
+                                   : outer_fwd<T, true>(P, X, sums + lane * GB_MAX_ISUM, O + lane * GB_WO, red);
     __syncwarp();
-    F.lo = __shfl_sync(0xffffffffu, F.lo, 0);
-    F.hi = __shfl_sync(0xffffffffu, F.hi, 0);
     return F;
 }
 
-__device__ __forceinline__ bool eval64_tab_child_w(const GbProg& P, const GbPool& pool, const GbParents& par,
-                                                   const GbTabs& Tb, const GbChildren& ch, long long ci,
-                                                   const GbSplit& sp, double gub_prev, unsigned long long* gkey,
-                                                   bool* has_key, int& red, int& pops, int lane, const WScratch& ws) {
+// FP64 part of one child by a warp (its sums in the scratch): midpoint sample,
+// F(X), cut-off, first-order test.
+__device__ __forceinline__ void eval64_tab_child_w(const GbProg& P, const GbPool& pool, const GbParents& par,
+                                                   const GbTabs& Tb, const GbChildren& ch, const ChildCtx& c,
+                                                   const GbSplitPos& SP, long long ci, const GbSplit& sp,
+                                                   double gub_prev, unsigned long long& key, int& red, int& pops,
+                                                   int lane, const WScratch& ws) {
+    const View<double> X = view64(pool, par, c, sp);
+    const iv64 F = outer_w<double, 4>(P, PointView{X, lane >> 1}, ws.S64, ws.O64, lane, red);
+    if (lane == 2 && F.hi == F.hi) key = min(key, gb_order_key(F.hi));
+    const double lo = __shfl_sync(0xffffffffu, F.lo, 0);
+    bool keep = !(lo > gub_prev);   // the same in every lane
+    if (keep) keep = !tab_mono_w<double>(P, Tb, c.p, SP, c.info.z, c.r, X, ws, red, pops, lane);
+    if (lane == 0) {
+        ch.flo[ci] = canon_lo(lo);
+        ch.flag[ci] = keep ? 1 : 0;
+    }
+}
+
+// FP32 part of one child by a warp: the cut-off and the first-order test.
+__device__ __forceinline__ bool eval32_tab_child_w(const GbProg& P, const GbPool& pool, const GbParents& par,
+                                                   const GbTabs& Tb, const ChildCtx& c, const GbSplitPos& SP,
+                                                   const GbSplit& sp, double gub_prev, int& red, int& pops, int lane,
+                                                   const WScratch& ws) {
+    const View<float> X = view32(pool, par, c, sp);
+    const View<double> X64 = view64(pool, par, c, sp);
+    const iv32 F = outer_w<float, 2>(P, X, ws.S32, ws.O32, lane, red);
+    const float lo = __shfl_sync(0xffffffffu, F.lo, 0);
+    bool keep = !((double)lo > gub_prev);   // the same in every lane
+    if (keep) keep = !tab_mono_w<float>(P, Tb, c.p, SP, c.info.z, c.r, X64, ws, red, pops, lane);
+    return keep;
+}
+
+// A warp's counters over its children.
+struct WCount {
+    int red32 = 0, pops32 = 0, red64 = 0, pops64 = 0;   // operations of the evaluating lanes, of the test's
+    unsigned long long nv = 0, n32 = 0, key = ~0ull;    // valid children, those in FP64, smallest sample
+    // into the problem's state.  The lanes of a pair count the same operations.
+    __device__ __forceinline__ void add(GbState* st, bool f32, int lane) const {
+        warp_min_gub(key, key != ~0ull, st);
+        const bool first = lane == 0 || lane == 2;
+        if (f32) warp_add_ops((first ? red32 : 0) + pops32, &st->ops32);
+        warp_add_ops((first ? red64 : 0) + pops64, &st->ops64);
+        if (lane == 0 && nv) {
+            if (f32) atomicAdd((unsigned long long*)&st->evals32, nv);
+            atomicAdd((unsigned long long*)&st->children, nv);
+        }
+        if (lane == 0 && n32) {
+            atomicAdd((unsigned long long*)&st->evals64, n32);
+            atomicAdd((unsigned long long*)&st->mids, n32);
+            if (f32) {
+                atomicAdd((unsigned long long*)&st->kept32, n32);
+                atomicAdd((unsigned long long*)&st->n32, n32);
+            }
+        }
+    }
+};
+
+// One child by a warp.  F32: a child that passes the FP32 test is evaluated in
+// FP64 at once (the same children, the same previous GUB and the same
+// operations as an FP32 kernel, a survivor list and an FP64 kernel in
+// sequence, without the list).
+template <bool F32>
+__device__ __forceinline__ void child_w(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& Tb,
+                                        const GbChildren& ch, long long ci, const GbSplit& sp, double gub_prev,
+                                        WCount& n, int lane, const WScratch& ws) {
+    child_sums_w<F32, true>(P, Tb, ci, ws, lane);
     const ChildCtx c = child_ctx(par, ci, sp);
     const int spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
-    if (spi < 0) {
-        if (lane == 0) {
+    bool pass = spi >= 0;
+    if (pass) {
+        const GbSplitPos SP = P.sps[spi];
+        n.nv++;
+        __syncwarp();
+        if (F32) pass = eval32_tab_child_w(P, pool, par, Tb, c, SP, sp, gub_prev, n.red32, n.pops32, lane, ws);
+        if (pass) {
+            n.n32++;
+            eval64_tab_child_w(P, pool, par, Tb, ch, c, SP, ci, sp, gub_prev, n.key, n.red64, n.pops64, lane, ws);
+        }
+    }
+    if (lane == 0) {
+        if (F32) ch.flag32[ci] = pass ? 1 : 0;
+        if (!pass) {
             ch.flag[ci] = 0;
             ch.flo[ci] = __longlong_as_double(0x7ff0000000000000LL);
         }
-        return false;
     }
-    const GbSplitPos SP = P.sps[spi];
-    const int blk = c.info.z;
-    const View<double> X = view64(pool, par, c, sp);
-    const MidView MX{X};
-    const size_t rowbase = (size_t)c.p * Tb.max_rows, nbase = (size_t)c.p * Tb.tree_nodes;
-    const size_t sbase = (size_t)c.p * Tb.max_srows;
-    iv64 sums[GB_MAX_ISUM], msums[GB_MAX_ISUM];   // lane 0's
-    int dt = SP.seg0;
-    if (Tb.cs64) {   // computed by k_child_sums
-        if (lane == 0)
-            for (int k = 0; k < P.n_sum; k++) {
-                const double2 a = Tb.cs64[(size_t)ci * P.n_sum + k], b = Tb.csm64[(size_t)ci * P.n_sum + k];
-                sums[k] = iv64{a.x, a.y};
-                msums[k] = iv64{b.x, b.y};
-            }
-    } else
-    for (int k = 0; k < P.n_sum; k++) {
-        const GbSum S = P.sums[k];
-        const int2 dr = P.dirty[blk * P.n_sum + k];
-        iv64 curF[GB_TAB_MAX_DIRTY], curM[GB_TAB_MAX_DIRTY];
-        for (int g = dr.x; g < dr.y; g++) {
-            iv64 v2[2];
-            int cnt;
-            warp_group<iv64, 2>(P, SP, k, g, c.r, dt, lane,
-                                [&](const GbSeg& G, int at, iv64* v) {
-                                    const double2 a = G.level ? Tb.ts64[sbase + at] : Tb.tv64[rowbase + at];
-                                    const double2 b = G.level ? Tb.tsm64[sbase + at] : Tb.tm64[rowbase + at];
-                                    v[0] = iv64{a.x, a.y};
-                                    v[1] = iv64{b.x, b.y};
-                                }, v2, cnt);
-            if (lane == 0) {
-                curF[g - dr.x] = v2[0];
-                curM[g - dr.x] = v2[1];
-            }
-            red += 4 * (cnt > 0 ? cnt - 1 : 0);
-        }
-        const size_t nb = nbase + S.node0;
-        const iv64 a = tab_path_w(S, dr, curF, [&](int i) { return TabPrec<double>::node(Tb, nb + i); }, lane, red);
-        const iv64 b = tab_path_w(S, dr, curM, [&](int i) { return mid_node(Tb, nb + i); }, lane, red);
-        if (lane == 0) sums[k] = a, msums[k] = b;
-    }
-    const iv64 Fm = outer_w<double>(P, MX, msums, ws, lane, red);
-    if (lane == 0 && Fm.hi == Fm.hi) {
-        *gkey = gb_order_key(Fm.hi);
-        *has_key = true;
-    }
-    const iv64 F = outer_w<double>(P, X, sums, ws, lane, red);   // leaves the outer values of X in the scratch
-    bool keep = !(F.lo > gub_prev);   // the same in every lane
-    if (keep) keep = !tab_mono_w<double>(P, Tb, c.p, SP, blk, c.r, X, ws, red, pops, lane);
-    if (lane == 0) {
-        ch.flo[ci] = canon_lo(F.lo);
-        ch.flag[ci] = keep ? 1 : 0;
-    }
-    return true;
+    __syncwarp();   // the scratch is reused by the warp's next child
 }
 
-// cc: as k_eval3264_tabw.
-__global__ void __launch_bounds__(128, 1) k_eval64_tabw(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
-                                                     GbChildren ch, GbSplit sp, int from_list, GbState* st,
-                                                     GbGenConst G, int cc) {
-    if (st->halt) return;
-    const long long lim = from_list ? st->n32 : st->nch;
-    const double gub_prev = gb_key_value(st->gub_key);
-    const int lane = threadIdx.x & 31;
-    GB_WSCRATCH_DECL
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    unsigned long long key = ~0ull;
-    bool has = false;
-    int red = 0, pops = 0;
-    unsigned long long nv = 0;
-    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < lim; w += nw) {
-        const long long ci = from_list ? (long long)ch.list32[w] : w;
-        unsigned long long k2 = ~0ull;
-        bool h2 = false;
-        if (eval64_tab_child_w(P, pool, par, Tb, ch, ci, sp, gub_prev, &k2, &h2, red, pops, lane, ws)) nv++;
-        if (h2 && k2 < key) key = k2, has = true;
-    }
-    warp_min_gub(key, has, st);
-    warp_add_ops((lane == 0 ? red : 0) + pops, &st->ops64);
-    if (lane == 0 && nv) {
-        atomicAdd((unsigned long long*)&st->evals64, nv);
-        atomicAdd((unsigned long long*)&st->mids, nv);
-        if (!from_list) atomicAdd((unsigned long long*)&st->children, nv);
-    }
-    if (cc) list_survivors_last(ch, st->nch, G, st);
-}
-
-// FP32 pass of one child by a warp: writes flag32 (and resets the FP64 flag
-// and LB); returns -1 for an invalid child, else whether the child passed.
-__device__ __forceinline__ int eval32_tab_child_w(const GbProg& P, const GbPool& pool, const GbParents& par,
-                                                  const GbTabs& Tb, const GbChildren& ch, long long ci,
-                                                  const GbSplit& sp, double gub_prev, int& red, int& pops,
-                                                  int lane, const WScratch& ws) {
-    const ChildCtx c = child_ctx(par, ci, sp);
-    const int spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
-    if (lane == 0) {
-        ch.flag[ci] = 0;
-        ch.flo[ci] = __longlong_as_double(0x7ff0000000000000LL);
-    }
-    if (spi < 0) {
-        if (lane == 0) ch.flag32[ci] = 0;
-        return -1;
-    }
-    const GbSplitPos SP = P.sps[spi];
-    const int blk = c.info.z;
-    const View<float> X = view32(pool, par, c, sp);
-    const View<double> X64 = view64(pool, par, c, sp);
-    const size_t rowbase = (size_t)c.p * Tb.max_rows, nbase = (size_t)c.p * Tb.tree_nodes;
-    const size_t sbase = (size_t)c.p * Tb.max_srows;
-    iv32 sums[GB_MAX_ISUM];   // lane 0's
-    int dt = SP.seg0;
-    if (Tb.cs32) {   // computed by k_child_sums
-        if (lane == 0)
-            for (int k = 0; k < P.n_sum; k++) {
-                const float2 a = Tb.cs32[(size_t)ci * P.n_sum + k];
-                sums[k] = iv32{a.x, a.y};
-            }
-    } else
-    for (int k = 0; k < P.n_sum; k++) {
-        const GbSum S = P.sums[k];
-        const int2 dr = P.dirty[blk * P.n_sum + k];
-        iv32 cur[GB_TAB_MAX_DIRTY];
-        for (int g = dr.x; g < dr.y; g++) {
-            int cnt;
-            iv32 v;
-            warp_group<iv32, 1>(P, SP, k, g, c.r, dt, lane,
-                                [&](const GbSeg& G, int at, iv32* v) {
-                                    const float2 a = G.level ? Tb.ts32[sbase + at] : Tb.tv32[rowbase + at];
-                                    v[0] = iv32{a.x, a.y};
-                                }, &v, cnt);
-            if (lane == 0) cur[g - dr.x] = v;
-            red += 2 * (cnt > 0 ? cnt - 1 : 0);
-        }
-        const size_t nb = nbase + S.node0;
-        const iv32 a = tab_path_w(S, dr, cur, [&](int i) { return TabPrec<float>::node(Tb, nb + i); }, lane, red);
-        if (lane == 0) sums[k] = a;
-    }
-    const iv32 F = outer_w<float>(P, X, sums, ws, lane, red);
-    bool keep = !((double)F.lo > gub_prev);   // the same in every lane
-    if (keep) keep = !tab_mono_w<float>(P, Tb, c.p, SP, blk, c.r, X64, ws, red, pops, lane);
-    if (lane == 0) ch.flag32[ci] = keep ? 1 : 0;
-    return keep ? 1 : 0;
-}
-
-__global__ void __launch_bounds__(128) k_eval32_tabw(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
-                                                     GbChildren ch, GbSplit sp, GbState* st) {
-    if (st->halt) return;
-    const long long lim = st->nch;
-    const double gub_prev = gb_key_value(st->gub_key);
-    const int lane = threadIdx.x & 31;
-    GB_WSCRATCH_DECL
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    int red = 0, pops = 0;
-    unsigned long long nv = 0;
-    for (long long ci = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; ci < lim; ci += nw)
-        if (eval32_tab_child_w(P, pool, par, Tb, ch, ci, sp, gub_prev, red, pops, lane, ws) >= 0) nv++;
-    warp_add_ops((lane == 0 ? red : 0) + pops, &st->ops32);
-    if (lane == 0 && nv) {
-        atomicAdd((unsigned long long*)&st->evals32, nv);
-        atomicAdd((unsigned long long*)&st->children, nv);
-    }
-}
-
-// FP32 prefilter and FP64 evaluation in one pass, one child per warp: a warp
-// whose child passes the FP32 test evaluates it in FP64 at once (the same
-// children, the same previous GUB and the same operations as the FP32 kernel,
-// the survivor list and the FP64 kernel in sequence, without the list).
-// With `cc` (at most 2^16 children) the last block to finish lists the
-// generation's survivors against the final incumbent (k_cc_small's work).
-__global__ void __launch_bounds__(128, 1) k_eval3264_tabw(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
-                                                       GbChildren ch, GbSplit sp, GbState* st, GbGenConst G,
-                                                       int cc) {
+// Every child of a generation.  With `cc` (at most 64 children per thread of a
+// block) the last block to finish lists the generation's survivors against the
+// final incumbent (k_cc_small's work).
+template <bool F32>
+__global__ void __launch_bounds__(128, 1) k_eval_tabw(GbProg P, GbPool pool, GbParents par, GbTabs Tb, GbChildren ch,
+                                                      GbSplit sp, GbState* st, GbGenConst G, int cc) {
     gb_grid_trigger();
     gb_grid_wait();
+    __shared__ WProg s_prog;
+    stage_prog(P, s_prog);
     if (st->halt) return;
     const long long lim = st->nch;
     const double gub_prev = gb_key_value(st->gub_key);
     const int lane = threadIdx.x & 31;
     GB_WSCRATCH_DECL
+    __syncthreads();
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    int red32 = 0, pops32 = 0, red64 = 0, pops64 = 0;
-    unsigned long long nv = 0, n32 = 0, key = ~0ull;
-    bool has = false;
-    for (long long ci = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; ci < lim; ci += nw) {
-        const int v = eval32_tab_child_w(P, pool, par, Tb, ch, ci, sp, gub_prev, red32, pops32, lane, ws);
-        if (v < 0) continue;
-        nv++;
-        if (v == 0) continue;
-        n32++;
-        unsigned long long k2 = ~0ull;
-        bool h2 = false;
-        eval64_tab_child_w(P, pool, par, Tb, ch, ci, sp, gub_prev, &k2, &h2, red64, pops64, lane, ws);
-        if (h2 && k2 < key) key = k2, has = true;
-    }
-    warp_min_gub(key, has, st);
-    warp_add_ops((lane == 0 ? red32 : 0) + pops32, &st->ops32);
-    warp_add_ops((lane == 0 ? red64 : 0) + pops64, &st->ops64);
-    if (lane == 0 && nv) {
-        atomicAdd((unsigned long long*)&st->evals32, nv);
-        atomicAdd((unsigned long long*)&st->children, nv);
-    }
-    if (lane == 0 && n32) {
-        atomicAdd((unsigned long long*)&st->evals64, n32);
-        atomicAdd((unsigned long long*)&st->mids, n32);
-        atomicAdd((unsigned long long*)&st->kept32, n32);
-        atomicAdd((unsigned long long*)&st->n32, n32);
-    }
+    WCount n;
+    for (long long ci = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; ci < lim; ci += nw)
+        child_w<F32>(P, pool, par, Tb, ch, ci, sp, gub_prev, n, lane, ws);
+    n.add(st, F32, lane);
     if (cc) list_survivors_last(ch, lim, G, st);
 }
 
@@ -1815,34 +1683,10 @@ __global__ void __launch_bounds__(128) k_eval3264_batch(const GbEvalDesc* __rest
         const double gub_prev = gb_key_value(st->gub_key);
         const long long c0 = (u - off[lo]) * GB_BATCH_UNIT;
         const long long c1 = min(lim, c0 + GB_BATCH_UNIT);
-        int red32 = 0, pops32 = 0, red64 = 0, pops64 = 0;
-        unsigned long long nv = 0, n32 = 0, key = ~0ull;
-        bool has = false;
-        for (long long ci = c0; ci < c1; ci++) {
-            const int v = eval32_tab_child_w(d.P, d.pool, d.par, d.Tb, d.ch, ci, d.sp, gub_prev, red32, pops32, lane,
-                                             ws);
-            if (v < 0) continue;
-            nv++;
-            if (v == 0) continue;
-            n32++;
-            unsigned long long k2 = ~0ull;
-            bool h2 = false;
-            eval64_tab_child_w(d.P, d.pool, d.par, d.Tb, d.ch, ci, d.sp, gub_prev, &k2, &h2, red64, pops64, lane, ws);
-            if (h2 && k2 < key) key = k2, has = true;
-        }
-        warp_min_gub(key, has, st);
-        warp_add_ops((lane == 0 ? red32 : 0) + pops32, &st->ops32);
-        warp_add_ops((lane == 0 ? red64 : 0) + pops64, &st->ops64);
-        if (lane == 0 && nv) {
-            atomicAdd((unsigned long long*)&st->evals32, nv);
-            atomicAdd((unsigned long long*)&st->children, nv);
-        }
-        if (lane == 0 && n32) {
-            atomicAdd((unsigned long long*)&st->evals64, n32);
-            atomicAdd((unsigned long long*)&st->mids, n32);
-            atomicAdd((unsigned long long*)&st->kept32, n32);
-            atomicAdd((unsigned long long*)&st->n32, n32);
-        }
+        WCount n;
+        for (long long ci = c0; ci < c1; ci++)
+            child_w<true>(d.P, d.pool, d.par, d.Tb, d.ch, ci, d.sp, gub_prev, n, lane, ws);
+        n.add(st, true, lane);
     }
 }
 
@@ -1878,13 +1722,7 @@ cudaError_t gb_launch_ptab(const GbProg& P, const GbPool& pool, const GbParents&
 cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, bool from_list,
                                  GbState* st, cudaStream_t s, const GbGenConst* cc) {
-    if (T.warp) {
-        unsigned g = grid_for(Cmax * 32, 128);
-        if (g > gb_sm_count() * 32) g = gb_sm_count() * 32;
-        k_eval64_tabw<<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, from_list ? 1 : 0, st, cc ? *cc : GbGenConst{},
-                                        cc ? 1 : 0);
-        return cudaGetLastError();
-    }
+    if (T.warp) return gb_launch_eval_tabw(P, pool, par, T, ch, Cmax, sp, false, st, s, cc);
     unsigned g = grid_for(Cmax, 128);
     if (T.dec) {
         const GbDec D{T.tv64, T.ts64, T.nf64, nullptr, T.max_rows, T.max_srows, T.tree_nodes, 0,
@@ -1925,24 +1763,18 @@ cudaError_t gb_launch_child_sums(const GbProg& P, const GbPool& pool, const GbPa
                         kinds, st, nch, base);
 }
 
-cudaError_t gb_launch_eval3264_tabw(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
-                                    const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
-                                    cudaStream_t s, const GbGenConst* cc) {
+cudaError_t gb_launch_eval_tabw(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
+                                const GbChildren& ch, long long Cmax, const GbSplit& sp, bool fp32, GbState* st,
+                                cudaStream_t s, const GbGenConst* cc) {
     unsigned g = grid_for(Cmax * 32, 128);
     if (g > gb_sm_count() * 32) g = gb_sm_count() * 32;
-    return gb_launch_ex(k_eval3264_tabw, g, 128, 0, s, true, P, pool, par, T, ch, sp, st, cc ? *cc : GbGenConst{},
-                        cc ? 1 : 0);
+    return gb_launch_ex(fp32 ? k_eval_tabw<true> : k_eval_tabw<false>, g, 128, 0, s, true, P, pool, par, T, ch, sp, st,
+                        cc ? *cc : GbGenConst{}, cc ? 1 : 0);
 }
 
 cudaError_t gb_launch_eval32_tab(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
                                  cudaStream_t s) {
-    if (T.warp) {
-        unsigned g = grid_for(Cmax * 32, 128);
-        if (g > gb_sm_count() * 32) g = gb_sm_count() * 32;
-        k_eval32_tabw<<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, st);
-        return cudaGetLastError();
-    }
     unsigned g = grid_for(Cmax, 128);
     if (g > gb_sm_count() * GB_TAB_GRID) g = gb_sm_count() * GB_TAB_GRID;
     k_eval32_tab<<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, st);

@@ -227,7 +227,7 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
                                  cudaStream_t s);
 
 // One problem of a fused child evaluation: the arguments of its
-// k_eval3264_tabw launch (term tables, one child per warp, FP32 then FP64).
+// k_eval_tabw launch (term tables, one child per warp, FP32 then FP64).
 struct GbEvalDesc {
     GbProg P;
     GbPool pool;
@@ -331,10 +331,11 @@ cudaError_t gb_launch_ptab_d(const GbProg& P, const GbPool& pool, const GbParent
 cudaError_t gb_launch_child_sums(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbSplit& sp, long long Cmax, int fp32, GbState* st, cudaStream_t s,
                                  bool fixed = false);
+// One child per warp (tables), FP64 or FP32 prefilter and FP64 in one pass.
 // cc non-null (at most 2^16 children): the kernel's last block also lists the survivors.
-cudaError_t gb_launch_eval3264_tabw(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
-                                    const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
-                                    cudaStream_t s, const GbGenConst* cc = nullptr);
+cudaError_t gb_launch_eval_tabw(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
+                                const GbChildren& ch, long long Cmax, const GbSplit& sp, bool fp32, GbState* st,
+                                cudaStream_t s, const GbGenConst* cc = nullptr);
 cudaError_t gb_launch_eval32_tab(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
                                  cudaStream_t s);
