@@ -19,7 +19,7 @@ LIB = os.path.join(BUILD, "libgb.so")
 SOURCES = ["gb_kernels.cu", "gb_kernels_tab.cu", "gb_kernels_box.cu", "gb_kernels_paper.cu", "gb_api.cu",
            "gb_compile.cpp", "gb_noalloc.cu", "gb_server.cpp",
            "gb_tune.cpp"]
-HEADERS = ["gb_internal.h", "gb_interval.cuh", "gb_eval.cuh", "gb_launch.h", "gb_child.cuh", "gb_paper.cuh", "gb_dec.cuh"]
+HEADERS = ["gb_internal.h", "gb_interval.cuh", "gb_eval.cuh", "gb_launch.h", "gb_child.cuh", "gb_paper.cuh", "gb_dec.cuh", "gb_cut.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-fmad=false", "-Xcompiler", "-fPIC",
          "-Xcompiler", "-fno-fast-math"]

@@ -591,6 +591,10 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
                 GbUop* d_u;
                 if ((e = upload(&d_u, Hh.uops.data(), Hh.uops.size(), A))) return bad(e, "upload table layouts");
                 P.uops = d_u;
+                if (!fp32 && d * mshift >= GB_CUT_MIN &&
+                    ((e = alloc(&T.cut.tv, 2 * rows, A)) || (e = alloc(&T.cut.ts, 2 * K * (size_t)T.max_srows, A)) ||
+                     (e = alloc(&T.cut.td, K * (size_t)T.max_drows, A))))
+                    return bad(e, "allocate hull tables");
             }
             T.max_sum_nodes = 1;
             for (const GbSum& S : Hh.sums) T.max_sum_nodes = std::max(T.max_sum_nodes, (int)S.nnodes);
@@ -651,6 +655,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         P.contribs = d_cb;
         P.jkd = d_jkd;
         P.segs = d_segs;
+        P.max_nseg = Hh.max_nseg;
         T.nk = 1 + (opt.samples > 0 ? opt.samples : 1);
         T.n_hoist = (int)Hh.hoist_node.size();
         T.n_oprog = (int)Hh.oprog.size();
@@ -674,6 +679,36 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             cudaGetLastError();   // no room for the tables: the interpreter
         else
             p->use_paper = true;
+        // groups of children (gb_cut.cuh): the operations a child applies to its reductions are isotone
+        bool iso = true;
+        for (const GbOIns& o : Hh.oprog) iso = iso && o.op != D_EXP && o.op != D_SIN && o.op != D_COS;
+        if (p->use_paper && iso && d * mshift >= GB_CUT_MIN &&
+            ((e = alloc(&T.cut.tv, kk * T.arows, A)) || (e = alloc(&T.cut.ts, kk * T.srows, A)) ||
+             (e = alloc(&T.cut.hv, kk * T.hrows, A)) || (e = alloc(&T.cut.td, K * (size_t)T.drows, A)))) {
+            cudaGetLastError();   // no room: every child by itself
+            T.cut = GbCut{};
+        }
+    }
+    // the sums' outer adjoints, where they are the same for every box: every
+    // node from the sum to the root passes its adjoint on, or times a constant
+    if (p->tabs.cut.tv || p->paper.cut.tv) {
+        std::vector<char> fixed(H.outer.size(), 1);
+        auto live = [&](int t) { return (H.outer[t].pad & GB_RV_LIVE) != 0; };
+        for (int t = (int)H.outer.size() - 1; t >= 0; t--) {
+            const GbIns& I = H.outer[t];
+            const bool pass = I.op == D_ADD || I.op == D_SUB || I.op == D_NEG || I.op == D_SCALE;
+            const bool prod = I.op == D_MUL || I.op == D_DIV;
+            if (I.pad & GB_RV_A) fixed[I.a] = fixed[I.a] && fixed[t] && (pass || (prod && !live(I.b)));
+            if (I.pad & GB_RV_B) fixed[I.b] = fixed[I.b] && fixed[t] && (pass || (I.op == D_MUL && !live(I.a)));
+        }
+        bool all = !H.any_prod;
+        for (const GbSum& S : H.sums) all = all && fixed[S.outer_reg];
+        double2* d_adj;
+        if (all) {
+            if ((e = alloc(&d_adj, (size_t)GB_MAX_ISUM, A)) || (e = gb_launch_outer_adj(P, d_adj, p->stream)))
+                return bad(e, "outer adjoints");
+            P.sum_adj = d_adj;
+        }
     }
     p->G.K = p->K;
     p->G.flog2 = d * mshift;

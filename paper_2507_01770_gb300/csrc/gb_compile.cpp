@@ -598,12 +598,6 @@ bool build_endpoint_programs(GbHostProg* P, bool paper) {
         if (!B.outer(P->outer_root) || B.max_depth > GB_DEC_DEPTH) return false;
         sp.u0 = (int)P->uops.size();
         sp.nu = (int)B.u.size();
-        sp.nsuf = 0;
-        while (sp.nsuf < sp.nu) {
-            const GbUop& x = B.u[sp.nu - 1 - sp.nsuf];
-            if (x.op <= U_ADD || ((x.op == U_ADDH || x.op == U_SUBH || x.op == U_MULH) && x.mask != 0)) break;
-            sp.nsuf++;
-        }
         P->uops.insert(P->uops.end(), B.u.begin(), B.u.end());
     }
     return true;

@@ -105,7 +105,7 @@ struct GbSplitPos {
     // tabulated are those of coordinates [ja, jb), the block and a term's reach beyond it
     int32_t nx, ja, jb;
     int32_t hrows;            // rows of the hoisted outer values
-    int32_t u0, nu, nsuf;     // endpoint program uops [u0, u0 + nu); the last nsuf read no digit and push nothing
+    int32_t u0, nu;           // endpoint program uops [u0, u0 + nu)
 };
 // Endpoint program of a split position: F's lower end (or a sample's upper
 // end) of a child as a postfix program over one double per stack entry, for
@@ -235,6 +235,8 @@ struct GbProg {
     int32_t outer_sum;               // 1: the outer expression is one sum (F = that sum, adjoint [1, 1])
     int32_t outer_unit;              // 1: every sum's outer adjoint is exactly [1, 1] and no outer VAR
                                      //    leaf: the first-order test needs no reverse sweep of the outer
+    const double2* sum_adj;          // [n_sum] the sums' outer adjoints where the outer expression fixes them
+                                     //    (child groups, gb_cut.cuh); null: they depend on the box, or a product
     int32_t samples;                 // GUB samples per box (0: midpoint; S: diagonal points j / (S + 1))
     int32_t mono_all;                // first-order test on every coordinate
     int32_t any_prod;                // some reduction is an IPROD
@@ -329,7 +331,7 @@ struct GbState {
     long long sel_need;         // ties (key == sel_T) to take, the last ones in pool order
     long long sel_ties;         // active entries with key == sel_T
     long long radix_rank;       // radix select: remaining rank
-    long long n32;              // length of the FP32-survivor list
+    long long n32;              // length of the FP32-survivor list; without the FP32 pass, of the list of child groups
     long long nfree_base;       // free-list size when the pool partition starts (set by k_stats)
     unsigned long long gub_key;     // incumbent upper bound (order key)
     unsigned long long gub_new_key; // min over this generation's samples

@@ -16,11 +16,14 @@
 // Every value comes from the interpreter's operations in the interpreter's
 // order, so the results are bit-identical.
 //
-// Bound: the FP64 pipe (one addition per table entry and endpoint).  Measured on
-// GB300, whole solves with 4^10 children a generation: Levy n = 30, 27
-// generations, 1172 ms with the interpreter, 42.3 ms here; Griewank n = 16, 10
-// generations, 1507 and 39.7 ms (its survivors' caches, too, come from the
-// tables: k_materialize 73 -> 0.2 ms a generation).
+// Bound: the FP64 pipe (one addition per table entry and endpoint), where
+// most children are cut off in groups (gb_cut.cuh) the latency of the rest.
+// Measured on GB300, whole solves with 4^10 children a generation: Levy n = 30,
+// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 18.6
+// with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 33.4 ms
+// (its survivors' caches, too, come from the tables: k_materialize 73 -> 0.2 ms
+// a generation; two thirds of a million of its children survive, and what
+// bounds those is the product's first-order test).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -265,6 +268,33 @@ __device__ __forceinline__ iv64 paper_outer(const GbProg& P, const GbPaper& T, i
     return O[P.outer_root];
 }
 
+// The adjoints of all m <= PP_TREE items of a pairwise product tree with adjoint
+// a, from the top level down (tree_item_adjoint's products, each formed once).
+// node: the items, room for the other levels after them.
+constexpr int PP_TREE = 16;
+__device__ __forceinline__ void tree_adjoints(iv64 a, int m, iv64* node, iv64* out, int& ops) {
+    int off[6], L = 0;
+    off[0] = 0;
+    for (int sz = m; sz > 1; sz = (sz + 1) / 2) {
+        off[L + 1] = off[L] + sz;
+        for (int i = 0; i < (sz + 1) / 2; i++) {
+            iv64 v = node[off[L] + 2 * i];
+            if (2 * i + 1 < sz) v = imul(v, node[off[L] + 2 * i + 1]), ops += 8;
+            node[off[L + 1] + i] = v;
+        }
+        L++;
+    }
+    out[0] = a;
+    for (int l = L - 1; l >= 0; l--) {
+        const int sz = off[l + 1] - off[l];
+        for (int i = sz - 1; i >= 0; i--) {   // (a node's adjoint is read before its place is taken)
+            const iv64 up = out[i >> 1];
+            out[i] = (i ^ 1) < sz ? imul(up, node[off[l] + (i ^ 1)]) : up;
+            ops += 8;
+        }
+    }
+}
+
 // First-order test of a child that passed the cut-off.  Sums: the block's
 // coordinates and those within a term's reach of it from the tabulated D, the
 // others (every coordinate tested) from the parent's cached D, or swept when
@@ -285,6 +315,12 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
         const double2* tv = T.tv + (size_t)c.p * T.nk * T.arows;
         const double2* ts = T.ts + (size_t)c.p * T.nk * T.srows;
         const CacheRef<double2> cf = cache64(pool, P, c.slot, 0);
+        // A group's term adjoints come from one sweep down its tree when the
+        // trees are small (the coordinates ask for a group's terms in turn);
+        // one term at a time, every partner product is formed again for each
+        // (Griewank n = 16, 6.8e5 children kept in a generation: 20 ms of it).
+        iv64 gv[PP_TREE], nodes[2 * PP_TREE], adj[PP_TREE];
+        int gk = -1, ak = -1, ag = -1;   // gv holds reduction gk's group values; adj group ag of reduction ak
         auto seed = [&](int k, int tt) -> iv64 {
             const GbSum S = P.sums[k];
             const GbPaperSum ps = T.psums[spi * P.n_sum + k];
@@ -295,6 +331,7 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
                 else hi = mid - 1;
             }
             const GbGroup G = P.groups[S.group0 + lo];
+            if (ak == k && ag == lo) return adj[tt - G.t0];
             const int2 dr = P.dirty[blk * P.n_sum + k];
             auto gval = [&](int g) {
                 if (g >= dr.x && g < dr.y) {
@@ -312,9 +349,21 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
                 const double2 v = tv[D.row + (int)((c.r >> D.dshift) & ((1u << (D.w * P.mshift)) - 1u))];
                 return iv64{v.x, v.y};
             };
-            iv64 a{1.0, 1.0};
-            a = tree_item_adjoint(a, S.ngroups, lo, gval, ops);
-            return tree_item_adjoint(a, G.count, tt - G.t0, tval, ops);
+            const iv64 one{1.0, 1.0};
+            if (S.ngroups > PP_TREE || G.count > PP_TREE) {
+                const iv64 a = tree_item_adjoint(one, S.ngroups, lo, gval, ops);
+                return tree_item_adjoint(a, G.count, tt - G.t0, tval, ops);
+            }
+            if (gk != k) {
+                for (int g = 0; g < S.ngroups; g++) gv[g] = gval(g);
+                gk = k;
+            }
+            const iv64 a = tree_item_adjoint(one, S.ngroups, lo, [&](int g) { return gv[g]; }, ops);
+            for (int t = 0; t < G.count; t++) nodes[t] = tval(t);
+            tree_adjoints(a, G.count, nodes, adj, ops);
+            ak = k;
+            ag = lo;
+            return adj[tt - G.t0];
         };
         if (!P.mono_all)
             return block_mono<true, double>(P, blk, X, X, O, OA, R, RA, (double*)nullptr,
@@ -384,90 +433,135 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
     return false;
 }
 
-// One child per thread.  The children of a warp that pass the cut-off are
-// queued in shared memory and tested 32 at a time, every lane busy (few pass).
+// The child evaluator of gb_cut.cuh over the interval walk.
+template <bool PR> struct PaperEval {
+    const GbProg& P;
+    const GbPaper& T;
+    __device__ __forceinline__ iv64 value(const ChildCtx& c, int spi, int kind, int& ops) const {
+        const GbSplitPos SP = P.sps[spi];
+        iv64 O[GB_MAX_OREGS], sums[GB_MAX_ISUM];
+        int sg = SP.seg0;
+        for (int k = 0; k < P.n_sum; k++) sums[k] = paper_sum<PR>(P, T, SP, c.p, k, c.info.z, c.r, kind, sg, ops);
+        return paper_outer(P, T, spi, c.p, c.r, kind, sums, O, ops);
+    }
+    __device__ __forceinline__ double lower(const ChildCtx& c, int spi, int kind, int& ops) const {
+        return value(c, spi, kind, ops).lo;
+    }
+    __device__ __forceinline__ void samples(const ChildCtx& c, int spi, unsigned long long& key, int& ops) const {
+        for (int kind = 1; kind < T.nk; kind++) {
+            const iv64 F = value(c, spi, kind, ops);
+            if (F.hi == F.hi) key = min(key, gb_order_key(F.hi));
+        }
+    }
+};
+
 template <bool PR>
 __global__ void __launch_bounds__(128) k_pp_eval(GbProg P, GbPool pool, GbParents par, GbPaper T, GbChildren ch,
-                                                 GbSplit sp, GbState* st) {
+                                                 GbSplit sp, int mode, GbState* st) {
     if (st->halt) return;
-    __shared__ unsigned s_queue[4][64];   // per warp: at most 31 left over + 32 new
-    const long long lim = st->nch;
-    const double gub_prev = gb_key_value(st->gub_key);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    unsigned* q = s_queue[threadIdx.x >> 5];
-    int qn = 0;   // warp-uniform queue length
-    int ops = 0;
-    unsigned long long key = ~0ull, nvalid = 0;
-    bool has = false;
-    auto test = [&](unsigned ci) {
-        const ChildCtx c = child_ctx(par, ci, sp);
-        ch.flag[ci] = paper_mono<PR>(P, pool, par, T, c, sp, P.sp_of_cyc[c.info.x], ops) ? 0 : 1;
-    };
-    for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < lim; base += stride) {
-        const long long ci = base + lane;
-        bool valid = false, need = false;
-        if (ci < lim) {
-            const ChildCtx c = child_ctx(par, ci, sp);
-            const int spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
-            ch.flag[ci] = 0;
-            if (spi < 0) {
-                ch.flo[ci] = __longlong_as_double(0x7ff0000000000000LL);
-            } else {
-                valid = true;
-                const GbSplitPos SP = P.sps[spi];
-                for (int kind = T.nk - 1; kind >= 0; kind--) {
-                    iv64 O[GB_MAX_OREGS], sums[GB_MAX_ISUM];
-                    int sg = SP.seg0;
-                    for (int k = 0; k < P.n_sum; k++)
-                        sums[k] = paper_sum<PR>(P, T, SP, c.p, k, c.info.z, c.r, kind, sg, ops);
-                    const iv64 F = paper_outer(P, T, spi, c.p, c.r, kind, sums, O, ops);
-                    if (kind > 0) {
-                        if (F.hi == F.hi) {
-                            const unsigned long long k2 = gb_order_key(F.hi);
-                            key = k2 < key ? k2 : key;
-                            has = true;
-                        }
-                    } else {
-                        need = !(F.lo > gub_prev);
-                        ch.flo[ci] = canon_lo(F.lo);
-                    }
-                }
-            }
-        }
-        nvalid += __popc(__ballot_sync(0xffffffffu, valid));
-        const unsigned bal = __ballot_sync(0xffffffffu, need);
-        if (need) q[qn + __popc(bal & ((1u << lane) - 1u))] = (unsigned)ci;
-        qn += __popc(bal);
-        __syncwarp();
-        if (qn >= 32) {
-            test(q[qn - 32 + lane]);
-            qn -= 32;
-            __syncwarp();
-        }
-    }
-    if (lane < qn) test(q[lane]);   // the rest of the queue
-    __syncwarp();
-    warp_min_gub(key, has, st);
-    warp_add_ops(ops, &st->ops64);
-    if (lane == 0 && nvalid) {
-        atomicAdd((unsigned long long*)&st->evals64, nvalid);
-        atomicAdd((unsigned long long*)&st->mids, nvalid * (unsigned long long)(T.nk - 1));
-        atomicAdd((unsigned long long*)&st->children, nvalid);
-    }
+    __shared__ unsigned s_queue[4][64];
+    cut_children(P, par, ch, sp, T.nk, mode, st, s_queue[threadIdx.x >> 5], PaperEval<PR>{P, T},
+                 [&](const ChildCtx& c, int spi, int& ops) { return paper_mono<PR>(P, pool, par, T, c, sp, spi, ops); });
 }
 
 // The same from the endpoint programs.
 __global__ void __launch_bounds__(128) k_pp_dec(GbProg P, GbPool pool, GbParents par, GbPaper T, GbDec D, GbChildren ch,
-                                                GbSplit sp, int one, GbState* st) {
+                                                GbSplit sp, int mode, GbState* st) {
     if (st->halt) return;
     __shared__ unsigned s_queue[4][64];
+    cut_children(P, par, ch, sp, T.nk, mode, st, s_queue[threadIdx.x >> 5], DecEval<5>{P, D},
+                 [&](const ChildCtx& c, int spi, int& ops) { return paper_mono<false>(P, pool, par, T, c, sp, spi, ops); });
+}
+
+// ---------------------------------------------------------------------------
+// Hull tables (GbCut): a block per (field, kind, parent); a field is the
+// entries of a term row, a segment, a hoisted value or (kind 0) a coordinate's
+// partial sum.  A warp takes 32 of its entries; the aligned runs of at most 32
+// are reduced by shuffles, as order keys (the FP64 pipe would take 16 clocks a
+// comparison).  An entry that is not a number becomes the whole line (the
+// children decide for themselves).
+__global__ void __launch_bounds__(128) k_cut_tabs(GbProg P, GbParents par, GbDec D, GbDec out, int n_hoist,
+                                                  const GbHoistPos* hoist_pos, GbState* st) {
+    if (st->halt) return;
+    const long long p = blockIdx.z;
+    const int kind = blockIdx.y;
+    if (p >= st->parents) return;
+    const int spi = P.sp_of_cyc[par.info[p].x];
+    if (spi < 0) return;
+    const GbSplitPos SP = P.sps[spi];
+    int f = blockIdx.x;
+    int base, shift, mask;
+    const double2 *src, *dst;
+    if (f < SP.nseg) {
+        const GbSeg G = P.segs[SP.seg0 + f];
+        base = G.base;
+        shift = G.shift;
+        mask = G.mask;
+        src = G.level ? D.ts + p * D.tsp + kind * D.tsk : D.tv + p * D.tvp + kind * D.tvk;
+        dst = G.level ? out.ts + p * out.tsp + kind * out.tsk : out.tv + p * out.tvp + kind * out.tvk;
+    } else if ((f -= SP.nseg) < n_hoist) {
+        const GbHoistPos H = hoist_pos[spi * n_hoist + f];
+        base = H.base;
+        shift = H.shift;
+        mask = H.mask;
+        src = D.hv + p * D.hvp + kind * D.hvk;
+        dst = out.hv + p * out.hvp + kind * out.hvk;
+    } else if (kind == 0 && (f -= n_hoist) < (SP.jb - SP.ja) * P.n_sum) {
+        const GbJkD J = P.jkd[SP.jk0 + f];
+        if (J.shift < 0) return;
+        base = J.base;
+        shift = J.shift;
+        mask = J.mask;
+        src = D.td + p * D.tdp;
+        dst = out.td + p * out.tdp;
+    } else {
+        return;
+    }
+    const int free_bits = min(max(GB_CUT_LOG2 - shift, 0), __popc((unsigned)mask));
+    const unsigned long long neg_inf = gb_order_key(-__longlong_as_double(0x7ff0000000000000LL)),
+                             pos_inf = gb_order_key(__longlong_as_double(0x7ff0000000000000LL));
+    for (int i0 = threadIdx.x & ~31; i0 <= mask; i0 += blockDim.x) {
+        const int i = i0 + (threadIdx.x & 31);
+        unsigned long long lo = pos_inf, hi = neg_inf;
+        if (i <= mask) {
+            const double2 v = src[base + i];
+            const bool ok = magkey(v.x) <= 0x7ff0000000000000ULL && magkey(v.y) <= 0x7ff0000000000000ULL;
+            lo = ok ? gb_order_key(v.x) : neg_inf;
+            hi = ok ? gb_order_key(v.y) : pos_inf;
+        }
+        for (int o = 1; o < 1 << free_bits; o <<= 1) {
+            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        if (i <= mask) const_cast<double2*>(dst)[base + i] = make_double2(gb_key_value(lo), gb_key_value(hi));
+    }
+}
+
+// The reverse sweep of the outer expression over its constants (the values it
+// reads on the way to a sum whose adjoint is fixed are constants).
+__global__ void k_outer_adj(GbProg P, double2* adj) {
+    iv64 O[GB_MAX_OREGS], A[GB_MAX_OREGS];
     int ops = 0;
-    dec_children<6>(P, par, ch, sp, D, false, one != 0, st, s_queue[threadIdx.x >> 5], [&](unsigned ci) {
-        const ChildCtx c = child_ctx(par, ci, sp);
-        return paper_mono<false>(P, pool, par, T, c, sp, P.sp_of_cyc[c.info.x], ops);
-    });
-    warp_add_ops(ops, &st->ops64);
+    for (int t = 0; t < P.n_outer; t++) {
+        const GbIns in = P.outer[t];
+        O[t] = A[t] = iv64{0.0, 0.0};
+        if (!(in.pad & GB_RV_LIVE)) O[t] = outer_ins<double>(in, View<double>{}, (const iv64*)nullptr, O);
+    }
+    A[P.outer_root] = iv64{1.0, 1.0};
+    reverse_sweep<double>(P.outer, P.n_outer, O, A, ops);
+    for (int k = 0; k < P.n_sum; k++) adj[k] = make_double2(A[P.sums[k].outer_reg].lo, A[P.sums[k].outer_reg].hi);
+}
+
+__global__ void __launch_bounds__(128) k_cut_dec(GbProg P, GbPool pool, GbParents par, GbDec D, GbChildren ch,
+                                                 GbSplit sp, GbState* st) {
+    if (st->halt) return;
+    cut_groups(P, pool, par, ch, sp, D.nk, D.td, D.tdp, st, DecEval<1>{P, D});
+}
+template <bool PR>
+__global__ void __launch_bounds__(128) k_cut_paper(GbProg P, GbPool pool, GbParents par, GbPaper T, GbChildren ch,
+                                                   GbSplit sp, GbState* st) {
+    if (st->halt) return;
+    cut_groups(P, pool, par, ch, sp, T.nk, T.cut.td, T.drows, st, PaperEval<PR>{P, T});
 }
 
 unsigned grid_for(long long items, int per_block) {
@@ -494,19 +588,57 @@ cudaError_t gb_launch_paper_tables(const GbProg& P, const GbPool& pool, const Gb
 cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbParents& par, const GbPaper& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
                                  cudaStream_t s) {
-    gb_launch_count++;
-    if (T.dec) {
-        const GbDec D{T.tv, T.ts, T.nd, T.hv, (long long)T.nk * T.arows, (long long)T.nk * T.srows,
-                      (long long)T.nk * T.tree_nodes, (long long)T.nk * T.hrows, T.arows, T.srows, T.tree_nodes, T.hrows,
-                      T.nk};
-        const bool one = (Cmax >> sp.flog2) <= 1;
-        // one parent: as many threads as stay resident, each taking several children
-        const unsigned gd = std::min<unsigned>(grid_for(Cmax, 128), (unsigned)gb_sm_count() * (one ? 8 : 32));
-        k_pp_dec<<<gd, 128, 0, s>>>(P, pool, par, T, D, ch, sp, one ? 1 : 0, st);
-        return cudaGetLastError();
+    GbDec D{T.tv, T.ts, T.nd, T.hv, (long long)T.nk * T.arows, (long long)T.nk * T.srows,
+            (long long)T.nk * T.tree_nodes, (long long)T.nk * T.hrows, T.arows, T.srows, T.tree_nodes, T.hrows,
+            T.nk, T.td, T.drows};
+    const int mode = T.cut.tv ? CUT_GROUPS : CUT_ALL;
+    cudaError_t e;
+    if (mode == CUT_GROUPS) {
+        GbDec C = D;
+        C.tv = T.cut.tv;
+        C.ts = T.cut.ts;
+        C.hv = T.cut.hv;
+        C.td = T.cut.td;
+        if ((e = gb_launch_cut_tabs(P, par, D, C, T.n_hoist, T.hoist_pos, Cmax >> sp.flog2, st, s)) != cudaSuccess) return e;
+        if (T.dec) {
+            if ((e = gb_launch_cut_dec(P, pool, par, C, ch, Cmax, sp, st, s)) != cudaSuccess) return e;
+        } else {
+            GbPaper H = T;
+            H.tv = T.cut.tv;
+            H.ts = T.cut.ts;
+            H.hv = T.cut.hv;
+            gb_launch_count++;
+            const unsigned g = std::min<unsigned>(grid_for(Cmax >> GB_CUT_LOG2, 128), (unsigned)gb_sm_count() * 16);
+            if (P.any_prod) k_cut_paper<true><<<g, 128, 0, s>>>(P, pool, par, H, ch, sp, st);
+            else k_cut_paper<false><<<g, 128, 0, s>>>(P, pool, par, H, ch, sp, st);
+        }
     }
-    const unsigned g = std::min<unsigned>(grid_for(Cmax, 128), (unsigned)gb_sm_count() * 32);
-    if (P.any_prod) k_pp_eval<true><<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, st);
-    else k_pp_eval<false><<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, st);
+    gb_launch_count++;
+    const unsigned g = std::min<unsigned>(grid_for(Cmax, 128), (unsigned)gb_sm_count() * (mode == CUT_GROUPS ? 8 : 32));
+    if (T.dec) k_pp_dec<<<g, 128, 0, s>>>(P, pool, par, T, D, ch, sp, mode, st);
+    else if (P.any_prod) k_pp_eval<true><<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, mode, st);
+    else k_pp_eval<false><<<g, 128, 0, s>>>(P, pool, par, T, ch, sp, mode, st);
+    return cudaGetLastError();
+}
+
+cudaError_t gb_launch_cut_tabs(const GbProg& P, const GbParents& par, const GbDec& D, const GbDec& out, int n_hoist,
+                               const GbHoistPos* hoist_pos, long long K, GbState* st, cudaStream_t s) {
+    gb_launch_count++;
+    const int fields = std::max(1, P.max_nseg + n_hoist + (P.B + 2 * GB_MAX_WIN) * P.n_sum);
+    k_cut_tabs<<<dim3((unsigned)fields, (unsigned)D.nk, (unsigned)K), 128, 0, s>>>(P, par, D, out, n_hoist, hoist_pos, st);
+    return cudaGetLastError();
+}
+
+cudaError_t gb_launch_outer_adj(const GbProg& P, double2* adj, cudaStream_t s) {
+    gb_launch_count++;
+    k_outer_adj<<<1, 1, 0, s>>>(P, adj);
+    return cudaGetLastError();
+}
+
+cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParents& par, const GbDec& C,
+                              const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st, cudaStream_t s) {
+    gb_launch_count++;
+    const unsigned g = std::min<unsigned>(grid_for(Cmax >> GB_CUT_LOG2, 128), (unsigned)gb_sm_count() * 16);
+    k_cut_dec<<<g, 128, 0, s>>>(P, pool, par, C, ch, sp, st);
     return cudaGetLastError();
 }

@@ -1213,15 +1213,14 @@ __global__ void __launch_bounds__(128, REG ? GB_TAB_MINB_REG : GB_TAB_MINB) k_ev
 // One child per thread from the endpoint programs (every sum enters F with
 // adjoint [1, 1], so the first-order test needs no outer values).
 __global__ void __launch_bounds__(128) k_eval64_dec(GbProg P, GbPool pool, GbParents par, GbTabs Tb, GbDec D,
-                                                    GbChildren ch, GbSplit sp, int from_list, int one, GbState* st) {
+                                                    GbChildren ch, GbSplit sp, int mode, GbState* st) {
     gb_grid_trigger();
     gb_grid_wait();
     if (st->halt) return;
     __shared__ unsigned s_queue[4][64];
-    int ops = 0;
-    dec_children<2>(P, par, ch, sp, D, from_list != 0, one != 0, st, s_queue[threadIdx.x >> 5], [&](unsigned ci) {
-        const ChildCtx c = child_ctx(par, ci, sp);
-        const GbSplitPos SP = P.sps[P.sp_of_cyc[c.info.x]];
+    cut_children(P, par, ch, sp, D.nk, mode, st, s_queue[threadIdx.x >> 5], DecEval<1>{P, D},
+                 [&](const ChildCtx& c, int spi, int& ops) {
+        const GbSplitPos SP = P.sps[spi];
         const View<double> X = view64(pool, par, c, sp);
         const int c0 = c.info.z * P.B, c1 = min(P.n, c0 + P.B);
         const double2* tl = leaf_tab<double>(Tb, c.p);
@@ -1232,7 +1231,6 @@ __global__ void __launch_bounds__(128) k_eval64_dec(GbProg P, GbPool pool, GbPar
         }
         return false;
     });
-    warp_add_ops(ops, &st->ops64);
 }
 
 __global__ void __launch_bounds__(128, GB_TAB_MINB) k_eval32_tab(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
@@ -1725,13 +1723,24 @@ cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbPa
     if (T.warp) return gb_launch_eval_tabw(P, pool, par, T, ch, Cmax, sp, false, st, s, cc);
     unsigned g = grid_for(Cmax, 128);
     if (T.dec) {
+        const long long K = Cmax >> sp.flog2;
         const GbDec D{T.tv64, T.ts64, T.nf64, nullptr, T.max_rows, T.max_srows, T.tree_nodes, 0,
-                      T.tm64 - T.tv64, T.tsm64 - T.ts64, T.nm64 - T.nf64, 0, 2};
-        const bool one = (Cmax >> sp.flog2) <= 1;
-        // one parent: as many threads as stay resident, each taking several children
-        g = std::min<unsigned>(g, (unsigned)gb_sm_count() * (one ? 12 : 32));
-        return gb_launch_ex(k_eval64_dec, g, 128, 0, s, true, P, pool, par, T, D, ch, sp, from_list ? 1 : 0, one ? 1 : 0,
-                            st);
+                      T.tm64 - T.tv64, T.tsm64 - T.ts64, T.nm64 - T.nf64, 0, 2, T.td64, T.max_drows};
+        const int mode = from_list ? CUT_LIST : T.cut.tv ? CUT_GROUPS : CUT_ALL;
+        if (mode == CUT_GROUPS) {
+            GbDec C = D;
+            C.tv = T.cut.tv;
+            C.ts = T.cut.ts;
+            C.td = T.cut.td;
+            C.tvk = K * T.max_rows;
+            C.tsk = K * T.max_srows;
+            cudaError_t e;
+            if ((e = gb_launch_cut_tabs(P, par, D, C, 0, nullptr, K, st, s)) != cudaSuccess ||
+                (e = gb_launch_cut_dec(P, pool, par, C, ch, Cmax, sp, st, s)) != cudaSuccess)
+                return e;
+        }
+        g = std::min<unsigned>(g, (unsigned)gb_sm_count() * (mode == CUT_GROUPS ? 12 : 32));
+        return gb_launch_ex(k_eval64_dec, g, 128, 0, s, true, P, pool, par, T, D, ch, sp, mode, st);
     }
     if (g > gb_sm_count() * GB_TAB_GRID) g = gb_sm_count() * GB_TAB_GRID;
     return gb_launch_ex(P.outer_sum ? (T.reg ? k_eval64_tab<true, true> : k_eval64_tab<true, false>)

@@ -71,6 +71,17 @@ struct GbSplit {
     int dmax;                  // boundary table stride (coordinates)
 };
 
+// Hull tables of the groups of 2^GB_CUT_LOG2 children (gb_cut.cuh): every
+// entry of the term rows, segments, hoisted values and partial sums replaced
+// by the hull of the aligned run of entries that a group reads.  Laid out as
+// the tables they stand for.  null: no groups.  Taken from a fan-out of
+// 2^GB_CUT_MIN children on.
+struct GbCut {
+    double2 *tv, *ts, *hv, *td;
+};
+constexpr int GB_CUT_LOG2 = 5;
+constexpr int GB_CUT_MIN = 10;   // log2
+
 // Per-parent term tables (rows indexed by parent * max_rows + row) and the
 // parent's group-sum trees (nodes indexed by parent * tree_nodes + node).
 struct GbTabs {
@@ -115,6 +126,7 @@ struct GbTabs {
     // most GB_REG_DIRTY groups of fewer than 2^GB_REG_LEVELS terms each)
     int reg;
     int dec;          // one child per thread: endpoint programs (P.uops) evaluate the children
+    GbCut cut;        // with dec
 };
 // Paper mode (diagonal samples, first-order test on every coordinate) from
 // per-parent tables.  Kind 0 is the box, kinds 1 .. nk - 1 its sample points
@@ -135,6 +147,7 @@ struct GbPaper {
     const GbOIns* oprog;
     uint32_t indep;
     int dec;          // 1: endpoint programs (P.uops) evaluate the children
+    GbCut cut;
 };
 // Tables of the endpoint programs (gb_dec.cuh): kind 0's arrays with the
 // strides of a parent (p) and of the next kind (k).
@@ -143,6 +156,8 @@ struct GbDec {
     long long tvp, tsp, ndp, hvp;
     long long tvk, tsk, ndk, hvk;
     int nk;
+    const double2* td;   // partial sums, tdp per parent
+    long long tdp;
 };
 constexpr int GB_CG = GB_MAX_ISUM * GB_TAB_MAX_DIRTY;
 constexpr int GB_MV_BITS = 6;
@@ -225,6 +240,15 @@ cudaError_t gb_launch_paper_tables(const GbProg& P, const GbPool& pool, const Gb
 cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbParents& par, const GbPaper& T,
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
                                  cudaStream_t s);
+
+// The hull tables of every parent (in D's order, strides per parent and kind in each).
+cudaError_t gb_launch_cut_tabs(const GbProg& P, const GbParents& par, const GbDec& D, const GbDec& out, int n_hoist,
+                               const GbHoistPos* hoist_pos, long long K, GbState* st, cudaStream_t s);
+// The sums' outer adjoints of an objective that fixes them (GbProg::sum_adj).
+cudaError_t gb_launch_outer_adj(const GbProg& P, double2* adj, cudaStream_t s);
+// The groups by the endpoint programs over the hull tables C.
+cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParents& par, const GbDec& C,
+                              const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st, cudaStream_t s);
 
 // One problem of a fused child evaluation: the arguments of its
 // k_eval_tabw launch (term tables, one child per warp, FP32 then FP64).
