@@ -696,6 +696,37 @@ __device__ __noinline__ void block_D(const GbProg& P, int blk, const V& X, iv64*
     }
 }
 
+// D of one coordinate and sum (block_D's value): every term whose range
+// reaches j, in ascending order.
+template <typename V>
+__device__ __forceinline__ double2 coord_D(const GbProg& P, int k, int j, const V& X, int& ops) {
+    const GbSum S = P.sums[k];
+    iv64 D{0.0, 0.0};
+    bool touched = false;
+    if (S.has_var) {
+        iv64 R[GB_MAX_TREGS], RA[GB_MAX_TREGS];
+        const GbIns* ins = P.tins + S.ins0;
+        const int need = j - S.off_max - S.first;
+        for (int t = need <= 0 ? 0 : (need + S.step - 1) / S.step;
+             t < S.count && S.first + t * S.step + S.off_min <= j; t++) {
+            const int i = S.first + t * S.step;
+            term_fwd<double>(P, S, i, X, R, ops);
+            for (int q = 0; q < S.nins; q++) RA[q] = iv64{0.0, 0.0};
+            RA[S.nins - 1] = iv64{1.0, 1.0};
+            reverse_sweep<double>(ins, S.nins, R, RA, ops);
+            for (int q = 0; q < S.nins; q++) {
+                if (ins[q].op != D_IVAR || i + ins[q].aux != j) continue;
+                D = iadd(D, RA[q]);
+                touched = true;
+                ops += 2;
+            }
+        }
+    }
+    if (!touched) return make_double2(__longlong_as_double(0x7ff0000000000000LL),
+                                      __longlong_as_double((long long)0xfff0000000000000ULL));
+    return make_double2(D.lo, D.hi);
+}
+
 // Blocks whose D a split of block blk changes: the blocks with a coordinate
 // within the widest term's reach (its IDX_VAR offset range) of the block.
 __device__ __forceinline__ int2 d_affected(const GbProg& P, int blk) {

@@ -57,11 +57,16 @@ __device__ __forceinline__ int block_prefix(bool f, int* smem_warp, int* total) 
 }
 
 // ---------------------------------------------------------------------------
-// Root box: the whole domain [l, u] (section 3.1 "initialization").
-template <bool PR>
-__global__ void k_root_init(GbProg P, GbPool pool, GbEntries E, double tol_x, GbState* st) {
+// Root box: the whole domain [l, u] (section 3.1 "initialization"), in three
+// launches: its coordinates; its caches, one group and point a warp (lanes the
+// terms) and one coordinate partial a thread; F, the samples and the state.
+// (One block with a group a thread, every point and every partial one after
+// the other, and the samples in thread 0 took 1.1 ms for the n = 100 chain and
+// for Levy n = 30 at 10 samples, a twentieth of those solves.)
+__global__ void __launch_bounds__(256) k_root_box(GbProg P, GbPool pool, double tol_x) {
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
     const int n = P.n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    for (int j = i0; j < n; j += step) {
         double l = P.l[j], u = P.u[j];
         // dense: slot 0's row; records: record b = j / B holds block b
         pool.recs ? (pool.rlo[j] = l) : (pool.lo64[j] = l);
@@ -73,79 +78,125 @@ __global__ void k_root_init(GbProg P, GbPool pool, GbEntries E, double tol_x, Gb
         }
     }
     if (pool.recs)
-        for (int b = threadIdx.x; b < pool.nb; b += blockDim.x) {
+        for (int b = i0; b < pool.nb; b += step) {
             pool.rid[b] = (unsigned)b;
             bool wide = false;
             for (int j = b * pool.B; j < min(n, (b + 1) * pool.B); j++)
                 if (!(__dsub_rn(P.u[j], P.l[j]) < tol_x)) wide = true;
             pool.rwide[b] = wide ? 1 : 0;
         }
+}
+
+// Group g of sum S by a warp, in lane 0: a lane takes an aligned run of 2^sub
+// terms, then lane i adds lane i + s (group_reduce's in-place pairwise tree).
+template <bool PROD, typename T, typename V>
+__device__ __forceinline__ typename Prec<T>::I group_warp(const GbProg& P, const GbSum& S, int g, const V& X,
+                                                          typename Prec<T>::I* R, int lane, int& ops) {
+    typedef typename Prec<T>::I I;
+    const GbGroup G = P.groups[S.group0 + g];
+    int sub = 0;
+    while (((G.count + (1 << sub) - 1) >> sub) > 32) sub++;
+    const int nr = (G.count + (1 << sub) - 1) >> sub;
+    Tree<I, PROD> tr;
+    tr.init();
+    for (int t = lane << sub; t < min((lane + 1) << sub, G.count); t++)
+        tr.push(term_fwd<T>(P, S, S.first + (G.t0 + t) * S.step, X, R, ops));
+    I v = tr.result();
+    for (int d = 1; d < nr; d <<= 1) {
+        const I o = shfl_iv(v, (lane + d) & 31);
+        if ((lane & (2 * d - 1)) == 0 && lane + d < nr) v = Tree<I, PROD>::comb(v, o);
+    }
+    return v;
+}
+
+template <bool PR>
+__global__ void __launch_bounds__(128) k_root_caches(GbProg P, GbPool pool) {
+    const int lane = threadIdx.x & 31;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    const View<double> X = box_view64(pool, 0);
+    const MidView MX{X};
+    int ops = 0;
+    // points of a group: F, midpoint, (FP32), (diagonal samples)
+    const int pf = pool.fp32 ? 1 : 0, np = 2 + pf + (has_samp(pool) ? pool.S : 0);
+    const long long njob = (long long)P.n_groups * np;
+    const bool dp = pool.gdp || pool.rgdp;
+    const long long nd = dp ? ((long long)P.n * P.n_sum + 31) / 32 : 0;
+    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < njob + nd; w += nw) {
+        if (w >= njob) {   // coordinate partials of the domain (block_D's terms and order, one per thread)
+            const long long it = (w - njob) * 32 + lane;
+            if (it >= (long long)P.n * P.n_sum) continue;
+            const int k = (int)(it / P.n), j = (int)(it - (long long)k * P.n);
+            const double2 v = coord_D(P, k, j, X, ops);
+            if (pool.gdp) pool.gdp[(size_t)k * P.n + j] = v;
+            else pool.rgdp[((size_t)(j / pool.B) * P.n_sum + k) * pool.B + j % pool.B] = v;
+            continue;
+        }
+        const int gg = (int)(w / np), pt = (int)(w - (long long)gg * np);
+        int k = 0;
+        while (k + 1 < P.n_sum && P.sums[k + 1].group0 <= gg) k++;
+        const GbSum S = P.sums[k];
+        const int g = gg - S.group0;
+        const size_t at = pool.recs ? (size_t)P.gown[gg].x * pool.GPB + P.gown[gg].y : (size_t)gg;
+        if (pf && pt == 2) {
+            iv32 R32[GB_MAX_TREGS];
+            const View<float> X32 = box_view32(pool, 0);
+            const iv32 c = PR && S.prod ? group_warp<true, float>(P, S, g, X32, R32, lane, ops)
+                                        : group_warp<false, float>(P, S, g, X32, R32, lane, ops);
+            if (lane == 0) (pool.recs ? pool.rgsum32 : pool.gsum32)[at] = make_float2(c.lo, c.hi);
+            continue;
+        }
+        iv64 R[GB_MAX_TREGS];
+        auto value = [&](const auto& V) {
+            return PR && S.prod ? group_warp<true, double>(P, S, g, V, R, lane, ops)
+                                : group_warp<false, double>(P, S, g, V, R, lane, ops);
+        };
+        const int j = pt - 1 - pf;   // diagonal sample
+        const iv64 v = pt == 0 ? value(X) : pt == 1 ? value(MX) : value(SampleView{X, j, pool.S + 1});
+        if (lane != 0) continue;
+        const double2 o = make_double2(v.lo, v.hi);
+        if (pt == 0) (pool.recs ? pool.rgsum : pool.gsum)[at] = o;
+        else if (pt == 1) (pool.recs ? pool.rgmid : pool.gmid)[at] = o;
+        else if (pool.recs) pool.rgsamp[(size_t)(j - 1) * pool.R * pool.GPB + at] = o;
+        else pool.gsamp[(size_t)(j - 1) * pool.NG + gg] = o;
+    }
+}
+
+constexpr int ROOT_T = 96;   // F and up to 64 samples, one per thread
+template <bool PR>
+__global__ void __launch_bounds__(ROOT_T) k_root_init(GbProg P, GbPool pool, GbEntries E, GbState* st) {
+    // F and the samples from the group sums just cached (the same group values
+    // and tree as a full evaluation)
+    __shared__ double s_lo, s_hi[ROOT_T];
+    const View<double> X = box_view64(pool, 0);
+    iv64 R[GB_MAX_TREGS], sums[GB_MAX_ISUM], O[GB_MAX_OREGS];
+    int ops = 0;
+    const int t = threadIdx.x, nsamp = P.samples > 0 ? P.samples : 1;
+    if (t == 0) {
+        const CacheRef<double2> cf = cache64(pool, P, 0, 0);
+        sum_values<PR, double>(P, -1, X, &cf, R, sums, ops);
+        s_lo = outer_fwd<double>(P, X, sums, O, ops).lo;
+    } else if (t <= nsamp && P.samples > 0) {   // diagonal samples of the domain
+        const SampleView SV{X, t, P.samples + 1};
+        const CacheRef<double2> cs = samp64(pool, P, 0, t);
+        sum_values<PR, double>(P, -1, SV, has_samp(pool) ? &cs : (const CacheRef<double2>*)nullptr, R, sums, ops);
+        s_hi[t] = outer_fwd<double>(P, SV, sums, O, ops).hi;
+    } else if (t <= nsamp) {
+        const MidView MX{X};
+        const CacheRef<double2> cm = cache64(pool, P, 0, 1);
+        sum_values<PR, double>(P, -1, MX, &cm, R, sums, ops);
+        s_hi[t] = outer_fwd<double>(P, MX, sums, O, ops).hi;
+    }
     __syncthreads();
-    if (pool.recs && threadIdx.x == 0) {
+    if (threadIdx.x != 0) return;
+    if (pool.recs) {
         int w = 0;
         for (int b = 0; b < pool.nb; b++) w += pool.rwide[b];
         pool.swide[0] = w;
     }
-    View<double> X = box_view64(pool, 0);
-    MidView MX{X};
-    View<float> X32 = box_view32(pool, 0);
-    iv64 R[GB_MAX_TREGS];
-    iv32 R32[GB_MAX_TREGS];
-    int ops = 0;
-    for (int k = 0; k < P.n_sum; k++) {
-        GbSum S = P.sums[k];
-        for (int g = threadIdx.x; g < S.ngroups; g += blockDim.x) {
-            const int gg = S.group0 + g;
-            const size_t at = pool.recs ? (size_t)P.gown[gg].x * pool.GPB + P.gown[gg].y : (size_t)gg;
-            iv64 a = group_sum<PR, double>(P, S, g, X, R, ops);
-            iv64 b = group_sum<PR, double>(P, S, g, MX, R, ops);
-            (pool.recs ? pool.rgsum : pool.gsum)[at] = make_double2(a.lo, a.hi);
-            (pool.recs ? pool.rgmid : pool.gmid)[at] = make_double2(b.lo, b.hi);
-            if (pool.fp32) {
-                iv32 c = group_sum<PR, float>(P, S, g, X32, R32, ops);
-                (pool.recs ? pool.rgsum32 : pool.gsum32)[at] = make_float2(c.lo, c.hi);
-            }
-            for (int j = 1; has_samp(pool) && j <= pool.S; j++) {
-                const iv64 v = group_sum<PR, double>(P, S, g, SampleView{X, j, pool.S + 1}, R, ops);
-                if (pool.recs) pool.rgsamp[(size_t)(j - 1) * pool.R * pool.GPB + at] = make_double2(v.lo, v.hi);
-                else pool.gsamp[(size_t)(j - 1) * pool.NG + gg] = make_double2(v.lo, v.hi);
-            }
-        }
-    }
-    if (pool.gdp) {   // coordinate partials of the domain, every block
-        iv64 RA[GB_MAX_TREGS];
-        for (int b = threadIdx.x; b < P.nb; b += blockDim.x) block_D(P, b, X, R, RA, pool.gdp, n, 0, ops);
-    }
-    if (pool.rgdp) {   // the same per block record (the root's record of block b is b)
-        iv64 RA[GB_MAX_TREGS];
-        for (int b = threadIdx.x; b < P.nb; b += blockDim.x)
-            block_D(P, b, X, R, RA, pool.rgdp + (size_t)b * P.n_sum * pool.B, pool.B, b * pool.B, ops);
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    // F and the midpoint sample from the group sums just cached (the same
-    // group values and tree as a full evaluation)
-    iv64 sums[GB_MAX_ISUM], O[GB_MAX_OREGS];
-    const CacheRef<double2> cf = cache64(pool, P, 0, 0), cm = cache64(pool, P, 0, 1);
-    sum_values<PR, double>(P, -1, X, &cf, R, sums, ops);
-    iv64 F = outer_fwd<double>(P, X, sums, O, ops);
     double gub = __longlong_as_double(0x7ff0000000000000LL);
-    long long nsamp = 1;
-    if (P.samples > 0) {   // diagonal samples of the domain
-        nsamp = P.samples;
-        for (int j = 1; j <= P.samples; j++) {
-            const SampleView SV{X, j, P.samples + 1};
-            const CacheRef<double2> cs = samp64(pool, P, 0, j);
-            sum_values<PR, double>(P, -1, SV, has_samp(pool) ? &cs : (const CacheRef<double2>*)nullptr, R, sums, ops);
-            const iv64 Fs = outer_fwd<double>(P, SV, sums, O, ops);
-            if (Fs.hi < gub) gub = Fs.hi;
-        }
-    } else {
-        sum_values<PR, double>(P, -1, MX, &cm, R, sums, ops);
-        const iv64 Fm = outer_fwd<double>(P, MX, sums, O, ops);
-        if (Fm.hi == Fm.hi) gub = Fm.hi;
-    }
-    E.flo[0] = canon_lo(F.lo);
+    for (int j = 1; j <= nsamp; j++)
+        if (s_hi[j] < gub) gub = s_hi[j];
+    E.flo[0] = canon_lo(s_lo);
     E.slot[0] = 0;
     E.cyc[0] = 0;
     GbState s0 = {};
@@ -1838,9 +1889,19 @@ int gb_sm_count() {
 }
 cudaError_t gb_launch_root_init(const GbProg& P, const GbPool& pool, const GbEntries& E, double tol_x,
                                 GbState* st, cudaStream_t s) {
-    gb_launch_count++;
-    if (P.any_prod) k_root_init<true><<<1, 256, 0, s>>>(P, pool, E, tol_x, st);
-    else k_root_init<false><<<1, 256, 0, s>>>(P, pool, E, tol_x, st);
+    gb_launch_count += 3;
+    const unsigned sms = (unsigned)gb_sm_count();
+    k_root_box<<<std::min<unsigned>(grid_for(P.n, 256), sms * 2), 256, 0, s>>>(P, pool, tol_x);
+    const int np = 2 + (pool.fp32 ? 1 : 0) + pool.S;
+    const long long jobs = (long long)P.n_groups * np + ((long long)P.n * P.n_sum + 31) / 32;
+    const unsigned g = std::min<unsigned>(grid_for(jobs * 32, 128), sms * 16);
+    if (P.any_prod) {
+        k_root_caches<true><<<g, 128, 0, s>>>(P, pool);
+        k_root_init<true><<<1, ROOT_T, 0, s>>>(P, pool, E, st);
+    } else {
+        k_root_caches<false><<<g, 128, 0, s>>>(P, pool);
+        k_root_init<false><<<1, ROOT_T, 0, s>>>(P, pool, E, st);
+    }
     return cudaGetLastError();
 }
 
