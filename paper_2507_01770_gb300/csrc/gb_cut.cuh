@@ -14,7 +14,11 @@
 //     every child; or
 //   - some partial's enclosure has a fixed sign and no child touches the bound
 //     the sign points to (every child is ruled out by the first-order test),
-//     and no sample of any child can lower the incumbent.
+//     and no sample of any child can lower the incumbent.  To know early what
+//     the incumbent comes to, the group with the smallest bound of its samples
+//     is sampled first (by the last block of the group pass); the others are
+//     compared with the incumbent as it stands when their turn comes, and of
+//     those still walked the samples alone are taken.
 // The others are walked one child per thread.  Of a child that the cut-off
 // removes no sample is needed: its lower bound is above the incumbent, and each
 // sample's upper end is above the value of f at that point, which is above the
@@ -24,7 +28,9 @@
 // Bound: the FP64 pipe while every child was walked.  Measured on GB300 with
 // 4^10 children a generation, whole solves: chain n = 100 (128 generations)
 // 26.4 -> 20.5 ms, a child kernel of 110 us -> 17 after 26 for the groups;
-// paper mode, Levy n = 30 (27 generations) 34.3 -> 18.6 ms.  From a fan-out of
+// paper mode, Levy n = 30 (27 generations) 34.3 -> 9.2 ms (18.6
+// before a group is sampled first, its samples taken five at a time and the
+// test's fixed adjoints used first).  From a fan-out of
 // 2^10 on: the hull tables and the groups take two launches (8 + 10 us at
 // least) and a smaller fan-out is one latency chain either way.
 #pragma once
@@ -78,15 +84,19 @@ __device__ __forceinline__ bool group_ruled_out(const GbProg& P, const GbPool& p
 
 // Groups: appends those to walk to ch.list32 (their number in st->n32, zero
 // at the start of a generation), clears every flag and counts the children.
-// e: the child evaluator over the hull tables; td, tdp: the partial sums' hulls.
-template <typename E>
+// The first child's place in ch.flo tells why a group is walked: the bound of
+// its samples when the first-order test rules it out, else -inf.
+// e: the child evaluator over the hull tables, er over the children's own; td,
+// tdp: the partial sums' hulls.
+template <typename E, typename R>
 __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, const GbParents& par,
                                            const GbChildren& ch, const GbSplit& sp, int nk, const double2* td,
-                                           long long tdp, GbState* st, const E& e) {
+                                           long long tdp, GbState* st, const E& e, const R& er) {
     const double gub_prev = gb_key_value(st->gub_key);
     const long long total = st->nch >> GB_CUT_LOG2, stride = (long long)gridDim.x * blockDim.x;
+    const unsigned long long gmask = total > 1 ? ~0ull >> __clzll(total - 1) : 0;
     const int lane = threadIdx.x & 31;
-    unsigned long long nvalid = 0;
+    unsigned long long nvalid = 0, seed = ~0ull;
     int ops = 0;
     for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
         const long long g = base + lane;
@@ -99,10 +109,15 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
             f[0] = f[1] = make_uint4(0, 0, 0, 0);
             if (spi >= 0) {
                 n = min(1u << GB_CUT_LOG2, (1u << (c.info.y * sp.mshift)) - c.r);
-                walk = !(e.lower(c, spi, 0, ops) > gub_prev);
-                if (walk && group_ruled_out(P, pool, par, sp, P.sps[spi], c, td + c.p * tdp, ops)) {
-                    walk = false;
-                    for (int kind = 1; kind < nk && !walk; kind++) walk = !(e.lower(c, spi, kind, ops) >= gub_prev);
+                walk = !(e.lower(c, spi, ops) > gub_prev);
+                if (walk) {
+                    unsigned long long k = 0;   // below every key of a number
+                    if (group_ruled_out(P, pool, par, sp, P.sps[spi], c, td + c.p * tdp, ops)) {
+                        k = e.bound(c, spi, ops);
+                        walk = k < st->gub_key;
+                        if (walk) seed = min(seed, (k & ~gmask) | (unsigned long long)g);
+                    }
+                    if (walk) ch.flo[g << GB_CUT_LOG2] = k ? gb_key_value(k) : -__longlong_as_double(0x7ff0000000000000LL);
                 }
             }
         }
@@ -113,12 +128,36 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
         at = __shfl_sync(0xffffffffu, at, 0);
         if (walk) ch.list32[at + __popc(bal & ((1u << lane) - 1u))] = (unsigned)g;
     }
-    for (int o = 16; o; o >>= 1) nvalid += __shfl_down_sync(0xffffffffu, nvalid, o);
+    for (int o = 16; o; o >>= 1) {
+        nvalid += __shfl_down_sync(0xffffffffu, nvalid, o);
+        seed = min(seed, __shfl_down_sync(0xffffffffu, seed, o));
+    }
     if (lane == 0 && nvalid) {
         atomicAdd((unsigned long long*)&st->evals64, nvalid);
         atomicAdd((unsigned long long*)&st->mids, nvalid * (unsigned long long)(nk - 1));
         atomicAdd((unsigned long long*)&st->children, nvalid);
     }
+    if (lane == 0 && seed != ~0ull) atomicMin(&st->cut_seed, seed);
+    warp_add_ops(ops, &st->ops64);
+    __shared__ bool s_last;
+    if (!arrive_last(&st->cc_done, gridDim.x, &s_last)) return;
+    seed = __ldcg(&st->cut_seed);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        st->cc_done = 0;
+        st->cut_seed = ~0ull;
+    }
+    if (seed == ~0ull) return;
+    // a warp's share of the kinds, a child per lane
+    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, per = (nk - 1 + nw - 1) / nw;
+    const int k0 = 1 + w * per, k1 = min(nk, k0 + per);
+    unsigned long long key = ~0ull;
+    ops = 0;
+    if (k0 < k1) {
+        const ChildCtx c = child_ctx(par, (long long)((seed & gmask) << GB_CUT_LOG2) + lane, sp);
+        if (c.valid) key = er.samples(c, P.sp_of_cyc[c.info.x], k0, k1, ~0ull, ops);
+    }
+    warp_min_gub(key, key != ~0ull, st);
     warp_add_ops(ops, &st->ops64);
 }
 
@@ -139,32 +178,43 @@ __device__ __forceinline__ void cut_children(const GbProg& P, const GbParents& p
     int qn = 0;   // warp-uniform queue length
     int ops = 0;
     unsigned long long key = ~0ull, nvalid = 0;
-    auto test = [&](unsigned ci) {
+    constexpr unsigned RULED_OUT = 0x80000000u;   // (fewer than 2^31 children)
+    auto test = [&](unsigned e0) {
+        const unsigned ci = e0 & ~RULED_OUT;
         const ChildCtx c = child_ctx(par, ci, sp);
         const int spi = P.sp_of_cyc[c.info.x];
-        e.samples(c, spi, key, ops);
-        ch.flag[ci] = mono(c, spi, ops) ? 0 : 1;
+        key = min(key, e.samples(c, spi, 1, nk, ~0ull, ops));
+        if (!(e0 & RULED_OUT)) ch.flag[ci] = mono(c, spi, ops) ? 0 : 1;
     };
     for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < lim; base += stride) {
         const long long idx = base + lane;
         bool need = false, valid = false;
         long long ci = 0;
+        unsigned ruled = 0;
+        if (mode == CUT_GROUPS) {   // (the warp's children are one group)
+            const long long c0 = (long long)ch.list32[base >> GB_CUT_LOG2] << GB_CUT_LOG2;
+            const double b = ch.flo[c0];
+            __syncwarp();
+            if (gb_order_key(b) >= *(volatile unsigned long long*)&st->gub_new_key) continue;
+            if (b > -__longlong_as_double(0x7ff0000000000000LL)) ruled = RULED_OUT;
+            ci = c0 + lane;
+        } else if (idx < lim) {
+            ci = mode == CUT_LIST ? (long long)ch.list32[idx] : idx;
+        }
         if (idx < lim) {
-            ci = mode == CUT_GROUPS ? ((long long)ch.list32[idx >> GB_CUT_LOG2] << GB_CUT_LOG2) + lane
-                 : mode == CUT_LIST ? (long long)ch.list32[idx] : idx;
             const ChildCtx c = child_ctx(par, ci, sp);
             const int spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
             if (mode != CUT_GROUPS) ch.flag[ci] = 0;
             if (spi >= 0) {
                 valid = true;
-                const double lo = e.lower(c, spi, 0, ops);
+                const double lo = e.lower(c, spi, ops);
                 need = !(lo > gub_prev);
                 if (need) ch.flo[ci] = canon_lo(lo);
             }
         }
         nvalid += __popc(__ballot_sync(0xffffffffu, valid));
         const unsigned bal = __ballot_sync(0xffffffffu, need);
-        if (need) q[qn + __popc(bal & ((1u << lane) - 1u))] = (unsigned)ci;
+        if (need) q[qn + __popc(bal & ((1u << lane) - 1u))] = (unsigned)ci | ruled;
         qn += __popc(bal);
         __syncwarp();
         if (qn >= 32) {

@@ -78,24 +78,31 @@ template <int NQ> struct DecEval {
         dec_exec<N, LO>(P.uops + SP.u0, 0, SP.nu, D, D.tv + c.p * D.tvp + q0 * D.tvk, D.ts + c.p * D.tsp + q0 * D.tsk,
                         D.nd + c.p * D.ndp + q0 * D.ndk, D.hv + c.p * D.hvp + q0 * D.hvk, off, c.r, v, ops);
     }
-    __device__ __forceinline__ double lower(const ChildCtx& c, int spi, int kind, int& ops) const {
+    __device__ __forceinline__ double lower(const ChildCtx& c, int spi, int& ops) const {
         const int off[1] = {0};
         double v[GB_DEC_DEPTH][1];
-        exec<1, true>(P.sps[spi], c, kind, off, v, ops);
+        exec<1, true>(P.sps[spi], c, 0, off, v, ops);
         return v[0][0];
     }
-    __device__ __forceinline__ void samples(const ChildCtx& c, int spi, unsigned long long& key, int& ops) const {
+    // smallest order key of the samples' upper ends, kinds [k0, k1); a value that is not a number counts as `nan`
+    __device__ __forceinline__ unsigned long long samples(const ChildCtx& c, int spi, int k0, int k1,
+                                                          unsigned long long nan, int& ops) const {
         const GbSplitPos SP = P.sps[spi];
-        for (int q0 = 1; q0 < D.nk; q0 += NQ) {
+        unsigned long long key = ~0ull;
+        for (int q0 = k0; q0 < k1; q0 += NQ) {
             int off[NQ];
 #pragma unroll
-            for (int i = 0; i < NQ; i++) off[i] = min(q0 + i, D.nk - 1) - q0;
+            for (int i = 0; i < NQ; i++) off[i] = min(q0 + i, k1 - 1) - q0;
             double v[GB_DEC_DEPTH][NQ];
             exec<NQ, false>(SP, c, q0, off, v, ops);
 #pragma unroll
-            for (int i = 0; i < NQ; i++)
-                if (!nan_bits(v[0][i])) key = min(key, gb_order_key(v[0][i]));
+            for (int i = 0; i < NQ; i++) key = min(key, nan_bits(v[0][i]) ? nan : gb_order_key(v[0][i]));
         }
+        return key;
+    }
+    // over the hull tables: no sample of the group is below the key
+    __device__ __forceinline__ unsigned long long bound(const ChildCtx& c, int spi, int& ops) const {
+        return samples(c, spi, 1, D.nk, 0, ops);
     }
 };
 

@@ -349,6 +349,7 @@ struct GbState {
     unsigned stats_done;               // blocks of k_stats finished (the last one starts the generation)
     unsigned cc_done;                  // blocks of the child kernel finished (the last one lists the survivors)
     int cc_listed;                     // the child kernel has listed the survivors (written by k_child_box alone)
+    unsigned long long cut_seed;       // child groups: smallest sample bound of a group, its low bits the group (~0: none)
     unsigned part_done;                // blocks of the partition finished (the last one combines their keys)
     unsigned long long min_key;        // smallest active key (K = 1 selection)
     long long evals32, evals64, mids;  // running counters

@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(ROOT_T) k_root_init(GbProg P, GbPool pool, GbE
     s0.gub_key = gb_order_key(gub);
     s0.gub_new_key = s0.gub_key;
     s0.sel_T = ~0ull;
-    s0.min_key = ~0ull;
+    s0.min_key = s0.cut_seed = ~0ull;
     s0.evals64 = 1;
     s0.mids = nsamp;
     s0.rec_bump = pool.recs ? pool.nb : 0;
@@ -1779,7 +1779,7 @@ __global__ void k_resume_state(long long count, double gub, GbState* st) {
     s0.gub_key = gb_order_key(gub);
     s0.gub_new_key = s0.gub_key;
     s0.sel_T = ~0ull;
-    s0.min_key = ~0ull;
+    s0.min_key = s0.cut_seed = ~0ull;
     *st = s0;
 }
 

@@ -19,8 +19,8 @@
 // Bound: the FP64 pipe (one addition per table entry and endpoint), where
 // most children are cut off in groups (gb_cut.cuh) the latency of the rest.
 // Measured on GB300, whole solves with 4^10 children a generation: Levy n = 30,
-// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 18.6
-// with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 33.4 ms
+// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 9.2
+// with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 32.5 ms
 // (its survivors' caches, too, come from the tables: k_materialize 73 -> 0.2 ms
 // a generation; two thirds of a million of its children survive, and what
 // bounds those is the product's first-order test).
@@ -307,11 +307,11 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
     const int blk = c.info.z;
     const View<double> X = view64(pool, par, c, sp);
     iv64 O[GB_MAX_OREGS], OA[GB_MAX_OREGS], sums[GB_MAX_ISUM];
-    int sg = SP.seg0;
-    for (int k = 0; k < P.n_sum; k++) sums[k] = paper_sum<PR>(P, T, SP, c.p, k, blk, c.r, 0, sg, ops);
-    outer_fwd<double>(P, X, sums, O, ops);
     iv64 R[GB_MAX_TREGS], RA[GB_MAX_TREGS];
     if constexpr (PR) {
+        int sg = SP.seg0;
+        for (int k = 0; k < P.n_sum; k++) sums[k] = paper_sum<PR>(P, T, SP, c.p, k, blk, c.r, 0, sg, ops);
+        outer_fwd<double>(P, X, sums, O, ops);
         const double2* tv = T.tv + (size_t)c.p * T.nk * T.arows;
         const double2* ts = T.ts + (size_t)c.p * T.nk * T.srows;
         const CacheRef<double2> cf = cache64(pool, P, c.slot, 0);
@@ -374,15 +374,17 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
                 return true;
         return false;
     }
-    for (int t = 0; t < P.n_outer; t++) OA[t] = iv64{0.0, 0.0};
-    OA[P.outer_root] = iv64{1.0, 1.0};
-    reverse_sweep<double>(P.outer, P.n_outer, O, OA, ops);
     const int c0 = blk * P.B, c1 = min(P.n, c0 + P.B);
     const int ja = P.mono_all ? SP.ja : c0, jb = P.mono_all ? SP.jb : c1;
     auto hit = [&](int j, const iv64& g) {
         if (!gt_zero(g.lo) && !lt_zero(g.hi)) return false;
         const iv64 x = X.get(j);
         return (gt_zero(g.lo) && !same_value(x.lo, __ldg(P.l + j))) || (lt_zero(g.hi) && !same_value(x.hi, __ldg(P.u + j)));
+    };
+    auto leaf = [&](int j) {
+        bool l = false;
+        for (int v = 0; v < P.n_var_leaves; v++) l |= P.var_leaves[v].coord == j;
+        return l;
     };
     auto leaves = [&](int j) {
         iv64 g{0.0, 0.0};
@@ -392,38 +394,58 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
         }
         return g;
     };
-    for (int j = ja; j < jb; j++) {
-        iv64 g = leaves(j);
-        for (int k = 0; k < P.n_sum; k++) {
-            iv64 D;
-            if (!paper_D(P, T, SP, c.p, j, k, c.r, D)) continue;
-            g = iadd(g, imul(OA[P.sums[k].outer_reg], D));
-            ops += 4;
+    // Where the sums' outer adjoints are the same for every box, the coordinates
+    // that the outer expression does not read need nothing of it and go first
+    // (nearly every child is ruled out by one of them, and the outer expression
+    // with its sines and its reverse sweep is most of the test).
+    const bool cached = pool.gdp || pool.rgdp;
+    for (int pass = P.sum_adj ? 0 : 1; pass < 2; pass++) {
+        if (pass) {
+            int sg = SP.seg0;
+            for (int k = 0; k < P.n_sum; k++) sums[k] = paper_sum<PR>(P, T, SP, c.p, k, blk, c.r, 0, sg, ops);
+            outer_fwd<double>(P, X, sums, O, ops);
+            for (int t = 0; t < P.n_outer; t++) OA[t] = iv64{0.0, 0.0};
+            OA[P.outer_root] = iv64{1.0, 1.0};
+            reverse_sweep<double>(P.outer, P.n_outer, O, OA, ops);
         }
-        if (hit(j, g)) return true;
-    }
-    if (!P.mono_all) return false;
-    if (pool.gdp || pool.rgdp) {
-        for (int j = 0; j < P.n; j++) {
+        auto adj = [&](int k) {
+            if (pass) return OA[P.sums[k].outer_reg];
+            const double2 a = P.sum_adj[k];
+            return iv64{a.x, a.y};
+        };
+        auto mine = [&](int j) { return P.sum_adj == nullptr || leaf(j) == (pass == 1); };
+        for (int j = ja; j < jb; j++) {
+            if (!mine(j)) continue;
+            iv64 g = pass ? leaves(j) : iv64{0.0, 0.0};
+            for (int k = 0; k < P.n_sum; k++) {
+                iv64 D;
+                if (!paper_D(P, T, SP, c.p, j, k, c.r, D)) continue;
+                g = iadd(g, imul(adj(k), D));
+                ops += 4;
+            }
+            if (hit(j, g)) return true;
+        }
+        for (int j = 0; P.mono_all && cached && j < P.n; j++) {
             if (j == ja) j = jb;
             if (j >= P.n) break;
+            if (!mine(j)) continue;
             const int b = j / P.B;
             const double2* row = pool.recs
                 ? pool.rgdp + (size_t)pool.rid[(size_t)c.slot * pool.nb + b] * P.n_sum * pool.B + (j - b * P.B)
                 : pool.gdp + (size_t)c.slot * P.n_sum * P.n + j;
             const int stride = pool.recs ? pool.B : P.n;
-            iv64 g = leaves(j);
+            iv64 g = pass ? leaves(j) : iv64{0.0, 0.0};
             for (int k = 0; k < P.n_sum; k++) {
                 if (!P.sums[k].has_var) continue;
                 const double2 d = row[(size_t)k * stride];
                 if (!d_touched(d)) continue;
-                g = iadd(g, imul(OA[P.sums[k].outer_reg], iv64{d.x, d.y}));
+                g = iadd(g, imul(adj(k), iv64{d.x, d.y}));
                 ops += 4;
             }
             if (hit(j, g)) return true;
         }
-        return false;
     }
+    if (!P.mono_all || cached) return false;
     for (int b = 0; b < P.nb; b++) {   // no cache: sweep the blocks beyond the tabulated coordinates
         if (b * P.B >= ja && min(P.n, (b + 1) * P.B) <= jb) continue;
         if (block_mono<false, double>(P, b, X, X, O, OA, R, RA, (double*)nullptr, (const CacheRef<double2>*)nullptr, -1,
@@ -444,14 +466,25 @@ template <bool PR> struct PaperEval {
         for (int k = 0; k < P.n_sum; k++) sums[k] = paper_sum<PR>(P, T, SP, c.p, k, c.info.z, c.r, kind, sg, ops);
         return paper_outer(P, T, spi, c.p, c.r, kind, sums, O, ops);
     }
-    __device__ __forceinline__ double lower(const ChildCtx& c, int spi, int kind, int& ops) const {
-        return value(c, spi, kind, ops).lo;
+    __device__ __forceinline__ double lower(const ChildCtx& c, int spi, int& ops) const {
+        return value(c, spi, 0, ops).lo;
     }
-    __device__ __forceinline__ void samples(const ChildCtx& c, int spi, unsigned long long& key, int& ops) const {
-        for (int kind = 1; kind < T.nk; kind++) {
-            const iv64 F = value(c, spi, kind, ops);
-            if (F.hi == F.hi) key = min(key, gb_order_key(F.hi));
+    __device__ __forceinline__ unsigned long long samples(const ChildCtx& c, int spi, int k0, int k1,
+                                                          unsigned long long nan, int& ops) const {
+        unsigned long long key = ~0ull;
+        for (int kind = k0; kind < k1; kind++) {
+            const double v = value(c, spi, kind, ops).hi;
+            key = min(key, nan_bits(v) ? nan : gb_order_key(v));
         }
+        return key;
+    }
+    __device__ __forceinline__ unsigned long long bound(const ChildCtx& c, int spi, int& ops) const {
+        unsigned long long key = ~0ull;   // (below each sample's upper end: its enclosure's lower end over the hulls)
+        for (int kind = 1; kind < T.nk; kind++) {
+            const double v = value(c, spi, kind, ops).lo;
+            key = min(key, nan_bits(v) ? 0ull : gb_order_key(v));
+        }
+        return key;
     }
 };
 
@@ -479,9 +512,11 @@ __global__ void __launch_bounds__(128) k_pp_dec(GbProg P, GbPool pool, GbParents
 // partial sum.  A warp takes 32 of its entries; the aligned runs of at most 32
 // are reduced by shuffles, as order keys (the FP64 pipe would take 16 clocks a
 // comparison).  An entry that is not a number becomes the whole line (the
-// children decide for themselves).
+// children decide for themselves).  ends: the samples' tables are read by the
+// endpoint programs for a lower bound of upper ends, so theirs hold the largest
+// lower and the smallest upper end of a run.
 __global__ void __launch_bounds__(128) k_cut_tabs(GbProg P, GbParents par, GbDec D, GbDec out, int n_hoist,
-                                                  const GbHoistPos* hoist_pos, GbState* st) {
+                                                  const GbHoistPos* hoist_pos, int ends, GbState* st) {
     if (st->halt) return;
     const long long p = blockIdx.z;
     const int kind = blockIdx.y;
@@ -520,20 +555,23 @@ __global__ void __launch_bounds__(128) k_cut_tabs(GbProg P, GbParents par, GbDec
     const int free_bits = min(max(GB_CUT_LOG2 - shift, 0), __popc((unsigned)mask));
     const unsigned long long neg_inf = gb_order_key(-__longlong_as_double(0x7ff0000000000000LL)),
                              pos_inf = gb_order_key(__longlong_as_double(0x7ff0000000000000LL));
+    const bool inner = ends && kind > 0;
     for (int i0 = threadIdx.x & ~31; i0 <= mask; i0 += blockDim.x) {
         const int i = i0 + (threadIdx.x & 31);
+        // the run's smallest of one end in lo, its largest of the other in hi
         unsigned long long lo = pos_inf, hi = neg_inf;
         if (i <= mask) {
             const double2 v = src[base + i];
             const bool ok = magkey(v.x) <= 0x7ff0000000000000ULL && magkey(v.y) <= 0x7ff0000000000000ULL;
-            lo = ok ? gb_order_key(v.x) : neg_inf;
-            hi = ok ? gb_order_key(v.y) : pos_inf;
+            lo = ok ? gb_order_key(inner ? v.y : v.x) : neg_inf;
+            hi = ok ? gb_order_key(inner ? v.x : v.y) : pos_inf;
         }
         for (int o = 1; o < 1 << free_bits; o <<= 1) {
             lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
             hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         }
-        if (i <= mask) const_cast<double2*>(dst)[base + i] = make_double2(gb_key_value(lo), gb_key_value(hi));
+        if (i <= mask) const_cast<double2*>(dst)[base + i] = inner ? make_double2(gb_key_value(hi), gb_key_value(lo))
+                                                                  : make_double2(gb_key_value(lo), gb_key_value(hi));
     }
 }
 
@@ -552,16 +590,18 @@ __global__ void k_outer_adj(GbProg P, double2* adj) {
     for (int k = 0; k < P.n_sum; k++) adj[k] = make_double2(A[P.sums[k].outer_reg].lo, A[P.sums[k].outer_reg].hi);
 }
 
-__global__ void __launch_bounds__(128) k_cut_dec(GbProg P, GbPool pool, GbParents par, GbDec D, GbChildren ch,
+// D: the hull tables; R: the children's own.
+template <int NQ>
+__global__ void __launch_bounds__(128) k_cut_dec(GbProg P, GbPool pool, GbParents par, GbDec D, GbDec R, GbChildren ch,
                                                  GbSplit sp, GbState* st) {
     if (st->halt) return;
-    cut_groups(P, pool, par, ch, sp, D.nk, D.td, D.tdp, st, DecEval<1>{P, D});
+    cut_groups(P, pool, par, ch, sp, D.nk, D.td, D.tdp, st, DecEval<NQ>{P, D}, DecEval<NQ>{P, R});
 }
 template <bool PR>
-__global__ void __launch_bounds__(128) k_cut_paper(GbProg P, GbPool pool, GbParents par, GbPaper T, GbChildren ch,
-                                                   GbSplit sp, GbState* st) {
+__global__ void __launch_bounds__(128) k_cut_paper(GbProg P, GbPool pool, GbParents par, GbPaper T, GbPaper R,
+                                                   GbChildren ch, GbSplit sp, GbState* st) {
     if (st->halt) return;
-    cut_groups(P, pool, par, ch, sp, T.nk, T.cut.td, T.drows, st, PaperEval<PR>{P, T});
+    cut_groups(P, pool, par, ch, sp, T.nk, T.cut.td, T.drows, st, PaperEval<PR>{P, T}, PaperEval<PR>{P, R});
 }
 
 unsigned grid_for(long long items, int per_block) {
@@ -599,9 +639,9 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
         C.ts = T.cut.ts;
         C.hv = T.cut.hv;
         C.td = T.cut.td;
-        if ((e = gb_launch_cut_tabs(P, par, D, C, T.n_hoist, T.hoist_pos, Cmax >> sp.flog2, st, s)) != cudaSuccess) return e;
+        if ((e = gb_launch_cut_tabs(P, par, D, C, T.n_hoist, T.hoist_pos, Cmax >> sp.flog2, T.dec != 0, st, s)) != cudaSuccess) return e;
         if (T.dec) {
-            if ((e = gb_launch_cut_dec(P, pool, par, C, ch, Cmax, sp, st, s)) != cudaSuccess) return e;
+            if ((e = gb_launch_cut_dec(P, pool, par, C, D, ch, Cmax, sp, st, s)) != cudaSuccess) return e;
         } else {
             GbPaper H = T;
             H.tv = T.cut.tv;
@@ -609,8 +649,8 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
             H.hv = T.cut.hv;
             gb_launch_count++;
             const unsigned g = std::min<unsigned>(grid_for(Cmax >> GB_CUT_LOG2, 128), (unsigned)gb_sm_count() * 16);
-            if (P.any_prod) k_cut_paper<true><<<g, 128, 0, s>>>(P, pool, par, H, ch, sp, st);
-            else k_cut_paper<false><<<g, 128, 0, s>>>(P, pool, par, H, ch, sp, st);
+            if (P.any_prod) k_cut_paper<true><<<g, 128, 0, s>>>(P, pool, par, H, T, ch, sp, st);
+            else k_cut_paper<false><<<g, 128, 0, s>>>(P, pool, par, H, T, ch, sp, st);
         }
     }
     gb_launch_count++;
@@ -622,10 +662,11 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
 }
 
 cudaError_t gb_launch_cut_tabs(const GbProg& P, const GbParents& par, const GbDec& D, const GbDec& out, int n_hoist,
-                               const GbHoistPos* hoist_pos, long long K, GbState* st, cudaStream_t s) {
+                               const GbHoistPos* hoist_pos, long long K, bool ends, GbState* st, cudaStream_t s) {
     gb_launch_count++;
     const int fields = std::max(1, P.max_nseg + n_hoist + (P.B + 2 * GB_MAX_WIN) * P.n_sum);
-    k_cut_tabs<<<dim3((unsigned)fields, (unsigned)D.nk, (unsigned)K), 128, 0, s>>>(P, par, D, out, n_hoist, hoist_pos, st);
+    k_cut_tabs<<<dim3((unsigned)fields, (unsigned)D.nk, (unsigned)K), 128, 0, s>>>(P, par, D, out, n_hoist, hoist_pos,
+                                                                                 ends ? 1 : 0, st);
     return cudaGetLastError();
 }
 
@@ -635,10 +676,11 @@ cudaError_t gb_launch_outer_adj(const GbProg& P, double2* adj, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParents& par, const GbDec& C,
+cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParents& par, const GbDec& C, const GbDec& D,
                               const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st, cudaStream_t s) {
     gb_launch_count++;
     const unsigned g = std::min<unsigned>(grid_for(Cmax >> GB_CUT_LOG2, 128), (unsigned)gb_sm_count() * 16);
-    k_cut_dec<<<g, 128, 0, s>>>(P, pool, par, C, ch, sp, st);
+    if (D.nk > 2) k_cut_dec<5><<<g, 128, 0, s>>>(P, pool, par, C, D, ch, sp, st);
+    else k_cut_dec<1><<<g, 128, 0, s>>>(P, pool, par, C, D, ch, sp, st);
     return cudaGetLastError();
 }

@@ -1735,8 +1735,8 @@ cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbPa
             C.tvk = K * T.max_rows;
             C.tsk = K * T.max_srows;
             cudaError_t e;
-            if ((e = gb_launch_cut_tabs(P, par, D, C, 0, nullptr, K, st, s)) != cudaSuccess ||
-                (e = gb_launch_cut_dec(P, pool, par, C, ch, Cmax, sp, st, s)) != cudaSuccess)
+            if ((e = gb_launch_cut_tabs(P, par, D, C, 0, nullptr, K, true, st, s)) != cudaSuccess ||
+                (e = gb_launch_cut_dec(P, pool, par, C, D, ch, Cmax, sp, st, s)) != cudaSuccess)
                 return e;
         }
         g = std::min<unsigned>(g, (unsigned)gb_sm_count() * (mode == CUT_GROUPS ? 12 : 32));

@@ -241,13 +241,14 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
                                  const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st,
                                  cudaStream_t s);
 
-// The hull tables of every parent (in D's order, strides per parent and kind in each).
+// The hull tables of every parent (in D's order, strides per parent and kind in
+// each); ends: for the endpoint programs.
 cudaError_t gb_launch_cut_tabs(const GbProg& P, const GbParents& par, const GbDec& D, const GbDec& out, int n_hoist,
-                               const GbHoistPos* hoist_pos, long long K, GbState* st, cudaStream_t s);
+                               const GbHoistPos* hoist_pos, long long K, bool ends, GbState* st, cudaStream_t s);
 // The sums' outer adjoints of an objective that fixes them (GbProg::sum_adj).
 cudaError_t gb_launch_outer_adj(const GbProg& P, double2* adj, cudaStream_t s);
-// The groups by the endpoint programs over the hull tables C.
-cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParents& par, const GbDec& C,
+// The groups by the endpoint programs over the hull tables C (D: the children's own).
+cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParents& par, const GbDec& C, const GbDec& D,
                               const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st, cudaStream_t s);
 
 // One problem of a fused child evaluation: the arguments of its
