@@ -252,28 +252,50 @@ class Result:
     trace: dict
 
 
+class _Owner:
+    """One array that the library allocated, freed with the last numpy view of it."""
+
+    def __init__(self, struct, free):
+        self.struct, self.free = struct, free
+
+    def __del__(self):
+        self.free(ctypes.byref(self.struct))
+
+
+def _adopt(s, field: str, count: int, ctype, free):
+    """The library's array s.field as a numpy array that owns it (no copy: the
+    regions of a large pool are tens of MB); s no longer refers to it."""
+    own = type(s)()
+    ptr = getattr(s, field)
+    setattr(own, field, ptr)
+    buf = (ctype * count).from_address(ctypes.addressof(ptr.contents))
+    buf._owner = _Owner(own, free)   # buf is the base of every view
+    setattr(s, field, None)
+    return np.frombuffer(buf, dtype=np.dtype(ctype))
+
+
 def _result(r: gb_result, n: int, rc: int | None = None) -> Result:
     """The host copy of a result; `rc` (the call's return code) is the
     status whenever it is given, so a failed call never reads as OK."""
     nb = r.n_boxes
 
-    def arr(ptr, count):
-        if not ptr or count == 0:
+    def arr(field, count):
+        if not getattr(r, field) or count == 0:
             return None
-        return np.ctypeslib.as_array(ptr, shape=(count,)).copy()
+        return _adopt(r, field, count, ctypes.c_double, load().gb_free_result)
 
-    lo = arr(r.box_lo, nb * n)
-    hi = arr(r.box_hi, nb * n)
-    tr = {k: [] for k in ("parents", "children", "kept32", "kept", "pool", "gub")}
-    for t in range(r.n_trace):
-        g = r.trace[t]
-        for k in tr:
-            tr[k].append(getattr(g, k))
-    tr = {k: np.array(v) for k, v in tr.items()}
+    lo = arr("box_lo", nb * n)
+    hi = arr("box_hi", nb * n)
+    keys = ("parents", "children", "kept32", "kept", "pool", "gub")
+    if r.n_trace:   # one row per generation: columns of the array of structs
+        rows = np.ctypeslib.as_array(r.trace, shape=(r.n_trace,))
+        tr = {k: rows[k].copy() for k in keys}
+    else:
+        tr = {k: np.array([]) for k in keys}
     return Result(r.fmin_lo, r.fmin_hi, r.status if rc is None else int(rc), nb,
                   lo.reshape(nb, n) if lo is not None else None,
                   hi.reshape(nb, n) if hi is not None else None,
-                  arr(r.box_flo, nb), r.generations, r.box_evals_fp32, r.box_evals_fp64,
+                  arr("box_flo", nb), r.generations, r.box_evals_fp32, r.box_evals_fp64,
                   r.mid_evals, r.solve_ms, r.device_ms, r.eval64_ms, r.eval32_ms,
                   r.eval64_launches, r.eval32_launches, r.kernel_launches, r.ops64, r.ops32,
                   r.queue_ms, r.latency_ms, r.pool_mode, r.record_gcs, tr)
@@ -364,14 +386,14 @@ def gb_snapshot_take(prob: "_Problem") -> Snapshot:
             raise GbError(rc, gb_last_error())
         c, n = int(s.count), int(s.n)
 
-        def arr(ptr, count, dt):
+        def arr(field, count, ctype):
             if count == 0:
-                return np.zeros(0, dtype=dt)
-            return np.ctypeslib.as_array(ptr, shape=(count,)).astype(dt, copy=True)
+                return np.zeros(0, dtype=np.dtype(ctype))
+            return _adopt(s, field, count, ctype, L.gb_free_snapshot)
 
-        return Snapshot(n, int(s.block), arr(s.lo, c * n, np.float64).reshape(c, n),
-                        arr(s.hi, c * n, np.float64).reshape(c, n), arr(s.flo, c, np.float64),
-                        arr(s.cyc, c, np.int32), float(s.gub), int(s.generations))
+        return Snapshot(n, int(s.block), arr("lo", c * n, ctypes.c_double).reshape(c, n),
+                        arr("hi", c * n, ctypes.c_double).reshape(c, n), arr("flo", c, ctypes.c_double),
+                        arr("cyc", c, ctypes.c_int32), float(s.gub), int(s.generations))
     finally:
         L.gb_free_snapshot(ctypes.byref(s))
 
