@@ -915,9 +915,14 @@ __attribute__((visibility("hidden"))) int solve_advance(gb_problem* p, bool bloc
         if ((e = cudaGraphLaunch(p->gexec[cur], s)) != cudaSuccess) return stop(cuda_fail(e, "cudaGraphLaunch"));
         R.launches += p->graph_kernels;
     } else {
+        // the host has just read the pool's size and the active count: the
+        // launches and their grids follow them, not the largest pool (an
+        // n = 2 generation of a few parents: 7 launches instead of 13)
+        const long long pool_now = std::max(1LL, h.pool);
+        const long long kids_now = std::min(p->K, std::max(1LL, h.active)) << p->sp.flog2;
         long long nl = 0;
         e = gb_launch_generation(p->P, p->pool, p->E[cur], p->E[1 - cur], p->par, p->ch, p->sp, p->sc,
-                                 p->use_tabs ? &p->tabs : nullptr, p->G, p->cap, p->Cmax, p->st, s, &p->ev[2], &nl, 0,
+                                 p->use_tabs ? &p->tabs : nullptr, p->G, pool_now, kids_now, p->st, s, &p->ev[2], &nl, 0,
                                  &p->fork, p->use_paper ? &p->paper : nullptr);
         if (e != cudaSuccess) return stop(cuda_fail(e, "generation launch"));
         R.timed64 = true;

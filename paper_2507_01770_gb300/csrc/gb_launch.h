@@ -217,7 +217,8 @@ cudaError_t gb_launch_resume(const GbProg& P, const GbPool& pool, const GbEntrie
 // One generation: select, partition, prepare parents, (term tables), evaluate
 // children (FP32 pass, compaction, FP64 pass), compact survivors,
 // materialise, free parents, finish, and the active count of the new pool.
-// Every size is read from the device state.  ev (4 events or null) brackets
+// Every size is read from the device state; cap and Cmax bound the pool before
+// it and its children (grids, and which of the equivalent kernels run).  ev (4 events or null) brackets
 // the FP64 and FP32 evaluation kernels.  Returns the kernels launched in
 // *nlaunch.  part 1 stops before the child evaluation and part 2 starts
 // after it (a fused evaluation over several problems goes between them).
