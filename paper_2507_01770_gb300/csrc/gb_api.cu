@@ -506,7 +506,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     if ((e = alloc(&p->par.slot, K, A)) || (e = alloc(&p->par.cyc, K, A)) ||
         (e = alloc(&p->par.flo, K, A)) || (e = alloc(&p->par.info, K, A)) ||
         (e = alloc(&p->par.bnd, bt, A)) || (e = alloc(&p->par.bnd_rd, bt, A)) ||
-        (e = alloc(&p->par.bnd_ru, bt, A)))
+        (e = alloc(&p->par.bnd_ru, bt, A)) || (e = alloc(&p->par.spos, K, A)))
         return bad(e, "allocate parent buffers");
     const size_t C = (size_t)p->Cmax;
     if ((e = alloc(&p->ch.flo, C, A)) || (e = alloc(&p->ch.flag, C, A)) ||
@@ -520,6 +520,9 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             const bool warp = opt.eval_mode == 4 || (opt.eval_mode != 3 && gb_warp_per_child(p->Cmax));
             const bool dec = !warp && P.n_var_leaves == 0 && (P.outer_unit || (P.outer_sum && P.n_sum == 1)) &&
                              gb_build_endpoints(&p->hp, false);
+            // children 32 to a block, verdicts by lookup (k_unit)
+            const bool unit = warp && P.n_var_leaves == 0 && (P.outer_unit || (P.outer_sum && P.n_sum == 1)) &&
+                              d * mshift >= 5 && P.B <= GB_UNIT_B && gb_build_verdicts(&p->hp, GB_MV_BITS);
             const GbHostProg& Hh = p->hp;
             int32_t* d_spc;
             GbSplitPos* d_sps;
@@ -528,6 +531,12 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             GbContrib* d_cb;
             GbJkD* d_jkd;
             GbSeg* d_segs;
+            uint16_t* d_mvf;
+            if (unit) {
+                if ((e = upload(&d_mvf, Hh.mvf.data(), Hh.mvf.size(), A))) return bad(e, "upload table layouts");
+                P.mvf = d_mvf;
+                p->tabs.unit = 1;
+            }
             if ((e = upload(&d_jkd, Hh.jkd.data(), Hh.jkd.size(), A)) ||
                 (e = upload(&d_segs, Hh.segs.data(), Hh.segs.size(), A)) ||
                 (e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||

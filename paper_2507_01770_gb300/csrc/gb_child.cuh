@@ -304,16 +304,21 @@ __device__ __forceinline__ long long survivor_list_block(const GbChildren& ch, l
 // The generation's survivor count and what it implies: overflow when the
 // pool cannot take them or their block records do not fit (after the
 // generation's record collection, if it ran).
+__device__ __forceinline__ bool survivors_overflow(const GbGenConst& G, const GbState* st, long long S) {
+    const long long room = st->nfree + (st->cap - st->bump);
+    return S > room || (G.nrec && S * G.nrec > st->rec_nfree + (G.R - st->rec_bump));
+}
 __device__ __forceinline__ void set_survivors(const GbGenConst& G, GbState* st, long long S) {
     st->kept = S;
-    const long long room = st->nfree + (st->cap - st->bump);
-    st->overflow = (S > room || (G.nrec && S * G.nrec > st->rec_nfree + (G.R - st->rec_bump))) ? 1 : 0;
+    st->overflow = survivors_overflow(G, st, S) ? 1 : 0;
 }
 
 // The kernel's last block to finish lists the generation's survivors (at most
-// 64 children per thread of it) against the final incumbent.
+// 64 children per thread of it) against the final incumbent.  late: the pool
+// partition may be running; whether the survivors fit is decided by the
+// materialisation, after it.
 __device__ __forceinline__ void list_survivors_last(const GbChildren& ch, long long nch, const GbGenConst& G,
-                                                    GbState* st) {
+                                                    GbState* st, bool late = false) {
     __shared__ int s_sw[32];
     __shared__ bool s_last;
     if (!arrive_last(&st->cc_done, gridDim.x, &s_last)) return;
@@ -321,7 +326,8 @@ __device__ __forceinline__ void list_survivors_last(const GbChildren& ch, long l
     const long long S = survivor_list_block(ch, nch, gub_new, true, s_sw);
     if (threadIdx.x == 0) {
         st->cc_done = 0;
-        set_survivors(G, st, S);
+        if (late) st->kept = S;
+        else set_survivors(G, st, S);
     }
 }
 

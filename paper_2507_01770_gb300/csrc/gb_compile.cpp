@@ -605,6 +605,34 @@ bool build_endpoint_programs(GbHostProg* P, bool paper) {
 
 }  // namespace
 
+bool gb_build_verdicts(GbHostProg* P, int bits) {
+    P->mvf.clear();
+    if (!P->tab_ok) return false;
+    const int ns = (int)P->sums.size();
+    for (GbSplitPos& sp : P->sps) {
+        sp.mv0 = (int)P->mvf.size();
+        const int c0 = sp.block * P->B, c1 = std::min(P->n, c0 + P->B);
+        for (int j = c0; j < c1; j++) {
+            int a = 32, b = 0;   // the digit bits its contributions and its own piece read
+            auto field = [&](int shift, int n) {
+                if (n <= 0) return;
+                a = std::min(a, shift);
+                b = std::max(b, shift + n);
+            };
+            for (int k = 0; k < ns; k++) {
+                const int2 rg = P->jk[(size_t)sp.jk0 + (size_t)(j - c0) * ns + k];
+                for (int q = rg.x; q < rg.y; q++)
+                    field(P->contribs[q].dshift, __builtin_popcount(P->contribs[q].mask));
+            }
+            if (j >= sp.c0 && j < sp.c0 + sp.dd) field((j - sp.c0) * P->mshift, P->mshift);
+            if (b <= a) a = b = 0;
+            if (b - a > bits) return false;
+            P->mvf.push_back((uint16_t)(a | (b - a) << 8));
+        }
+    }
+    return true;
+}
+
 bool gb_build_endpoints(GbHostProg* P, bool paper) { return P->tab_ok && build_endpoint_programs(P, paper); }
 
 void gb_build_tables(GbHostProg* P, int m, int d, int sbits, bool paper) {

@@ -105,6 +105,7 @@ struct GbSplitPos {
     // tabulated are those of coordinates [ja, jb), the block and a term's reach beyond it
     int32_t nx, ja, jb;
     int32_t hrows;            // rows of the hoisted outer values
+    int32_t mv0;              // GbProg::mvf of the block's coordinates (GbTabs::unit)
     int32_t u0, nu;           // endpoint program uops [u0, u0 + nu)
 };
 // Endpoint program of a split position: F's lower end (or a sample's upper
@@ -229,6 +230,7 @@ struct GbProg {
     const GbContrib* contribs;
     const GbJkD* jkd;                // parallel to jk: partial-table rows
     int32_t max_drows;
+    const uint16_t* mvf;             // digit field of a block coordinate's first-order verdict: first bit | bits << 8
     const GbUop* uops;               // endpoint programs of every split position
     const GbSeg* segs;               // term-tree segments of every split position
     int32_t max_srows, max_nseg;
@@ -269,6 +271,7 @@ struct GbHostProg {
     std::vector<int32_t> hoist_node;     // outer register, | 1 << 16: its reciprocal
     std::vector<GbOIns> oprog;
     std::vector<GbUop> uops;
+    std::vector<uint16_t> mvf;
     int32_t max_arows = 0, max_hrows = 0;
     uint32_t indep = 0;                  // outer registers that depend on no reduction
     // block records: group ownership (a group lives in the record of its lowest touched block)
@@ -292,6 +295,9 @@ struct GbHostProg {
 // sbits: largest digit-bit count of a tabulated term-tree segment (<= GB_TAB_SBITS).
 // paper: layouts of the paper-mode tables (products included; see GbSplitPos).
 void gb_build_tables(GbHostProg* P, int m, int d, int sbits = GB_TAB_SBITS, bool paper = false);
+// Digit fields of the first-order verdicts (GbProg::mvf) of every split position, for objectives whose sums enter
+// with adjoint [1, 1]; false: a coordinate's verdict depends on more than `bits` digit bits.
+bool gb_build_verdicts(GbHostProg* P, int bits);
 // Endpoint programs (GbUop) of every split position of the layouts just built; false: not for this objective.
 bool gb_build_endpoints(GbHostProg* P, bool paper);
 // Compiles and validates a DAG; returns an empty string or an error message.

@@ -1612,8 +1612,8 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
 template <bool PR, bool RECS, int TAB>
 __global__ void __launch_bounds__(128) k_materialize(GbProg P, GbPool pool, GbParents par, GbChildren ch,
                                                      GbSplit sp, GbEntries En, double tol_x, GbState* st,
-                                                     GbTabs Tb, GbPaper PT, GbGenConst G, int npart, unsigned long long* pkey,
-                                                     long long* ppos) {
+                                                     GbTabs Tb, GbPaper PT, GbGenConst G, int late, int npart,
+                                                     unsigned long long* pkey, long long* ppos) {
     gb_grid_trigger();
     gb_grid_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1623,7 +1623,9 @@ __global__ void __launch_bounds__(128) k_materialize(GbProg P, GbPool pool, GbPa
     __shared__ long long s_bq[4];
     __shared__ bool s_last;
     if (st->halt) return;
-    const long long kept = st->overflow ? 0 : st->kept;
+    // late: the survivors were listed beside the partition, whose counts say whether they fit
+    const bool overflow = late ? survivors_overflow(G, st, st->kept) : st->overflow != 0;
+    const long long kept = overflow ? 0 : st->kept;
     const long long kept_old = st->kept_old;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     unsigned long long bk = ~0ull;
@@ -1649,6 +1651,10 @@ __global__ void __launch_bounds__(128) k_materialize(GbProg P, GbPool pool, GbPa
         ppos[npart + blockIdx.x] = bq;
     }
     if (!arrive_last(&st->stats_done, gridDim.x, &s_last)) return;
+    if (late) {
+        if (threadIdx.x == 0) st->overflow = overflow ? 1 : 0;
+        __syncthreads();
+    }
     free_parents(par, pool, En, st, threadIdx.x, blockDim.x);
     unsigned long long mk;
     long long mq;
@@ -1984,6 +1990,8 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
     // pairs and k_materialize's last block ends the generation
     const bool fuse_end = G.K == 1 && gtile_pool <= (unsigned)GB_STAT_BLOCKS && 1 + gmat_max <= (unsigned)GB_STAT_BLOCKS;
     bool cc_done = false;   // the survivor list came with the child kernel
+    bool late = false;      // beside the partition (its overflow is decided by k_materialize)
+    const bool unit = tabs && tabs->unit && part == 0;
     // part 0: the whole generation; 1: up to the child evaluation; 2: after it
     if (part == 2) goto after_eval;
     {
@@ -2015,7 +2023,16 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
         if ((et = gb_launch_ptab(P, pool, par, *tabs, G.K, sp, st, ts, sel_tabs ? &E : nullptr)) != cudaSuccess)
             return et;
         gb_launch_count++;
-        if ((et = gb_launch_ptab_d(P, pool, par, *tabs, G.K, P.B, st, ts, sel_tabs)) != cudaSuccess) return et;
+        if ((et = gb_launch_ptab_d(P, pool, par, *tabs, sp, G.K, st, ts, sel_tabs, unit)) != cudaSuccess) return et;
+        if (unit) {   // the children too: with one parent they need nothing from the partition
+            if (ev) cudaEventRecord(ev[2], ts), cudaEventRecord(ev[3], ts);
+            gb_launch_count++;
+            cc_done = Cmax <= 64LL * gb_unit_threads(P, G.fp32);
+            late = cc_done && ts != s;
+            et = gb_launch_unit(P, pool, par, *tabs, ch, Cmax, sp, G.fp32, st, ts, sel_tabs, cc_done ? &G : nullptr, late);
+            if (ev) cudaEventRecord(ev[1], ts);
+            return et;
+        }
         if (tabs->cs64) {
             gb_launch_count++;
             if ((et = gb_launch_child_sums(P, pool, par, *tabs, sp, Cmax, G.fp32, st, ts, sel_tabs)) != cudaSuccess)
@@ -2066,7 +2083,9 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
         return cudaGetLastError();
     }
     const bool fused = G.fp32 && tabs && tabs->warp;
-    if (fused) {
+    if (unit) {
+        // (with the tables)
+    } else if (fused) {
         // FP32 prefilter and FP64 evaluation in one warp-per-child kernel
         if (ev) cudaEventRecord(ev[2], s), cudaEventRecord(ev[3], s);
         gb_launch_count++;
@@ -2142,7 +2161,7 @@ after_eval:
     const int np = 1;   // the partition's combined pair
 #define GB_MAT(PR, RECS, TAB)                                                                                      \
     e = gb_launch_ex(k_materialize<PR, RECS, TAB>, gmat, 128, 0, s, true, P, pool, par, ch, sp, E_new, G.tol_x,   \
-                     st, Tb, PT, G, np, pk, pq)
+                     st, Tb, PT, G, late ? 1 : 0, np, pk, pq)
     if (paper) {   // (products included: a group's value comes from the tables)
         if (pool.recs) GB_MAT(false, true, 2);
         else GB_MAT(false, false, 2);

@@ -205,6 +205,10 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
     }
     int4 info = make_int4(0, 0, 0, 0);
     if (rows) info = parent_split(P, pool, par, sp, p, slot, cyc, s_bnd, s_brd, s_bru, blockIdx.x == 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // the split position for the later kernels
+        if (spi < 0) SP.ndterm = -1;
+        par.spos[p] = SP;
+    }
     __syncthreads();
     if (spi < 0) return;
     if (!rows) {
@@ -333,26 +337,73 @@ template <typename I> __device__ __forceinline__ I shfl_down_iv(I v, int d) {
     return v;
 }
 
-__global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents par, GbTabs T,
-                                                GbState* st, int fixed) {
+// UNIT (GbTabs::unit): instead of (1) the verdict tables, one thread per (block
+// coordinate, digit combination): the coordinate's partial for a child with
+// those digits (unit adjoints: the sum of its leaf adjoints, summed as in (1))
+// and the first-order test, FP32 and FP64.
+// The blocks below nd_blocks take (1), the others (2): one latency chain each.
+__device__ bool mono_hit(const GbProg& P, const View<double>& X64, int j, bool pos, bool neg);
+template <bool UNIT>
+__global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents par, GbTabs T, GbSplit sp,
+                                                GbState* st, int nd_blocks, int fixed) {
     gb_grid_trigger();
     gb_grid_wait();
     if (st->halt) return;
     const long long p = blockIdx.y;
     if (!fixed && p >= st->parents) return;
-    const int4 info = par.info[p];
-    const int spi = P.sp_of_cyc[info.x];
-    if (spi < 0) return;
-    const GbSplitPos SP = P.sps[spi];
-    const int c0 = info.z * P.B, c1 = min(P.n, c0 + P.B);
+    const GbSplitPos SP = par.spos[p];
+    if (SP.ndterm < 0) return;
+    const int c0 = SP.block * P.B, c1 = min(P.n, c0 + P.B);
     const int nent = (c1 - c0) * P.n_sum;
     const double2* tl = T.tl64 + (size_t)p * T.max_rows * T.max_leaves;
     const float2* tl32 = pool.fp32 ? T.tl32 + (size_t)p * T.max_rows * T.max_leaves : nullptr;
     const int nd_items = nent << GB_TAB_DBITS;
     const int lane = threadIdx.x & 31;
     int ops = 0, ops32 = 0;
+    if (UNIT && (int)blockIdx.x < nd_blocks) {
+        const int4 info = par.info[p];
+        ChildCtx c;
+        c.p = p;
+        c.info = info;
+        c.slot = par.slot[p];
+        c.valid = true;
+        for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < (c1 - c0) << GB_MV_BITS; item += nd_blocks * blockDim.x) {
+            const int jl = item >> GB_MV_BITS, combo = item & ((1 << GB_MV_BITS) - 1), j = c0 + jl;
+            const unsigned f = P.mvf[SP.mv0 + jl];
+            if (combo >> (f >> 8)) continue;
+            c.r = (unsigned)combo << (f & 0xffu);
+            iv64 g{0.0, 0.0};
+            iv32 g32{0.f, 0.f};
+            bool have = false;
+            for (int k = 0; k < P.n_sum; k++) {
+                const int2 rg = P.jk[SP.jk0 + jl * P.n_sum + k];
+                if (rg.x == rg.y) continue;
+                iv64 D{0.0, 0.0};
+                iv32 D32{0.f, 0.f};
+                for (int q = rg.x; q < rg.y; q++) {
+                    const GbContrib C = P.contribs[q];
+                    const int at = C.base + (int)((c.r >> C.dshift) & C.mask) * T.max_leaves;
+                    const double2 v = tl[at];
+                    D = q > rg.x ? iadd(D, iv64{v.x, v.y}) : iv64{v.x, v.y};
+                    if (tl32) {
+                        const float2 v32 = tl32[at];
+                        D32 = q > rg.x ? iadd(D32, iv32{v32.x, v32.y}) : iv32{v32.x, v32.y};
+                    }
+                }
+                ops += 2 * (rg.y - rg.x);
+                if (tl32) ops32 += 2 * (rg.y - rg.x);
+                g = have ? iadd(g, D) : D;
+                g32 = have ? iadd(g32, D32) : D32;
+                have = true;
+            }
+            const View<double> X = view64(pool, par, c, sp);
+            const bool h64 = mono_hit(P, X, j, gt_zero(g.lo), lt_zero(g.hi));
+            const bool h32 = tl32 && mono_hit(P, X, j, gt_zero(g32.lo), lt_zero(g32.hi));
+            T.mv64[(((size_t)p * P.B + jl) << GB_MV_BITS) + combo] = (h32 ? 1 : 0) | (h64 ? 2 : 0);
+        }
+    }
     // (1) partial tables
-    for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < nd_items; item += gridDim.x * blockDim.x) {
+    for (int item = blockIdx.x * blockDim.x + threadIdx.x; !UNIT && item < nd_items; item += nd_blocks * blockDim.x) {
         const int e = item >> GB_TAB_DBITS, c = item & ((1 << GB_TAB_DBITS) - 1);
         const GbJkD J = P.jkd[SP.jk0 + e];
         if (J.shift < 0 || c > (int)J.mask) continue;
@@ -380,9 +431,9 @@ __global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents
     }
     // (2) segment tables
     const int nw_items = SP.srows;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const int nwarps = ((gridDim.x - nd_blocks) * blockDim.x) >> 5;
     const size_t rb = (size_t)p * T.max_rows;
-    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw_items; w += nwarps) {
+    for (int w = (((int)blockIdx.x - nd_blocks) * (int)blockDim.x + (int)threadIdx.x) >> 5; w >= 0 && w < nw_items; w += nwarps) {
         // the tabulated segment owning row w (a lane per segment)
         int si = -1;
         for (int s0 = 0; s0 < SP.nseg && si < 0; s0 += 32) {
@@ -447,11 +498,33 @@ __global__ void __launch_bounds__(128) k_ptab_d(GbProg P, GbPool pool, GbParents
 // ---------------------------------------------------------------------------
 // tab_path for 32 lanes that walk the same path (same tree and dirty range)
 // over their own dirty values: the sibling nodes are loaded once across the
-// lanes (lane t the t-th one the walk reads) and handed out by shuffles;
-// every lane computes its own walk.  Same operations in the same order as
-// tab_path.
+// lanes (lane t the t-th one the walk reads; tab_path_pre, ahead of the dirty
+// values, which it does not need) and handed out by shuffles; every lane
+// computes its own walk.  Same operations in the same order as tab_path.
 template <typename I, typename N>
-__device__ __forceinline__ I tab_path_lanes(const GbSum& S, int2 dr, I* cur, N node, int lane, int& ops) {
+__device__ __forceinline__ I tab_path_pre(const GbSum& S, int2 dr, N node, int lane) {
+    I pre;
+    pre.lo = 0;
+    pre.hi = 0;
+    if (S.ngroups == 0 || S.nnodes <= 0 || dr.x >= dr.y) return pre;
+    int mine = -1, cnt = 0;
+    int lo = dr.x, hi = dr.y, off = 0;
+    for (int mL = S.ngroups; mL > 1; mL = (mL + 1) / 2) {
+        const int nlo = lo >> 1, nhi = ((hi - 1) >> 1) + 1;
+        for (int q = nlo; q < nhi; q++) {
+            const int a = 2 * q;
+            if (!(a >= lo && a < hi)) mine = cnt++ == lane ? off + a : mine;
+            if (a + 1 < mL && !(a + 1 >= lo && a + 1 < hi)) mine = cnt++ == lane ? off + a + 1 : mine;
+        }
+        lo = nlo;
+        hi = nhi;
+        off += mL;
+    }
+    if (mine >= 0) pre = node(mine);
+    return pre;
+}
+template <typename I, typename N>
+__device__ __forceinline__ I tab_path_lanes(const GbSum& S, int2 dr, I pre, I* cur, N node, int& ops) {
     if (S.ngroups == 0 || S.nnodes <= 0) {
         I z;
         z.lo = 0;
@@ -459,25 +532,6 @@ __device__ __forceinline__ I tab_path_lanes(const GbSum& S, int2 dr, I* cur, N n
         return z;
     }
     if (dr.x >= dr.y) return node(S.nnodes - 1);
-    int mine = -1, cnt = 0;
-    {
-        int lo = dr.x, hi = dr.y, off = 0;
-        for (int mL = S.ngroups; mL > 1; mL = (mL + 1) / 2) {
-            const int nlo = lo >> 1, nhi = ((hi - 1) >> 1) + 1;
-            for (int q = nlo; q < nhi; q++) {
-                const int a = 2 * q;
-                if (!(a >= lo && a < hi)) mine = cnt++ == lane ? off + a : mine;
-                if (a + 1 < mL && !(a + 1 >= lo && a + 1 < hi)) mine = cnt++ == lane ? off + a + 1 : mine;
-            }
-            lo = nlo;
-            hi = nhi;
-            off += mL;
-        }
-    }
-    I pre;
-    pre.lo = 0;
-    pre.hi = 0;
-    if (mine >= 0) pre = node(mine);
     I tmp[GB_TAB_MAX_DIRTY];
     int lo = dr.x, hi = dr.y, off = 0, used = 0;
     auto take = [&](int idx) {
@@ -517,17 +571,23 @@ __device__ __forceinline__ I tab_path_lanes(const GbSum& S, int2 dr, I* cur, N n
 // are consecutive children of the same (sum, kind), so a warp follows one
 // control path; the ~10^4 short chains run side by side instead of one
 // child's chains one after another in a warp.
+// Bound: latency.  What a chain reads to find its values (sums, dirty ranges,
+// segments) is staged in shared memory when the block's children share a
+// parent, a segment run's values are loaded CS_BATCH at a time, the tree
+// path's sibling nodes before them; one after the other, each of these missed
+// L1 at ~700 clocks (13k clocks a chain, n = 10^4 family).
+constexpr int CS_SEGS = 256;   // segments staged (more: read where they are)
+constexpr int CS_BATCH = 4;
 template <typename I, typename P2>
-__device__ __forceinline__ void child_sum(const GbProg& P, const GbSplitPos& SP, int k, int blk, unsigned r,
+__device__ __forceinline__ void child_sum(const GbSum& S, int2 dr, const GbSeg* seg, int nseg, int k, unsigned r,
                                           const P2* trow, const P2* tseg, const P2* nodes, I* gout, I* sout,
                                           bool lanes, int& ops) {
-    const GbSum S = P.sums[k];
-    const int2 dr = P.dirty[blk * P.n_sum + k];
-    int sg = SP.seg0;
-    const int send = SP.seg0 + SP.nseg;
-    while (sg < send) {   // the run of (k, first dirty group): segments are ordered by sum, group, term
-        const GbSeg G = P.segs[sg];
-        if (G.sum > k || (G.sum == k && G.group >= dr.x)) break;
+    auto node = [&](int i) { const P2 v = nodes[S.node0 + i]; return mk<decltype(v.x)>(v.x, v.y); };
+    I pre;
+    if (lanes) pre = tab_path_pre<I>(S, dr, node, threadIdx.x & 31);
+    int sg = 0;
+    while (sg < nseg) {   // the run of (k, first dirty group): segments are ordered by sum, group, term
+        if (seg[sg].sum > k || (seg[sg].sum == k && seg[sg].group >= dr.x)) break;
         sg++;
     }
     I cur[GB_TAB_MAX_DIRTY];
@@ -535,21 +595,31 @@ __device__ __forceinline__ void child_sum(const GbProg& P, const GbSplitPos& SP,
         Tree<I> tr;
         tr.init();
         int ns = 0;
-        while (sg < send) {
-            const GbSeg G = P.segs[sg];
-            if (G.sum != k || G.group != g) break;
-            const int at = G.base + (int)((r >> G.shift) & G.mask);
-            const P2 v = G.level ? tseg[at] : trow[at];
-            tr.push_level(mk<decltype(v.x)>(v.x, v.y), G.level);
-            ns++;
-            sg++;
+        for (;;) {
+            P2 v[CS_BATCH];
+            int lev[CS_BATCH], m = 0;
+#pragma unroll
+            for (int u = 0; u < CS_BATCH; u++) {
+                if (m < u || sg + u >= nseg) continue;
+                const GbSeg G = seg[sg + u];
+                if (G.sum != k || G.group != g) continue;
+                const int at = G.base + (int)((r >> G.shift) & G.mask);
+                v[u] = G.level ? tseg[at] : trow[at];
+                lev[u] = G.level;
+                m = u + 1;
+            }
+#pragma unroll
+            for (int u = 0; u < CS_BATCH; u++)
+                if (u < m) tr.push_level(mk<decltype(v[u].x)>(v[u].x, v[u].y), lev[u]);
+            ns += m;
+            sg += m;
+            if (m < CS_BATCH) break;
         }
         ops += 2 * (ns > 0 ? ns - 1 : 0);
         cur[g - dr.x] = tr.result();
         gout[k * GB_TAB_MAX_DIRTY + (g - dr.x)] = cur[g - dr.x];
     }
-    auto node = [&](int i) { const P2 v = nodes[S.node0 + i]; return mk<decltype(v.x)>(v.x, v.y); };
-    *sout = lanes ? tab_path_lanes(S, dr, cur, node, threadIdx.x & 31, ops) : tab_path(S, dr, cur, node, ops);
+    *sout = lanes ? tab_path_lanes(S, dr, pre, cur, node, ops) : tab_path(S, dr, cur, node, ops);
 }
 
 // The first-order verdict of one (parent, kind, block coordinate, digit
@@ -572,38 +642,60 @@ __global__ void __launch_bounds__(128) k_child_sums(GbProg P, GbPool pool, GbPar
         warp_add_ops(o32, &st->ops32);
         return;
     }
+    const int n_sum = P.n_sum > 0 ? P.n_sum : 1;
     const long long ci = t % Cmax, rest = t / Cmax;
-    const int k = (int)(rest % (P.n_sum > 0 ? P.n_sum : 1)), kind = (int)(rest / (P.n_sum > 0 ? P.n_sum : 1));
+    const int k = (int)(rest % n_sum), kind = (int)(rest / n_sum);
     int ops = 0;
+    const long long nch = nch_fixed >= 0 ? nch_fixed : st->nch;
+    // the block's children share a parent (the decision is the block's)
+    const long long b0 = (t - threadIdx.x) % Cmax;
+    const bool one = b0 + blockDim.x <= Cmax && b0 >> sp.flog2 == (b0 + blockDim.x - 1) >> sp.flog2 && b0 < nch;
+    __shared__ GbSum s_sum[GB_MAX_ISUM];
+    __shared__ int2 s_dirty[GB_MAX_ISUM];
+    __shared__ GbSeg s_seg[CS_SEGS];
+    bool staged = false;
+    if (one) {
+        const GbSplitPos SP = par.spos[b0 >> sp.flog2];
+        staged = SP.nseg <= CS_SEGS;
+        if (threadIdx.x < P.n_sum) {
+            s_sum[threadIdx.x] = P.sums[threadIdx.x];
+            s_dirty[threadIdx.x] = P.dirty[SP.block * P.n_sum + threadIdx.x];
+        }
+        if (staged)
+            for (int i = threadIdx.x; i < SP.nseg; i += blockDim.x) s_seg[i] = P.segs[SP.seg0 + i];
+        __syncthreads();
+    }
     // the warp's 32 children share one path when they share a parent and a
     // (sum, kind) and all of them are evaluated (the decision is the warp's)
     const long long t0 = t - (threadIdx.x & 31);
     bool lanes = t0 % Cmax + 31 < Cmax && (t0 % Cmax) >> sp.flog2 == (t0 % Cmax + 31) >> sp.flog2 &&
                  t0 + 31 < (long long)gridDim.x * blockDim.x;
-    const bool live0 = P.n_sum > 0 && kind < kinds && ci < (nch_fixed >= 0 ? nch_fixed : st->nch);
+    const bool live0 = P.n_sum > 0 && kind < kinds && ci < nch;
     ChildCtx c{};
-    int spi = -1;
+    GbSplitPos SP{};
+    bool live = false;
     if (live0) {
         c = child_ctx(par, ci, sp);
-        spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
+        SP = par.spos[c.p];
+        live = c.valid && SP.ndterm >= 0;
     }
-    if (lanes) lanes = __all_sync(0xffffffffu, live0 && spi >= 0);
-    {
-        if (live0 && spi >= 0) {
-            const GbSplitPos SP = P.sps[spi];
-            const size_t rowb = (size_t)c.p * Tb.max_rows, segb = (size_t)c.p * Tb.max_srows,
-                         nodeb = (size_t)c.p * Tb.tree_nodes;
-            const size_t so = (size_t)ci * P.n_sum + k, go = (size_t)ci * GB_CG;
-            if (kind == 0)
-                child_sum<iv64>(P, SP, k, c.info.z, c.r, Tb.tv64 + rowb, Tb.ts64 + segb, Tb.nf64 + nodeb,
-                                (iv64*)(Tb.cg64 + go), (iv64*)(Tb.cs64 + so), lanes, ops);
-            else if (kind == 1)
-                child_sum<iv64>(P, SP, k, c.info.z, c.r, Tb.tm64 + rowb, Tb.tsm64 + segb, Tb.nm64 + nodeb,
-                                (iv64*)(Tb.cgm64 + go), (iv64*)(Tb.csm64 + so), lanes, ops);
-            else
-                child_sum<iv32>(P, SP, k, c.info.z, c.r, Tb.tv32 + rowb, Tb.ts32 + segb, Tb.nf32 + nodeb,
-                                (iv32*)(Tb.cg32 + go), (iv32*)(Tb.cs32 + so), lanes, ops);
-        }
+    if (lanes) lanes = __all_sync(0xffffffffu, live);
+    if (live) {
+        const GbSum S = one ? s_sum[k] : P.sums[k];
+        const int2 dr = one ? s_dirty[k] : P.dirty[c.info.z * P.n_sum + k];
+        const GbSeg* seg = staged ? s_seg : P.segs + SP.seg0;
+        const size_t rowb = (size_t)c.p * Tb.max_rows, segb = (size_t)c.p * Tb.max_srows,
+                     nodeb = (size_t)c.p * Tb.tree_nodes;
+        const size_t so = (size_t)ci * P.n_sum + k, go = (size_t)ci * GB_CG;
+        if (kind == 0)
+            child_sum<iv64>(S, dr, seg, SP.nseg, k, c.r, Tb.tv64 + rowb, Tb.ts64 + segb, Tb.nf64 + nodeb,
+                            (iv64*)(Tb.cg64 + go), (iv64*)(Tb.cs64 + so), lanes, ops);
+        else if (kind == 1)
+            child_sum<iv64>(S, dr, seg, SP.nseg, k, c.r, Tb.tm64 + rowb, Tb.tsm64 + segb, Tb.nm64 + nodeb,
+                            (iv64*)(Tb.cgm64 + go), (iv64*)(Tb.csm64 + so), lanes, ops);
+        else
+            child_sum<iv32>(S, dr, seg, SP.nseg, k, c.r, Tb.tv32 + rowb, Tb.ts32 + segb, Tb.nf32 + nodeb,
+                            (iv32*)(Tb.cg32 + go), (iv32*)(Tb.cs32 + so), lanes, ops);
     }
     warp_add_ops(kind < 2 ? ops : 0, &st->ops64);
     warp_add_ops(kind == 2 ? ops : 0, &st->ops32);
@@ -734,7 +826,7 @@ __device__ __forceinline__ unsigned unit_sums(const GbProg& P, const I* OA) {
 
 // The first-order test discards the box when a partial has a fixed sign and
 // the box does not touch the bound the sign points to.
-__device__ __forceinline__ bool mono_hit(const GbProg& P, const View<double>& X64, int j, bool pos, bool neg) {
+__device__ bool mono_hit(const GbProg& P, const View<double>& X64, int j, bool pos, bool neg) {
     if (!pos && !neg) return false;
     const iv64 x = X64.get(j);
     return (pos && !same_value(x.lo, __ldg(P.l + j))) || (neg && !same_value(x.hi, __ldg(P.u + j)));
@@ -791,9 +883,8 @@ __device__ void mono_fill(const GbProg& P, const GbPool& pool, const GbParents& 
     const int jl = (int)((rem >> GB_MV_BITS) % P.B), combo = (int)(rem & ((1 << GB_MV_BITS) - 1));
     if (!Tb.mv64 || p >= npar) return;
     const int4 info = par.info[p];
-    const int spi = P.sp_of_cyc[info.x];
-    if (spi < 0) return;
-    const GbSplitPos SP = P.sps[spi];
+    const GbSplitPos SP = par.spos[p];
+    if (SP.ndterm < 0) return;
     const int c0 = info.z * P.B, c1 = min(P.n, c0 + P.B), j = c0 + jl;
     if (j >= c1) return;
     auto meta = [&](int k, int& x, int& y, int& shift, unsigned& mask) {
@@ -1599,10 +1690,9 @@ __device__ __forceinline__ void child_w(const GbProg& P, const GbPool& pool, con
                                         WCount& n, int lane, const WScratch& ws) {
     child_sums_w<F32, true>(P, Tb, ci, ws, lane);
     const ChildCtx c = child_ctx(par, ci, sp);
-    const int spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
-    bool pass = spi >= 0;
+    const GbSplitPos SP = par.spos[c.p];
+    bool pass = c.valid && SP.ndterm >= 0;
     if (pass) {
-        const GbSplitPos SP = P.sps[spi];
         n.nv++;
         __syncwarp();
         if (F32) pass = eval32_tab_child_w(P, pool, par, Tb, c, SP, sp, gub_prev, n.red32, n.pops32, lane, ws);
@@ -1643,6 +1733,141 @@ __global__ void __launch_bounds__(128, 1) k_eval_tabw(GbProg P, GbPool pool, GbP
         child_w<F32>(P, pool, par, Tb, ch, ci, sp, gub_prev, n, lane, ws);
     n.add(st, F32, lane);
     if (cc) list_survivors_last(ch, lim, G, st);
+}
+
+// GbTabs::unit: the children of a parent 32 to a block.  A warp per (sum, kind)
+// forms the block's 32 sums (child_sum, a child per lane) while every warp
+// looks the block coordinates' verdicts up in shared memory; then one warp
+// each takes F in FP32, F and the midpoint through the outer expression, a
+// child per lane, and the first one decides: a child passes FP32, its sample
+// counts, it is kept -- the tests, values and order of k_child_sums and
+// k_eval_tabw (whose warp per child spent its time in one lane, three dependent
+// lookups deep).  With one parent it runs beside the pool partition.
+// Bound: latency (one chain of loads, the sums, the outer expression, the
+// block's arrival).  Measured on GB300, 2^10 children of the n = 10^4 family:
+// 16.6 us where k_child_sums (10.2, beside the partition) and k_eval_tabw (16,
+// after it) took 26; a solve of 21,897 generations 1490 -> 1288 ms.  Blocks of
+// 32 children from 32 children per parent on; fewer leave lanes idle.
+template <bool F32>
+__global__ void __launch_bounds__(32 * 3 * GB_MAX_ISUM) k_unit(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
+                                                               GbChildren ch, GbSplit sp, GbState* st,
+                                                               long long nch_fixed, GbGenConst G, int cc, int late) {
+    gb_grid_trigger();
+    gb_grid_wait();
+    __shared__ WProg s_prog;
+    __shared__ int2 s_dirty[GB_MAX_ISUM];
+    __shared__ GbSeg s_seg[CS_SEGS];
+    __shared__ uint4 s_mv[GB_UNIT_B << (GB_MV_BITS - 4)];
+    __shared__ uint16_t s_mvf[GB_UNIT_B];
+    __shared__ iv64 s_s64[2][GB_MAX_ISUM][32];
+    __shared__ iv32 s_s32[GB_MAX_ISUM][32];
+    __shared__ unsigned s_hit[2], s_above[2];   // children: ruled out (FP32, FP64), F above the incumbent
+    __shared__ double s_lo[32], s_mid[32];
+    stage_prog(P, s_prog);
+    if (st->halt) return;
+    const long long nch = nch_fixed >= 0 ? nch_fixed : st->nch;
+    const long long c0 = blockIdx.x * 32LL;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+    int n = 0;   // valid children of the block
+    int ops = 0, ops32 = 0;
+    if (c0 < nch) {
+        const long long p = c0 >> sp.flog2;
+        const unsigned r0 = (unsigned)(c0 & ((1LL << sp.flog2) - 1));
+        const int4 info = par.info[p];
+        const GbSplitPos SP = par.spos[p];
+        const unsigned top = 1u << (info.y * sp.mshift);
+        n = SP.ndterm >= 0 && r0 < top ? (int)min(32u, top - r0) : 0;
+        if (n) {
+            const double gub_prev = gb_key_value(st->gub_key);
+            const int cb = min(P.B, P.n - info.z * P.B);   // coordinates of the block
+            const bool staged = SP.nseg <= CS_SEGS;
+            if (threadIdx.x < P.n_sum) s_dirty[threadIdx.x] = P.dirty[info.z * P.n_sum + threadIdx.x];
+            if (threadIdx.x < 2) s_hit[threadIdx.x] = s_above[threadIdx.x] = 0;
+            for (int i = threadIdx.x; staged && i < SP.nseg; i += blockDim.x) s_seg[i] = P.segs[SP.seg0 + i];
+            const uint4* mv = reinterpret_cast<const uint4*>(Tb.mv64 + ((size_t)p * P.B << GB_MV_BITS));
+            for (int i = threadIdx.x; i < cb << (GB_MV_BITS - 4); i += blockDim.x) s_mv[i] = mv[i];
+            for (int i = threadIdx.x; i < cb; i += blockDim.x) s_mvf[i] = P.mvf[SP.mv0 + i];
+            __syncthreads();
+            const unsigned r = r0 + lane;
+            const int kinds = F32 ? 3 : 2;
+            for (int job = w; job < P.n_sum * kinds; job += W) {
+                const int k = job % P.n_sum, kind = job / P.n_sum;
+                if (lane >= n) continue;
+                const GbSum S = P.sums[k];
+                const int2 dr = s_dirty[k];
+                const GbSeg* seg = staged ? s_seg : P.segs + SP.seg0;
+                const size_t rowb = (size_t)p * Tb.max_rows, segb = (size_t)p * Tb.max_srows, nodeb = (size_t)p * Tb.tree_nodes;
+                const size_t go = (size_t)(c0 + lane) * GB_CG;
+                const bool lanes = n == 32;
+                if (kind == 0)
+                    child_sum<iv64>(S, dr, seg, SP.nseg, k, r, Tb.tv64 + rowb, Tb.ts64 + segb, Tb.nf64 + nodeb,
+                                    (iv64*)(Tb.cg64 + go), &s_s64[0][k][lane], lanes, ops);
+                else if (kind == 1)
+                    child_sum<iv64>(S, dr, seg, SP.nseg, k, r, Tb.tm64 + rowb, Tb.tsm64 + segb, Tb.nm64 + nodeb,
+                                    (iv64*)(Tb.cgm64 + go), &s_s64[1][k][lane], lanes, ops);
+                else if (F32)
+                    child_sum<iv32>(S, dr, seg, SP.nseg, k, r, Tb.tv32 + rowb, Tb.ts32 + segb, Tb.nf32 + nodeb,
+                                    (iv32*)(Tb.cg32 + go), &s_s32[k][lane], lanes, ops32);
+            }
+            unsigned hit = 0;
+            const unsigned char* mvb = reinterpret_cast<const unsigned char*>(s_mv);
+            for (int j = w; j < cb; j += W) {
+                const unsigned f = s_mvf[j];
+                hit |= mvb[(j << GB_MV_BITS) + ((r >> (f & 0xffu)) & ((1u << (f >> 8)) - 1u))];
+            }
+            const unsigned h32 = __ballot_sync(0xffffffffu, hit & 1u), h64 = __ballot_sync(0xffffffffu, hit & 2u);
+            if (lane == 0 && h32) atomicOr(&s_hit[0], h32);
+            if (lane == 0 && h64) atomicOr(&s_hit[1], h64);
+            __syncthreads();
+            if (w < 2) {   // warp 0 F in FP64, warp 1 the midpoint
+                iv64 sums[GB_MAX_ISUM], O[GB_MAX_OREGS];
+                for (int k = 0; k < P.n_sum; k++) sums[k] = s_s64[w][k][lane];
+                const iv64 F = outer_value<double>(P, View<double>{}, sums, O, ops);
+                if (w == 0) {
+                    s_lo[lane] = F.lo;
+                    const unsigned b = __ballot_sync(0xffffffffu, F.lo > gub_prev);
+                    if (lane == 0) s_above[1] = b;
+                } else {
+                    s_mid[lane] = F.hi;
+                }
+            } else if (F32 && w == 2) {
+                iv32 sums[GB_MAX_ISUM], O[GB_MAX_OREGS];
+                for (int k = 0; k < P.n_sum; k++) sums[k] = s_s32[k][lane];
+                const iv32 F = outer_value<float>(P, View<float>{}, sums, O, ops32);
+                const unsigned b = __ballot_sync(0xffffffffu, (double)F.lo > gub_prev);
+                if (lane == 0) s_above[0] = b;
+            }
+            __syncthreads();
+        }
+        if (w == 0) {
+            const unsigned bit = 1u << lane;
+            const bool valid = lane < n;
+            const bool pass = valid && (!F32 || !((s_above[0] | s_hit[0]) & bit));
+            const bool keep = pass && !((s_above[1] | s_hit[1]) & bit);
+            unsigned long long key = ~0ull;
+            if (pass && s_mid[lane] == s_mid[lane]) key = gb_order_key(s_mid[lane]);
+            if (F32) ch.flag32[c0 + lane] = pass ? 1 : 0;
+            ch.flag[c0 + lane] = keep ? 1 : 0;
+            ch.flo[c0 + lane] = pass ? canon_lo(s_lo[lane]) : __longlong_as_double(0x7ff0000000000000LL);
+            warp_min_gub(key, key != ~0ull, st);
+            const unsigned long long n32 = __popc(__ballot_sync(0xffffffffu, pass));
+            if (lane == 0 && n) {
+                if (F32) atomicAdd((unsigned long long*)&st->evals32, (unsigned long long)n);
+                atomicAdd((unsigned long long*)&st->children, (unsigned long long)n);
+            }
+            if (lane == 0 && n32) {
+                atomicAdd((unsigned long long*)&st->evals64, n32);
+                atomicAdd((unsigned long long*)&st->mids, n32);
+                if (F32) {
+                    atomicAdd((unsigned long long*)&st->kept32, n32);
+                    atomicAdd((unsigned long long*)&st->n32, n32);
+                }
+            }
+        }
+    }
+    warp_add_ops(ops, &st->ops64);
+    if (F32) warp_add_ops(ops32, &st->ops32);
+    if (cc) list_survivors_last(ch, nch, G, st, late != 0);
 }
 
 // The same FP32-then-FP64 warp-per-child evaluation over the children of
@@ -1749,13 +1974,24 @@ cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbPa
 }
 
 cudaError_t gb_launch_ptab_d(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
-                             long long K, int B, GbState* st, cudaStream_t s, bool fixed) {
-    // threads for the partial-table entries, warps for the segment entries
-    const long long items = std::max<long long>((long long)B * P.n_sum << GB_TAB_DBITS,
-                                                (long long)P.max_srows << 5);
-    unsigned g = grid_for(items, 128);
-    if (g > (unsigned)gb_sm_count() * 16) g = gb_sm_count() * 16;
-    return gb_launch_ex(k_ptab_d, dim3(g, (unsigned)K), 128, 0, s, true, P, pool, par, T, st, fixed ? 1 : 0);
+                             const GbSplit& sp, long long K, GbState* st, cudaStream_t s, bool fixed, bool unit) {
+    // threads for the partial-table (verdict) entries, then warps for the segment entries
+    const unsigned cap = (unsigned)gb_sm_count() * 8;
+    const unsigned nd = std::min<unsigned>(grid_for((long long)P.B * (unit ? 1 : P.n_sum) << GB_TAB_DBITS, 128), cap);
+    const unsigned ng = std::min<unsigned>(grid_for((long long)P.max_srows << 5, 128), cap);
+    static_assert(GB_TAB_DBITS == GB_MV_BITS, "one grid for either table");
+    return gb_launch_ex(unit ? k_ptab_d<true> : k_ptab_d<false>, dim3(nd + ng, (unsigned)K), 128, 0, s, true, P, pool,
+                        par, T, sp, st, (int)nd, fixed ? 1 : 0);
+}
+
+int gb_unit_threads(const GbProg& P, bool fp32) { return 32 * std::max(4, P.n_sum * (fp32 ? 3 : 2)); }
+
+cudaError_t gb_launch_unit(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
+                           const GbChildren& ch, long long Cmax, const GbSplit& sp, bool fp32, GbState* st,
+                           cudaStream_t s, bool fixed, const GbGenConst* cc, bool late) {
+    const long long nch = fixed ? (1LL << sp.flog2) : -1;
+    return gb_launch_ex(fp32 ? k_unit<true> : k_unit<false>, grid_for(Cmax, 32), gb_unit_threads(P, fp32), 0, s, true, P,
+                        pool, par, T, ch, sp, st, nch, cc ? *cc : GbGenConst{}, cc ? 1 : 0, late ? 1 : 0);
 }
 
 cudaError_t gb_launch_child_sums(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,

@@ -56,6 +56,8 @@ struct GbParents {
     double* bnd;      // [K][dmax][m+1] piece boundaries
     float* bnd_rd;    // boundaries rounded down / up to float
     float* bnd_ru;
+    GbSplitPos* spos; // term tables: the parent's split position (ndterm < 0: it has none), written by k_ptab --
+                      // one load where the cycling position's lookup takes three dependent ones
 };
 
 struct GbChildren {
@@ -127,6 +129,11 @@ struct GbTabs {
     int reg;
     int dec;          // one child per thread: endpoint programs (P.uops) evaluate the children
     GbCut cut;        // with dec
+    // one child per warp, objectives as for the verdict tables, at least 32
+    // children per parent, every coordinate's verdict within GB_MV_BITS digit
+    // bits: k_unit takes the children 32 to a block instead (mv64 then holds
+    // bit 0 the FP32, bit 1 the FP64 verdict)
+    int unit;
 };
 // Paper mode (diagonal samples, first-order test on every coordinate) from
 // per-parent tables.  Kind 0 is the box, kinds 1 .. nk - 1 its sample points
@@ -161,6 +168,7 @@ struct GbDec {
 };
 constexpr int GB_CG = GB_MAX_ISUM * GB_TAB_MAX_DIRTY;
 constexpr int GB_MV_BITS = 6;
+constexpr int GB_UNIT_B = 256;   // block coordinates k_unit stages the verdicts of
 constexpr int GB_REG_DIRTY = 4;
 constexpr int GB_REG_LEVELS = 5;
 
@@ -351,8 +359,16 @@ cudaError_t gb_launch_eval64_tab(const GbProg& P, const GbPool& pool, const GbPa
 // FP32 prefilter + FP64 evaluation fused, one child per warp (tables).
 // Partial tables of every parent (after gb_launch_ptab).
 // fixed: the generation has K parents for certain (do not read the count the partition writes).
+// unit: the verdict tables of k_unit instead of the partial tables.
 cudaError_t gb_launch_ptab_d(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
-                             long long K, int B, GbState* st, cudaStream_t s, bool fixed = false);
+                             const GbSplit& sp, long long K, GbState* st, cudaStream_t s, bool fixed, bool unit);
+// GbTabs::unit: every child's sums, values and verdicts (tables first).  fixed: one parent, nothing read that the
+// partition writes.  cc non-null: the last block lists the survivors (late: whether they fit is left to
+// k_materialize).
+int gb_unit_threads(const GbProg& P, bool fp32);
+cudaError_t gb_launch_unit(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
+                           const GbChildren& ch, long long Cmax, const GbSplit& sp, bool fp32, GbState* st,
+                           cudaStream_t s, bool fixed, const GbGenConst* cc, bool late);
 // One child per warp: every child's sums and dirty group values (tables first).
 cudaError_t gb_launch_child_sums(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                                  const GbSplit& sp, long long Cmax, int fp32, GbState* st, cudaStream_t s,
