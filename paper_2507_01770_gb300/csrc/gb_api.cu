@@ -536,6 +536,8 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
                 if ((e = upload(&d_mvf, Hh.mvf.data(), Hh.mvf.size(), A))) return bad(e, "upload table layouts");
                 P.mvf = d_mvf;
                 p->tabs.unit = 1;
+            } else if (warp && d * mshift >= 5 && P.n_sum > 0) {
+                p->tabs.unit = 2;
             }
             if ((e = upload(&d_jkd, Hh.jkd.data(), Hh.jkd.size(), A)) ||
                 (e = upload(&d_segs, Hh.segs.data(), Hh.segs.size(), A)) ||

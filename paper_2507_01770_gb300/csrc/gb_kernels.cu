@@ -2023,11 +2023,11 @@ cudaError_t gb_launch_generation(const GbProg& P, const GbPool& pool, const GbEn
         if ((et = gb_launch_ptab(P, pool, par, *tabs, G.K, sp, st, ts, sel_tabs ? &E : nullptr)) != cudaSuccess)
             return et;
         gb_launch_count++;
-        if ((et = gb_launch_ptab_d(P, pool, par, *tabs, sp, G.K, st, ts, sel_tabs, unit)) != cudaSuccess) return et;
+        if ((et = gb_launch_ptab_d(P, pool, par, *tabs, sp, G.K, st, ts, sel_tabs, unit && tabs->unit == 1)) != cudaSuccess) return et;
         if (unit) {   // the children too: with one parent they need nothing from the partition
             if (ev) cudaEventRecord(ev[2], ts), cudaEventRecord(ev[3], ts);
             gb_launch_count++;
-            cc_done = Cmax <= 64LL * gb_unit_threads(P, G.fp32);
+            cc_done = Cmax <= 64LL * gb_unit_threads(P, *tabs, G.fp32);
             late = cc_done && ts != s;
             et = gb_launch_unit(P, pool, par, *tabs, ch, Cmax, sp, G.fp32, st, ts, sel_tabs, cc_done ? &G : nullptr, late);
             if (ev) cudaEventRecord(ev[1], ts);

@@ -1735,6 +1735,63 @@ __global__ void __launch_bounds__(128, 1) k_eval_tabw(GbProg P, GbPool pool, GbP
     if (cc) list_survivors_last(ch, lim, G, st);
 }
 
+// The sums of a block's 32 children (n of them valid, child indices r = r0 +
+// lane of parent p), a warp per (sum, kind), a child per lane.
+template <bool F32>
+__device__ __forceinline__ void block_sums(const GbProg& P, const GbTabs& Tb, const GbSplitPos& SP, long long p,
+                                           long long c0, unsigned r, int n, const GbSeg* seg, const int2* dirty,
+                                           iv64 (*s64)[GB_MAX_ISUM][32], iv32 (*s32)[32], int& ops, int& ops32) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+    const size_t rowb = (size_t)p * Tb.max_rows, segb = (size_t)p * Tb.max_srows, nodeb = (size_t)p * Tb.tree_nodes;
+    const size_t go = (size_t)(c0 + lane) * GB_CG;
+    const bool lanes = n == 32;
+    for (int job = w; job < P.n_sum * (F32 ? 3 : 2); job += W) {
+        if (lane >= n) continue;
+        const int k = job % P.n_sum, kind = job / P.n_sum;
+        const GbSum S = P.sums[k];
+        const int2 dr = dirty[k];
+        if (kind == 0)
+            child_sum<iv64>(S, dr, seg, SP.nseg, k, r, Tb.tv64 + rowb, Tb.ts64 + segb, Tb.nf64 + nodeb,
+                            (iv64*)(Tb.cg64 + go), &s64[0][k][lane], lanes, ops);
+        else if (kind == 1)
+            child_sum<iv64>(S, dr, seg, SP.nseg, k, r, Tb.tm64 + rowb, Tb.tsm64 + segb, Tb.nm64 + nodeb,
+                            (iv64*)(Tb.cgm64 + go), &s64[1][k][lane], lanes, ops);
+        else if (F32)
+            child_sum<iv32>(S, dr, seg, SP.nseg, k, r, Tb.tv32 + rowb, Tb.ts32 + segb, Tb.nf32 + nodeb,
+                            (iv32*)(Tb.cg32 + go), &s32[k][lane], lanes, ops32);
+    }
+}
+
+// What becomes of a block's children, by its first warp: out32, out64 are the
+// children that the FP32 and the FP64 tests remove.  A child that passes FP32
+// counts as evaluated in FP64 and its sample counts.
+template <bool F32>
+__device__ __forceinline__ void block_decide(const GbChildren& ch, GbState* st, long long c0, int n, unsigned out32,
+                                             unsigned out64, const double* lo, const double* mid) {
+    const int lane = threadIdx.x & 31;
+    const unsigned bit = 1u << lane;
+    const bool pass = lane < n && (!F32 || !(out32 & bit)), keep = pass && !(out64 & bit);
+    unsigned long long key = ~0ull;
+    if (pass && mid[lane] == mid[lane]) key = gb_order_key(mid[lane]);
+    if (F32) ch.flag32[c0 + lane] = pass ? 1 : 0;
+    ch.flag[c0 + lane] = keep ? 1 : 0;
+    ch.flo[c0 + lane] = pass ? canon_lo(lo[lane]) : __longlong_as_double(0x7ff0000000000000LL);
+    warp_min_gub(key, key != ~0ull, st);
+    const unsigned long long n32 = __popc(__ballot_sync(0xffffffffu, pass));
+    if (lane == 0 && n) {
+        if (F32) atomicAdd((unsigned long long*)&st->evals32, (unsigned long long)n);
+        atomicAdd((unsigned long long*)&st->children, (unsigned long long)n);
+    }
+    if (lane == 0 && n32) {
+        atomicAdd((unsigned long long*)&st->evals64, n32);
+        atomicAdd((unsigned long long*)&st->mids, n32);
+        if (F32) {
+            atomicAdd((unsigned long long*)&st->kept32, n32);
+            atomicAdd((unsigned long long*)&st->n32, n32);
+        }
+    }
+}
+
 // GbTabs::unit: the children of a parent 32 to a block.  A warp per (sum, kind)
 // forms the block's 32 sums (child_sum, a child per lane) while every warp
 // looks the block coordinates' verdicts up in shared memory; then one warp
@@ -1789,26 +1846,7 @@ __global__ void __launch_bounds__(32 * 3 * GB_MAX_ISUM) k_unit(GbProg P, GbPool 
             for (int i = threadIdx.x; i < cb; i += blockDim.x) s_mvf[i] = P.mvf[SP.mv0 + i];
             __syncthreads();
             const unsigned r = r0 + lane;
-            const int kinds = F32 ? 3 : 2;
-            for (int job = w; job < P.n_sum * kinds; job += W) {
-                const int k = job % P.n_sum, kind = job / P.n_sum;
-                if (lane >= n) continue;
-                const GbSum S = P.sums[k];
-                const int2 dr = s_dirty[k];
-                const GbSeg* seg = staged ? s_seg : P.segs + SP.seg0;
-                const size_t rowb = (size_t)p * Tb.max_rows, segb = (size_t)p * Tb.max_srows, nodeb = (size_t)p * Tb.tree_nodes;
-                const size_t go = (size_t)(c0 + lane) * GB_CG;
-                const bool lanes = n == 32;
-                if (kind == 0)
-                    child_sum<iv64>(S, dr, seg, SP.nseg, k, r, Tb.tv64 + rowb, Tb.ts64 + segb, Tb.nf64 + nodeb,
-                                    (iv64*)(Tb.cg64 + go), &s_s64[0][k][lane], lanes, ops);
-                else if (kind == 1)
-                    child_sum<iv64>(S, dr, seg, SP.nseg, k, r, Tb.tm64 + rowb, Tb.tsm64 + segb, Tb.nm64 + nodeb,
-                                    (iv64*)(Tb.cgm64 + go), &s_s64[1][k][lane], lanes, ops);
-                else if (F32)
-                    child_sum<iv32>(S, dr, seg, SP.nseg, k, r, Tb.tv32 + rowb, Tb.ts32 + segb, Tb.nf32 + nodeb,
-                                    (iv32*)(Tb.cg32 + go), &s_s32[k][lane], lanes, ops32);
-            }
+            block_sums<F32>(P, Tb, SP, p, c0, r, n, staged ? s_seg : P.segs + SP.seg0, s_dirty, s_s64, s_s32, ops, ops32);
             unsigned hit = 0;
             const unsigned char* mvb = reinterpret_cast<const unsigned char*>(s_mv);
             for (int j = w; j < cb; j += W) {
@@ -1839,31 +1877,147 @@ __global__ void __launch_bounds__(32 * 3 * GB_MAX_ISUM) k_unit(GbProg P, GbPool 
             }
             __syncthreads();
         }
-        if (w == 0) {
-            const unsigned bit = 1u << lane;
-            const bool valid = lane < n;
-            const bool pass = valid && (!F32 || !((s_above[0] | s_hit[0]) & bit));
-            const bool keep = pass && !((s_above[1] | s_hit[1]) & bit);
-            unsigned long long key = ~0ull;
-            if (pass && s_mid[lane] == s_mid[lane]) key = gb_order_key(s_mid[lane]);
-            if (F32) ch.flag32[c0 + lane] = pass ? 1 : 0;
-            ch.flag[c0 + lane] = keep ? 1 : 0;
-            ch.flo[c0 + lane] = pass ? canon_lo(s_lo[lane]) : __longlong_as_double(0x7ff0000000000000LL);
-            warp_min_gub(key, key != ~0ull, st);
-            const unsigned long long n32 = __popc(__ballot_sync(0xffffffffu, pass));
-            if (lane == 0 && n) {
-                if (F32) atomicAdd((unsigned long long*)&st->evals32, (unsigned long long)n);
-                atomicAdd((unsigned long long*)&st->children, (unsigned long long)n);
-            }
-            if (lane == 0 && n32) {
-                atomicAdd((unsigned long long*)&st->evals64, n32);
-                atomicAdd((unsigned long long*)&st->mids, n32);
-                if (F32) {
-                    atomicAdd((unsigned long long*)&st->kept32, n32);
-                    atomicAdd((unsigned long long*)&st->n32, n32);
+        if (w == 0)
+            block_decide<F32>(ch, st, c0, n, s_above[0] | s_hit[0], s_above[1] | s_hit[1], s_lo, s_mid);
+    }
+    warp_add_ops(ops, &st->ops64);
+    if (F32) warp_add_ops(ops32, &st->ops32);
+    if (cc) list_survivors_last(ch, nch, G, st, late != 0);
+}
+
+// The same for any outer expression: its values and adjoints per child.  The
+// FP32 test (forward, reverse, coordinates) runs in one warp, a child per lane,
+// beside the FP64 values of every child and of its midpoint, two lanes a child
+// (the pair shares the endpoints of exp, sin and cos); the FP64 reverse sweep
+// and coordinates follow for the children that pass.  A warp per child did
+// these one after the other (FP32 32k clocks, then FP64 60k, n = 1000
+// exp/sqrt/cos family), most of it instructions issued for two lanes of 32.
+// Bound: latency.  Measured on GB300, 2^10 children of that family: 44 us where
+// k_child_sums (9.3, beside the partition) and k_eval_tabw (47, after it) took
+// 56; a solve of 2,634 generations 235 -> 204 ms.
+template <bool F32>
+__global__ void __launch_bounds__(32 * 3 * GB_MAX_ISUM) k_outer32(GbProg P, GbPool pool, GbParents par, GbTabs Tb,
+                                                                  GbChildren ch, GbSplit sp, GbState* st,
+                                                                  long long nch_fixed, GbGenConst G, int cc, int late) {
+    gb_grid_trigger();
+    gb_grid_wait();
+    __shared__ WProg s_prog;
+    __shared__ int2 s_dirty[GB_MAX_ISUM];
+    __shared__ GbSeg s_seg[CS_SEGS];
+    __shared__ iv64 s_s64[2][GB_MAX_ISUM][32];
+    __shared__ iv32 s_s32[GB_MAX_ISUM][32];
+    __shared__ __align__(16) iv64 s_o64[32][GB_WO];   // a child's outer values, then (swept) its adjoints
+    __shared__ iv32 s_oa32[32][GB_WO];                // a child's FP32 adjoints
+    __shared__ unsigned s_out[2], s_unit[2][32];      // children removed by the FP32, FP64 tests
+    __shared__ double s_lo[32], s_mid[32];
+    stage_prog(P, s_prog);
+    if (st->halt) return;
+    const long long nch = nch_fixed >= 0 ? nch_fixed : st->nch;
+    const long long c0 = blockIdx.x * 32LL;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+    int n = 0;   // valid children of the block
+    int ops = 0, ops32 = 0;
+    if (c0 < nch) {
+        ChildCtx c;
+        c.p = c0 >> sp.flog2;
+        const unsigned r0 = (unsigned)(c0 & ((1LL << sp.flog2) - 1));
+        c.info = par.info[c.p];
+        c.slot = par.slot[c.p];
+        c.valid = true;
+        const GbSplitPos SP = par.spos[c.p];
+        const unsigned top = 1u << (c.info.y * sp.mshift);
+        n = SP.ndterm >= 0 && r0 < top ? (int)min(32u, top - r0) : 0;
+        if (n) {
+            const double gub_prev = gb_key_value(st->gub_key);
+            const bool staged = SP.nseg <= CS_SEGS;
+            if (threadIdx.x < P.n_sum) s_dirty[threadIdx.x] = P.dirty[c.info.z * P.n_sum + threadIdx.x];
+            if (threadIdx.x < 2) s_out[threadIdx.x] = 0;
+            for (int i = threadIdx.x; staged && i < SP.nseg; i += blockDim.x) s_seg[i] = P.segs[SP.seg0 + i];
+            __syncthreads();
+            block_sums<F32>(P, Tb, SP, c.p, c0, r0 + lane, n, staged ? s_seg : P.segs + SP.seg0, s_dirty, s_s64, s_s32,
+                            ops, ops32);
+            __syncthreads();
+            // child of this thread in the FP64 phases: 16 pairs a warp
+            const int pi = lane >> 1;
+            if (w < 4) {   // warps 0, 1 the box, 2, 3 the midpoint
+                const int i = (w & 1) * 16 + pi;
+                if (i < n) {
+                    c.r = r0 + i;
+                    iv64 sums[GB_MAX_ISUM], O[GB_MAX_OREGS];
+                    for (int k = 0; k < P.n_sum; k++) sums[k] = s_s64[w >> 1][k][i];
+                    int o = 0;
+                    const PointView X{view64(pool, par, c, sp), w >> 1};
+                    const iv64 F = outer_fwd<double, true>(P, X, sums, O, o);
+                    if (!(lane & 1)) {
+                        ops += o;
+                        (w < 2 ? s_lo : s_mid)[i] = w < 2 ? F.lo : F.hi;
+                        for (int t = 0; w < 2 && t < P.n_outer; t++) s_o64[i][t] = O[t];
+                        if (w < 2 && F.lo > gub_prev) atomicOr(&s_out[1], 1u << i);
+                    }
+                }
+            } else if (F32 && w == 4 && lane < n) {   // FP32: value, adjoints
+                c.r = r0 + lane;
+                iv32 sums[GB_MAX_ISUM], O[GB_MAX_OREGS], A[GB_MAX_OREGS];
+                for (int k = 0; k < P.n_sum; k++) sums[k] = s_s32[k][lane];
+                const iv32 F = outer_fwd<float>(P, view32(pool, par, c, sp), sums, O, ops32);
+                if ((double)F.lo > gub_prev) {
+                    atomicOr(&s_out[0], 1u << lane);
+                } else {
+                    for (int t = 0; t < P.n_outer; t++) A[t] = iv32{0.f, 0.f};
+                    A[P.outer_root] = iv32{1.f, 1.f};
+                    reverse_sweep<float>(P.outer, P.n_outer, O, A, ops32);
+                    for (int t = 0; t < P.n_outer; t++) s_oa32[lane][t] = A[t];
+                    s_unit[0][lane] = unit_sums(P, A);
                 }
             }
+            __syncthreads();
+            const int b0 = c.info.z * P.B, cb = min(P.n, b0 + P.B) - b0;   // the block's coordinates
+            if (F32) {   // FP32 first-order test: a child per lane, the coordinates over the warps
+                const unsigned out = s_out[0];
+                const bool live = lane < n && !((out >> lane) & 1u);
+                c.r = r0 + lane;
+                const View<double> X = view64(pool, par, c, sp);
+                bool hit = false;
+                for (int j = b0 + w; live && !hit && j < b0 + cb; j += W) {
+                    const iv32 g = tab_partial<float>(P, Tb, leaf_tab<float>(Tb, c.p), part_tab<float>(Tb, c.p), SP, j,
+                                                      b0, c.r, s_oa32[lane], s_unit[0][lane], ops32);
+                    hit = mono_hit(P, X, j, gt_zero(g.lo), lt_zero(g.hi));
+                }
+                const unsigned h = __ballot_sync(0xffffffffu, hit);
+                __syncthreads();   // (every warp has read s_out)
+                if (lane == 0 && h) atomicOr(&s_out[0], h);
+                __syncthreads();
+            }
+            // FP64 adjoints of the children left, one pair of lanes each
+            const unsigned left = ~((F32 ? s_out[0] : 0u) | s_out[1]) & (n == 32 ? 0xffffffffu : (1u << n) - 1u);
+            const int nleft = __popc(left);
+            for (int q = w * 16 + pi; q < nleft; q += W * 16) {
+                const int i = __fns(left, 0, q + 1);
+                iv64 A[GB_MAX_OREGS];
+                for (int t = 0; t < P.n_outer; t++) A[t] = iv64{0.0, 0.0};
+                A[P.outer_root] = iv64{1.0, 1.0};
+                int o = 0;
+                reverse_sweep<double, true>(P.outer, P.n_outer, s_o64[i], A, o);
+                __syncwarp(3u << (lane & 30));   // the pair has read the values
+                if (!(lane & 1)) {
+                    ops += o;
+                    for (int t = 0; t < P.n_outer; t++) s_o64[i][t] = A[t];
+                    s_unit[1][i] = unit_sums(P, A);
+                }
+            }
+            __syncthreads();
+            unsigned hit = 0;
+            for (int q = threadIdx.x; q < nleft * cb; q += blockDim.x) {   // and their coordinates
+                const int i = __fns(left, 0, q / cb + 1), j = b0 + q % cb;
+                c.r = r0 + i;
+                const iv64 g = tab_partial<double>(P, Tb, leaf_tab<double>(Tb, c.p), part_tab<double>(Tb, c.p), SP, j,
+                                                   b0, c.r, s_o64[i], s_unit[1][i], ops);
+                if (mono_hit(P, view64(pool, par, c, sp), j, gt_zero(g.lo), lt_zero(g.hi))) hit |= 1u << i;
+            }
+            if (hit) atomicOr(&s_out[1], hit);
+            __syncthreads();
         }
+        if (w == 0) block_decide<F32>(ch, st, c0, n, F32 ? s_out[0] : 0u, s_out[1], s_lo, s_mid);
     }
     warp_add_ops(ops, &st->ops64);
     if (F32) warp_add_ops(ops32, &st->ops32);
@@ -1984,14 +2138,16 @@ cudaError_t gb_launch_ptab_d(const GbProg& P, const GbPool& pool, const GbParent
                         par, T, sp, st, (int)nd, fixed ? 1 : 0);
 }
 
-int gb_unit_threads(const GbProg& P, bool fp32) { return 32 * std::max(4, P.n_sum * (fp32 ? 3 : 2)); }
+int gb_unit_threads(const GbProg& P, const GbTabs& T, bool fp32) {
+    return 32 * std::max(T.unit == 2 ? 8 : 4, P.n_sum * (fp32 ? 3 : 2));
+}
 
 cudaError_t gb_launch_unit(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                            const GbChildren& ch, long long Cmax, const GbSplit& sp, bool fp32, GbState* st,
                            cudaStream_t s, bool fixed, const GbGenConst* cc, bool late) {
     const long long nch = fixed ? (1LL << sp.flog2) : -1;
-    return gb_launch_ex(fp32 ? k_unit<true> : k_unit<false>, grid_for(Cmax, 32), gb_unit_threads(P, fp32), 0, s, true, P,
-                        pool, par, T, ch, sp, st, nch, cc ? *cc : GbGenConst{}, cc ? 1 : 0, late ? 1 : 0);
+    const auto k = T.unit == 2 ? (fp32 ? k_outer32<true> : k_outer32<false>) : (fp32 ? k_unit<true> : k_unit<false>);
+    return gb_launch_ex(k, grid_for(Cmax, 32), gb_unit_threads(P, T, fp32), 0, s, true, P, pool, par, T, ch, sp, st, nch, cc ? *cc : GbGenConst{}, cc ? 1 : 0, late ? 1 : 0);
 }
 
 cudaError_t gb_launch_child_sums(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,

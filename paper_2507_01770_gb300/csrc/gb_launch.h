@@ -129,10 +129,10 @@ struct GbTabs {
     int reg;
     int dec;          // one child per thread: endpoint programs (P.uops) evaluate the children
     GbCut cut;        // with dec
-    // one child per warp, objectives as for the verdict tables, at least 32
-    // children per parent, every coordinate's verdict within GB_MV_BITS digit
-    // bits: k_unit takes the children 32 to a block instead (mv64 then holds
-    // bit 0 the FP32, bit 1 the FP64 verdict)
+    // one child per warp, at least 32 children per parent: the children are
+    // taken 32 to a block instead.  1 (k_unit): objectives as for the verdict
+    // tables, every coordinate's verdict within GB_MV_BITS digit bits (mv64 then
+    // holds bit 0 the FP32, bit 1 the FP64 verdict); 2 (k_outer32): any other
     int unit;
 };
 // Paper mode (diagonal samples, first-order test on every coordinate) from
@@ -365,7 +365,7 @@ cudaError_t gb_launch_ptab_d(const GbProg& P, const GbPool& pool, const GbParent
 // GbTabs::unit: every child's sums, values and verdicts (tables first).  fixed: one parent, nothing read that the
 // partition writes.  cc non-null: the last block lists the survivors (late: whether they fit is left to
 // k_materialize).
-int gb_unit_threads(const GbProg& P, bool fp32);
+int gb_unit_threads(const GbProg& P, const GbTabs& T, bool fp32);
 cudaError_t gb_launch_unit(const GbProg& P, const GbPool& pool, const GbParents& par, const GbTabs& T,
                            const GbChildren& ch, long long Cmax, const GbSplit& sp, bool fp32, GbState* st,
                            cudaStream_t s, bool fixed, const GbGenConst* cc, bool late);

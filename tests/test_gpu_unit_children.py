@@ -1,5 +1,6 @@
-"""Children 32 to a block with the first-order verdicts looked up (objectives
-whose sums enter with adjoint [1, 1]) against the interpreter: the same run bit
+"""Children 32 to a block, with the first-order verdicts looked up (objectives
+whose sums enter with adjoint [1, 1]) or the outer expression swept per child
+(any other, also with coordinates of its own), against the interpreter: the same run bit
 for bit -- fan-outs from exactly 32 on, ragged last blocks (fewer valid children
 than a block of threads), one and several parents, FP32 first or not, both
 pools, launches one by one and replayed, a pool too small for the survivors
@@ -37,12 +38,12 @@ def _same_run(p, **opts):
     return a
 
 
-@pytest.mark.parametrize("fam", ["chain", "sep_cos", "mixed"])
+@pytest.mark.parametrize("fam", ["chain", "sep_cos", "mixed", "ackley", "paper_rastrigin", "paper_salomon", "paper_rosenbrock", "paper_levy"])
 @pytest.mark.parametrize("fp32", [0, 1])
 @pytest.mark.parametrize("n,B,m,d,K", [(23, 10, 2, 5, 16), (21, 10, 2, 10, 1), (19, 9, 2, 6, 3), (13, 6, 4, 3, 4),
                                        (44, 21, 4, 6, 1), (30, 10, 2, 10, 12)])
 def test_same_run_as_the_interpreter(fam, fp32, n, B, m, d, K):
-    p = S.make(fam, n=n, block=B, seed=7)
+    p = S.make(fam, n=n, block=B, **({} if fam.startswith("paper") else {"seed": 7}))
     _same_run(p, block=B, split_m=m, split_d=d, max_children=K * m ** d, fp32_prefilter=fp32, max_generations=40,
               tol_f=1e-6)
 
