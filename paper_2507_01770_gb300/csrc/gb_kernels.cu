@@ -1174,11 +1174,12 @@ __device__ __forceinline__ void tab_dirty_groups(const GbProg& P, const GbPool& 
                                                  const ChildCtx& c, long long ci, int lane, double2* shF,
                                                  double2* shM, float2* sh32) {
     if (Tb.cg64) {   // computed by k_child_sums: copy the slots
-        for (int q = lane; q < GB_SHG; q += 32) {
+        for (int q = lane; q < P.n_sum * GB_TAB_MAX_DIRTY; q += 32) {
             const size_t at = (size_t)ci * GB_CG + q;
-            shF[q] = Tb.cg64[at];
-            shM[q] = Tb.cgm64[at];
+            const double2 f = Tb.cg64[at], m = Tb.cgm64[at];
             if (pool.fp32) sh32[q] = Tb.cg32[at];
+            shF[q] = f;
+            shM[q] = m;
         }
         __syncwarp();
         return;
@@ -1440,20 +1441,52 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
     const long long rnf = st->rec_nfree, rbump = st->rec_bump;
     const long long ci = ch.surv[s];
     const ChildCtx c = child_ctx(par, ci, sp);
-    if (tab) tab_dirty_groups(P, pool, Tb, c, ci, lane, shF, shM, sh32);
-    const unsigned ns = (s < nfree) ? pool.freel[nfree - 1 - s] : (unsigned)(bump + (s - nfree));
     const int n = pool.n, nb = pool.nb, B = pool.B, GPB = pool.GPB, nrec = pool.nrec;
+    // Bound: latency.  Every load that depends on the survivor alone is issued
+    // before the first result is used (a warp stalls at a use, and a load takes
+    // ~700 clocks): the dirty group values, the slots, the records' ids, then
+    // what these name.  One after the other they took 14k clocks a survivor of
+    // the n = 10^4 family.
+    auto record = [&](int t) {   // the survivor's t-th new record
+        const long long q = s * nrec + t;
+        return q < rnf ? pool.rfree[rnf - 1 - q] : (unsigned)(rbump + (q - rnf));
+    };
+    const unsigned ns = (s < nfree) ? pool.freel[nfree - 1 - s] : (unsigned)(bump + (s - nfree));
+    const double flo = ch.flo[ci];
     const int blk = c.info.z;
     const unsigned* prow = pool.rid + (size_t)c.slot * nb;
     unsigned* crow = pool.rid + (size_t)ns * nb;
-    for (int b = lane; b < nb; b += 32) {
-        const int t = blk - b;
-        unsigned id = prow[b];
-        if (t >= 0 && t < nrec) {
-            const long long q = s * nrec + t;
-            id = q < rnf ? pool.rfree[rnf - 1 - q] : (unsigned)(rbump + (q - rnf));
+    // lane t: the t-th new record and the one it replaces (t >= 32: looked up where needed)
+    unsigned nid = 0, oid = 0;
+    if (lane < nrec && blk - lane >= 0) {
+        nid = record(lane);
+        oid = prow[blk - lane];
+    }
+    auto new_id = [&](int t) { return t < 32 ? __shfl_sync(0xffffffffu, nid, t) : record(t); };   // (t the warp's)
+    auto old_id = [&](int t) { return t < 32 ? __shfl_sync(0xffffffffu, oid, t) : prow[blk - t]; };
+    int g0 = 0;           // lane k: sum k's first group and dirty range
+    int2 dk = make_int2(0, 0);
+    if (tab && lane < P.n_sum) {
+        g0 = P.sums[lane].group0;
+        dk = P.dirty[blk * P.n_sum + lane];
+    }
+    if (tab) tab_dirty_groups(P, pool, Tb, c, ci, lane, shF, shM, sh32);
+    int ow = 0;
+    if (lane < nrec && blk - lane >= 0) ow = (int)pool.rwide[oid];
+    const int pw = pool.swide[c.slot];
+    for (int b0 = 0; b0 < nb; b0 += 128) {
+        unsigned id[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int b = b0 + u * 32 + lane;
+            if (b < nb) id[u] = prow[b];
         }
-        crow[b] = id;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int b = b0 + u * 32 + lane, t = blk - b;
+            const unsigned r = __shfl_sync(0xffffffffu, nid, t & 31);
+            if (b < nb) crow[b] = t >= 0 && t < nrec ? (t < 32 ? r : record(t)) : id[u];
+        }
     }
     __syncwarp();
     const View<double> X = view64(pool, par, c, sp);
@@ -1468,7 +1501,9 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
     const size_t bo = (size_t)c.p * sp.dmax * (sp.m + 1);
     for (int t = 0; t < nrec && blk - t >= 0; t++) {
         const int b = blk - t, j0 = b * B, j1 = min(n, j0 + B);
-        const size_t o = (size_t)crow[b] * B, src = (size_t)prow[b] * B;
+        const unsigned idn = new_id(t);
+        const size_t o = (size_t)idn * B, src = (size_t)old_id(t) * B;
+        const int was = t < 32 ? __shfl_sync(0xffffffffu, ow, t) : (int)pool.rwide[prow[b]];
         bool wide = false;
         for (int jb = j0; jb < j1; jb += 32 * BATCH) {
             double xl[BATCH], xh[BATCH];
@@ -1511,8 +1546,8 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
         }
         wide = __any_sync(0xffffffffu, wide);
         if (lane == 0) {
-            pool.rwide[crow[b]] = wide ? 1 : 0;
-            wide_delta += (wide ? 1 : 0) - (int)pool.rwide[prow[b]];
+            pool.rwide[idn] = wide ? 1 : 0;
+            wide_delta += (wide ? 1 : 0) - was;
         }
     }
     const MidView MX{X};
@@ -1527,7 +1562,35 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
             else if (P.samples == 0) pool.rgmid[at] = make_double2(v.lo, v.hi);
             else pool.rgsamp[(size_t)(kind - 1) * pool.R * GPB + at] = make_double2(v.lo, v.hi);
         });
-    for (int it = lane; it < nrec * GPB; it += 32) {
+    for (int i0 = 0; tab && i0 < nrec * GPB; i0 += 32) {   // (whole warps: the sums are handed out by shuffles)
+        const int it = i0 + lane, t = it / GPB, o = it - t * GPB, b = blk - t;
+        const bool in = it < nrec * GPB && b >= 0;
+        const int g = in ? P.owned[(size_t)b * GPB + o] : -1;
+        int k = 0;
+        for (int q = 1; q < P.n_sum; q++)
+            if (__shfl_sync(0xffffffffu, g0, q) <= g) k = q;
+        const int gl = g - __shfl_sync(0xffffffffu, g0, k);
+        const int d0 = __shfl_sync(0xffffffffu, dk.x, k), d1 = __shfl_sync(0xffffffffu, dk.y, k);
+        const unsigned rn = __shfl_sync(0xffffffffu, nid, t & 31), ro = __shfl_sync(0xffffffffu, oid, t & 31);
+        if (g < 0) continue;
+        const size_t dst = (size_t)(t < 32 ? rn : record(t)) * GPB + o, src = (size_t)(t < 32 ? ro : prow[b]) * GPB + o;
+        double2 f, m;
+        float2 f32 = make_float2(0.f, 0.f);
+        if (gl < d0 || gl >= d1) {
+            f = pool.rgsum[src];
+            m = pool.rgmid[src];
+            if (pool.fp32) f32 = pool.rgsum32[src];
+        } else {
+            const int at = k * GB_TAB_MAX_DIRTY + (gl - d0);
+            f = shF[at];
+            m = shM[at];
+            if (pool.fp32) f32 = sh32[at];
+        }
+        pool.rgsum[dst] = f;
+        pool.rgmid[dst] = m;
+        if (pool.fp32) pool.rgsum32[dst] = f32;
+    }
+    for (int it = lane; !tab && it < nrec * GPB; it += 32) {
         const int t = it / GPB, o = it - t * GPB, b = blk - t;
         if (b < 0) continue;
         const int g = P.owned[(size_t)b * GPB + o];
@@ -1552,22 +1615,16 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
                 const iv64 v = group_sum<PR, double>(P, S, gl, SampleView{X, j, pool.S + 1}, R, ops);
                 pool.rgsamp[(j - 1) * sstep + dst] = make_double2(v.lo, v.hi);
             }
-        iv64 a, m;
-        if constexpr (tab) {
-            const int at = k * GB_TAB_MAX_DIRTY + (gl - dr.x);
-            a = iv64{shF[at].x, shF[at].y};
-            m = iv64{shM[at].x, shM[at].y};
-            if (pool.fp32) pool.rgsum32[dst] = sh32[at];
-        } else {
-            a = group_sum<PR, double>(P, S, gl, X, R, ops);
-            m = group_sum<PR, double>(P, S, gl, MX, R, ops);
+        if constexpr (!tab) {
+            const iv64 a = group_sum<PR, double>(P, S, gl, X, R, ops);
+            const iv64 m = group_sum<PR, double>(P, S, gl, MX, R, ops);
             if (pool.fp32) {
                 const iv32 f = group_sum<PR, float>(P, S, gl, X32, R32, ops);
                 pool.rgsum32[dst] = make_float2(f.lo, f.hi);
             }
+            pool.rgsum[dst] = make_double2(a.lo, a.hi);
+            pool.rgmid[dst] = make_double2(m.lo, m.hi);
         }
-        pool.rgsum[dst] = make_double2(a.lo, a.hi);
-        pool.rgmid[dst] = make_double2(m.lo, m.hi);
     }
     if (TAB == 2 && pool.rgdp) {   // coordinate partials of each new record's block, from the tables or the parent's
         const GbSplitPos SP = P.sps[P.sp_of_cyc[c.info.x]];
@@ -1590,11 +1647,11 @@ __device__ __forceinline__ void materialize_rec(const GbProg& P, const GbPool& p
         }
     }
     if (lane == 0) {
-        const int w = pool.swide[c.slot] + wide_delta;
+        const int w = pw + wide_delta;
         pool.swide[ns] = w;
         const bool narrow = tol_x > 0.0 && w == 0;
         const long long e = kept_old + s;
-        En.flo[e] = ch.flo[ci];
+        En.flo[e] = flo;
         En.slot[e] = ns;
         En.cyc[e] = (int)((unsigned)c.info.w | (narrow ? GB_FINAL_BIT : 0u));
     }
