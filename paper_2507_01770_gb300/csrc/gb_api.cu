@@ -690,6 +690,16 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             cudaGetLastError();   // no room for the tables: the interpreter
         else
             p->use_paper = true;
+        // products: forward values and reverse factors of their term rows (64 MiB at most, or the sweeps form them)
+        if (p->use_paper && P.any_prod) {
+            for (const GbSum& S : Hh.sums)
+                if (S.prod) T.pw = std::max(T.pw, (int)S.nins);
+            const size_t pc = K * (size_t)T.arows * T.pw;
+            if (pc * sizeof(double2) <= (32u << 20) && (alloc(&T.pv, pc, A) || alloc(&T.pf, pc, A))) {
+                cudaGetLastError();
+                T.pv = T.pf = nullptr;
+            }
+        }
         // groups of children (gb_cut.cuh): the operations a child applies to its reductions are isotone
         bool iso = true;
         for (const GbOIns& o : Hh.oprog) iso = iso && o.op != D_EXP && o.op != D_SIN && o.op != D_COS;

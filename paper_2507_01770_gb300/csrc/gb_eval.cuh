@@ -350,6 +350,60 @@ __device__ __forceinline__ void reverse_sweep(const GbIns* ins, int nins, const 
     }
 }
 
+// What a push through node t multiplies the adjoint with, for the operations
+// whose factor is a function of the forward values alone (FP64): the sweep
+// below takes it from a table instead of calling the library again.
+__device__ __forceinline__ bool rev_factor(const GbIns& in, const iv64* V, int t, iv64& f) {
+    switch (in.op) {
+    case D_DIV: f = ircp(V[in.b]); return true;
+    case D_SQRT: f = iscale(ircp(V[t]), 0.5); return true;
+    case D_SIN: f = itrig(V[in.a], true); return true;
+    case D_COS: f = ineg(itrig(V[in.a], false)); return true;
+    default: return false;
+    }
+}
+// reverse_sweep of a template from tabulated forward values and factors
+// (entry t: node t): slow_rev's products in its order.
+__device__ __forceinline__ void reverse_sweep_tab(const GbIns* ins, int nins, const double2* V, const double2* F, iv64* A,
+                                                  int& ops) {
+    auto at = [](const double2* q, int t) { const double2 v = q[t]; return iv64{v.x, v.y}; };
+    for (int t = nins - 1; t >= 0; t--) {
+        const GbIns in = ins[t];
+        ops += (in.pad >> 8) & 0xff;
+        if (!(in.pad & (GB_RV_A | GB_RV_B))) continue;
+        const iv64 g = A[t];
+        iv64 da = g, db = g;
+        switch (in.op) {
+        case D_SUB: db = ineg(g); break;
+        case D_MUL:
+            if (in.pad & GB_RV_A) da = imul(g, at(V, in.b));
+            if (in.pad & GB_RV_B) db = imul(g, at(V, in.a));
+            break;
+        case D_DIV: {
+            const iv64 rb = at(F, t);
+            da = imul(g, rb);
+            if (in.pad & GB_RV_B) db = imul(g, ineg(imul(at(V, t), rb)));
+            break;
+        }
+        case D_NEG: da = ineg(g); break;
+        case D_SQR: da = imul(g, iscale(at(V, in.a), 2.0)); break;
+        case D_EXP: da = imul(g, at(V, t)); break;
+        case D_SQRT:
+        case D_SIN:
+        case D_COS: da = imul(g, at(F, t)); break;
+        case D_STEP: {
+            const iv64 va = at(V, in.a);
+            slow_rev(in.op, g, va, va, va, &da, &db);
+            break;
+        }
+        case D_SCALE: da = iscale(g, in.c); break;
+        default: break;   // D_ADD
+        }
+        if (in.pad & GB_RV_A) adj_push(A[in.a], da, (in.pad & GB_RV_A0) != 0);
+        if (in.pad & GB_RV_B) adj_push(A[in.b], db, (in.pad & GB_RV_B0) != 0);
+    }
+}
+
 // Sum (IPROD: product) of the terms of one group (local group g of sum S).
 template <bool PROD, typename T, typename V>
 __device__ __forceinline__ typename Prec<T>::I group_reduce(const GbProg& P, const GbSum& S, int g, const V& X,
@@ -546,7 +600,8 @@ __device__ __forceinline__ typename Prec<T>::I outer_fwd(const GbProg& P, const 
 // forward pass.  A product's term templates are seeded with the term's
 // adjoint in the product (prod_term_seed; group values from gcache except
 // the groups dirty for block dblk, all recomputed when gcache is null), or by
-// seeder(k, term ordinal) when it is not a null pointer.
+// seeder(k, term ordinal) when it is not a null pointer; seeder.sweep may then
+// give a term's leaf adjoints itself.
 template <bool PR, typename T, typename V, typename C, typename Seed = const int*>
 __device__ __forceinline__ bool block_mono(const GbProg& P, int blk, const V& X, const View<double>& X64,
                                            const typename Prec<T>::I* O, typename Prec<T>::I* OA,
@@ -593,11 +648,15 @@ __device__ __forceinline__ bool block_mono(const GbProg& P, int blk, const V& X,
                             seed = seeder(k, cur[k]);
                     }
                 }
-                term_fwd<T>(P, S, i, X, R, ops);
-                for (int t = 0; t < S.nins; t++) RA[t] = mk<T>((T)0, (T)0);
-                RA[S.nins - 1] = seed;
                 const GbIns* ins = P.tins + S.ins0;
-                reverse_sweep<T>(ins, S.nins, R, RA, ops);
+                bool swept = false;   // the leaf adjoints from the caller's tables
+                if constexpr (!std::is_pointer<Seed>::value) swept = seeder.sweep(k, cur[k], S, seed, RA, ops);
+                if (!swept) {
+                    term_fwd<T>(P, S, i, X, R, ops);
+                    for (int t = 0; t < S.nins; t++) RA[t] = mk<T>((T)0, (T)0);
+                    RA[S.nins - 1] = seed;
+                    reverse_sweep<T>(ins, S.nins, R, RA, ops);
+                }
                 for (int t = 0; t < S.nins; t++) {
                     GbIns in = ins[t];
                     if (in.op != D_IVAR) continue;

@@ -20,10 +20,11 @@
 // most children are cut off in groups (gb_cut.cuh) the latency of the rest.
 // Measured on GB300, whole solves with 4^10 children a generation: Levy n = 30,
 // 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 9.2
-// with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 32.5 ms
+// with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 19.5 ms
 // (its survivors' caches, too, come from the tables: k_materialize 73 -> 0.2 ms
 // a generation; two thirds of a million of its children survive, and what
-// bounds those is the product's first-order test).
+// bounds those is the product's first-order test, which takes the templates'
+// forward values and library factors from the term rows: 32.5 ms before).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -114,6 +115,16 @@ __global__ void __launch_bounds__(PP_T) k_pp_rows(GbProg P, GbPool pool, GbParen
             iv64 R[GB_MAX_TREGS];
             const iv64 v = term_fwd<double>(P, S, i, X, R, ops);
             T.tv[((size_t)p * T.nk + kind) * T.arows + row] = make_double2(v.lo, v.hi);
+            if (kind == 0 && S.prod && T.pv) {   // what its reverse sweep reads
+                const GbIns* ins = P.tins + S.ins0;
+                const size_t o = ((size_t)p * T.arows + row) * T.pw;
+                for (int t = 0; t < S.nins; t++) {
+                    if (!(ins[t].pad & GB_RV_LIVE) && !(ins[t].pad & GB_RV_VAL)) continue;
+                    T.pv[o + t] = make_double2(R[t].lo, R[t].hi);
+                    iv64 f;
+                    if ((ins[t].pad & GB_RV_LIVE) && rev_factor(ins[t], R, t, f)) T.pf[o + t] = make_double2(f.lo, f.hi);
+                }
+            }
             if (kind == 0 && !S.prod) {
                 iv64 RA[GB_MAX_TREGS];
                 for (int t = 0; t < S.nins; t++) RA[t] = iv64{0.0, 0.0};
@@ -295,6 +306,16 @@ __device__ __forceinline__ void tree_adjoints(iv64 a, int m, iv64* node, iv64* o
     }
 }
 
+// block_mono's seeder: a term's adjoint in its product, and its sweep.
+template <typename F, typename G> struct PaperSeed {
+    F& f;
+    G& g;
+    __device__ __forceinline__ iv64 operator()(int k, int tt) const { return f(k, tt); }
+    __device__ __forceinline__ bool sweep(int k, int tt, const GbSum& S, iv64 sd, iv64* A, int& o) const {
+        return g(k, tt, S, sd, A, o);
+    }
+};
+
 // First-order test of a child that passed the cut-off.  Sums: the block's
 // coordinates and those within a term's reach of it from the tabulated D, the
 // others (every coordinate tested) from the parent's cached D, or swept when
@@ -321,7 +342,13 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
         // (Griewank n = 16, 6.8e5 children kept in a generation: 20 ms of it).
         iv64 gv[PP_TREE], nodes[2 * PP_TREE], adj[PP_TREE];
         int gk = -1, ak = -1, ag = -1;   // gv holds reduction gk's group values; adj group ag of reduction ak
-        auto seed = [&](int k, int tt) -> iv64 {
+        auto term_row = [&](const GbPaperSum& ps, int tt) {   // the table row of a product's term for this child
+            const int q = tt >= ps.t_lo && tt < ps.t_hi ? ps.d0 + (tt - ps.t_lo)
+                                                        : ps.x0 + (tt < ps.t_lo ? tt : tt - (ps.t_hi - ps.t_lo));
+            const GbDTerm D = P.dterms[SP.dterm0 + q];
+            return D.row + (int)((c.r >> D.dshift) & ((1u << (D.w * P.mshift)) - 1u));
+        };
+        auto seed_of = [&](int k, int tt) -> iv64 {
             const GbSum S = P.sums[k];
             const GbPaperSum ps = T.psums[spi * P.n_sum + k];
             int lo = 0, hi = S.ngroups - 1;   // the term's group
@@ -342,11 +369,7 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
                 return iv64{v.x, v.y};
             };
             auto tval = [&](int t) {   // t: index in the group
-                const int tt2 = G.t0 + t;
-                const int q = tt2 >= ps.t_lo && tt2 < ps.t_hi ? ps.d0 + (tt2 - ps.t_lo)
-                                                              : ps.x0 + (tt2 < ps.t_lo ? tt2 : tt2 - (ps.t_hi - ps.t_lo));
-                const GbDTerm D = P.dterms[SP.dterm0 + q];
-                const double2 v = tv[D.row + (int)((c.r >> D.dshift) & ((1u << (D.w * P.mshift)) - 1u))];
+                const double2 v = tv[term_row(ps, G.t0 + t)];
                 return iv64{v.x, v.y};
             };
             const iv64 one{1.0, 1.0};
@@ -365,6 +388,16 @@ __device__ __noinline__ bool paper_mono(const GbProg& P, const GbPool& pool, con
             ag = lo;
             return adj[tt - G.t0];
         };
+        // a product's term swept from its row's values and factors
+        auto sweep_of = [&](int k, int tt, const GbSum& S, iv64 sd, iv64* A, int& o) {
+            if (!S.prod || !T.pv) return false;
+            const size_t at = ((size_t)c.p * T.arows + term_row(T.psums[spi * P.n_sum + k], tt)) * T.pw;
+            for (int t = 0; t < S.nins; t++) A[t] = iv64{0.0, 0.0};
+            A[S.nins - 1] = sd;
+            reverse_sweep_tab(P.tins + S.ins0, S.nins, T.pv + at, T.pf + at, A, o);
+            return true;
+        };
+        const PaperSeed<decltype(seed_of), decltype(sweep_of)> seed{seed_of, sweep_of};
         if (!P.mono_all)
             return block_mono<true, double>(P, blk, X, X, O, OA, R, RA, (double*)nullptr,
                                             (const CacheRef<double2>*)nullptr, blk, ops, seed);

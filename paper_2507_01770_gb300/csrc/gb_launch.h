@@ -148,6 +148,8 @@ struct GbPaper {
     double2* nd;      // group trees of the parent's cached values
     double2* td;      // partial sums D by digit combination
     double2* hv;      // hoisted outer values
+    double2 *pv, *pf; // products' term rows: forward values and reverse factors, pw nodes per row (null: none kept)
+    int pw;
     const GbPaperSum* psums;
     const GbHoistPos* hoist_pos;
     const int32_t* hoist_node;
