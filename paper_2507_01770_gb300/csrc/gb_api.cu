@@ -604,8 +604,10 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
                 P.uops = d_u;
                 if (!fp32 && d * mshift >= GB_CUT_MIN &&
                     ((e = alloc(&T.cut.tv, 2 * rows, A)) || (e = alloc(&T.cut.ts, 2 * K * (size_t)T.max_srows, A)) ||
-                     (e = alloc(&T.cut.td, K * (size_t)T.max_drows, A))))
-                    return bad(e, "allocate hull tables");
+                     (e = alloc(&T.cut.td, K * (size_t)T.max_drows, A)))) {
+                    cudaGetLastError();   // no room: every child by itself
+                    T.cut = GbCut{};
+                }
             }
             T.max_sum_nodes = 1;
             for (const GbSum& S : Hh.sums) T.max_sum_nodes = std::max(T.max_sum_nodes, (int)S.nnodes);

@@ -115,7 +115,7 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
                     if (group_ruled_out(P, pool, par, sp, P.sps[spi], c, td + c.p * tdp, ops)) {
                         k = e.bound(c, spi, ops);
                         walk = k < st->gub_key;
-                        if (walk) seed = min(seed, (k & ~gmask) | (unsigned long long)g);
+                        if (walk && nk > 2) seed = min(seed, (k & ~gmask) | (unsigned long long)g);
                     }
                     if (walk) ch.flo[g << GB_CUT_LOG2] = k ? gb_key_value(k) : -__longlong_as_double(0x7ff0000000000000LL);
                 }
@@ -139,6 +139,7 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
     }
     if (lane == 0 && seed != ~0ull) atomicMin(&st->cut_seed, seed);
     warp_add_ops(ops, &st->ops64);
+    if (nk == 2) return;   // (one sample a child: the groups' own bounds come too late to save as much)
     __shared__ bool s_last;
     if (!arrive_last(&st->cc_done, gridDim.x, &s_last)) return;
     seed = __ldcg(&st->cut_seed);

@@ -294,6 +294,13 @@ __device__ __forceinline__ void stage_term(const GbIns* ins, int nins, int i, co
     __syncwarp();
 }
 
+// The forward values that the reverse sweep of a term reads, no others.
+template <typename T, typename V>
+__device__ __forceinline__ void term_vals(const GbProg& P, const GbSum& S, int i, const V& X, typename Prec<T>::I* R,
+                                          int& ops, const GbIns* sins = nullptr) {
+    term_fwd<T, V, false, true>(P, S, i, X, R, ops, sins);
+}
+
 // A push of d into an adjoint: its first one is [0, 0] + d without the two
 // additions (RU(+0 + -0) is +0, the other sums are d's own ends).
 template <typename I> __device__ __forceinline__ void adj_push(I& A, I d, bool first) {
@@ -652,7 +659,7 @@ __device__ __forceinline__ bool block_mono(const GbProg& P, int blk, const V& X,
                 bool swept = false;   // the leaf adjoints from the caller's tables
                 if constexpr (!std::is_pointer<Seed>::value) swept = seeder.sweep(k, cur[k], S, seed, RA, ops);
                 if (!swept) {
-                    term_fwd<T>(P, S, i, X, R, ops);
+                    term_vals<T>(P, S, i, X, R, ops);
                     for (int t = 0; t < S.nins; t++) RA[t] = mk<T>((T)0, (T)0);
                     RA[S.nins - 1] = seed;
                     reverse_sweep<T>(ins, S.nins, R, RA, ops);
@@ -726,7 +733,7 @@ __device__ __noinline__ void block_D(const GbProg& P, int blk, const V& X, iv64*
             if (S.has_var) {
                 while (cur[k] < S.count && S.first + cur[k] * S.step + S.off_min <= j) {
                     int i = S.first + cur[k] * S.step;
-                    term_fwd<double>(P, S, i, X, R, ops);
+                    term_vals<double>(P, S, i, X, R, ops);
                     for (int t = 0; t < S.nins; t++) RA[t] = iv64{0.0, 0.0};
                     RA[S.nins - 1] = iv64{1.0, 1.0};
                     const GbIns* ins = P.tins + S.ins0;
@@ -769,7 +776,7 @@ __device__ __forceinline__ double2 coord_D(const GbProg& P, int k, int j, const 
         for (int t = need <= 0 ? 0 : (need + S.step - 1) / S.step;
              t < S.count && S.first + t * S.step + S.off_min <= j; t++) {
             const int i = S.first + t * S.step;
-            term_fwd<double>(P, S, i, X, R, ops);
+            term_vals<double>(P, S, i, X, R, ops);
             for (int q = 0; q < S.nins; q++) RA[q] = iv64{0.0, 0.0};
             RA[S.nins - 1] = iv64{1.0, 1.0};
             reverse_sweep<double>(ins, S.nins, R, RA, ops);

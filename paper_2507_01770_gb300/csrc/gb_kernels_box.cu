@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(C::THREADS) k_box(GbProg P, const GbBoxTile* _
             const int tz = z < 0 ? 0 : min(S.count, z / S.step + 1);
             for (int t = ta + lane; t < tz; t += W) {
                 I RA[GB_MAX_TREGS];
-                term_fwd<T>(P, S, S.first + t * S.step, X, R, ops, ins);
+                term_vals<T>(P, S, S.first + t * S.step, X, R, ops, ins);
                 for (int i = 0; i < S.nins; i++) RA[i] = zero_iv<I>();
                 RA[S.nins - 1] = mk<T>((T)1, (T)1);
                 reverse_sweep<T>(ins, S.nins, R, RA, ops);
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(128) k_child_box(GbProg P, GbPool pool, GbPare
             const int tz = z < 0 ? 0 : min(S.count, z / S.step + 1);
             for (int t = ta + lane; t < tz; t += W) {
                 iv64 RA[GB_MAX_TREGS];
-                term_fwd<double>(P, S, S.first + t * S.step, X, R, ops, ins);
+                term_vals<double>(P, S, S.first + t * S.step, X, R, ops, ins);
                 for (int i = 0; i < S.nins; i++) RA[i] = iv64{0.0, 0.0};
                 RA[S.nins - 1] = iv64{1.0, 1.0};
                 reverse_sweep<double>(ins, S.nins, R, RA, ops);
