@@ -84,9 +84,6 @@ FP32_OPS_PER_SM_CLK = 128.0  # 128 FP32 lanes per SM (directed add / mul at full
 WORKLOADS = {
     "chain100": dict(family="chain", n=100, block=10, split_m=4, split_d=10, max_children=1 << 20, fp32=0,
                      gens_per_sync=0, pool_gb=16.0, cpu_parents=4, cpu_split_m=2, cpu_split_d=10, cpu_gens=20,
-                     # DRAM bytes (read + write) of one k_eval64_tab launch, ncu capture in
-                     # profiles/k_eval64_tab_chain100.md
-                     traffic=0.645e6,
                      name="chain n=100 (coupled quartic, planted min 0), FP64, B=10, 4-way split of the 10 "
                           "block coordinates (4^10 children) of 1 best box per generation, tol_f=1e-6"),
     "ackley1000": dict(family="ackley", n=1000, block=10, split_m=2, split_d=10, max_children=1 << 10, fp32=1,
@@ -599,12 +596,15 @@ def roofline(m, w, opts, sm_mhz, sms, gb, local):
     achieved = eq / (ms * 1e-3) if ms > 0 else None
     warp = opts["max_children"] < (1 << 16)
     if w.get("paper"):
-        kname = "k_eval32 + k_eval64 (bytecode interpreter)" if w["fp32"] else "k_eval64 (bytecode interpreter)"
+        kname = "k_eval32 + k_eval64 (bytecode interpreter)" if w["fp32"] else "k_pp_rows + k_pp_seg + k_cut_* + k_pp_dec / k_pp_eval"
     elif w["fp32"] and warp:
-        kname = "k_ptab + k_ptab_d + k_eval_tabw (tables, then FP32 and FP64 in one warp-per-child kernel)"
+        kname = "k_ptab + k_ptab_d + k_unit / k_outer32 (tables, then FP32 and FP64, 32 children to a block)"
+    elif warp:
+        kname = "k_ptab + k_ptab_d + k_unit / k_outer32 (tables, then 32 children to a block)"
+    elif w["fp32"]:
+        kname = "k_ptab + k_ptab_d + k_eval32_tab + compaction + k_eval64_dec"
     else:
-        kname = ("k_ptab + k_ptab_d + " + ("k_eval32_tab + compaction + " if w["fp32"] else "") + "k_eval64_tab"
-                 + ("w" if warp else ""))
+        kname = "k_ptab + k_ptab_d + k_cut_tabs + k_cut_dec + k_eval64_dec (tables, child groups, children of those left)"
     try:
         probe64, _ = gb.gb_measure_peak(local, 0)
     except Exception:

@@ -163,8 +163,9 @@ typedef struct gb_result {
     double* box_flo;          /* lower bound of f on each box */
     int64_t generations;
     int64_t box_evals_fp32;   /* children evaluated in FP32 (F and gradient) */
-    int64_t box_evals_fp64;   /* children evaluated in FP64 (F and gradient) */
-    int64_t mid_evals;        /* FP64 midpoint samples */
+    int64_t box_evals_fp64;   /* children decided in FP64 (F and gradient): one by one, or (large fan-outs) with
+                                 their group of 32 from an enclosure of all of them, with the same verdict */
+    int64_t mid_evals;        /* FP64 samples of those children: taken, or shown not to lower the incumbent */
     double solve_ms;          /* wall time of the solve on the host clock */
     double device_ms;         /* CUDA-event time from the first to the last launch */
     double eval64_ms;         /* CUDA-event time of the child evaluation: per-parent term tables, FP32 pass

@@ -256,10 +256,10 @@ class _Owner:
     """One array that the library allocated, freed with the last numpy view of it."""
 
     def __init__(self, struct, free):
-        self.struct, self.free = struct, free
+        self.ref, self.free = ctypes.byref(struct), free   # (the reference keeps the struct)
 
     def __del__(self):
-        self.free(ctypes.byref(self.struct))
+        self.free(self.ref)
 
 
 def _adopt(s, field: str, count: int, ctype, free):

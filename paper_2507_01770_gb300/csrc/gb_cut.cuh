@@ -82,6 +82,17 @@ __device__ __forceinline__ bool group_ruled_out(const GbProg& P, const GbPool& p
     return false;
 }
 
+// Threads of a block that take a group each, and the roles that share its work:
+// the first bounds F and then tries the first-order test while the others
+// bound the samples of the groups that F does not cut off, a share of the kinds
+// each.  (One thread doing all of it was one chain of 170k clocks, Levy n = 30
+// at 10 samples: a solve 8.52 ms, 8.25 with the roles.)
+constexpr int CUT_T = 128, CUT_ROLES = 4;
+inline int cut_threads(int nk) {   // about five kinds a sample role
+    const int roles = 1 + (nk - 1 + 4) / 5;
+    return CUT_T * (roles < CUT_ROLES ? roles : CUT_ROLES);
+}
+
 // Groups: appends those to walk to ch.list32 (their number in st->n32, zero
 // at the start of a generation), clears every flag and counts the children.
 // The first child's place in ch.flo tells why a group is walked: the bound of
@@ -93,40 +104,63 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
                                            const GbChildren& ch, const GbSplit& sp, int nk, const double2* td,
                                            long long tdp, GbState* st, const E& e, const R& er) {
     const double gub_prev = gb_key_value(st->gub_key);
-    const long long total = st->nch >> GB_CUT_LOG2, stride = (long long)gridDim.x * blockDim.x;
+    const long long total = st->nch >> GB_CUT_LOG2, stride = (long long)gridDim.x * CUT_T;
     const unsigned long long gmask = total > 1 ? ~0ull >> __clzll(total - 1) : 0;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, t = threadIdx.x % CUT_T, role = threadIdx.x / CUT_T;
+    const int per = (nk - 1 + blockDim.x / CUT_T - 2) / (blockDim.x / CUT_T - 1);   // kinds of a sample role
+    __shared__ unsigned s_pass[CUT_T / 32];
+    __shared__ unsigned long long s_key[CUT_ROLES - 1][CUT_T];
     unsigned long long nvalid = 0, seed = ~0ull;
     int ops = 0;
-    for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
-        const long long g = base + lane;
-        bool walk = false;
-        unsigned n = 0;
+    for (long long base = blockIdx.x * (long long)CUT_T; base < total; base += stride) {
+        const long long g = base + t;
+        ChildCtx c{};
+        int spi = -1;
         if (g < total) {
-            const ChildCtx c = child_ctx(par, g << GB_CUT_LOG2, sp);
-            const int spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
-            uint4* f = reinterpret_cast<uint4*>(ch.flag + (g << GB_CUT_LOG2));
-            f[0] = f[1] = make_uint4(0, 0, 0, 0);
-            if (spi >= 0) {
-                n = min(1u << GB_CUT_LOG2, (1u << (c.info.y * sp.mshift)) - c.r);
-                walk = !(e.lower(c, spi, ops) > gub_prev);
-                if (walk) {
-                    unsigned long long k = 0;   // below every key of a number
-                    if (group_ruled_out(P, pool, par, sp, P.sps[spi], c, td + c.p * tdp, ops)) {
-                        k = e.bound(c, spi, ops);
-                        walk = k < st->gub_key;
-                        if (walk && nk > 2) seed = min(seed, (k & ~gmask) | (unsigned long long)g);
-                    }
-                    if (walk) ch.flo[g << GB_CUT_LOG2] = k ? gb_key_value(k) : -__longlong_as_double(0x7ff0000000000000LL);
-                }
-            }
+            c = child_ctx(par, g << GB_CUT_LOG2, sp);
+            spi = c.valid ? P.sp_of_cyc[c.info.x] : -1;
         }
-        nvalid += n;
-        const unsigned bal = __ballot_sync(0xffffffffu, walk);
-        unsigned at = 0;
-        if (lane == 0 && bal) at = (unsigned)atomicAdd((unsigned long long*)&st->n32, (unsigned long long)__popc(bal));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (walk) ch.list32[at + __popc(bal & ((1u << lane) - 1u))] = (unsigned)g;
+        bool walk = false, ruled = false;
+        if (role == 0) {
+            if (g < total) {
+                uint4* f = reinterpret_cast<uint4*>(ch.flag + (g << GB_CUT_LOG2));
+                f[0] = f[1] = make_uint4(0, 0, 0, 0);
+            }
+            if (spi >= 0) {
+                nvalid += min(1u << GB_CUT_LOG2, (1u << (c.info.y * sp.mshift)) - c.r);
+                walk = !(e.lower(c, spi, ops) > gub_prev);
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, walk);
+            if (lane == 0) s_pass[t >> 5] = b;
+        }
+        __syncthreads();
+        if (role == 0) {
+            ruled = walk && group_ruled_out(P, pool, par, sp, P.sps[spi], c, td + c.p * tdp, ops);
+        } else {
+            const int k0 = 1 + (role - 1) * per, k1 = min(nk, k0 + per);
+            unsigned long long k = ~0ull;
+            // (read only where the test can rule a group out)
+            if (P.sum_adj && k0 < k1 && ((s_pass[t >> 5] >> lane) & 1u)) k = e.bound(c, spi, k0, k1, ops);
+            s_key[role - 1][t] = k;
+        }
+        __syncthreads();
+        if (role == 0) {
+            if (walk) {
+                unsigned long long k = 0;   // below every key of a number
+                if (ruled) {
+                    k = ~0ull;
+                    for (int i = 0; i < (int)blockDim.x / CUT_T - 1; i++) k = min(k, s_key[i][t]);
+                    walk = k < st->gub_key;
+                    if (walk && nk > 2) seed = min(seed, (k & ~gmask) | (unsigned long long)g);
+                }
+                if (walk) ch.flo[g << GB_CUT_LOG2] = k ? gb_key_value(k) : -__longlong_as_double(0x7ff0000000000000LL);
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, walk);
+            unsigned at = 0;
+            if (lane == 0 && bal) at = (unsigned)atomicAdd((unsigned long long*)&st->n32, (unsigned long long)__popc(bal));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (walk) ch.list32[at + __popc(bal & ((1u << lane) - 1u))] = (unsigned)g;
+        }
     }
     for (int o = 16; o; o >>= 1) {
         nvalid += __shfl_down_sync(0xffffffffu, nvalid, o);
@@ -150,8 +184,8 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
     }
     if (seed == ~0ull) return;
     // a warp's share of the kinds, a child per lane
-    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, per = (nk - 1 + nw - 1) / nw;
-    const int k0 = 1 + w * per, k1 = min(nk, k0 + per);
+    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, share = (nk - 1 + nw - 1) / nw;
+    const int k0 = 1 + w * share, k1 = min(nk, k0 + share);
     unsigned long long key = ~0ull;
     ops = 0;
     if (k0 < k1) {

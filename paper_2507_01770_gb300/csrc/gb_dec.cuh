@@ -100,9 +100,9 @@ template <int NQ> struct DecEval {
         }
         return key;
     }
-    // over the hull tables: no sample of the group is below the key
-    __device__ __forceinline__ unsigned long long bound(const ChildCtx& c, int spi, int& ops) const {
-        return samples(c, spi, 1, D.nk, 0, ops);
+    // over the hull tables: no sample (kinds [k0, k1)) of the group is below the key
+    __device__ __forceinline__ unsigned long long bound(const ChildCtx& c, int spi, int k0, int k1, int& ops) const {
+        return samples(c, spi, k0, k1, 0, ops);
     }
 };
 

@@ -511,9 +511,9 @@ template <bool PR> struct PaperEval {
         }
         return key;
     }
-    __device__ __forceinline__ unsigned long long bound(const ChildCtx& c, int spi, int& ops) const {
+    __device__ __forceinline__ unsigned long long bound(const ChildCtx& c, int spi, int k0, int k1, int& ops) const {
         unsigned long long key = ~0ull;   // (below each sample's upper end: its enclosure's lower end over the hulls)
-        for (int kind = 1; kind < T.nk; kind++) {
+        for (int kind = k0; kind < k1; kind++) {
             const double v = value(c, spi, kind, ops).lo;
             key = min(key, nan_bits(v) ? 0ull : gb_order_key(v));
         }
@@ -625,13 +625,13 @@ __global__ void k_outer_adj(GbProg P, double2* adj) {
 
 // D: the hull tables; R: the children's own.
 template <int NQ>
-__global__ void __launch_bounds__(128) k_cut_dec(GbProg P, GbPool pool, GbParents par, GbDec D, GbDec R, GbChildren ch,
+__global__ void __launch_bounds__(CUT_T * CUT_ROLES) k_cut_dec(GbProg P, GbPool pool, GbParents par, GbDec D, GbDec R, GbChildren ch,
                                                  GbSplit sp, GbState* st) {
     if (st->halt) return;
     cut_groups(P, pool, par, ch, sp, D.nk, D.td, D.tdp, st, DecEval<NQ>{P, D}, DecEval<NQ>{P, R});
 }
 template <bool PR>
-__global__ void __launch_bounds__(128) k_cut_paper(GbProg P, GbPool pool, GbParents par, GbPaper T, GbPaper R,
+__global__ void __launch_bounds__(CUT_T * CUT_ROLES) k_cut_paper(GbProg P, GbPool pool, GbParents par, GbPaper T, GbPaper R,
                                                    GbChildren ch, GbSplit sp, GbState* st) {
     if (st->halt) return;
     cut_groups(P, pool, par, ch, sp, T.nk, T.cut.td, T.drows, st, PaperEval<PR>{P, T}, PaperEval<PR>{P, R});
@@ -682,8 +682,8 @@ cudaError_t gb_launch_paper_eval(const GbProg& P, const GbPool& pool, const GbPa
             H.hv = T.cut.hv;
             gb_launch_count++;
             const unsigned g = std::min<unsigned>(grid_for(Cmax >> GB_CUT_LOG2, 128), (unsigned)gb_sm_count() * 16);
-            if (P.any_prod) k_cut_paper<true><<<g, 128, 0, s>>>(P, pool, par, H, T, ch, sp, st);
-            else k_cut_paper<false><<<g, 128, 0, s>>>(P, pool, par, H, T, ch, sp, st);
+            if (P.any_prod) k_cut_paper<true><<<g, cut_threads(T.nk), 0, s>>>(P, pool, par, H, T, ch, sp, st);
+            else k_cut_paper<false><<<g, cut_threads(T.nk), 0, s>>>(P, pool, par, H, T, ch, sp, st);
         }
     }
     gb_launch_count++;
@@ -713,7 +713,7 @@ cudaError_t gb_launch_cut_dec(const GbProg& P, const GbPool& pool, const GbParen
                               const GbChildren& ch, long long Cmax, const GbSplit& sp, GbState* st, cudaStream_t s) {
     gb_launch_count++;
     const unsigned g = std::min<unsigned>(grid_for(Cmax >> GB_CUT_LOG2, 128), (unsigned)gb_sm_count() * 16);
-    if (D.nk > 2) k_cut_dec<5><<<g, 128, 0, s>>>(P, pool, par, C, D, ch, sp, st);
-    else k_cut_dec<1><<<g, 128, 0, s>>>(P, pool, par, C, D, ch, sp, st);
+    if (D.nk > 2) k_cut_dec<5><<<g, cut_threads(D.nk), 0, s>>>(P, pool, par, C, D, ch, sp, st);
+    else k_cut_dec<1><<<g, cut_threads(D.nk), 0, s>>>(P, pool, par, C, D, ch, sp, st);
     return cudaGetLastError();
 }
