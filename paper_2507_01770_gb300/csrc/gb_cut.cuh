@@ -27,8 +27,8 @@
 //
 // Bound: the FP64 pipe while every child was walked.  Measured on GB300 with
 // 4^10 children a generation, whole solves: chain n = 100 (128 generations)
-// 26.4 -> 20.5 ms, a child kernel of 110 us -> 17 after 26 for the groups;
-// paper mode, Levy n = 30 (27 generations) 34.3 -> 9.2 ms (18.6
+// 26.4 -> 19.4 ms, a child kernel of 110 us -> 20 after 30 for the groups;
+// paper mode, Levy n = 30 (27 generations) 34.3 -> 8.25 ms (18.6
 // before a group is sampled first, its samples taken five at a time and the
 // test's fixed adjoints used first).  From a fan-out of
 // 2^10 on: the hull tables and the groups take two launches (8 + 10 us at

@@ -19,7 +19,7 @@
 // Bound: the FP64 pipe (one addition per table entry and endpoint), where
 // most children are cut off in groups (gb_cut.cuh) the latency of the rest.
 // Measured on GB300, whole solves with 4^10 children a generation: Levy n = 30,
-// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 9.2
+// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 8.25
 // with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 19.5 ms
 // (its survivors' caches, too, come from the tables: k_materialize 73 -> 0.2 ms
 // a generation; two thirds of a million of its children survive, and what
