@@ -230,7 +230,9 @@ __device__ __forceinline__ void cut_children(const GbProg& P, const GbParents& p
             const long long c0 = (long long)ch.list32[base >> GB_CUT_LOG2] << GB_CUT_LOG2;
             const double b = ch.flo[c0];
             __syncwarp();
-            if (gb_order_key(b) >= *(volatile unsigned long long*)&st->gub_new_key) continue;
+            // Other warps lower the incumbent meanwhile, so two lanes may read two
+            // values: lane 0 decides for the warp (the ballots below need all lanes).
+            if (__shfl_sync(0xffffffffu, lane == 0 && gb_order_key(b) >= *(volatile unsigned long long*)&st->gub_new_key, 0)) continue;
             if (b > -__longlong_as_double(0x7ff0000000000000LL)) ruled = RULED_OUT;
             ci = c0 + lane;
         } else if (idx < lim) {
