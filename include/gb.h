@@ -231,6 +231,10 @@ gb_status gb_snapshot_take(gb_problem* prob, gb_snapshot* out);
  * With the same block, split and selection options the run continues
  * exactly as the uninterrupted solve would: the generations of the resumed
  * call follow those of the snapshot.  out->generations counts this call.
+ * A snapshot of another block or split can hold regions that wait at a
+ * coordinate where this problem's own splits never start; such a call
+ * evaluates its children by the bytecode interpreter (the same results,
+ * slower).
  * Needs dense rows (pool_mode 1).  GB_E_INVALID on a mismatched or
  * malformed snapshot (regions outside the bounds, lo > hi, a cycling word
  * out of range, a NaN bound), GB_E_CAPACITY if the regions do not fit. */

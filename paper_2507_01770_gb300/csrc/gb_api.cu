@@ -77,6 +77,7 @@ void float_bounds(double c, float* lo, float* hi) {
 
 struct SolveRun {
     bool active = false, loop_done = false;
+    bool interp = false;   // children by the interpreter whatever tables the problem has (tables_cover)
     int cur = 0;
     std::vector<gb_gen_stat> trace;
     long long last_par = 0, launches = 0;
@@ -115,10 +116,10 @@ struct gb_problem {
     SolveRun run;
     GbGenConst G{};
     gb_gen_stat* trace_dev = nullptr;
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};   // gens_per_sync generations starting on pool buffer 0 / 1
+    cudaGraphExec_t gexec[2][2] = {};   // [interpreter][pool buffer]: gens_per_sync generations starting on that buffer
     cudaGraphExec_t gpart[2][2] = {};  // fused serving: [pool buffer][before / after the child evaluation]
     long long part_kernels[2][2] = {};
-    long long graph_kernels = 0;
+    long long graph_kernels[2] = {};
     size_t device_bytes = 0;       // device memory held by the problem
     bool marks_used = false;       // a solve stamped record marks (cleared before the next one)
     bool have_pool = false;        // a solve has left a pool to snapshot
@@ -166,8 +167,9 @@ void gb_destroy_problem(gb_problem* p) {
     for (cudaEvent_t e : p->ev)
         if (e) cudaEventDestroy(e);
     if (p->ev_state) cudaEventDestroy(p->ev_state);
-    for (cudaGraphExec_t g : p->gexec)
-        if (g) cudaGraphExecDestroy(g);
+    for (auto& pp : p->gexec)
+        for (cudaGraphExec_t g : pp)
+            if (g) cudaGraphExecDestroy(g);
     for (auto& pp : p->gpart)
         for (cudaGraphExec_t g : pp)
             if (g) cudaGraphExecDestroy(g);
@@ -789,9 +791,21 @@ void gb_free_result(gb_result* r) {
 // its asynchronous copy has landed) and enqueues the next generation,
 // solve_finish gathers the output.  gb_solve runs the three blocking; the
 // serving loop interleaves many problems without blocking on any of them.
+// The tables are laid out at the positions that a solve from the domain splits
+// at.  A snapshot taken under another block or split can hold regions that wait
+// elsewhere; for these the tables have nothing, so such a solve runs on the
+// interpreter, which splits at any position (the same results).
+static bool tables_cover(const gb_problem* p, const gb_snapshot& s) {
+    if (!p->use_tabs && !p->use_paper) return true;
+    for (long long q = 0; q < s.count; q++)
+        if (s.cyc[q] >= 0 && p->hp.sp_of_cyc[s.cyc[q]] < 0) return false;   // (bit 31: final, never split)
+    return true;
+}
+
 static gb_status solve_begin_from(gb_problem* p, const gb_snapshot* snap) {
     SolveRun& R = p->run;
     R = SolveRun{};
+    R.interp = snap && !tables_cover(p, *snap);
     R.t0 = std::chrono::steady_clock::now();
     GB_CU(cudaSetDevice(p->device));
     const long long l0 = gb_launches_so_far();
@@ -849,6 +863,10 @@ static gb_status solve_begin_from(gb_problem* p, const gb_snapshot* snap) {
 
 __attribute__((visibility("hidden"))) gb_status solve_begin(gb_problem* p) { return solve_begin_from(p, nullptr); }
 
+// The tables that the running solve evaluates its children from.
+static const GbTabs* tabs_of(const gb_problem* p) { return p->use_tabs && !p->run.interp ? &p->tabs : nullptr; }
+static const GbPaper* paper_of(const gb_problem* p) { return p->use_paper && !p->run.interp ? &p->paper : nullptr; }
+
 // Captures gens_per_sync consecutive generations as one CUDA graph per
 // starting pool buffer (once per problem; every argument of a generation is
 // fixed, sizes come from the device state, and a generation that must not
@@ -856,9 +874,9 @@ __attribute__((visibility("hidden"))) gb_status solve_begin(gb_problem* p) { ret
 // state read.
 static cudaError_t capture_graphs(gb_problem* p) {
     cudaStream_t s = p->stream;
-    const int G = p->opt.gens_per_sync;
+    const int G = p->opt.gens_per_sync, in = p->run.interp ? 1 : 0;
     for (int par = 0; par < 2; par++) {
-        if (p->gexec[par]) continue;
+        if (p->gexec[in][par]) continue;
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return e;
@@ -867,8 +885,8 @@ static cudaError_t capture_graphs(gb_problem* p) {
             const int b = (par + k) & 1;
             long long n1 = 0;
             e = gb_launch_generation(p->P, p->pool, p->E[b], p->E[1 - b], p->par, p->ch, p->sp, p->sc,
-                                     p->use_tabs ? &p->tabs : nullptr, p->G, p->cap, p->Cmax, p->st, s, nullptr,
-                                     &n1, 0, &p->fork, p->use_paper ? &p->paper : nullptr);
+                                     tabs_of(p), p->G, p->cap, p->Cmax, p->st, s, nullptr, &n1, 0, &p->fork,
+                                     paper_of(p));
             nl += n1;
         }
         cudaError_t e2 = cudaStreamEndCapture(s, &g);
@@ -877,10 +895,10 @@ static cudaError_t capture_graphs(gb_problem* p) {
             return e;
         }
         if (e2 != cudaSuccess) return e2;
-        e = cudaGraphInstantiate(&p->gexec[par], g, 0);
+        e = cudaGraphInstantiate(&p->gexec[in][par], g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return e;
-        p->graph_kernels = nl;
+        p->graph_kernels[in] = nl;
     }
     return cudaSuccess;
 }
@@ -935,8 +953,8 @@ __attribute__((visibility("hidden"))) int solve_advance(gb_problem* p, bool bloc
     const int G = p->opt.gens_per_sync;
     if (G > 1) {
         if ((e = capture_graphs(p)) != cudaSuccess) return stop(cuda_fail(e, "graph capture"));
-        if ((e = cudaGraphLaunch(p->gexec[cur], s)) != cudaSuccess) return stop(cuda_fail(e, "cudaGraphLaunch"));
-        R.launches += p->graph_kernels;
+        if ((e = cudaGraphLaunch(p->gexec[R.interp][cur], s)) != cudaSuccess) return stop(cuda_fail(e, "cudaGraphLaunch"));
+        R.launches += p->graph_kernels[R.interp];
     } else {
         // the host has just read the pool's size and the active count: the
         // launches and their grids follow them, not the largest pool (an
@@ -945,8 +963,8 @@ __attribute__((visibility("hidden"))) int solve_advance(gb_problem* p, bool bloc
         const long long kids_now = std::min(p->K, std::max(1LL, h.active)) << p->sp.flog2;
         long long nl = 0;
         e = gb_launch_generation(p->P, p->pool, p->E[cur], p->E[1 - cur], p->par, p->ch, p->sp, p->sc,
-                                 p->use_tabs ? &p->tabs : nullptr, p->G, pool_now, kids_now, p->st, s, &p->ev[2], &nl, 0,
-                                 &p->fork, p->use_paper ? &p->paper : nullptr);
+                                 tabs_of(p), p->G, pool_now, kids_now, p->st, s, &p->ev[2], &nl, 0, &p->fork,
+                                 paper_of(p));
         if (e != cudaSuccess) return stop(cuda_fail(e, "generation launch"));
         R.timed64 = true;
         R.timed32 = p->opt.fp32_prefilter != 0;

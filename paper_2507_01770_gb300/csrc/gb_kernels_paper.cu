@@ -80,7 +80,10 @@ __global__ void __launch_bounds__(PP_T) k_pp_rows(GbProg P, GbPool pool, GbParen
     const long long p = blockIdx.y;
     if (p >= st->parents) return;
     const int spi = P.sp_of_cyc[par.info[p].x];
-    if (spi < 0) return;
+    if (spi < 0) {   // no layout (the host sends no such parent here): its children would be lost
+        if (threadIdx.x == 0) atomicOr(&st->error, 8);
+        return;
+    }
     const unsigned slot = par.slot[p];
     int ops = 0;
     if ((int)blockIdx.x >= row_blocks) {   // group tree (k, kind)

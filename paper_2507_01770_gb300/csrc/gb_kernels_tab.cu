@@ -206,7 +206,10 @@ __global__ void __launch_bounds__(PTAB_T) k_ptab(GbProg P, GbPool pool, GbParent
     int4 info = make_int4(0, 0, 0, 0);
     if (rows) info = parent_split(P, pool, par, sp, p, slot, cyc, s_bnd, s_brd, s_bru, blockIdx.x == 0);
     if (blockIdx.x == 0 && threadIdx.x == 0) {   // the split position for the later kernels
-        if (spi < 0) SP.ndterm = -1;
+        if (spi < 0) {   // no layout (the host sends no such parent here): its children would be lost
+            SP.ndterm = -1;
+            atomicOr(&st->error, 8);
+        }
         par.spos[p] = SP;
     }
     __syncthreads();
