@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "gb_child.cuh"
 #include "gb_launch.h"
@@ -301,12 +302,31 @@ __global__ void __launch_bounds__(C::THREADS) k_box(GbProg P, const GbBoxTile* _
     if (lane == 0 && live) mono[b] = *s_mono;
 }
 
+// Shared memory a block may take (of the 227 KB): one block per SM (the box
+// evaluation), two (the children).
+constexpr size_t BOX_SMEM = 200 * 1024, CHILD_SMEM = 100 * 1024;
+
+// Lets kernel K take `cap` bytes of dynamic shared memory.  The limit belongs
+// to the function and the device, not to a launch: set to a call's own size, it
+// could be lowered by another thread's call between the setting and the launch.
+// So it is set to the most that the dispatch allows, once per device.
+template <auto K> cudaError_t allow_smem(size_t cap) {
+    static std::atomic<bool> done[64];   // by device ordinal (above: set every time)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 64 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
+    if (e == cudaSuccess && dev < 64) done[dev].store(true, std::memory_order_release);
+    return e;
+}
+
 // Threads per box.  Small objectives (no sum over 16 terms): the next power
 // of two, several boxes per warp.  Else a warp per box once the boxes give
 // every SM 16 warps; with fewer boxes 128 and then 512 threads, so that a
 // handful of boxes still fills the chip.  The tiles must hold every group.
 struct BoxPick { int cfg, list; };
-template <typename C, typename I> bool fits_smem(const GbProg& P) { return box_smem_block<C, I>(P) <= 200 * 1024; }
+template <typename C, typename I> bool fits_smem(const GbProg& P) { return box_smem_block<C, I>(P) <= BOX_SMEM; }
 
 typedef BoxCfg<4, 4, 4> Cfg4;
 typedef BoxCfg<8, 8, 8> Cfg8;
@@ -553,7 +573,7 @@ cudaError_t launch_box(const GbProg& P, int list, const double* lo, const double
                        double* F, double* Fmid, double* G, int* mono, cudaStream_t s) {
     const size_t smem = box_smem_block<C, typename Prec<T>::I>(P);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_box<C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem<k_box<C, T>>(BOX_SMEM);
         if (e != cudaSuccess) return e;
     }
     k_box<C, T><<<(unsigned)((nbox + C::BPB - 1) / C::BPB), C::THREADS, smem, s>>>(
@@ -585,9 +605,9 @@ int gb_box_coop(const GbProg& P, long long nbox) { return box_pick(P, nbox).cfg 
 int gb_child_box(const GbProg& P) {
     if (P.any_prod || P.n_groups > 64) return 0;
     const int need = std::max(P.max_dirty_terms, P.B);
-    if (need <= 4 && box_smem_block<Cfg4, iv64>(P) <= 100 * 1024) return 4;
-    if (need <= 8 && box_smem_block<Cfg8, iv64>(P) <= 100 * 1024) return 8;
-    if (need <= 16 && box_smem_block<Cfg16, iv64>(P) <= 100 * 1024) return 16;
+    if (need <= 4 && box_smem_block<Cfg4, iv64>(P) <= CHILD_SMEM) return 4;
+    if (need <= 8 && box_smem_block<Cfg8, iv64>(P) <= CHILD_SMEM) return 8;
+    if (need <= 16 && box_smem_block<Cfg16, iv64>(P) <= CHILD_SMEM) return 16;
     return 0;
 }
 
@@ -597,7 +617,7 @@ cudaError_t launch_child_box(const GbProg& P, const GbPool& pool, const GbParent
                              long long Cmax, const GbSplit& sp, GbState* st, const GbGenConst& G, cudaStream_t s) {
     const size_t smem = box_smem_block<C, iv64>(P);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_child_box<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem<k_child_box<C>>(CHILD_SMEM);
         if (e != cudaSuccess) return e;
     }
     const unsigned g = (unsigned)std::min<long long>((Cmax + C::BPB - 1) / C::BPB, gb_sm_count() * 8);
