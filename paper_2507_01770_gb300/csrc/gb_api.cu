@@ -516,6 +516,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         (e = alloc(&p->ch.surv, C, A)))
         return bad(e, "allocate child buffers");
     // per-parent term tables
+    bool want_unit = false, want_dec = false;
     if (opt.eval_mode != 1) {
         const bool want = opt.eval_mode >= 2 || p->fan >= 16;
         if (p->hp.tab_ok && want) {
@@ -533,14 +534,9 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             GbContrib* d_cb;
             GbJkD* d_jkd;
             GbSeg* d_segs;
-            uint16_t* d_mvf;
-            if (unit) {
-                if ((e = upload(&d_mvf, Hh.mvf.data(), Hh.mvf.size(), A))) return bad(e, "upload table layouts");
-                P.mvf = d_mvf;
-                p->tabs.unit = 1;
-            } else if (warp && d * mshift >= 5 && P.n_sum > 0) {
-                p->tabs.unit = 2;
-            }
+            want_unit = unit;
+            want_dec = dec;
+            if (!unit && warp && d * mshift >= 5 && P.n_sum > 0) p->tabs.unit = 2;
             if ((e = upload(&d_jkd, Hh.jkd.data(), Hh.jkd.size(), A)) ||
                 (e = upload(&d_segs, Hh.segs.data(), Hh.segs.size(), A)) ||
                 (e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||
@@ -599,18 +595,6 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
                 }
                 T.reg = fits ? 1 : 0;
             }
-            T.dec = dec ? 1 : 0;
-            if (dec) {
-                GbUop* d_u;
-                if ((e = upload(&d_u, Hh.uops.data(), Hh.uops.size(), A))) return bad(e, "upload table layouts");
-                P.uops = d_u;
-                if (!fp32 && d * mshift >= GB_CUT_MIN &&
-                    ((e = alloc(&T.cut.tv, 2 * rows, A)) || (e = alloc(&T.cut.ts, 2 * K * (size_t)T.max_srows, A)) ||
-                     (e = alloc(&T.cut.td, K * (size_t)T.max_drows, A)))) {
-                    cudaGetLastError();   // no room: every child by itself
-                    T.cut = GbCut{};
-                }
-            }
             T.max_sum_nodes = 1;
             for (const GbSum& S : Hh.sums) T.max_sum_nodes = std::max(T.max_sum_nodes, (int)S.nnodes);
             // no opt-in needed: the table kernel's static shared memory (about 12 KB) and the
@@ -629,110 +613,6 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
                 }
             }
             p->use_tabs = true;
-        }
-    }
-    if (paper_tabs) {
-        const bool dec = gb_build_endpoints(&p->hp, true);
-        const GbHostProg& Hh = p->hp;
-        GbPaper& T = p->paper;
-        int32_t* d_spc;
-        GbSplitPos* d_sps;
-        GbDTerm* d_dt;
-        int2* d_jk;
-        GbContrib* d_cb;
-        GbJkD* d_jkd;
-        GbSeg* d_segs;
-        GbPaperSum* d_ps;
-        GbHoistPos* d_hp;
-        int32_t* d_hn;
-        GbOIns* d_op;
-        GbUop* d_u;
-        if ((e = upload(&d_u, Hh.uops.data(), Hh.uops.size(), A)) ||
-            (e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||
-            (e = upload(&d_sps, Hh.sps.data(), Hh.sps.size(), A)) ||
-            (e = upload(&d_dt, Hh.dterms.data(), Hh.dterms.size(), A)) ||
-            (e = upload(&d_jk, Hh.jk.data(), Hh.jk.size(), A)) ||
-            (e = upload(&d_cb, Hh.contribs.data(), Hh.contribs.size(), A)) ||
-            (e = upload(&d_jkd, Hh.jkd.data(), Hh.jkd.size(), A)) ||
-            (e = upload(&d_segs, Hh.segs.data(), Hh.segs.size(), A)) ||
-            (e = upload(&d_ps, Hh.psums.data(), Hh.psums.size(), A)) ||
-            (e = upload(&d_hp, Hh.hoist_pos.data(), Hh.hoist_pos.size(), A)) ||
-            (e = upload(&d_hn, Hh.hoist_node.data(), Hh.hoist_node.size(), A)) ||
-            (e = upload(&d_op, Hh.oprog.data(), Hh.oprog.size(), A)))
-            return bad(e, "upload table layouts");
-        P.m = Hh.m;
-        P.mshift = Hh.mshift;
-        P.max_rows = Hh.max_rows;
-        P.sp_of_cyc = d_spc;
-        P.sps = d_sps;
-        P.dterms = d_dt;
-        P.jk = d_jk;
-        P.contribs = d_cb;
-        P.jkd = d_jkd;
-        P.segs = d_segs;
-        P.max_nseg = Hh.max_nseg;
-        T.nk = 1 + (opt.samples > 0 ? opt.samples : 1);
-        T.n_hoist = (int)Hh.hoist_node.size();
-        T.n_oprog = (int)Hh.oprog.size();
-        T.arows = std::max(1, Hh.max_arows);
-        T.srows = std::max(1, Hh.max_srows);
-        T.drows = std::max(1, Hh.max_drows);
-        T.hrows = std::max(1, Hh.max_hrows);
-        T.tree_nodes = std::max(1, Hh.tree_nodes);
-        T.max_leaves = std::max(1, Hh.max_leaves);
-        T.psums = d_ps;
-        T.hoist_pos = d_hp;
-        T.hoist_node = d_hn;
-        T.oprog = d_op;
-        T.indep = Hh.indep;
-        T.dec = dec ? 1 : 0;
-        P.uops = d_u;
-        const size_t kk = K * (size_t)T.nk;
-        if ((e = alloc(&T.tv, kk * T.arows, A)) || (e = alloc(&T.ts, kk * T.srows, A)) ||
-            (e = alloc(&T.nd, kk * T.tree_nodes, A)) || (e = alloc(&T.hv, kk * T.hrows, A)) ||
-            (e = alloc(&T.tl, K * (size_t)T.arows * T.max_leaves, A)) || (e = alloc(&T.td, K * (size_t)T.drows, A)))
-            cudaGetLastError();   // no room for the tables: the interpreter
-        else
-            p->use_paper = true;
-        // products: forward values and reverse factors of their term rows (64 MiB at most, or the sweeps form them)
-        if (p->use_paper && P.any_prod) {
-            for (const GbSum& S : Hh.sums)
-                if (S.prod) T.pw = std::max(T.pw, (int)S.nins);
-            const size_t pc = K * (size_t)T.arows * T.pw;
-            if (pc * sizeof(double2) <= (32u << 20) && (alloc(&T.pv, pc, A) || alloc(&T.pf, pc, A))) {
-                cudaGetLastError();
-                T.pv = T.pf = nullptr;
-            }
-        }
-        // groups of children (gb_cut.cuh): the operations a child applies to its reductions are isotone
-        bool iso = true;
-        for (const GbOIns& o : Hh.oprog) iso = iso && o.op != D_EXP && o.op != D_SIN && o.op != D_COS;
-        if (p->use_paper && iso && d * mshift >= GB_CUT_MIN &&
-            ((e = alloc(&T.cut.tv, kk * T.arows, A)) || (e = alloc(&T.cut.ts, kk * T.srows, A)) ||
-             (e = alloc(&T.cut.hv, kk * T.hrows, A)) || (e = alloc(&T.cut.td, K * (size_t)T.drows, A)))) {
-            cudaGetLastError();   // no room: every child by itself
-            T.cut = GbCut{};
-        }
-    }
-    // the sums' outer adjoints, where they are the same for every box: every
-    // node from the sum to the root passes its adjoint on, or times a constant
-    if (p->tabs.cut.tv || p->paper.cut.tv) {
-        std::vector<char> fixed(H.outer.size(), 1);
-        auto live = [&](int t) { return (H.outer[t].pad & GB_RV_LIVE) != 0; };
-        for (int t = (int)H.outer.size() - 1; t >= 0; t--) {
-            const GbIns& I = H.outer[t];
-            const bool pass = I.op == D_ADD || I.op == D_SUB || I.op == D_NEG || I.op == D_SCALE;
-            const bool prod = I.op == D_MUL || I.op == D_DIV;
-            if (I.pad & GB_RV_A) fixed[I.a] = fixed[I.a] && fixed[t] && (pass || (prod && !live(I.b)));
-            if (I.pad & GB_RV_B) fixed[I.b] = fixed[I.b] && fixed[t] && (pass || (I.op == D_MUL && !live(I.a)));
-        }
-        bool all = !H.any_prod;
-        for (const GbSum& S : H.sums) all = all && fixed[S.outer_reg];
-        double2* d_adj;
-        if (all) {
-            if ((e = alloc(&d_adj, (size_t)GB_MAX_ISUM, A)) || (e = gb_launch_outer_adj(P, d_adj, p->stream)))
-                return bad(e, "outer adjoints");
-            P.sum_adj = d_adj;
         }
     }
     p->G.K = p->K;
@@ -757,6 +637,148 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         (e = alloc(&p->st, 1, A)))
         return bad(e, "allocate scan buffers");
     if ((e = cudaMemsetAsync(p->sc.hist, 0, 65536 * sizeof(unsigned), p->stream))) return bad(e, "cudaMemset");
+    // what only makes a solve faster, now that all it needs is there
+    auto optional = [&](size_t bytes, auto&& take) {
+        size_t left = 0, total = 0;
+        const size_t n0 = p->owned.size(), b0 = p->device_bytes;
+        if (cudaMemGetInfo(&left, &total) == cudaSuccess && bytes <= left / 2 && take() == cudaSuccess) return true;
+        cudaGetLastError();
+        for (; p->owned.size() > n0; p->owned.pop_back()) cudaFreeAsync(p->owned.back(), p->stream);
+        p->device_bytes = b0;
+        return false;
+    };
+    auto bytes_of = [](const auto& v) { return v.size() * sizeof(v[0]); };
+    if (want_unit) {
+        uint16_t* d_mvf;
+        if (optional(bytes_of(H.mvf), [&] { return upload(&d_mvf, H.mvf.data(), H.mvf.size(), A); })) {
+            P.mvf = d_mvf;
+            p->tabs.unit = 1;
+        }
+    }
+    if (want_dec) {
+        GbUop* d_u;
+        GbTabs& T = p->tabs;
+        if (optional(bytes_of(H.uops), [&] { return upload(&d_u, H.uops.data(), H.uops.size(), A); })) {
+            P.uops = d_u;
+            T.dec = 1;
+        }
+        const size_t rows = 2 * K * (size_t)T.max_rows, segs = 2 * K * (size_t)T.max_srows, parts = K * (size_t)T.max_drows;
+        if (T.dec && !fp32 && d * mshift >= GB_CUT_MIN && !optional((rows + segs + parts) * sizeof(double2), [&] {
+                (e = alloc(&T.cut.tv, rows, A)) || (e = alloc(&T.cut.ts, segs, A)) || (e = alloc(&T.cut.td, parts, A));
+                return e;
+            }))
+            T.cut = GbCut{};   // no room: every child by itself
+    }
+    if (paper_tabs) {
+        const bool dec = gb_build_endpoints(&p->hp, true);
+        GbPaper& T = p->paper;
+        T.nk = 1 + (opt.samples > 0 ? opt.samples : 1);
+        T.n_hoist = (int)H.hoist_node.size();
+        T.n_oprog = (int)H.oprog.size();
+        T.arows = std::max(1, H.max_arows);
+        T.srows = std::max(1, H.max_srows);
+        T.drows = std::max(1, H.max_drows);
+        T.hrows = std::max(1, H.max_hrows);
+        T.tree_nodes = std::max(1, H.tree_nodes);
+        T.max_leaves = std::max(1, H.max_leaves);
+        T.indep = H.indep;
+        T.dec = dec ? 1 : 0;
+        int32_t* d_spc;
+        GbSplitPos* d_sps;
+        GbDTerm* d_dt;
+        int2* d_jk;
+        GbContrib* d_cb;
+        GbJkD* d_jkd;
+        GbSeg* d_segs;
+        GbPaperSum* d_ps;
+        GbHoistPos* d_hp;
+        int32_t* d_hn;
+        GbOIns* d_op;
+        GbUop* d_u;
+        const size_t kk = K * (size_t)T.nk, parts = K * (size_t)T.drows;
+        const size_t layouts = bytes_of(H.uops) + bytes_of(H.sp_of_cyc) + bytes_of(H.sps) + bytes_of(H.dterms) +
+                               bytes_of(H.jk) + bytes_of(H.contribs) + bytes_of(H.jkd) + bytes_of(H.segs) +
+                               bytes_of(H.psums) + bytes_of(H.hoist_pos) + bytes_of(H.hoist_node) + bytes_of(H.oprog);
+        const size_t entries = kk * ((size_t)T.arows + T.srows + T.hrows + T.tree_nodes) +
+                               K * (size_t)T.arows * T.max_leaves + parts;
+        p->use_paper = optional(layouts + entries * sizeof(double2), [&] {
+            (e = upload(&d_u, H.uops.data(), H.uops.size(), A)) ||
+                (e = upload(&d_spc, H.sp_of_cyc.data(), H.sp_of_cyc.size(), A)) ||
+                (e = upload(&d_sps, H.sps.data(), H.sps.size(), A)) ||
+                (e = upload(&d_dt, H.dterms.data(), H.dterms.size(), A)) ||
+                (e = upload(&d_jk, H.jk.data(), H.jk.size(), A)) ||
+                (e = upload(&d_cb, H.contribs.data(), H.contribs.size(), A)) ||
+                (e = upload(&d_jkd, H.jkd.data(), H.jkd.size(), A)) ||
+                (e = upload(&d_segs, H.segs.data(), H.segs.size(), A)) ||
+                (e = upload(&d_ps, H.psums.data(), H.psums.size(), A)) ||
+                (e = upload(&d_hp, H.hoist_pos.data(), H.hoist_pos.size(), A)) ||
+                (e = upload(&d_hn, H.hoist_node.data(), H.hoist_node.size(), A)) ||
+                (e = upload(&d_op, H.oprog.data(), H.oprog.size(), A)) || (e = alloc(&T.tv, kk * T.arows, A)) ||
+                (e = alloc(&T.ts, kk * T.srows, A)) || (e = alloc(&T.nd, kk * T.tree_nodes, A)) ||
+                (e = alloc(&T.hv, kk * T.hrows, A)) || (e = alloc(&T.tl, K * (size_t)T.arows * T.max_leaves, A)) ||
+                (e = alloc(&T.td, parts, A));
+            return e;
+        });
+        if (p->use_paper) {   // (else the interpreter)
+            P.m = H.m;
+            P.mshift = H.mshift;
+            P.max_rows = H.max_rows;
+            P.sp_of_cyc = d_spc;
+            P.sps = d_sps;
+            P.dterms = d_dt;
+            P.jk = d_jk;
+            P.contribs = d_cb;
+            P.jkd = d_jkd;
+            P.segs = d_segs;
+            P.max_nseg = H.max_nseg;
+            P.uops = d_u;
+            T.psums = d_ps;
+            T.hoist_pos = d_hp;
+            T.hoist_node = d_hn;
+            T.oprog = d_op;
+        }
+        // products: forward values and reverse factors of their term rows (64 MiB at most, or the sweeps form them)
+        if (p->use_paper && P.any_prod) {
+            for (const GbSum& S : H.sums)
+                if (S.prod) T.pw = std::max(T.pw, (int)S.nins);
+            const size_t pc = K * (size_t)T.arows * T.pw;
+            if (pc * sizeof(double2) <= (32u << 20) && !optional(2 * pc * sizeof(double2), [&] {
+                    (e = alloc(&T.pv, pc, A)) || (e = alloc(&T.pf, pc, A));
+                    return e;
+                }))
+                T.pv = T.pf = nullptr;
+        }
+        // groups of children (gb_cut.cuh): the operations a child applies to its reductions are isotone
+        bool iso = true;
+        for (const GbOIns& o : H.oprog) iso = iso && o.op != D_EXP && o.op != D_SIN && o.op != D_COS;
+        if (p->use_paper && iso && d * mshift >= GB_CUT_MIN &&
+            !optional((kk * ((size_t)T.arows + T.srows + T.hrows) + parts) * sizeof(double2), [&] {
+                (e = alloc(&T.cut.tv, kk * T.arows, A)) || (e = alloc(&T.cut.ts, kk * T.srows, A)) ||
+                    (e = alloc(&T.cut.hv, kk * T.hrows, A)) || (e = alloc(&T.cut.td, parts, A));
+                return e;
+            }))
+            T.cut = GbCut{};   // no room: every child by itself
+    }
+    // the sums' outer adjoints, where they are the same for every box: every
+    // node from the sum to the root passes its adjoint on, or times a constant
+    if (p->tabs.cut.tv || p->paper.cut.tv) {
+        std::vector<char> fixed(H.outer.size(), 1);
+        auto live = [&](int t) { return (H.outer[t].pad & GB_RV_LIVE) != 0; };
+        for (int t = (int)H.outer.size() - 1; t >= 0; t--) {
+            const GbIns& I = H.outer[t];
+            const bool pass = I.op == D_ADD || I.op == D_SUB || I.op == D_NEG || I.op == D_SCALE;
+            const bool prod = I.op == D_MUL || I.op == D_DIV;
+            if (I.pad & GB_RV_A) fixed[I.a] = fixed[I.a] && fixed[t] && (pass || (prod && !live(I.b)));
+            if (I.pad & GB_RV_B) fixed[I.b] = fixed[I.b] && fixed[t] && (pass || (I.op == D_MUL && !live(I.a)));
+        }
+        bool all = !H.any_prod;
+        for (const GbSum& S : H.sums) all = all && fixed[S.outer_reg];
+        double2* d_adj;
+        if (all && optional(GB_MAX_ISUM * sizeof(double2), [&] { return alloc(&d_adj, (size_t)GB_MAX_ISUM, A); })) {
+            if ((e = gb_launch_outer_adj(P, d_adj, p->stream))) return bad(e, "outer adjoints");
+            P.sum_adj = d_adj;
+        }
+    }
     if ((e = cudaMallocHost((void**)&p->st_host, sizeof(GbState)))) return bad(e, "cudaMallocHost");
     for (cudaEvent_t& ev : p->ev)
         if ((e = cudaEventCreate(&ev))) return bad(e, "cudaEventCreate");
