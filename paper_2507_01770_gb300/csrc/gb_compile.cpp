@@ -803,9 +803,10 @@ void gb_build_tables(GbHostProg* P, int m, int d, int sbits, bool paper) {
                             if (t < ps.t_lo || t >= ps.t_hi) add(t);
                     } else if (S.has_var) {   // the clean terms that touch [ja, jb)
                         std::vector<int> before, after;
-                        for (int t = 0; t < S.count; t++) {
+                        const int need = sp.ja - S.off_max - S.first;
+                        for (int t = need <= 0 ? 0 : (need + S.step - 1) / S.step; t < S.count; t++) {
                             const int i = S.first + t * S.step;
-                            if (i + S.off_max < sp.ja || (t >= ps.t_lo && t < ps.t_hi)) continue;
+                            if (t >= ps.t_lo && t < ps.t_hi) continue;
                             if (i + S.off_min >= sp.jb) break;
                             (t < ps.t_lo ? before : after).push_back(add(t));
                         }
