@@ -67,6 +67,47 @@ cudaError_t alloc(T** dst, size_t count, DevAlloc& a) {
     return e;
 }
 
+// The outer expression is one sum.
+bool outer_is_sum(const GbHostProg& H) {
+    return H.outer.size() == 1 && H.outer[0].op == D_ISUMV && H.outer_root == 0 && !H.any_prod;
+}
+
+// Every sum's outer adjoint is exactly [1, 1] and no coordinate enters the
+// outer expression.  The outer adjoints that are exact constants: the root's
+// is [1, 1]; an addition passes its adjoint to both operands, a subtraction to
+// the left one (the right one gets its negation), a negation its negation;
+// anything else makes its operands' adjoints data-dependent.
+bool outer_is_unit(const GbHostProg& H) {
+    const int no = (int)H.outer.size();
+    std::vector<double> adj(no, 0.0);
+    std::vector<char> known(no, 1);
+    if (no > 0) adj[H.outer_root] = 1.0;
+    auto pass = [&](int r, double v, bool k) {
+        if (r < 0 || r >= no) return;
+        if (!k) known[r] = 0;
+        else adj[r] += v;
+    };
+    for (int t = no - 1; t >= 0; t--) {
+        const GbIns& I = H.outer[t];
+        const bool k = known[t] != 0;
+        switch (I.op) {
+        case D_ADD: pass(I.a, adj[t], k); pass(I.b, adj[t], k); break;
+        case D_SUB: pass(I.a, adj[t], k); pass(I.b, -adj[t], k); break;
+        case D_NEG: pass(I.a, -adj[t], k); break;
+        case D_CONST: case D_PI: case D_EULER: case D_VAR: case D_ISUMV: break;
+        default: pass(I.a, 0.0, false); pass(I.b, 0.0, false); break;
+        }
+    }
+    bool unit = !H.any_prod && H.var_leaves.empty() && !H.sums.empty();
+    for (const GbSum& S : H.sums) unit = unit && known[S.outer_reg] && adj[S.outer_reg] == 1.0;
+    return unit;
+}
+
+// Every sum enters F with adjoint [1, 1] and no coordinate of its own does.
+bool sums_alone(const GbHostProg& H) {
+    return H.var_leaves.empty() && (outer_is_unit(H) || (outer_is_sum(H) && H.sums.size() == 1));
+}
+
 void float_bounds(double c, float* lo, float* hi) {
     float f = (float)c;
     *lo = ((double)f <= c) ? f : std::nextafter(f, -INFINITY);
@@ -245,37 +286,66 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         }
         p->opt.eval_mode = opt.eval_mode = 1;
     }
+    // What the tables of all parents of a generation may take.
+    const double budget = std::max(64.0 * (1 << 20), (double)opt.pool_bytes / 8.0);
+    const int flog2 = opt.split_d * mshift;
+    const long long gen_parents = std::max(1LL, (long long)opt.max_children >> flog2);
+    const bool large = flog2 >= GB_CUT_MIN;   // children in groups (gb_cut.cuh)
     // term-table layouts also set each sum's tree offsets: build them before
     // the program is uploaded
+    bool tab_groups = false;   // with the hull tables of the child groups
     if (opt.eval_mode != 1) {
-        // segment tables are per parent: the widest segments whose tables for
-        // all parents of a generation fit max(64 MiB, pool budget / 8)
-        const int msh = opt.split_m == 2 ? 1 : 2;
-        const long long fan = 1LL << (opt.split_d * msh);
-        const long long K = std::max(1LL, (long long)opt.max_children / fan);
-        const double budget = std::max(64.0 * (1 << 20), (double)opt.pool_bytes / 8.0);
+        // segment tables are per parent: the widest segments whose tables,
+        // with the hulls that the groups read of them, keep to the budget; if
+        // none do, the widest without groups
+        const bool per_thread = opt.eval_mode == 3 || (opt.eval_mode != 4 && !gb_warp_per_child(gen_parents << flog2));
         const double per_row = opt.fp32_prefilter ? 40.0 : 32.0;
-        for (int sbits = GB_TAB_SBITS; sbits >= 0; sbits--) {
+        bool groups = large && per_thread && !opt.fp32_prefilter && sums_alone(p->hp), fits = false;
+        for (int sbits = GB_TAB_SBITS; !fits; sbits--) {
             gb_build_tables(&p->hp, opt.split_m, opt.split_d, sbits);
-            if (!p->hp.tab_ok || (double)K * p->hp.max_srows * per_row <= budget) break;
+            groups = groups && gb_build_endpoints(&p->hp, false);
+            fits = !p->hp.tab_ok || (double)gen_parents * p->hp.max_srows * (per_row + (groups ? 32.0 : 0.0)) <= budget;
+            if (sbits > 0 || fits) continue;
+            if (!groups) break;
+            groups = false;
+            sbits = GB_TAB_SBITS + 1;
         }
+        tab_groups = groups;
     }
-    // paper mode: tables when a parent has at least 16 children, they fit
-    // max(64 MiB, pool budget / 8) for all parents of a generation and the
-    // objective's outer expression allows them
+    // paper mode: tables when a parent has at least 16 children, they keep to
+    // the budget and the objective's outer expression allows them; with the
+    // hull tables of the groups (the operations a child applies to its
+    // reductions have to be isotone) and the rows of the products' sweeps when
+    // these fit beside them
+    bool paper_groups = false, paper_rows = false;
     if (paper_tabs) {
-        const int flog2 = opt.split_d * mshift;
-        const long long K = std::max(1LL, (long long)opt.max_children >> flog2);
+        const GbHostProg& T = p->hp;
         const int nk = 1 + (opt.samples > 0 ? opt.samples : 1);
-        const double budget = std::max(64.0 * (1 << 20), (double)opt.pool_bytes / 8.0);
-        paper_tabs = flog2 >= 4 && K <= 65535;
+        int pw = 0;   // nodes of the widest product template
+        for (const GbSum& S : T.sums)
+            if (S.prod) pw = std::max(pw, (int)S.nins);
+        paper_tabs = flog2 >= 4 && gen_parents <= 65535;
+        bool extra = true;   // the tables that the others can do without
         for (int sbits = GB_TAB_SBITS; paper_tabs; sbits--) {
             gb_build_tables(&p->hp, opt.split_m, opt.split_d, sbits, true);
-            const GbHostProg& T = p->hp;
-            const double per = 16.0 * (nk * ((double)T.max_arows + T.max_srows + T.max_hrows + T.tree_nodes) +
-                                       (double)T.max_arows * T.max_leaves + T.max_drows);
-            if (T.tab_ok && K * per <= budget) break;
-            if (!T.tab_ok || sbits == 0) paper_tabs = false;
+            if (!T.tab_ok) {
+                paper_tabs = false;
+                break;
+            }
+            paper_groups = extra && large;
+            for (const GbOIns& o : T.oprog) paper_groups = paper_groups && o.op != D_EXP && o.op != D_SIN && o.op != D_COS;
+            const double K16 = 16.0 * gen_parents, sweep = K16 * T.max_arows * pw;
+            paper_rows = extra && pw > 0 && sweep <= (32 << 20);   // (64 MiB at most, or the sweeps form the values)
+            const double per_kind = nk * ((double)T.max_arows + T.max_srows + T.max_hrows);
+            double need = K16 * (per_kind + nk * (double)T.tree_nodes + (double)T.max_arows * T.max_leaves + T.max_drows);
+            if (paper_groups) need += K16 * (per_kind + T.max_drows);
+            if (paper_rows) need += 2.0 * sweep;
+            if (need <= budget) break;
+            const double segs = K16 * nk * T.max_srows * (paper_groups ? 2 : 1);
+            if (sbits > 0 && need - segs <= budget) continue;   // narrower segments may do
+            if (!paper_groups && !paper_rows) paper_tabs = false;
+            extra = false;
+            sbits = GB_TAB_SBITS + 1;
         }
         if (!paper_tabs) p->hp.tab_ok = 0;
     }
@@ -313,36 +383,8 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     P.n_outer = (int)H.outer.size();
     P.outer_root = H.outer_root;
     P.n_var_leaves = (int)H.var_leaves.size();
-    P.outer_sum = (H.outer.size() == 1 && H.outer[0].op == D_ISUMV && H.outer_root == 0 && !H.any_prod) ? 1 : 0;
-    {
-        // the outer adjoints that are exact constants: the root's is [1, 1];
-        // an addition passes its adjoint to both operands, a subtraction to
-        // the left one (the right one gets its negation), a negation its
-        // negation; anything else makes its operands' adjoints data-dependent
-        const int no = (int)H.outer.size();
-        std::vector<double> adj(no, 0.0);
-        std::vector<char> known(no, 1);
-        if (no > 0) adj[H.outer_root] = 1.0;
-        auto pass = [&](int r, double v, bool k) {
-            if (r < 0 || r >= no) return;
-            if (!k) known[r] = 0;
-            else adj[r] += v;
-        };
-        for (int t = no - 1; t >= 0; t--) {
-            const GbIns& I = H.outer[t];
-            const bool k = known[t] != 0;
-            switch (I.op) {
-            case D_ADD: pass(I.a, adj[t], k); pass(I.b, adj[t], k); break;
-            case D_SUB: pass(I.a, adj[t], k); pass(I.b, -adj[t], k); break;
-            case D_NEG: pass(I.a, -adj[t], k); break;
-            case D_CONST: case D_PI: case D_EULER: case D_VAR: case D_ISUMV: break;
-            default: pass(I.a, 0.0, false); pass(I.b, 0.0, false); break;
-            }
-        }
-        bool unit = !H.any_prod && H.var_leaves.empty() && !H.sums.empty();
-        for (const GbSum& S : H.sums) unit = unit && known[S.outer_reg] && adj[S.outer_reg] == 1.0;
-        P.outer_unit = unit ? 1 : 0;
-    }
+    P.outer_sum = outer_is_sum(H) ? 1 : 0;
+    P.outer_unit = outer_is_unit(H) ? 1 : 0;
     P.any_prod = H.any_prod;
     P.samples = opt.samples;
     P.mono_all = opt.mono_all ? 1 : 0;
@@ -521,11 +563,10 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         const bool want = opt.eval_mode >= 2 || p->fan >= 16;
         if (p->hp.tab_ok && want) {
             const bool warp = opt.eval_mode == 4 || (opt.eval_mode != 3 && gb_warp_per_child(p->Cmax));
-            const bool dec = !warp && P.n_var_leaves == 0 && (P.outer_unit || (P.outer_sum && P.n_sum == 1)) &&
-                             gb_build_endpoints(&p->hp, false);
+            const bool dec = !warp && sums_alone(H) && gb_build_endpoints(&p->hp, false);
             // children 32 to a block, verdicts by lookup (k_unit)
-            const bool unit = warp && P.n_var_leaves == 0 && (P.outer_unit || (P.outer_sum && P.n_sum == 1)) &&
-                              d * mshift >= 5 && P.B <= GB_UNIT_B && gb_build_verdicts(&p->hp, GB_MV_BITS);
+            const bool unit = warp && sums_alone(H) && d * mshift >= 5 && P.B <= GB_UNIT_B &&
+                              gb_build_verdicts(&p->hp, GB_MV_BITS);
             const GbHostProg& Hh = p->hp;
             int32_t* d_spc;
             GbSplitPos* d_sps;
@@ -663,7 +704,7 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             T.dec = 1;
         }
         const size_t rows = 2 * K * (size_t)T.max_rows, segs = 2 * K * (size_t)T.max_srows, parts = K * (size_t)T.max_drows;
-        if (T.dec && !fp32 && d * mshift >= GB_CUT_MIN && !optional((rows + segs + parts) * sizeof(double2), [&] {
+        if (T.dec && tab_groups && !optional((rows + segs + parts) * sizeof(double2), [&] {
                 (e = alloc(&T.cut.tv, rows, A)) || (e = alloc(&T.cut.ts, segs, A)) || (e = alloc(&T.cut.td, parts, A));
                 return e;
             }))
@@ -737,21 +778,18 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             T.hoist_node = d_hn;
             T.oprog = d_op;
         }
-        // products: forward values and reverse factors of their term rows (64 MiB at most, or the sweeps form them)
-        if (p->use_paper && P.any_prod) {
+        // products: forward values and reverse factors of their term rows
+        if (p->use_paper && paper_rows) {
             for (const GbSum& S : H.sums)
                 if (S.prod) T.pw = std::max(T.pw, (int)S.nins);
             const size_t pc = K * (size_t)T.arows * T.pw;
-            if (pc * sizeof(double2) <= (32u << 20) && !optional(2 * pc * sizeof(double2), [&] {
+            if (!optional(2 * pc * sizeof(double2), [&] {
                     (e = alloc(&T.pv, pc, A)) || (e = alloc(&T.pf, pc, A));
                     return e;
                 }))
                 T.pv = T.pf = nullptr;
         }
-        // groups of children (gb_cut.cuh): the operations a child applies to its reductions are isotone
-        bool iso = true;
-        for (const GbOIns& o : H.oprog) iso = iso && o.op != D_EXP && o.op != D_SIN && o.op != D_COS;
-        if (p->use_paper && iso && d * mshift >= GB_CUT_MIN &&
+        if (p->use_paper && paper_groups &&
             !optional((kk * ((size_t)T.arows + T.srows + T.hrows) + parts) * sizeof(double2), [&] {
                 (e = alloc(&T.cut.tv, kk * T.arows, A)) || (e = alloc(&T.cut.ts, kk * T.srows, A)) ||
                     (e = alloc(&T.cut.hv, kk * T.hrows, A)) || (e = alloc(&T.cut.td, parts, A));

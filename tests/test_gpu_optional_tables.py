@@ -1,5 +1,6 @@
-"""Tables that only make a solve faster (paper mode's, the child groups'): a
-problem that fits the device without them is created whatever is left for them."""
+"""Tables that only make a solve faster (paper mode's, the child groups'): they
+keep to the stated budget, max(64 MiB, pool budget / 8), and a problem that fits
+the device without them is created whatever is left for them."""
 import ctypes
 
 import numpy as np
@@ -37,6 +38,14 @@ def _held(make):
     held = f0 - _free()
     s.close()
     return held
+
+
+@pytest.mark.parametrize("fam", ["paper_levy", "paper_griewank", "paper_rastrigin"])
+def test_budget_of_the_paper_mode_tables(fam):
+    without = _held(lambda: _paper(fam, 1, 1 << 30))
+    for pool in (1 << 29, 1 << 30, 2 << 30, 3 << 30, 4 << 30, 5 << 30, 6 << 30, 8 << 30, 12 << 30):
+        tables = _held(lambda: _paper(fam, 0, pool)) - without
+        assert tables <= max(64 * MIB, pool // 8) + GRAIN, (pool / MIB, tables / MIB)
 
 
 def _run(s):
