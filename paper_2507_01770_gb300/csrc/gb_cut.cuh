@@ -204,7 +204,7 @@ __device__ __forceinline__ void cut_groups(const GbProg& P, const GbPool& pool, 
 enum { CUT_ALL = 0, CUT_LIST = 1, CUT_GROUPS = 2 };
 template <typename E, typename M>
 __device__ __forceinline__ void cut_children(const GbProg& P, const GbParents& par, const GbChildren& ch,
-                                             const GbSplit& sp, int nk, int mode, GbState* st, unsigned* q, const E& e,
+                                             const GbSplit& sp, int nk, int mode, GbState* st, unsigned long long* q, const E& e,
                                              const M& mono) {
     const double gub_prev = gb_key_value(st->gub_key);
     const long long lim = mode == CUT_GROUPS ? st->n32 << GB_CUT_LOG2 : mode == CUT_LIST ? st->n32 : st->nch;
@@ -213,9 +213,9 @@ __device__ __forceinline__ void cut_children(const GbProg& P, const GbParents& p
     int qn = 0;   // warp-uniform queue length
     int ops = 0;
     unsigned long long key = ~0ull, nvalid = 0;
-    constexpr unsigned RULED_OUT = 0x80000000u;   // (fewer than 2^31 children)
-    auto test = [&](unsigned e0) {
-        const unsigned ci = e0 & ~RULED_OUT;
+    constexpr unsigned long long RULED_OUT = 1ull << 63;   // (a generation may hold up to 2^32 children)
+    auto test = [&](unsigned long long e0) {
+        const long long ci = (long long)(e0 & ~RULED_OUT);
         const ChildCtx c = child_ctx(par, ci, sp);
         const int spi = P.sp_of_cyc[c.info.x];
         key = min(key, e.samples(c, spi, 1, nk, ~0ull, ops));
@@ -225,7 +225,7 @@ __device__ __forceinline__ void cut_children(const GbProg& P, const GbParents& p
         const long long idx = base + lane;
         bool need = false, valid = false;
         long long ci = 0;
-        unsigned ruled = 0;
+        unsigned long long ruled = 0;
         if (mode == CUT_GROUPS) {   // (the warp's children are one group)
             const long long c0 = (long long)ch.list32[base >> GB_CUT_LOG2] << GB_CUT_LOG2;
             const double b = ch.flo[c0];
@@ -251,7 +251,7 @@ __device__ __forceinline__ void cut_children(const GbProg& P, const GbParents& p
         }
         nvalid += __popc(__ballot_sync(0xffffffffu, valid));
         const unsigned bal = __ballot_sync(0xffffffffu, need);
-        if (need) q[qn + __popc(bal & ((1u << lane) - 1u))] = (unsigned)ci | ruled;
+        if (need) q[qn + __popc(bal & ((1u << lane) - 1u))] = (unsigned long long)ci | ruled;
         qn += __popc(bal);
         __syncwarp();
         if (qn >= 32) {

@@ -528,7 +528,7 @@ template <bool PR>
 __global__ void __launch_bounds__(128) k_pp_eval(GbProg P, GbPool pool, GbParents par, GbPaper T, GbChildren ch,
                                                  GbSplit sp, int mode, GbState* st) {
     if (st->halt) return;
-    __shared__ unsigned s_queue[4][64];
+    __shared__ unsigned long long s_queue[4][64];
     cut_children(P, par, ch, sp, T.nk, mode, st, s_queue[threadIdx.x >> 5], PaperEval<PR>{P, T},
                  [&](const ChildCtx& c, int spi, int& ops) { return paper_mono<PR>(P, pool, par, T, c, sp, spi, ops); });
 }
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(128) k_pp_eval(GbProg P, GbPool pool, GbParent
 __global__ void __launch_bounds__(128) k_pp_dec(GbProg P, GbPool pool, GbParents par, GbPaper T, GbDec D, GbChildren ch,
                                                 GbSplit sp, int mode, GbState* st) {
     if (st->halt) return;
-    __shared__ unsigned s_queue[4][64];
+    __shared__ unsigned long long s_queue[4][64];
     cut_children(P, par, ch, sp, T.nk, mode, st, s_queue[threadIdx.x >> 5], DecEval<5>{P, D},
                  [&](const ChildCtx& c, int spi, int& ops) { return paper_mono<false>(P, pool, par, T, c, sp, spi, ops); });
 }

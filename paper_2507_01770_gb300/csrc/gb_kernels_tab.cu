@@ -1311,7 +1311,7 @@ __global__ void __launch_bounds__(128) k_eval64_dec(GbProg P, GbPool pool, GbPar
     gb_grid_trigger();
     gb_grid_wait();
     if (st->halt) return;
-    __shared__ unsigned s_queue[4][64];
+    __shared__ unsigned long long s_queue[4][64];
     cut_children(P, par, ch, sp, D.nk, mode, st, s_queue[threadIdx.x >> 5], DecEval<1>{P, D},
                  [&](const ChildCtx& c, int spi, int& ops) {
         const GbSplitPos SP = P.sps[spi];
