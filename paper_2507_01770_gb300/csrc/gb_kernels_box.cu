@@ -305,6 +305,9 @@ __global__ void __launch_bounds__(C::THREADS) k_box(GbProg P, const GbBoxTile* _
 // Shared memory a block may take (of the 227 KB): one block per SM (the box
 // evaluation), two (the children).
 constexpr size_t BOX_SMEM = 200 * 1024, CHILD_SMEM = 100 * 1024;
+// Dynamic shared memory a launch gets without asking: 48 KB less the kernel's
+// static arrays (k_child_box: 144 bytes).
+constexpr size_t FREE_SMEM = 47 * 1024;
 
 // Lets kernel K take `cap` bytes of dynamic shared memory.  The limit belongs
 // to the function and the device, not to a launch: set to a call's own size, it
@@ -572,7 +575,7 @@ template <typename C, typename T>
 cudaError_t launch_box(const GbProg& P, int list, const double* lo, const double* hi, long long nbox, int blk,
                        double* F, double* Fmid, double* G, int* mono, cudaStream_t s) {
     const size_t smem = box_smem_block<C, typename Prec<T>::I>(P);
-    if (smem > 48 * 1024) {
+    if (smem > FREE_SMEM) {
         const cudaError_t e = allow_smem<k_box<C, T>>(BOX_SMEM);
         if (e != cudaSuccess) return e;
     }
@@ -616,7 +619,7 @@ template <typename C>
 cudaError_t launch_child_box(const GbProg& P, const GbPool& pool, const GbParents& par, const GbChildren& ch,
                              long long Cmax, const GbSplit& sp, GbState* st, const GbGenConst& G, cudaStream_t s) {
     const size_t smem = box_smem_block<C, iv64>(P);
-    if (smem > 48 * 1024) {
+    if (smem > FREE_SMEM) {
         const cudaError_t e = allow_smem<k_child_box<C>>(CHILD_SMEM);
         if (e != cudaSuccess) return e;
     }

@@ -51,6 +51,27 @@ def test_small_fan_outs(fam, n, B, d, K, gens, sync):
     assert g.trace["children"].max() == K << d
 
 
+@pytest.mark.parametrize("groups", [56, 57, 58])
+def test_shared_memory_around_what_needs_no_asking(groups):
+    # 8 threads a child, a kernel of groups * 512 + nodes * 32 bytes and 20 KB more: every step of
+    # 32 bytes around the 48 KB that a launch gets, the kernel's own arrays included
+    n = 8 * groups
+    for nodes in range(17):
+        g = Dag()
+        t = g.sqr(g.ivar(0))
+        for _ in range(nodes):
+            t = g.neg(t)
+        if nodes % 2:
+            t = g.neg(t)
+        root = g.isum(t, 0, n, 1)
+        p = Problem("squares", n, g.nodes(), root, g.tables, np.full(n, -1.0), np.full(n, 2.0), 1e-6, 8,
+                    np.zeros(n), 0)
+        s = gb.Solver(p, block=8, split_m=2, split_d=3, max_children=8, max_generations=3, pool_bytes=1 << 26)
+        r = s.solve(raise_on_error=False)
+        s.close()
+        assert r.status == gb.GB_E_LIMIT and r.generations == 3, (groups, nodes, r.status, gb.gb_last_error())
+
+
 @pytest.mark.parametrize("sync", [0, 3])
 @pytest.mark.parametrize("pool_mode", [1, 2])
 @pytest.mark.parametrize("fam,mode,K,extra", [
