@@ -324,10 +324,13 @@ template <auto K> cudaError_t allow_smem(size_t cap) {
     return e;
 }
 
-// Threads per box.  Small objectives (no sum over 16 terms): the next power
-// of two, several boxes per warp.  Else a warp per box once the boxes give
-// every SM 16 warps; with fewer boxes 128 and then 512 threads, so that a
-// handful of boxes still fills the chip.  The tiles must hold every group.
+// Threads per box.  No sum of two terms: one (nothing runs side by side but F
+// and the midpoint, and the staging costs more than that saves: up to 3000
+// boxes of objectives without a sum, 73-80 us a call here, 64-68 by one thread
+// a box).  Small objectives (no sum over 16 terms): the next power of two,
+// several boxes per warp.  Else a warp per box once the boxes give every SM 16
+// warps; with fewer boxes 128 and then 512 threads, so that a handful of boxes
+// still fills the chip.  The tiles must hold every group.
 struct BoxPick { int cfg, list; };
 template <typename C, typename I> bool fits_smem(const GbProg& P) { return box_smem_block<C, I>(P) <= BOX_SMEM; }
 
@@ -340,8 +343,8 @@ typedef BoxCfg<512, 512, 128> Cfg512;
 
 BoxPick box_pick(const GbProg& P, long long nbox) {
     const BoxPick none{-1, 0};
-    if (P.any_prod || nbox > (1LL << 30)) return none;
-    const bool l0 = P.n_box_tiles[0] > 0 || P.max_terms == 0, l1 = P.n_box_tiles[1] > 0 || P.max_terms == 0;
+    if (P.any_prod || P.max_terms <= 1 || nbox > (1LL << 30)) return none;
+    const bool l0 = P.n_box_tiles[0] > 0, l1 = P.n_box_tiles[1] > 0;
     if (l0 && P.max_terms <= 4 && fits_smem<Cfg4, iv64>(P)) return BoxPick{0, 0};
     if (l0 && P.max_terms <= 8 && fits_smem<Cfg8, iv64>(P)) return BoxPick{1, 0};
     if (l0 && P.max_terms <= 16 && fits_smem<Cfg16, iv64>(P)) return BoxPick{2, 0};

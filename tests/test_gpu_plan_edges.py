@@ -93,3 +93,30 @@ def test_groups(fam, mode, K, extra, pool_mode, sync):
     assert np.array_equal(a.box_flo, b.box_flo)
     assert (a.box_evals_fp64, a.mid_evals) == (b.box_evals_fp64, b.mid_evals)
     assert a.ops64 < b.ops64   # (the work counted in the kernels: the tables were used)
+
+
+@pytest.mark.parametrize("terms", [0, 1, 2])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_boxes_of_objectives_with_hardly_a_term(terms, fp32):
+    # no sum, sums of one term (one thread a box) and of two (several)
+    n = 3
+    g = Dag()
+    root = g.mul(g.sqr(g.sub(g.var(0), g.const(0.25))), g.var(2))
+    for off in (0, 1):
+        if terms:
+            t = g.sqr(g.sub(g.ivar(off), g.const(0.5)))
+            root = g.add(root, g.isum(t, 0, terms, 1))
+    p = Problem("few_terms", n, g.nodes(), root, g.tables, np.full(n, -2.0), np.full(n, 3.0), 1e-6, 2, np.zeros(n), 0)
+    s = gb.Solver(p, block=2, pool_bytes=1 << 26)
+    orc = O.Oracle(p, block=2)
+    lo, hi = S.random_boxes(p, 150, seed=3)
+    dlo, dhi = torch.from_numpy(lo).cuda(), torch.from_numpy(hi).cuda()
+    for blk in (0, 1):
+        w = min(2, n - 2 * blk)
+        for noalloc in (False, True):
+            F, Fm, G, mono = (t.cpu().numpy() for t in gb.gb_eval_boxes(s.h, dlo, dhi, blk, fp32, noalloc=noalloc))
+            for k in range(0, 150, 7):
+                f, fm, gr, m = orc.eval_box(lo[k], hi[k], blk=blk, f32=fp32)
+                assert np.array_equal(F[k], f) and np.array_equal(Fm[k], fm)
+                assert np.array_equal(G[k, :w], np.asarray(gr)[:w]) and mono[k] == m
+    s.close()
