@@ -613,7 +613,9 @@ def roofline(m, w, opts, sm_mhz, sms, gb, local):
             "unit": "TFLOP/s", "frac": (achieved / peak64) if achieved else None, "traffic": w.get("traffic"),
             "kernel": kname,
             "ops": "directed-rounding FP64 operations plus FP32 operations x 2/128, executed by the per-parent "
-                   "table kernels and the child kernels (counted in the kernels)",
+                   "table kernels and the child kernels (counted in the kernels; with child groups the count varies "
+                   "a little from run to run)",
+            "ops_per_eval_are": "executed operations per child counted in box_evals (see evals_are)",
             "ops64_per_eval": o64 / max(1, evals), "ops32_per_eval": o32 / max(1, evals),
             "static_ops_per_eval": m["info"]["ops_eval"] + m["info"]["ops_mid"],
             "peak_source": f"{FP64_OPS_PER_SM_CLK:.0f} FP64 ops/SM/clk x {sms} SMs (device attribute) x "
@@ -631,7 +633,12 @@ def _summary(m, w, opts, sm_mhz, sms, gb, local):
     ok = all(r.status == 0 and r.fmin_lo <= fstar <= r.fmin_hi and
              (w.get("paper") or r.fmin_hi - r.fmin_lo <= m["p"].tol_f) for r in res)
     last = res[-1]
+    groups = not w["fp32"] and opts["split_m"] ** opts["split_d"] >= 1 << 10 and (
+        bool(w.get("paper")) or opts["max_children"] >= 1 << 16)
     return {"workload": w["name"], "box_evals_per_s": evals / (dev_ms * 1e-3), "ms_per_solve": dev_ms / len(res),
+            "evals_are": ("children decided: one by one, or with their group of 32 from an enclosure of all of them; "
+                          "samples taken, or shown not to lower the incumbent" if groups else
+                          "children evaluated, samples taken"),
             "solves_per_s": len(res) / (dev_ms * 1e-3), "solves_timed": len(res),
             "generations_per_solve": last.generations, "ms_per_generation": dev_ms / len(res) / max(1, last.generations),
             "kernel_launches_per_generation": last.kernel_launches / max(1, last.generations),

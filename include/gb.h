@@ -54,8 +54,8 @@ typedef enum gb_status {
  * index).  ISUM(a = template root, b = first, c = end, d = step) is the sum
  * over i in {b, b+d, ...} < c of the template sub-DAG rooted at a, and
  * IPROD (same fields) the product (the Griewank, Styblinski and Zabinsky
- * functions of the paper's SI Appendix A; IPROD problems run on the
- * interpreter kernels, eval_mode 0 or 1).  In a template
+ * functions of the paper's SI Appendix A; IPROD problems need eval_mode 0 or
+ * 1 and have tables in paper mode only).  In a template
  * IDX_VAR(b = offset) stands for x[i+offset] and IDX_COEF(a = table,
  * b = offset) for coef_tables[a][i+offset].  CONST(v) is the exact double v;
  * PI and EULER are the constants pi and e, enclosed by adjacent doubles;
@@ -98,10 +98,11 @@ typedef struct gb_options {
     size_t pool_bytes;        /* device memory budget for the pool (0: 16 GiB) */
     int32_t device;           /* CUDA device ordinal */
     int32_t eval_mode;        /* child evaluation: 0 auto (term tables when m^d >= 16 and they fit),
-                                 1 bytecode interpreter, 2 term tables when they fit (one child per warp
-                                 when a generation has fewer than 2^16 children, else per thread),
-                                 3 / 4 term tables with one child per thread / per warp; results are
-                                 identical */
+                                 1 bytecode interpreter, 2 term tables when they fit, 3 / 4 their forms for
+                                 large / small generations whatever the size (2^16 children and more: one
+                                 child per thread, from 2^10 children a parent on cut off in groups of 32
+                                 first where the objective allows it; fewer: 32 children to a block, or one
+                                 per warp below 32 children a parent); results are identical */
     int32_t gens_per_sync;    /* <= 1: the host reads the state after every generation (per-kernel timing);
                                  G > 1: generations run as replays of a captured CUDA graph, G between
                                  state reads (the search is the same) */
@@ -174,7 +175,9 @@ typedef struct gb_result {
     int64_t eval64_launches;
     int64_t eval32_launches;
     int64_t kernel_launches;  /* kernels the library launched for this solve */
-    int64_t ops64;            /* directed-rounding FP64 operations executed by the evaluation (tables, children) */
+    int64_t ops64;            /* directed-rounding FP64 operations executed by the evaluation (tables, children); with
+                                 child groups it varies a little from run to run: which of them the incumbent
+                                 lets skip depends on when it falls */
     int64_t ops32;            /* directed-rounding FP32 operations executed by the evaluation (tables, children) */
     double queue_ms;          /* serving: submit -> admission (host clock); 0 for gb_solve */
     double latency_ms;        /* serving: submit -> result ready (host clock); 0 for gb_solve */
@@ -321,7 +324,8 @@ gb_status gb_eval_boxes(gb_problem* prob, const double* d_lo, const double* d_hi
  * latency-critical thread that must not wait on the device allocator).
  * Same arguments and results as gb_eval_boxes.  The paper has no counterpart
  * of this entry point.
- *  - The FP32 copy of the boxes that fp32 = 1 needs is kept in a fixed array
+ *  - The FP32 copy of the boxes that fp32 = 1 may need (objectives that one
+ *    thread a box evaluates) is kept in a fixed array
  *    inside the library instead of a per-call buffer: at most 2^20
  *    coordinates (nbox * n <= 1048576) per FP32 call; larger FP32 calls
  *    return GB_E_INVALID with a message.  fp32 = 0 needs no scratch and has
@@ -360,8 +364,8 @@ gb_status gb_measure_peak(int32_t device, int32_t which, double* ops_per_s, doub
 /* Times complete solves of the problem (arguments as in gb_create_problem)
  * under candidate settings of the bisection fan-out (split_m in {2, 4},
  * split_d in {B, ceil(B/2)} with m^d <= 2^20), the parents per generation
- * (max_children = 1 or 4 times m^d) and the child-kernel shape (eval_mode 3:
- * one child per thread, 4: one child per warp, when term tables are used),
+ * (max_children = 1 or 4 times m^d) and the child-kernel shape (eval_mode 3
+ * or 4, when term tables are used),
  * starting from *base (NULL: defaults; its block, tolerances, precision,
  * pool and device are kept), and writes the fastest setting to *best and its
  * solve time (ms, host clock, second of two solves) to *best_ms.  Every

@@ -31,8 +31,10 @@
 // paper mode, Levy n = 30 (27 generations) 34.3 -> 8.25 ms (18.6
 // before a group is sampled first, its samples taken five at a time and the
 // test's fixed adjoints used first).  From a fan-out of
-// 2^10 on: the hull tables and the groups take two launches (8 + 10 us at
-// least) and a smaller fan-out is one latency chain either way.
+// 2^10 on: the hull tables and the groups take two launches (8.0 and 22.2 us
+// for the chain) and a smaller fan-out is one latency chain either way.
+// Not taken: after an FP32 pass (its list says which children are left), and
+// outside paper mode for outer expressions that are not a plain sum of sums.
 #pragma once
 #include "gb_child.cuh"
 

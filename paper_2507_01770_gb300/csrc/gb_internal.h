@@ -125,6 +125,11 @@ struct GbUop {
     int32_t pad3;
     double lo, hi;     // constant operand
 };  // 32 bytes
+// Stack entries of an endpoint program, kept in registers (two for each entry
+// and kind: 40 in the walk that takes five samples at a time).  An objective
+// that needs more at one split position takes no program at all and
+// k_eval64_tab walks its children: the chain needs 5 with blocks of 16, 24 and
+// 32 coordinates, the mixed family also with 15 (4-way also 17 to 20).
 #define GB_DEC_DEPTH 4
 // Paper mode, per (split position, reduction): its dirty terms [t_lo, t_hi)
 // are dterms d0 ..., the other terms of a product, in order, dterms x0 ...

@@ -14,7 +14,10 @@
 // calls); few boxes, the dependent chain of one term.  One thread per box
 // left both idle; measured on GB300, one call: 301 boxes of the mixed family,
 // n = 10,001, FP32: 87.6 ms with one thread per box, 0.71 ms here; 8192 boxes
-// of the chain, n = 100, FP64: 0.92 and 0.28 ms; one box, n = 2: 64 and 45 us.
+// of the chain, n = 100, FP64: 0.95 and 0.24 ms; one box, n = 2: 59 and 45 us.
+// One thread a box (k_eval_boxes) is left for products, objectives without a
+// sum of two terms, groups of more than 512 terms and group sums beyond the
+// shared memory (about 5,900 groups: chain of n = 29,500 with blocks of 10).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -19,12 +19,14 @@
 // Bound: the FP64 pipe (one addition per table entry and endpoint), where
 // most children are cut off in groups (gb_cut.cuh) the latency of the rest.
 // Measured on GB300, whole solves with 4^10 children a generation: Levy n = 30,
-// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 8.25
-// with the groups; Griewank n = 16, 10 generations, 1507, 34.6 and 19.5 ms
+// 27 generations, 1172 ms with the interpreter, 34.3 ms from the tables, 8.1
+// with the groups; Griewank n = 16, 10 generations, 1509, 34.6 and 19.6 ms
 // (its survivors' caches, too, come from the tables: k_materialize 73 -> 0.2 ms
-// a generation; two thirds of a million of its children survive, and what
-// bounds those is the product's first-order test, which takes the templates'
-// forward values and library factors from the term rows: 32.5 ms before).
+// a generation; 0.87 million of its children survive, and what bounds those is
+// the product's first-order test, which takes the templates' forward values and
+// library factors from the term rows: 32.5 ms before).  The domain decides how
+// many survive: over four of them, its bounds moved by up to 2 % of its width,
+// 0.52 .. 1.34 million, 1021 .. 2154 ms and 16.0 .. 23.6.
 #include <cuda_runtime.h>
 
 #include <algorithm>

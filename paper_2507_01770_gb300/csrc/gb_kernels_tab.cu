@@ -24,8 +24,9 @@ using namespace gb;
 #define GB_TAB_MINB 7
 #endif
 // The same for the register-resident single-sum kernel (80 registers, no
-// local memory to speak of; measured on the n = 100 chain, 4^10 children a
-// launch: 27.1 ms per solve at 6 blocks, 27.7 at 5 and at 7).
+// local memory to speak of; measured while it took the n = 100 chain at B = 10,
+// 4^10 children a launch, which the endpoint programs do now: 27.1 ms per solve
+// at 6 blocks, 27.7 at 5 and at 7).
 #ifndef GB_TAB_MINB_REG
 #define GB_TAB_MINB_REG 6
 #endif

@@ -311,10 +311,10 @@ int gb_sm_count();
 // `pdl` can overlap its launch and block scheduling with the end of its
 // predecessor in the stream.  A kernel launched without `pdl` waits as usual
 // and the two calls return at once.  The overlap is off unless the
-// environment sets GB_PDL=1: measured on GB300 it loses slightly (a C3
-// generation 80.8 us with it, 79.1 us without; served solves 50.7/s with
-// it, 53.4/s without), as the early blocks hold SM resources that the
-// kernels of the other stream, or of other requests, could use.
+// environment sets GB_PDL=1: measured on GB300 it loses (a solve of the
+// n = 10^4 mixed family, whose children run beside the partition, 1519 ms with
+// it, 1263 without), as the early blocks hold SM resources that the kernels
+// of the other stream, or of other requests, could use.
 // gb_pdl_thread(false) keeps it off for the calling thread's launches and
 // graph captures whatever the environment (the serving worker).
 bool gb_pdl_enabled();
