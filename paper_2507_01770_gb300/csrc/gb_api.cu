@@ -558,7 +558,6 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
         (e = alloc(&p->ch.surv, C, A)))
         return bad(e, "allocate child buffers");
     // per-parent term tables
-    bool want_unit = false, want_dec = false;
     if (opt.eval_mode != 1) {
         const bool want = opt.eval_mode >= 2 || p->fan >= 16;
         if (p->hp.tab_ok && want) {
@@ -575,9 +574,20 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
             GbContrib* d_cb;
             GbJkD* d_jkd;
             GbSeg* d_segs;
-            want_unit = unit;
-            want_dec = dec;
-            if (!unit && warp && d * mshift >= 5 && P.n_sum > 0) p->tabs.unit = 2;
+            uint16_t* d_mvf;
+            GbUop* d_u;
+            if (unit) {
+                if ((e = upload(&d_mvf, Hh.mvf.data(), Hh.mvf.size(), A))) return bad(e, "upload table layouts");
+                P.mvf = d_mvf;
+                p->tabs.unit = 1;
+            } else if (warp && d * mshift >= 5 && P.n_sum > 0) {
+                p->tabs.unit = 2;
+            }
+            if (dec) {
+                if ((e = upload(&d_u, Hh.uops.data(), Hh.uops.size(), A))) return bad(e, "upload table layouts");
+                P.uops = d_u;
+                p->tabs.dec = 1;
+            }
             if ((e = upload(&d_jkd, Hh.jkd.data(), Hh.jkd.size(), A)) ||
                 (e = upload(&d_segs, Hh.segs.data(), Hh.segs.size(), A)) ||
                 (e = upload(&d_spc, Hh.sp_of_cyc.data(), Hh.sp_of_cyc.size(), A)) ||
@@ -682,29 +692,20 @@ gb_status gb_create_problem(const gb_node* dag, int32_t n_nodes, int32_t root, c
     auto optional = [&](size_t bytes, auto&& take) {
         size_t left = 0, total = 0;
         const size_t n0 = p->owned.size(), b0 = p->device_bytes;
-        if (cudaMemGetInfo(&left, &total) == cudaSuccess && bytes <= left / 2 && take() == cudaSuccess) return true;
+        // (a small set is tried without asking: the question takes 50 us, of 700 for a whole small problem)
+        const bool ask = bytes > (1 << 20);
+        if ((!ask || (cudaMemGetInfo(&left, &total) == cudaSuccess && bytes <= left / 2)) && take() == cudaSuccess)
+            return true;
         cudaGetLastError();
         for (; p->owned.size() > n0; p->owned.pop_back()) cudaFreeAsync(p->owned.back(), p->stream);
         p->device_bytes = b0;
         return false;
     };
     auto bytes_of = [](const auto& v) { return v.size() * sizeof(v[0]); };
-    if (want_unit) {
-        uint16_t* d_mvf;
-        if (optional(bytes_of(H.mvf), [&] { return upload(&d_mvf, H.mvf.data(), H.mvf.size(), A); })) {
-            P.mvf = d_mvf;
-            p->tabs.unit = 1;
-        }
-    }
-    if (want_dec) {
-        GbUop* d_u;
+    if (p->tabs.dec && tab_groups) {
         GbTabs& T = p->tabs;
-        if (optional(bytes_of(H.uops), [&] { return upload(&d_u, H.uops.data(), H.uops.size(), A); })) {
-            P.uops = d_u;
-            T.dec = 1;
-        }
         const size_t rows = 2 * K * (size_t)T.max_rows, segs = 2 * K * (size_t)T.max_srows, parts = K * (size_t)T.max_drows;
-        if (T.dec && tab_groups && !optional((rows + segs + parts) * sizeof(double2), [&] {
+        if (!optional((rows + segs + parts) * sizeof(double2), [&] {
                 (e = alloc(&T.cut.tv, rows, A)) || (e = alloc(&T.cut.ts, segs, A)) || (e = alloc(&T.cut.td, parts, A));
                 return e;
             }))
