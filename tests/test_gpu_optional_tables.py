@@ -17,7 +17,7 @@ if not torch.cuda.is_available():
 import paper_2507_01770_gb300 as gb  # noqa: E402
 
 MIB = 1 << 20
-GRAIN = 96 * MIB   # what the driver's pool rounds a problem's memory up by
+GRAIN = 96 * MIB   # what CUDA's memory pool rounds a problem's memory up by
 
 
 def _free():
